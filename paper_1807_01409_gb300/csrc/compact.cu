@@ -1,24 +1,29 @@
-// Single-pass row compaction over tuple sets, and a device-wide exclusive scan.
+// Row selection over tuple sets, and a device-wide exclusive scan.
 //
-// One kernel template serves the operators that keep a subset of rows in
-// their original order and write k output columns:
+// Three kernels serve the operators that keep a subset of rows in their
+// original order and write k output columns:
 //   * bind     -- from triple indices, the terms at a pattern's variable slots,
 //                 dropping rows whose repeated variable disagrees; the FILTER
 //                 predicates of the subquery are applied in the same pass
 //                 (Section 4.3: the filter is applied while the matched triples
 //                 are extracted into the subquery's vector);
 //   * filter   -- a predicate on one column of a set;
+//   * member   -- rows whose key is in another set's key column (the join with
+//                 a set of keys only);
 //   * unique   -- after a sort, a row is kept when it differs from its
 //                 predecessor in sorted order (DISTINCT, Section 4.3), on
 //                 column rows or on packed row keys;
 //   * semijoin -- the entailment's keyed store pass (Section 5): a store triple
 //                 is kept when its term at the join position is one of the
 //                 first search's distinct terms (a hash probe).
-// A CTA owns 2048 consecutive rows (256 threads x 8, striped so each warp
-// instruction touches 32 consecutive rows); ranks come from ballots, the
-// tile offset from the decoupled look-back (lookback.cuh).
+// Short inputs: k_compact, one launch (ranks from ballots, tile offsets from
+// the decoupled look-back of lookback.cuh).  Long inputs: k_sel_mark, which
+// tests every row and writes one keep bit per row, and k_sel_expand, which
+// reads the kept rows' values and writes them in order; no CTA of either waits
+// for another.
 
 #include <algorithm>
+#include <type_traits>
 
 #include "lookback.cuh"
 #include "ops.cuh"
@@ -32,113 +37,178 @@ constexpr int CP_WARPS = CP_THREADS / 32;
 constexpr int CP_ITEMS = 8;
 constexpr int CP_TILE = CP_THREADS * CP_ITEMS;
 
-__device__ __forceinline__ bool pred_ok(const Pred &p, int32_t x) {
-    if (x == 0) return false;  // unbound never passes
-    switch (p.op) {
-        case TID_CMP_EQ: return x == p.a;
-        case TID_CMP_NE: return x != p.a;
-        case TID_CMP_LT: return x < p.a;
-        case TID_CMP_LE: return x <= p.a;
-        case TID_CMP_GT: return x > p.a;
-        case TID_CMP_GE: return x >= p.a;
-        case TID_CMP_RANGE: return p.a <= x && x <= p.b;
-        default: return false;
-    }
+__device__ __forceinline__ bool pred_ok(const Pred &p, int32_t x) {  // an unbound value never passes
+    return x != 0 && (((uint32_t)x - (uint32_t)p.lo <= p.span) != (p.neg != 0));
+}
+
+// Membership of a term in a set of terms held as a bit per term of [lo, lo + w)
+// (sort order); 0 (unbound) is never a member.
+__device__ __forceinline__ bool is_member(const Members &m, int32_t x) {
+    const uint32_t d = ((uint32_t)x ^ 0x80000000u) - m.lo;
+    return d < m.w && ((__ldg(m.bits + (d >> 5)) >> (d & 31)) & 1u);
 }
 
 // ---- row sources -----------------------------------------------------------
 
 // A row source says, for a row r < n, whether it is kept (keep: reads only
-// what the test needs) and gives its k output values (values: v[0..k)).
-// Column loops run to TID_MAX_COLS with a guard so v[] stays in registers.
+// what the test needs) and gives its K output values (values<K>: v[0..K)); at
+// most MAX_K columns.  keep_step tests a lane's 32 rows of a full step (rows
+// r0 + 128 g + (0..3), r0 a multiple of 4): bit e of m[g] is row r0 + 128 g + e.
+// It loads 16 bytes at a time and issues a group of loads before using any.
+__device__ __forceinline__ int4 ld4(const int32_t *p) { return __ldg(reinterpret_cast<const int4 *>(p)); }
 
-__device__ __forceinline__ bool preds_ok(const Pred *preds, int n_preds, const int32_t *v) {
-    bool ok = true;
-#pragma unroll
-    for (int q = 0; q < MAX_PREDS; ++q) {
-        if (q < n_preds) {
-            int32_t x = v[0];
-#pragma unroll
-            for (int c = 1; c < TID_MAX_COLS; ++c)
-                if (preds[q].col == c) x = v[c];
-            ok = ok && pred_ok(preds[q], x);
-        }
-    }
-    return ok;
+template <class F>
+__device__ __forceinline__ unsigned test4(int4 x, F f) {
+    return (unsigned)f(x.x) | ((unsigned)f(x.y) << 1) | ((unsigned)f(x.z) << 2) | ((unsigned)f(x.w) << 3);
 }
 
 struct BindRow {  // triple index -> variable values
+    static constexpr int MAX_K = 3;
     const int32_t *S, *P, *O;
     const int32_t *idx;
     int k;
     int need;                   // slots (bit 0 s, 1 p, 2 o) that carry a variable
+    int test;                   // slots that a test reads
     int8_t src[TID_MAX_COLS];   // slot (0,1,2) giving output column c
     int8_t eq_a[3], eq_b[3];    // pairs of slots that must be equal
     int n_eq;
-    Pred preds[MAX_PREDS];
+    Pred preds[MAX_PREDS];      // col: a slot
     int n_preds;
-    __device__ __forceinline__ void slots(int64_t r, int32_t &t0, int32_t &t1, int32_t &t2) const {
-        const int64_t t = idx[r];
-        // only the variable slots are read: a bound slot holds the key itself
-        t0 = (need & 1) ? S[t] : 0;
-        t1 = (need & 2) ? P[t] : 0;
-        t2 = (need & 4) ? O[t] : 0;
-    }
-    __device__ __forceinline__ void out_of(int32_t t0, int32_t t1, int32_t t2, int32_t *v) const {
-#pragma unroll
-        for (int c = 0; c < TID_MAX_COLS; ++c)
-            if (c < k) v[c] = src[c] == 0 ? t0 : (src[c] == 1 ? t1 : t2);
-    }
-    __device__ __forceinline__ bool keep(int64_t r) const {
-        if (n_eq == 0 && n_preds == 0) return true;
-        int32_t t0, t1, t2, v[TID_MAX_COLS];
-        slots(r, t0, t1, t2);
+    int32_t *stash;             // row r's value of the one tested slot, written by keep_step (or null)
+    Members mem[MAX_MEMBERS];   // terms a slot's value must be among
+    int8_t mem_slot[MAX_MEMBERS];
+    int n_mem;
+    __device__ __forceinline__ bool ok(int32_t t0, int32_t t1, int32_t t2) const {
+        auto at = [&](int slot) { return slot == 0 ? t0 : (slot == 1 ? t1 : t2); };
         bool ok = true;
 #pragma unroll
-        for (int e = 0; e < 3; ++e) {
-            if (e < n_eq) {
-                const int32_t a = eq_a[e] == 0 ? t0 : (eq_a[e] == 1 ? t1 : t2);
-                const int32_t b = eq_b[e] == 0 ? t0 : (eq_b[e] == 1 ? t1 : t2);
-                ok = ok && a == b;
+        for (int e = 0; e < 3; ++e)
+            if (e < n_eq) ok = ok && at(eq_a[e]) == at(eq_b[e]);
+#pragma unroll
+        for (int q = 0; q < MAX_PREDS; ++q)
+            if (q < n_preds) ok = ok && pred_ok(preds[q], at(preds[q].col));
+#pragma unroll
+        for (int q = 0; q < MAX_MEMBERS; ++q)
+            if (q < n_mem) ok = ok && is_member(mem[q], at(mem_slot[q]));
+        return ok;
+    }
+    __device__ __forceinline__ bool keep(int64_t r) const {
+        const int64_t t = idx[r];
+        if (stash) stash[r] = (test & 1) ? S[t] : ((test & 2) ? P[t] : O[t]);
+        return keep_at(t);
+    }
+    __device__ __forceinline__ bool keep_at(int64_t t) const {
+        return ok((test & 1) ? S[t] : 0, (test & 2) ? P[t] : 0, (test & 4) ? O[t] : 0);
+    }
+    __device__ __forceinline__ void keep_step(uint32_t r0, unsigned *m) const {
+#pragma unroll 1
+        for (int h = 0; h < 8; h += 4) {  // 16 rows at a time: their indices, then their gathers, in flight
+            int4 t[4];
+#pragma unroll
+            for (int g = 0; g < 4; ++g) t[g] = ld4(idx + r0 + (h + g) * 128);
+            unsigned k4[4];
+            if (n_eq == 0 && (test & (test - 1)) == 0) {  // one slot is tested
+                const int32_t *col = test == 1 ? S : (test == 2 ? P : O);
+                int4 x[4];
+#pragma unroll
+                for (int g = 0; g < 4; ++g) x[g] = make_int4(col[t[g].x], col[t[g].y], col[t[g].z], col[t[g].w]);
+#pragma unroll
+                for (int g = 0; g < 4; ++g) {
+                    k4[g] = test4(x[g], [&](int32_t v) { return ok(v, v, v); });
+                    if (stash) *reinterpret_cast<int4 *>(stash + r0 + (h + g) * 128) = x[g];
+                }
+            } else {
+#pragma unroll
+                for (int g = 0; g < 4; ++g) k4[g] = test4(t[g], [&](int32_t i) { return keep_at(i); });
+            }
+#pragma unroll
+            for (int g = 0; g < 4; ++g) {
+                if (h == 0) m[g] = k4[g];
+                else m[g + 4] = k4[g];
             }
         }
-        out_of(t0, t1, t2, v);
-        return ok && preds_ok(preds, n_preds, v);
     }
+    template <int K>
     __device__ __forceinline__ void values(int64_t r, int32_t *v) const {
-        int32_t t0, t1, t2;
-        slots(r, t0, t1, t2);
-        out_of(t0, t1, t2, v);
+        const int64_t t = idx[r];
+        // only the variable slots are read: a bound slot holds the key itself.
+        // The tested slot of a kept row comes from the stash: at one kept triple
+        // in sixteen its column's gather would read nearly every line again.
+        const int skip = stash ? test : 0;
+        const int32_t x = skip ? stash[r] : 0;
+        const int32_t t0 = (skip & 1) ? x : ((need & 1) ? S[t] : 0), t1 = (skip & 2) ? x : ((need & 2) ? P[t] : 0),
+                      t2 = (skip & 4) ? x : ((need & 4) ? O[t] : 0);
+#pragma unroll
+        for (int c = 0; c < K; ++c)
+            if (c < k) v[c] = src[c] == 0 ? t0 : (src[c] == 1 ? t1 : t2);
     }
 };
 
 struct FilterRow {
+    static constexpr int MAX_K = TID_MAX_COLS;
     const int32_t *col[TID_MAX_COLS];
     int k;
     Pred preds[MAX_PREDS];
     int n_preds;
+    __device__ __forceinline__ const int32_t *column(int c) const {  // constant indices: no local copy of col[]
+        const int32_t *p = col[0];
+#pragma unroll
+        for (int i = 1; i < TID_MAX_COLS; ++i)
+            if (c == i) p = col[i];
+        return p;
+    }
     __device__ __forceinline__ bool keep(int64_t r) const {  // the predicates' columns only
         bool ok = true;
 #pragma unroll
-        for (int q = 0; q < MAX_PREDS; ++q) {
-            if (q < n_preds) {
-                const int32_t *cp = col[0];  // selected with constant indices (no local copy of col[])
-#pragma unroll
-                for (int c = 1; c < TID_MAX_COLS; ++c)
-                    if (preds[q].col == c) cp = col[c];
-                ok = ok && pred_ok(preds[q], cp[r]);
-            }
-        }
+        for (int q = 0; q < MAX_PREDS; ++q)
+            if (q < n_preds) ok = ok && pred_ok(preds[q], column(preds[q].col)[r]);
         return ok;
     }
+    __device__ __forceinline__ void keep_step(uint32_t r0, unsigned *m) const {
+#pragma unroll
+        for (int g = 0; g < 8; ++g) m[g] = 0xFu;
+#pragma unroll 1
+        for (int q = 0; q < n_preds; ++q) {
+            const Pred p = preds[q];
+            const int32_t *cp = column(p.col);
+            int4 x[8];
+#pragma unroll
+            for (int g = 0; g < 8; ++g) x[g] = ld4(cp + r0 + g * 128);
+#pragma unroll
+            for (int g = 0; g < 8; ++g) m[g] &= test4(x[g], [&](int32_t v) { return pred_ok(p, v); });
+        }
+    }
+    template <int K>
     __device__ __forceinline__ void values(int64_t r, int32_t *v) const {
 #pragma unroll
-        for (int c = 0; c < TID_MAX_COLS; ++c)
+        for (int c = 0; c < K; ++c)
+            if (c < k) v[c] = col[c][r];
+    }
+};
+
+struct MemberRow {  // rows of a set whose first column is among the members
+    static constexpr int MAX_K = TID_MAX_COLS;
+    const int32_t *col[TID_MAX_COLS];
+    int k;
+    Members m;
+    __device__ __forceinline__ bool keep(int64_t r) const { return is_member(m, col[0][r]); }
+    __device__ __forceinline__ void keep_step(uint32_t r0, unsigned *k4) const {
+        int4 x[8];
+#pragma unroll
+        for (int g = 0; g < 8; ++g) x[g] = ld4(col[0] + r0 + g * 128);
+#pragma unroll
+        for (int g = 0; g < 8; ++g) k4[g] = test4(x[g], [&](int32_t v) { return is_member(m, v); });
+    }
+    template <int K>
+    __device__ __forceinline__ void values(int64_t r, int32_t *v) const {
+#pragma unroll
+        for (int c = 0; c < K; ++c)
             if (c < k) v[c] = col[c][r];
     }
 };
 
 struct UniqueRow {  // rows in perm order; keep the first of each run of equal rows
+    static constexpr int MAX_K = TID_MAX_COLS;
     const int32_t *col[TID_MAX_COLS];
     const int32_t *perm;  // may be null (rows already in order)
     int k;
@@ -152,16 +222,25 @@ struct UniqueRow {  // rows in perm order; keep the first of each run of equal r
             if (c < k) same = same && col[c][b] == col[c][a];
         return !same;
     }
+    __device__ __forceinline__ void keep_step(uint32_t r0, unsigned *m) const {
+#pragma unroll
+        for (int g = 0; g < 8; ++g) {
+            const uint32_t r = r0 + g * 128;
+            m[g] = test4(make_int4(0, 1, 2, 3), [&](int32_t e) { return keep(r + e); });
+        }
+    }
+    template <int K>
     __device__ __forceinline__ void values(int64_t r, int32_t *v) const {
         const int64_t a = perm ? perm[r] : r;
 #pragma unroll
-        for (int c = 0; c < TID_MAX_COLS; ++c)
+        for (int c = 0; c < K; ++c)
             if (c < k) v[c] = col[c][a];
     }
 };
 
 struct SemiJoinRow {  // store triple r, kept when a slot holds a fixed term and another slot's
                       // term is in a key set (open-addressing table of keys, 0 = empty)
+    static constexpr int MAX_K = 3;
     const int32_t *S, *P, *O;
     int need;                   // slots read (bit 0 s, 1 p, 2 o)
     int fixed_slot;             // -1: none
@@ -169,6 +248,7 @@ struct SemiJoinRow {  // store triple r, kept when a slot holds a fixed term and
     int key_slot;
     const int32_t *table;
     int tbits;                  // log2 of the table size
+    int vec;                    // the columns are 16-byte aligned
     int k;
     int8_t src[TID_MAX_COLS];   // slot giving output column c
     __device__ __forceinline__ const int32_t *column(int slot) const { return slot == 0 ? S : (slot == 1 ? P : O); }
@@ -195,26 +275,66 @@ struct SemiJoinRow {  // store triple r, kept when a slot holds a fixed term and
         }
         return false;
     }
+    __device__ __forceinline__ void keep_step(uint32_t r0, unsigned *m) const {
+        const int32_t *first = first_column();
+        int4 v[8];
+#pragma unroll
+        for (int g = 0; g < 8; ++g) {
+            const int32_t *p = first + r0 + g * 128;
+            v[g] = vec ? ld4(p) : make_int4(p[0], p[1], p[2], p[3]);
+        }
+#pragma unroll
+        for (int g = 0; g < 8; ++g) {
+            const uint32_t r = r0 + g * 128;
+            m[g] = (unsigned)keep_given(r, v[g].x) | ((unsigned)keep_given(r + 1, v[g].y) << 1) |
+                   ((unsigned)keep_given(r + 2, v[g].z) << 2) | ((unsigned)keep_given(r + 3, v[g].w) << 3);
+        }
+    }
+    template <int K>
     __device__ __forceinline__ void values(int64_t r, int32_t *v) const {
         const int32_t t0 = (need & 1) ? S[r] : 0;
         const int32_t t1 = (need & 2) ? P[r] : 0;
         const int32_t t2 = (need & 4) ? O[r] : 0;
 #pragma unroll
-        for (int c = 0; c < TID_MAX_COLS; ++c)
+        for (int c = 0; c < K; ++c)
             if (c < k) v[c] = src[c] == 0 ? t0 : (src[c] == 1 ? t1 : t2);
     }
 };
 
-template <typename K>
+template <typename W>
 struct PackedUniqueRow {  // sorted packed keys; keep the first of each run of equal keys
-    const K *keys;
+    static constexpr int MAX_K = TID_MAX_COLS;
+    const W *keys;
     PackSpec ps;
     int k;
     __device__ __forceinline__ bool keep(int64_t r) const { return r == 0 || keys[r - 1] != keys[r]; }
-    __device__ __forceinline__ void values(int64_t r, int32_t *v) const {
-        const K key = keys[r];
+    __device__ __forceinline__ void keep_step(uint32_t r0, unsigned *m) const {
+        W x[8][4], before[8];
 #pragma unroll
-        for (int c = 0; c < TID_MAX_COLS; ++c) {
+        for (int g = 0; g < 8; ++g) {
+            const uint32_t r = r0 + g * 128;
+            const int4 a = ld4(reinterpret_cast<const int32_t *>(keys + r));
+            if constexpr (sizeof(W) == 4) {
+                x[g][0] = a.x, x[g][1] = a.y, x[g][2] = a.z, x[g][3] = a.w;
+            } else {
+                const int4 b = ld4(reinterpret_cast<const int32_t *>(keys + r + 2));
+                x[g][0] = (W)(uint32_t)a.x | ((W)(uint32_t)a.y << 32);
+                x[g][1] = (W)(uint32_t)a.z | ((W)(uint32_t)a.w << 32);
+                x[g][2] = (W)(uint32_t)b.x | ((W)(uint32_t)b.y << 32);
+                x[g][3] = (W)(uint32_t)b.z | ((W)(uint32_t)b.w << 32);
+            }
+            before[g] = keys[r > 0 ? r - 1 : 0];
+        }
+#pragma unroll
+        for (int g = 0; g < 8; ++g)
+            m[g] = (unsigned)(x[g][0] != before[g] || r0 + g * 128 == 0) | ((unsigned)(x[g][1] != x[g][0]) << 1) |
+                   ((unsigned)(x[g][2] != x[g][1]) << 2) | ((unsigned)(x[g][3] != x[g][2]) << 3);
+    }
+    template <int K>
+    __device__ __forceinline__ void values(int64_t r, int32_t *v) const {
+        const W key = keys[r];
+#pragma unroll
+        for (int c = 0; c < K; ++c) {
             if (c < k) {
                 const uint32_t f = ps.mask[c] ? (uint32_t)((key >> ps.shift[c]) & ps.mask[c]) : 0u;
                 v[c] = (int32_t)((f + ps.min[c]) ^ 0x80000000u);
@@ -224,10 +344,11 @@ struct PackedUniqueRow {  // sorted packed keys; keep the first of each run of e
 };
 
 // bounds (sort order) of the values a thread wrote, merged per warp into mm
+template <int K>
 __device__ __forceinline__ void merge_bounds(uint32_t *mm, int k_out, const uint32_t *lo, const uint32_t *hi) {
     const unsigned lane = threadIdx.x & 31;
 #pragma unroll
-    for (int c = 0; c < TID_MAX_COLS; ++c) {
+    for (int c = 0; c < K; ++c) {
         if (c < k_out) {
             uint32_t a = lo[c], b = hi[c];
 #pragma unroll
@@ -303,7 +424,7 @@ k_compact(Row row, int64_t n, int k_out, OutCols out, int64_t cap, int64_t *__re
         for (int j = 0; j < CP_ITEMS; ++j) {
             if (!((keep >> j) & 1u)) continue;
             int32_t v[TID_MAX_COLS];
-            row.values(base + j * CP_THREADS + threadIdx.x, v);
+            row.template values<TID_MAX_COLS>(base + j * CP_THREADS + threadIdx.x, v);
             const unsigned at = s_off[j * CP_WARPS + warp] + wpre[j];
 #pragma unroll
             for (int c = 0; c < TID_MAX_COLS; ++c)
@@ -343,393 +464,251 @@ k_compact(Row row, int64_t n, int k_out, OutCols out, int64_t cap, int64_t *__re
             }
         }
     }
-    if (mm) merge_bounds(mm, k_out, lo, hi);  // column bounds of the kept rows
+    if (mm) merge_bounds<TID_MAX_COLS>(mm, k_out, lo, hi);  // column bounds of the kept rows
 }
 
-// ---- two-kernel compaction (dense keeps over long inputs) -------------------------
+// ---- mark and expand (long inputs) -------------------------------------------------
 //
-// k_tile_counts: every CTA tests its 2048-row tile and writes the tile's count;
-// the counts are scanned (k_scan_u32); k_tile_write tests the tile again, ranks
-// its kept rows (ballots and a block scan), stages their values in shared memory
-// and writes them at the tile's offset with coalesced stores.  No CTA waits for
-// another; the test columns are read twice.
+// k_sel_mark: a warp tests a step of 1024 rows, writes the step's 32 keep words
+// (bit b of word w: row 1024 j + 32 w + b) and its count, and adds the count to
+// the total of the range of steps that holds it; the last CTA to finish turns
+// the totals into the ranges' first output rows.  k_sel_expand: a CTA owns one
+// range; each of its warps scans the range's step counts and takes every eighth
+// step, so its warps never wait for each other.  A step that keeps many rows is
+// read word by word (lane l the word's row l: coalesced loads and stores); of
+// one that keeps few, the positions go to shared memory first and only the kept
+// rows are read, all lanes at work.  The test's columns are read twice, every
+// other value once, and no CTA waits for another: in the one-launch form a tile
+// waits for its predecessors' counts longer than its own work takes.
+// Bound: memory latency of the expansion's dependent loads (ncu: 57 % of DRAM
+// throughput binding 23.6M triples, long-scoreboard stalls).  Measured on GB300
+// (kernels, before -> after this form): FILTER of 24M two-column rows, half kept,
+// 227 -> 115 us; bind of 23.6M triples of a 200M store with a range FILTER
+// 700 -> 400 us (the tested column is gathered once and stashed); before, per
+// 2048-row tile: a count and a write launch (filter), one look-back launch (bind).
+// A mark phase with 4-byte loads in place of 16-byte ones took 58 us on the
+// filter against 32 us; one large range per resident CTA with block scans took
+// 97 us to expand against 83 us.
 
-template <class Row>
-__global__ void __launch_bounds__(CP_THREADS) k_tile_counts(Row row, int64_t n, uint32_t *__restrict__ counts) {
-    __shared__ unsigned s_w[CP_WARPS];
-    const unsigned lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int64_t base = (int64_t)blockIdx.x * CP_TILE;
-    bool kp[CP_ITEMS];
-#pragma unroll
-    for (int j = 0; j < CP_ITEMS; ++j) {
-        const int64_t r = base + j * CP_THREADS + threadIdx.x;
-        kp[j] = row.keep(r < n ? r : n - 1) && r < n;
-    }
-    unsigned c = 0;
-#pragma unroll
-    for (int j = 0; j < CP_ITEMS; ++j) c += __popc(__ballot_sync(0xffffffffu, kp[j]));
-    if (lane == 0) s_w[warp] = c;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        unsigned t = 0;
-        for (int w = 0; w < CP_WARPS; ++w) t += s_w[w];
-        counts[blockIdx.x] = t;
-    }
-}
+constexpr int SEL_THREADS = 256;
+constexpr int SEL_WARPS = SEL_THREADS / 32;
+constexpr int SEL_STEP = 1024;         // rows per step
+constexpr unsigned SEL_DENSE = 256;    // kept rows from which a step is read word by word
+constexpr int64_t SEL_MIN_ROWS = (int64_t)1 << 18;  // below this, the single-pass kernel
 
-template <class Row>
-__global__ void __launch_bounds__(CP_THREADS)
-k_tile_write(Row row, int64_t n, int k_out, OutCols out, int64_t cap, const uint32_t *__restrict__ offs,
-             const uint32_t *__restrict__ counts, unsigned tiles, int64_t *__restrict__ d_rows,
-             int64_t *__restrict__ h_rows, uint32_t *__restrict__ mm) {
-    extern __shared__ int32_t s_vals[];  // column c of staged row i at s_vals[c * CP_TILE + i]
-    __shared__ unsigned s_off[CP_ITEMS * CP_WARPS];
-    __shared__ unsigned s_total;
-    const unsigned lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const unsigned lt = (1u << lane) - 1u;
-    const int64_t base = (int64_t)blockIdx.x * CP_TILE;
-    if (blockIdx.x == 0 && threadIdx.x == 0) {  // the result's row count
-        const int64_t total = (int64_t)offs[tiles - 1] + counts[tiles - 1];
-        *d_rows = total;
-        *h_rows = total;
-    }
-    bool kp[CP_ITEMS];
-#pragma unroll
-    for (int j = 0; j < CP_ITEMS; ++j) {
-        const int64_t r = base + j * CP_THREADS + threadIdx.x;
-        kp[j] = row.keep(r < n ? r : n - 1) && r < n;
-    }
-    unsigned keep = 0, wpre[CP_ITEMS];
-#pragma unroll
-    for (int j = 0; j < CP_ITEMS; ++j) {
-        keep |= (unsigned)kp[j] << j;
-        const unsigned b = __ballot_sync(0xffffffffu, kp[j]);
-        wpre[j] = __popc(b & lt);
-        if (lane == 0) s_off[j * CP_WARPS + warp] = __popc(b);
-    }
-    __syncthreads();
-    if (warp == 0) {
-        const unsigned a0 = s_off[2 * lane], a1 = s_off[2 * lane + 1];
-        unsigned x = a0 + a1;
-#pragma unroll
-        for (int d = 1; d < 32; d <<= 1) {
-            const unsigned y = __shfl_up_sync(0xffffffffu, x, d);
-            if ((int)lane >= d) x += y;
-        }
-        const unsigned ex = x - a0 - a1;
-        s_off[2 * lane] = ex;
-        s_off[2 * lane + 1] = ex + a0;
-        if (lane == 31) s_total = x;
-    }
-    __syncthreads();
-#pragma unroll
-    for (int j = 0; j < CP_ITEMS; ++j) {
-        if (!((keep >> j) & 1u)) continue;
-        int32_t v[TID_MAX_COLS];
-        row.values(base + j * CP_THREADS + threadIdx.x, v);
-        const unsigned at = s_off[j * CP_WARPS + warp] + wpre[j];
-#pragma unroll
-        for (int c = 0; c < TID_MAX_COLS; ++c)
-            if (c < k_out) s_vals[c * CP_TILE + at] = v[c];
-    }
-    __syncthreads();
-    const unsigned total = s_total;
-    const long long o0 = offs[blockIdx.x];
-    uint32_t lo[TID_MAX_COLS], hi[TID_MAX_COLS];
-#pragma unroll
-    for (int c = 0; c < TID_MAX_COLS; ++c) {
-        lo[c] = 0xFFFFFFFFu;
-        hi[c] = 0u;
-    }
-    for (unsigned i = threadIdx.x; i < total; i += CP_THREADS) {
-        const long long pos = o0 + i;
-#pragma unroll
-        for (int c = 0; c < TID_MAX_COLS; ++c) {
-            if (c < k_out) {
-                const int32_t v = s_vals[c * CP_TILE + i];
-                if (pos < cap) out.col[c][pos] = v;
-                const uint32_t u = (uint32_t)v ^ 0x80000000u;
-                lo[c] = min(lo[c], u);
-                hi[c] = max(hi[c], u);
-            }
-        }
-    }
-    if (mm) merge_bounds(mm, k_out, lo, hi);
-}
-
-// ---- bitmap compaction (large inputs): K1's structure for rows --------------------
-//
-// One cooperative launch.  Phase A: warps draw runs of BC_DRAW steps of 1024
-// rows from one counter; for step j a warp tests rows 1024 j + 32 w + lane
-// (w = 0..31, BC_INFLIGHT tests in flight per lane), keeps the 32 ballots as the
-// step's keep words and its count, and adds the count to the total of the CTA
-// whose fixed range of steps holds it.  Bounded grid barrier.  Phase C: CTA
-// c's offset is the sum of the earlier CTAs' totals; it block-scans its steps'
-// counts and a warp expands a step: the kept rows' positions in the step go
-// to a shared-memory stage (popc, warp scan, set bits), then the warp reads
-// the kept rows' values in row order and writes them with coalesced stores.
-// A tile never waits for a slower predecessor: the only wait is the barrier.
-
-constexpr int BC_THREADS = 256;
-constexpr int BC_WARPS = BC_THREADS / 32;
-constexpr int BC_INFLIGHT = 16;    // rows a lane tests at once (their loads in flight together)
-
-// kp[u] = row.keep(row base + 32 u) for u < BC_INFLIGHT (false past n)
-template <class Row>
-__device__ __forceinline__ void keep_batch(const Row &row, int64_t base, int64_t n, bool *kp) {
-#pragma unroll
-    for (int u = 0; u < BC_INFLIGHT; ++u) {  // rows past n test row n - 1 (in bounds, no branch) and drop it
-        const int64_t r = base + (int64_t)u * 32;
-        kp[u] = row.keep(r < n ? r : n - 1) && r < n;
-    }
-}
-// The keyed pass: the first tested column of all BC_INFLIGHT rows is loaded
-// before any row is tested, since a test's early exit would otherwise keep
-// the next row's load from being issued ahead of it.
-__device__ __forceinline__ void keep_batch(const SemiJoinRow &row, int64_t base, int64_t n, bool *kp) {
-    const int32_t *first = row.first_column();
-    int32_t v[BC_INFLIGHT];
-#pragma unroll
-    for (int u = 0; u < BC_INFLIGHT; ++u) {
-        const int64_t r = base + (int64_t)u * 32;
-        v[u] = first[r < n ? r : n - 1];
-    }
-#pragma unroll
-    for (int u = 0; u < BC_INFLIGHT; ++u) {
-        const int64_t r = base + (int64_t)u * 32;
-        kp[u] = r < n && row.keep_given(r, v[u]);
-    }
-}
-constexpr int BC_STEP = 1024;      // rows per warp step (32 keep words)
-constexpr int BC_DRAW = 8;         // steps per draw from the counter
-constexpr int BC_CHUNK = BC_THREADS;  // steps scanned per round of phase C
-constexpr int BC_TICKET = 32;      // step counter's word in the control block
-constexpr size_t BC_CTL_BYTES = 256;
-constexpr int64_t BC_MIN_ROWS = (int64_t)1 << 18;  // below this, the single-pass kernel
-
-struct BcScratch {
-    uint32_t *bits;      // 32 keep words per step
-    uint32_t *cnt;       // kept rows per step
-    unsigned *ctl;       // [1] grid barrier, [BC_TICKET] step counter
-    unsigned *cta_tot;   // kept rows per CTA range
-    int *err;
-    int64_t steps;
+struct SelScratch {
+    uint32_t *bits;           // 32 keep words per step
+    uint32_t *cnt;            // kept rows per step
+    unsigned *done;           // CTAs of k_sel_mark that have finished
+    unsigned *tot;            // kept rows per range
+    unsigned long long *off;  // first output row per range
+    unsigned steps, per, ranges;  // range b owns steps [b per, (b + 1) per), per <= 32
 };
 
 template <class Row>
-__global__ void __launch_bounds__(BC_THREADS, 3)
-k_compact_bitmap(Row row, int64_t n, int k_out, OutCols out, int64_t cap, int64_t *__restrict__ d_rows,
-                 int64_t *__restrict__ h_rows, BcScratch sc, uint32_t *__restrict__ mm) {
-    __shared__ uint16_t s_stage[BC_WARPS][BC_STEP];
-    __shared__ uint32_t s_cnt[BC_CHUNK], s_off[BC_CHUNK];
-    __shared__ unsigned s_red[BC_WARPS];
-    __shared__ unsigned long long s_pre[BC_WARPS], s_all[BC_WARPS];
-    __shared__ long long s_base;
+__global__ void __launch_bounds__(SEL_THREADS)
+k_sel_mark(Row row, uint32_t n, SelScratch sc, int64_t *__restrict__ d_rows, int64_t *__restrict__ h_rows) {
     const unsigned lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int64_t per = (sc.steps + gridDim.x - 1) / gridDim.x;  // CTA c owns steps [c per, (c+1) per)
-
-    // ---- phase A: keep words and counts per step
-    {
-        unsigned *ticket = sc.ctl + BC_TICKET;
-        unsigned t = 0;
-        if (lane == 0) t = atomicAdd(ticket, (unsigned)BC_DRAW);
-        t = __shfl_sync(0xffffffffu, t, 0);
-        unsigned k = 0;
-        while ((int64_t)(t + k) < sc.steps) {
-            const int64_t step = (int64_t)t + k;
-            unsigned nxt = 0;
-            if (lane == 0 && k + 1 == (unsigned)BC_DRAW) nxt = atomicAdd(ticket, (unsigned)BC_DRAW);
-            const int64_t base = step * BC_STEP + lane;
-            uint32_t word = 0;
-            unsigned c = 0;
+    const unsigned sub = lane & 7u;
+    for (unsigned step = blockIdx.x * SEL_WARPS + warp; step < sc.steps; step += gridDim.x * SEL_WARPS) {
+        const uint32_t base = step * SEL_STEP + lane * 4;  // < 2^32: n < 2^31
+        unsigned m[8];
+        if ((step + 1) * SEL_STEP <= n) {
+            row.keep_step(base, m);
+        } else {  // ragged last step
 #pragma unroll 1
-            for (int w0 = 0; w0 < 32; w0 += BC_INFLIGHT) {
-                bool kp[BC_INFLIGHT];
-                keep_batch(row, base + (int64_t)w0 * 32, n, kp);
-#pragma unroll
-                for (int u = 0; u < BC_INFLIGHT; ++u) {
-                    const unsigned b = __ballot_sync(0xffffffffu, kp[u]);
-                    if ((int)lane == w0 + u) word = b;
-                    c += __popc(b);
+            for (int g = 0; g < 8; ++g) {
+                unsigned k4 = 0;
+                for (int e = 0; e < 4; ++e) {
+                    const uint32_t r = base + g * 128 + e;
+                    if (r < n && row.keep(r)) k4 |= 1u << e;
                 }
-            }
-            __stcg(sc.bits + step * 32 + lane, word);
-            if (lane == 0) {
-                __stcg(sc.cnt + step, c);
-                if (c) atomicAdd(sc.cta_tot + step / per, c);
-            }
-            if (++k == (unsigned)BC_DRAW) {
-                t = __shfl_sync(0xffffffffu, nxt, 0);
-                k = 0;
+#pragma unroll
+                for (int q = 0; q < 8; ++q)
+                    if (q == g) m[q] = k4;
             }
         }
-    }
-    if (!grid_barrier(sc.ctl + 1, gridDim.x, sc.err)) return;
-
-    // ---- phase C: this range's offset, then ordered expansion
-    const int64_t r0 = min((int64_t)blockIdx.x * per, sc.steps), r1 = min(r0 + per, sc.steps);
-    const unsigned mine = __ldcg(sc.cta_tot + blockIdx.x);
-    unsigned long long pre = 0, all = 0;
-    for (unsigned c = threadIdx.x; c < gridDim.x; c += BC_THREADS) {
-        const unsigned v = __ldcg(sc.cta_tot + c);
-        all += v;
-        if (c < blockIdx.x) pre += v;
-    }
+        // lanes 8k .. 8k + 7 together hold word 4 g + k; lane 8k + g keeps it
+        uint32_t word = 0;
 #pragma unroll
-    for (int d = 16; d > 0; d >>= 1) {
-        pre += __shfl_xor_sync(0xffffffffu, pre, d);
-        all += __shfl_xor_sync(0xffffffffu, all, d);
+        for (int g = 0; g < 8; ++g) {
+            uint32_t v = m[g] << (4 * sub);
+            v |= __shfl_xor_sync(0xffffffffu, v, 1);
+            v |= __shfl_xor_sync(0xffffffffu, v, 2);
+            v |= __shfl_xor_sync(0xffffffffu, v, 4);
+            if (sub == (unsigned)g) word = v;
+        }
+        sc.bits[(size_t)step * 32 + sub * 4 + (lane >> 3)] = word;
+        const unsigned c = __reduce_add_sync(0xffffffffu, __popc(word));
+        if (lane == 0) {
+            sc.cnt[step] = c;
+            if (c) atomicAdd(sc.tot + step / sc.per, c);
+        }
     }
-    if (lane == 0) {
-        s_pre[warp] = pre;
-        s_all[warp] = all;
-    }
+    // the last CTA: exclusive scan of the ranges' totals
+    __shared__ unsigned s_last;
+    __shared__ unsigned long long s_w[SEL_WARPS];
     __syncthreads();
     if (threadIdx.x == 0) {
-        unsigned long long p = 0, a = 0;
-        for (int w = 0; w < BC_WARPS; ++w) {
-            p += s_pre[w];
-            a += s_all[w];
-        }
-        s_base = (long long)p;
-        if (blockIdx.x == 0) {
-            *d_rows = (int64_t)a;
-            *h_rows = (int64_t)a;
-        }
+        __threadfence();
+        s_last = atomicAdd(sc.done, 1u) == gridDim.x - 1;
+        __threadfence();
     }
     __syncthreads();
-    if (mine == 0) return;
-    uint32_t lo[TID_MAX_COLS], hi[TID_MAX_COLS];
+    if (!s_last) return;
+    unsigned long long carry = 0;
+    for (unsigned b0 = 0; b0 < sc.ranges; b0 += SEL_THREADS) {
+        const unsigned b = b0 + threadIdx.x;
+        const unsigned long long c = b < sc.ranges ? __ldcg(sc.tot + b) : 0u;
+        unsigned long long x = c;
 #pragma unroll
-    for (int c = 0; c < TID_MAX_COLS; ++c) {
+        for (int d = 1; d < 32; d <<= 1) {
+            const unsigned long long y = __shfl_up_sync(0xffffffffu, x, d);
+            if ((int)lane >= d) x += y;
+        }
+        if (lane == 31) s_w[warp] = x;
+        __syncthreads();
+        unsigned long long wb = 0, all = 0;
+        for (int w = 0; w < SEL_WARPS; ++w) {
+            if (w < (int)warp) wb += s_w[w];
+            all += s_w[w];
+        }
+        if (b < sc.ranges) sc.off[b] = carry + wb + x - c;
+        carry += all;
+        __syncthreads();  // s_w is rewritten by the next round
+    }
+    if (threadIdx.x == 0) {
+        *d_rows = (int64_t)carry;
+        *h_rows = (int64_t)carry;
+    }
+}
+
+template <class Row, int K, bool BOUNDS>
+__global__ void __launch_bounds__(SEL_THREADS, K == 2 ? 5 : (K <= 3 ? 4 : 2))
+k_sel_expand(Row row, int k_out, OutCols out, int64_t cap, SelScratch sc, uint32_t *__restrict__ mm) {
+    __shared__ uint16_t s_stage[SEL_WARPS][SEL_DENSE];
+    const unsigned lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const unsigned lt = (1u << lane) - 1u;
+    uint32_t lo[K], hi[K];
+#pragma unroll
+    for (int c = 0; c < K; ++c) {
         lo[c] = 0xFFFFFFFFu;
         hi[c] = 0u;
     }
-    long long run = s_base;
-    for (int64_t q0 = r0; q0 < r1; q0 += BC_CHUNK) {
-        const int64_t j = q0 + threadIdx.x;
-        const unsigned c = j < r1 ? __ldcg(sc.cnt + j) : 0u;
-        unsigned x = c;
+    auto put = [&](const int32_t *v, unsigned long long pos) {
+#pragma unroll
+        for (int c = 0; c < K; ++c) {
+            if (c < k_out) {
+                if (pos < (unsigned long long)cap) out.col[c][pos] = v[c];
+                if (BOUNDS) {
+                    const uint32_t u = (uint32_t)v[c] ^ 0x80000000u;
+                    lo[c] = min(lo[c], u);
+                    hi[c] = max(hi[c], u);
+                }
+            }
+        }
+    };
+    constexpr int UX = K == 1 ? 8 : 4;  // rows per lane read together
+    const unsigned r0 = blockIdx.x * sc.per, here = min(sc.per, sc.steps - r0);
+    const unsigned cnt = lane < here ? sc.cnt[r0 + lane] : 0u;
+    uint32_t next = warp < here ? sc.bits[(size_t)(r0 + warp) * 32 + lane] : 0u;
+    unsigned first = cnt;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        const unsigned y = __shfl_up_sync(0xffffffffu, first, d);
+        if ((int)lane >= d) first += y;
+    }
+    first -= cnt;  // of step r0 + lane
+    const unsigned long long o_range = sc.off[blockIdx.x];
+    for (unsigned li = warp; li < here; li += SEL_WARPS) {
+        const uint32_t word = next;
+        if (li + SEL_WARPS < here) next = sc.bits[(size_t)(r0 + li + SEL_WARPS) * 32 + lane];
+        const unsigned sn = __shfl_sync(0xffffffffu, cnt, li);
+        if (sn == 0) continue;
+        const unsigned long long o0 = o_range + __shfl_sync(0xffffffffu, first, li);
+        const unsigned pc = __popc(word);
+        unsigned xo = pc;
 #pragma unroll
         for (int d = 1; d < 32; d <<= 1) {
-            const unsigned y = __shfl_up_sync(0xffffffffu, x, d);
-            if ((int)lane >= d) x += y;
+            const unsigned y = __shfl_up_sync(0xffffffffu, xo, d);
+            if ((int)lane >= d) xo += y;
         }
-        if (lane == 31) s_red[warp] = x;
-        __syncthreads();
-        unsigned wb = 0, rt = 0;
-        for (int w = 0; w < BC_WARPS; ++w) {
-            if (w < (int)warp) wb += s_red[w];
-            rt += s_red[w];
-        }
-        s_cnt[threadIdx.x] = c;
-        s_off[threadIdx.x] = wb + x - c;
-        __syncthreads();
-        uint16_t *stage = s_stage[warp];
-        for (int i = 0; i < 32; ++i) {  // warp w expands steps q0 + 32 w .. + 31
-            const int li = (int)warp * 32 + i;
-            const int64_t step = q0 + li;
-            if (step >= r1) break;
-            const unsigned sn = s_cnt[li];
-            if (sn == 0) continue;
-            // keep word w of a step holds rows 32 w + (0..31): lane w stages its word's rows
-            uint32_t word = __ldcg(sc.bits + step * 32 + lane);
-            const unsigned pc = __popc(word);
-            unsigned xo = pc;
+        xo -= pc;
+        const int64_t base = (int64_t)(r0 + li) * SEL_STEP;
+        if (sn >= SEL_DENSE) {
+#pragma unroll 1
+            for (int w0 = 0; w0 < 32; w0 += UX) {
+                int32_t v[UX][K];
+                unsigned bw[UX];
 #pragma unroll
-            for (int d = 1; d < 32; d <<= 1) {
-                const unsigned y = __shfl_up_sync(0xffffffffu, xo, d);
-                if ((int)lane >= d) xo += y;
+                for (int u = 0; u < UX; ++u) {
+                    bw[u] = __shfl_sync(0xffffffffu, word, w0 + u);
+                    if ((bw[u] >> lane) & 1u) row.template values<K>(base + (w0 + u) * 32 + lane, v[u]);
+                }
+#pragma unroll
+                for (int u = 0; u < UX; ++u) {
+                    const unsigned at = __shfl_sync(0xffffffffu, xo, w0 + u) + __popc(bw[u] & lt);
+                    if ((bw[u] >> lane) & 1u) put(v[u], o0 + at);
+                }
             }
-            unsigned at = xo - pc;
-            while (word) {
-                const int b = __ffs(word) - 1;
-                stage[at++] = (uint16_t)(lane * 32 + b);
-                word &= word - 1;
+        } else {
+            uint16_t *stage = s_stage[warp];
+            uint32_t w = word;
+            while (w) {
+                stage[xo++] = (uint16_t)(lane * 32 + __ffs(w) - 1);
+                w &= w - 1;
             }
             __syncwarp();
-            const long long o0 = run + s_off[li];
-#pragma unroll 4
-            for (unsigned e = lane; e < sn; e += 32) {
-                int32_t v[TID_MAX_COLS];
-                row.values(step * BC_STEP + stage[e], v);
-                const long long pos = o0 + e;
+#pragma unroll 1
+            for (unsigned e0 = 0; e0 < sn; e0 += 32 * UX) {
+                int32_t v[UX][K];
 #pragma unroll
-                for (int cc = 0; cc < TID_MAX_COLS; ++cc) {
-                    if (cc < k_out) {
-                        if ((unsigned long long)pos < (unsigned long long)cap) out.col[cc][pos] = v[cc];
-                        const uint32_t u = (uint32_t)v[cc] ^ 0x80000000u;
-                        lo[cc] = min(lo[cc], u);
-                        hi[cc] = max(hi[cc], u);
-                    }
+                for (int u = 0; u < UX; ++u) {
+                    const unsigned e = e0 + u * 32 + lane;
+                    if (e < sn) row.template values<K>(base + stage[e], v[u]);
+                }
+#pragma unroll
+                for (int u = 0; u < UX; ++u) {
+                    const unsigned e = e0 + u * 32 + lane;
+                    if (e < sn) put(v[u], o0 + e);
                 }
             }
             __syncwarp();
         }
-        run += rt;
-        __syncthreads();  // s_red, s_cnt, s_off are reused
     }
-    if (mm) merge_bounds(mm, k_out, lo, hi);
+    if (BOUNDS) merge_bounds<K>(mm, k_out, lo, hi);
 }
 
+template <class Row, int K>
+int expand_k(tid_ctx *ctx, const Row &row, int k_out, const OutCols &out, int64_t cap, const SelScratch &sc,
+             uint32_t *mm) {
+    if (mm) k_sel_expand<Row, K, true><<<sc.ranges, SEL_THREADS, 0, ctx->stream>>>(row, k_out, out, cap, sc, mm);
+    else k_sel_expand<Row, K, false><<<sc.ranges, SEL_THREADS, 0, ctx->stream>>>(row, k_out, out, cap, sc, mm);
+    return launch_check("k_sel_expand");
+}
+
+// grid of k_sel_mark: every CTA resident at once
 template <class Row>
-int bitmap_grid(unsigned *grid) {
+unsigned mark_grid() {
     static unsigned cached = 0;
     if (!cached) {
         int v = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, k_compact_bitmap<Row>, BC_THREADS, 0) != cudaSuccess ||
-            v <= 0)
-            return fail(TID_ERR_CUDA, "k_compact_bitmap: no resident CTA");
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, k_sel_mark<Row>, SEL_THREADS, 0) != cudaSuccess || v <= 0)
+            v = 1;
         cached = (unsigned)(v * sm_count());
     }
-    *grid = cached;
-    return TID_OK;
+    return cached;
 }
 
-// Which kernel compacts a long input.  Single pass: a tile's offset comes from
-// the decoupled look-back, and profiles show tiles waiting there for their
-// predecessors far longer than their own work takes; it serves short inputs
-// and bind with tests (its tests are random gathers: two kernels would gather
-// them twice, and measured no faster).  Two kernels (filters, distinct rows):
-// the test columns are read twice and no CTA waits for another.  Bitmap
-// (sparse keeps over the store: the keyed pass): one cooperative launch, the
-// kept rows' values read once after the grid barrier.
-enum CompactMode { CP_SINGLE, CP_TWO, CP_BITMAP };
-
 template <class Row>
-int launch_compact(tid_ctx *ctx, const Row &row, int64_t n, int k_out, const OutCols &out, int64_t cap,
-                   int64_t *d_rows, int64_t *h_rows_dev, uint32_t *mm = nullptr, CompactMode mode = CP_TWO) {
+int launch_compact(tid_ctx *ctx, Row row, int64_t n, int k_out, const OutCols &out, int64_t cap,
+                   int64_t *d_rows, int64_t *h_rows_dev, uint32_t *mm = nullptr) {
     if (n == 0) {
         TID_TRY_CUDA(cudaMemsetAsync(d_rows, 0, sizeof(int64_t), ctx->stream), "memset rows");
         TID_TRY_CUDA(cudaMemsetAsync(h_rows_dev, 0, sizeof(int64_t), ctx->stream), "memset rows");
         return TID_OK;
     }
-    if (n >= BC_MIN_ROWS && mode == CP_TWO) {
-        static bool opted = false;
-        if (!opted) {
-            TID_TRY_CUDA(cudaFuncSetAttribute(k_tile_write<Row>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                              (int)(sizeof(int32_t) * TID_MAX_COLS * CP_TILE)),
-                         "k_tile_write smem");
-            opted = true;
-        }
-        const unsigned tiles = (unsigned)ceil_div(n, CP_TILE);
-        void *blk = nullptr;
-        TID_TRY(dev_alloc(ctx, &blk, sizeof(uint32_t) * 2 * (size_t)tiles + 256));
-        uint32_t *counts = (uint32_t *)blk, *offs = counts + tiles;
-        int rc = TID_OK;
-        k_tile_counts<Row><<<tiles, CP_THREADS, 0, ctx->stream>>>(row, n, counts);
-        rc = launch_check("k_tile_counts");
-        if (rc == TID_OK) rc = scan_exclusive_u32(ctx, counts, offs, tiles, nullptr);
-        if (rc == TID_OK) {
-            const size_t smem = sizeof(int32_t) * (size_t)std::max(1, k_out) * CP_TILE;
-            k_tile_write<Row><<<tiles, CP_THREADS, smem, ctx->stream>>>(row, n, k_out, out, cap, offs, counts, tiles,
-                                                                        d_rows, h_rows_dev, mm);
-            rc = launch_check("k_tile_write");
-        }
-        dev_free(ctx, blk);
-        return rc;
-    }
-    if (n < BC_MIN_ROWS || mode == CP_SINGLE) {
+    if (n < SEL_MIN_ROWS) {
         static bool opted = false;  // staging of up to TID_MAX_COLS columns of a tile
         if (!opted) {
             TID_TRY_CUDA(cudaFuncSetAttribute(k_compact<Row>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -744,32 +723,40 @@ int launch_compact(tid_ctx *ctx, const Row &row, int64_t n, int k_out, const Out
         k_compact<Row><<<tiles, CP_THREADS, smem, ctx->stream>>>(row, n, k_out, out, cap, d_rows, h_rows_dev, lb, mm);
         return launch_check("k_compact");
     }
-    unsigned grid = 0;
-    TID_TRY(bitmap_grid<Row>(&grid));
-    const int64_t steps = ceil_div(n, (int64_t)BC_STEP);
-    grid = (unsigned)std::min<int64_t>(grid, steps);
-    const size_t bits_b = (size_t)steps * 32 * 4, cnt_b = ((size_t)steps * 4 + 255) / 256 * 256;
-    const size_t tot_b = (size_t)grid * 4;
+    SelScratch sc{};
+    sc.steps = (unsigned)ceil_div(n, (int64_t)SEL_STEP);
+    // a range is one step per warp, or four once that still gives every SM eight CTAs
+    sc.per = sc.steps >= (unsigned)sm_count() * 256 ? 32 : SEL_WARPS;
+    sc.ranges = (unsigned)ceil_div(sc.steps, (int64_t)sc.per);
+    const size_t bits_b = (size_t)sc.steps * 32 * 4, off_b = (size_t)sc.ranges * 8;
+    const size_t cnt_b = ((size_t)sc.steps * 4 + 255) / 256 * 256, tot_b = ((size_t)sc.ranges + 1) * 4;
+    size_t stash_b = 0;
+    if constexpr (std::is_same_v<Row, BindRow>) {
+        if (row.n_eq == 0 && (row.test & (row.test - 1)) == 0) stash_b = (size_t)n * 4;
+    }
     void *blk = nullptr;
-    TID_TRY(dev_alloc(ctx, &blk, bits_b + cnt_b + BC_CTL_BYTES + tot_b));
-    BcScratch sc{};
+    TID_TRY(dev_alloc(ctx, &blk, stash_b + bits_b + off_b + cnt_b + tot_b + 256));
+    if constexpr (std::is_same_v<Row, BindRow>) {
+        if (stash_b) row.stash = (int32_t *)((char *)blk + (bits_b + off_b + cnt_b + tot_b + 255) / 256 * 256);
+    }
     sc.bits = (uint32_t *)blk;
-    sc.cnt = (uint32_t *)((char *)blk + bits_b);
-    sc.ctl = (unsigned *)((char *)blk + bits_b + cnt_b);
-    sc.cta_tot = (unsigned *)((char *)blk + bits_b + cnt_b + BC_CTL_BYTES);
-    sc.err = ctx->err_dev;
-    sc.steps = steps;
+    sc.off = (unsigned long long *)((char *)blk + bits_b);
+    sc.cnt = (uint32_t *)((char *)blk + bits_b + off_b);
+    sc.done = (unsigned *)((char *)blk + bits_b + off_b + cnt_b);
+    sc.tot = sc.done + 1;
     int rc = TID_OK;
-    cudaError_t e = cudaMemsetAsync(sc.ctl, 0, BC_CTL_BYTES + tot_b, ctx->stream);
-    if (e != cudaSuccess) rc = fail_cuda(e, "k_compact_bitmap control words");
+    cudaError_t e = cudaMemsetAsync(sc.done, 0, tot_b, ctx->stream);
+    if (e != cudaSuccess) rc = fail_cuda(e, "row selection totals");
     if (rc == TID_OK) {
-        Row r = row;
-        OutCols oc = out;
-        void *args[] = {(void *)&r, (void *)&n, (void *)&k_out, (void *)&oc, (void *)&cap, (void *)&d_rows,
-                        (void *)&h_rows_dev, (void *)&sc, (void *)&mm};
-        e = cudaLaunchCooperativeKernel((const void *)k_compact_bitmap<Row>, dim3(grid), dim3(BC_THREADS), args, 0,
-                                        ctx->stream);
-        if (e != cudaSuccess) rc = fail_cuda(e, "k_compact_bitmap");
+        const unsigned grid = (unsigned)std::min<int64_t>(mark_grid<Row>(), ceil_div(sc.steps, (int64_t)SEL_WARPS));
+        k_sel_mark<Row><<<grid, SEL_THREADS, 0, ctx->stream>>>(row, (uint32_t)n, sc, d_rows, h_rows_dev);
+        rc = launch_check("k_sel_mark");
+    }
+    if (rc == TID_OK) {
+        if (k_out <= 1) rc = expand_k<Row, 1>(ctx, row, k_out, out, cap, sc, mm);
+        else if (k_out == 2) rc = expand_k<Row, 2>(ctx, row, k_out, out, cap, sc, mm);
+        else if (Row::MAX_K == 3 || k_out == 3) rc = expand_k<Row, 3>(ctx, row, k_out, out, cap, sc, mm);
+        else if constexpr (Row::MAX_K > 3) rc = expand_k<Row, Row::MAX_K>(ctx, row, k_out, out, cap, sc, mm);
     }
     dev_free(ctx, blk);
     return rc;
@@ -780,33 +767,47 @@ int launch_compact(tid_ctx *ctx, const Row &row, int64_t n, int k_out, const Out
 // compaction -- with the column bounds of the output.
 __global__ void __launch_bounds__(256) k_bind_gather(BindRow row, int64_t n, OutCols out, uint32_t *__restrict__ mm,
                                                      int64_t *__restrict__ d_rows, int64_t *__restrict__ h_rows) {
-    uint32_t lo[TID_MAX_COLS], hi[TID_MAX_COLS];
+    constexpr int K = 3, U = 4;  // a pattern has at most three variables; rows per thread in flight
+    uint32_t lo[K], hi[K];
 #pragma unroll
-    for (int c = 0; c < TID_MAX_COLS; ++c) {
+    for (int c = 0; c < K; ++c) {
         lo[c] = 0xFFFFFFFFu;
         hi[c] = 0u;
     }
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    const int64_t n_iter = ceil_div(n, stride) * stride;
-    for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < n_iter; r += stride) {
-        if (r < n) {
-            int32_t v[TID_MAX_COLS];
-            row.values(r, v);
+    const int64_t stride = (int64_t)gridDim.x * (256 * U);
+    for (int64_t r0 = (int64_t)blockIdx.x * (256 * U) + threadIdx.x; r0 < n; r0 += stride) {
+        int32_t v[U][K];
 #pragma unroll
-            for (int c = 0; c < TID_MAX_COLS; ++c) {
+        for (int u = 0; u < U; ++u) row.template values<K>(min(r0 + u * 256, n - 1), v[u]);
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int64_t r = r0 + u * 256;
+            if (r >= n) continue;
+#pragma unroll
+            for (int c = 0; c < K; ++c) {
                 if (c < row.k) {
-                    out.col[c][r] = v[c];
-                    const uint32_t u = (uint32_t)v[c] ^ 0x80000000u;
-                    lo[c] = min(lo[c], u);
-                    hi[c] = max(hi[c], u);
+                    out.col[c][r] = v[u][c];
+                    const uint32_t x = (uint32_t)v[u][c] ^ 0x80000000u;
+                    lo[c] = min(lo[c], x);
+                    hi[c] = max(hi[c], x);
                 }
             }
         }
     }
-    if (mm) merge_bounds(mm, row.k, lo, hi);
+    if (mm) merge_bounds<K>(mm, row.k, lo, hi);
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         *d_rows = n;
         *h_rows = n;
+    }
+}
+
+// bits: one per term of the column that lies in [lo, lo + w); 0 sets none
+__global__ void __launch_bounds__(256) k_member_bits(const int32_t *__restrict__ col, int64_t n, uint32_t lo,
+                                                     uint32_t w, uint32_t *__restrict__ bits) {
+    for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < n; i += (int64_t)gridDim.x * 256) {
+        const int32_t x = col[i];
+        const uint32_t d = ((uint32_t)x ^ 0x80000000u) - lo;
+        if (x != 0 && d < w) atomicOr(bits + (d >> 5), 1u << (d & 31));
     }
 }
 
@@ -946,7 +947,7 @@ int scan_exclusive_u32(tid_ctx *ctx, const uint32_t *in, uint32_t *out, int64_t 
 }
 
 int compact_bind(tid_ctx *ctx, const tid_store *st, const tid_pattern &pat, const int32_t *idx, int64_t n,
-                 const Pred *preds, int n_preds, tid_set *out, uint32_t *mm) {
+                 const Pred *preds, int n_preds, const BindMember *mem, int n_mem, tid_set *out, uint32_t *mm) {
     BindRow r{};
     r.S = st->s;
     r.P = st->p;
@@ -972,14 +973,25 @@ int compact_bind(tid_ctx *ctx, const tid_store *st, const tid_pattern &pat, cons
                 r.n_eq++;
             }
     r.n_preds = n_preds;
-    for (int q = 0; q < n_preds; ++q) r.preds[q] = preds[q];
+    for (int q = 0; q < n_preds; ++q) {  // a test reads a slot of the triple
+        r.preds[q] = preds[q];
+        r.preds[q].col = r.src[preds[q].col];
+        r.test |= 1 << r.preds[q].col;
+    }
+    for (int e = 0; e < r.n_eq; ++e) r.test |= (1 << r.eq_a[e]) | (1 << r.eq_b[e]);
+    r.n_mem = n_mem;
+    for (int q = 0; q < n_mem; ++q) {
+        r.mem[q] = mem[q].m;
+        r.mem_slot[q] = r.src[mem[q].col];
+        r.test |= 1 << r.mem_slot[q];
+    }
     OutCols oc{};
     for (int c = 0; c < out->k; ++c) oc.col[c] = out->col[c];
-    if (n > 0 && r.n_eq == 0 && r.n_preds == 0 && n <= out->cap) {
-        k_bind_gather<<<grid_for(n, 256, 8), 256, 0, ctx->stream>>>(r, n, oc, mm, out->d_rows, out->slot.dev);
+    if (n > 0 && r.test == 0 && n <= out->cap) {
+        k_bind_gather<<<grid_for(n, 256 * 4, 8), 256, 0, ctx->stream>>>(r, n, oc, mm, out->d_rows, out->slot.dev);
         return launch_check("k_bind_gather");
     }
-    return launch_compact(ctx, r, n, out->k, oc, out->cap, out->d_rows, out->slot.dev, mm, CP_SINGLE);
+    return launch_compact(ctx, r, n, out->k, oc, out->cap, out->d_rows, out->slot.dev, mm);
 }
 
 int compact_semijoin(tid_ctx *ctx, const tid_store *st, int fixed_slot, int32_t fixed_val, int key_slot,
@@ -993,6 +1005,7 @@ int compact_semijoin(tid_ctx *ctx, const tid_store *st, int fixed_slot, int32_t 
     r.key_slot = key_slot;
     r.table = table;
     r.tbits = tbits;
+    r.vec = st->aligned16;
     r.k = out->k;
     r.need = (fixed_slot >= 0 ? 1 << fixed_slot : 0) | (1 << key_slot);
     for (int c = 0; c < out->k; ++c) {
@@ -1001,7 +1014,7 @@ int compact_semijoin(tid_ctx *ctx, const tid_store *st, int fixed_slot, int32_t 
     }
     OutCols oc{};
     for (int c = 0; c < out->k; ++c) oc.col[c] = out->col[c];
-    return launch_compact(ctx, r, st->n, out->k, oc, out->cap, out->d_rows, out->slot.dev, nullptr, CP_BITMAP);
+    return launch_compact(ctx, r, st->n, out->k, oc, out->cap, out->d_rows, out->slot.dev);
 }
 
 int compact_filter(tid_ctx *ctx, const tid_set *in, int64_t n, const Pred *preds, int n_preds, tid_set *out) {
@@ -1010,6 +1023,37 @@ int compact_filter(tid_ctx *ctx, const tid_set *in, int64_t n, const Pred *preds
     for (int c = 0; c < in->k; ++c) r.col[c] = in->col[c];
     r.n_preds = n_preds;
     for (int q = 0; q < n_preds; ++q) r.preds[q] = preds[q];
+    OutCols oc{};
+    for (int c = 0; c < out->k; ++c) oc.col[c] = out->col[c];
+    return launch_compact(ctx, r, n, out->k, oc, out->cap, out->d_rows, out->slot.dev);
+}
+
+int member_bits(tid_ctx *ctx, const int32_t *col, int64_t n, uint32_t lo, uint32_t hi, Members *m) {
+    const uint64_t w = (uint64_t)hi - lo + 1;
+    const size_t words = (size_t)((w + 31) / 32);
+    void *p = nullptr;
+    TID_TRY(dev_alloc(ctx, &p, words * 4));
+    m->bits = (uint32_t *)p;
+    m->lo = lo;
+    m->w = (uint32_t)std::min<uint64_t>(w, 0xFFFFFFFFu);
+    cudaError_t e = cudaMemsetAsync(p, 0, words * 4, ctx->stream);
+    int rc = e == cudaSuccess ? TID_OK : fail_cuda(e, "member bits");
+    if (rc == TID_OK && n > 0) {
+        k_member_bits<<<grid_for(n, 256, 8), 256, 0, ctx->stream>>>(col, n, m->lo, m->w, (uint32_t *)p);
+        rc = launch_check("k_member_bits");
+    }
+    if (rc != TID_OK) {
+        dev_free(ctx, p);
+        m->bits = nullptr;
+    }
+    return rc;
+}
+
+int compact_member(tid_ctx *ctx, const tid_set *in, int64_t n, const Members &m, tid_set *out) {
+    MemberRow r{};
+    r.k = in->k;
+    for (int c = 0; c < in->k; ++c) r.col[c] = in->col[c];
+    r.m = m;
     OutCols oc{};
     for (int c = 0; c < out->k; ++c) oc.col[c] = out->col[c];
     return launch_compact(ctx, r, n, out->k, oc, out->cap, out->d_rows, out->slot.dev);

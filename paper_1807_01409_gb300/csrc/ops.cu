@@ -33,7 +33,20 @@ int make_preds(const int8_t *vars, int k, const tid_pred *preds, int n_preds, Pr
         if (col < 0) return fail(TID_ERR_ARG, "%s: predicate on variable %d not in the set", who, preds[q].var);
         if (preds[q].op < TID_CMP_EQ || preds[q].op > TID_CMP_RANGE)
             return fail(TID_ERR_ARG, "%s: unknown comparison %d", who, preds[q].op);
-        out[q] = Pred{col, preds[q].op, preds[q].a, preds[q].b};
+        int32_t lo = INT32_MIN, hi = INT32_MAX;
+        const int32_t a = preds[q].a;
+        bool none = false;  // no value passes
+        switch (preds[q].op) {
+            case TID_CMP_EQ:
+            case TID_CMP_NE: lo = hi = a; break;
+            case TID_CMP_LT: none = a == INT32_MIN; hi = none ? hi : a - 1; break;
+            case TID_CMP_LE: hi = a; break;
+            case TID_CMP_GT: none = a == INT32_MAX; lo = none ? lo : a + 1; break;
+            case TID_CMP_GE: lo = a; break;
+            default: none = a > preds[q].b; lo = none ? lo : a; hi = none ? hi : preds[q].b; break;  // RANGE
+        }
+        const Pred p{col, none || preds[q].op == TID_CMP_NE, lo, (uint32_t)hi - (uint32_t)lo};
+        out[q] = p;
     }
     return TID_OK;
 }
@@ -95,7 +108,7 @@ int bind_set(tid_ctx *ctx, const tid_store *st, const tid_pattern &pat, const ti
         if (e == cudaSuccess) e = cudaMemsetAsync(mm + TID_MAX_COLS, 0, TID_MAX_COLS * sizeof(uint32_t), ctx->stream);
         if (e != cudaSuccess) rc = fail_cuda(e, "tid_bind");
     }
-    if (rc == TID_OK) rc = compact_bind(ctx, st, pat, idx->col[0], n, pr, n_preds, tmp, mm);
+    if (rc == TID_OK) rc = compact_bind(ctx, st, pat, idx->col[0], n, pr, n_preds, nullptr, 0, tmp, mm);
     uint32_t hb[2 * TID_MAX_COLS];
     if (rc == TID_OK) {
         cudaError_t e = cudaMemcpyAsync(hb, mm, sizeof hb, cudaMemcpyDeviceToHost, ctx->stream);

@@ -8,10 +8,23 @@ namespace tid {
 
 constexpr int MAX_PREDS = 4;  // predicates fused into one compaction pass
 
-struct Pred {  // a FILTER predicate on column `col` of the set being produced
+struct Pred {  // a FILTER predicate on column `col` of the set being produced: a value passes
+               // when it is bound (not 0) and (lo <= value <= lo + span) != neg
     int col;
-    int op;
-    int32_t a, b;
+    int neg;
+    int32_t lo;
+    uint32_t span;
+};
+
+// A set of terms as a bitmap over [lo, lo + w) in sort order (int32 ^ 0x80000000)
+struct Members {
+    const uint32_t *bits;
+    uint32_t lo, w;
+};
+constexpr int MAX_MEMBERS = 2;
+struct BindMember {  // a bound row is kept when its column `col` is a member
+    Members m;
+    int col;
 };
 
 struct OutCols {
@@ -38,11 +51,16 @@ struct Bounds {
 int scan_exclusive_u32(tid_ctx *ctx, const uint32_t *in, uint32_t *out, int64_t n,
                        unsigned long long *total_dev);
 
-// single-pass compactions (compact.cu); `out` must have capacity >= n
+// row selections (compact.cu); `out` must have capacity >= n
 // bind; if mm is not null, mm[c] / mm[8 + c] receive (atomic min / max) the
 // sort-order bounds of output column c over the kept rows (caller presets them)
 int compact_bind(tid_ctx *ctx, const tid_store *st, const tid_pattern &pat, const int32_t *idx, int64_t n,
-                 const Pred *preds, int n_preds, tid_set *out, uint32_t *mm);
+                 const Pred *preds, int n_preds, const BindMember *mem, int n_mem, tid_set *out, uint32_t *mm);
+// the terms of col[0, n) in [lo, hi] (sort order, hi - lo < 2^32 - 1) as a bitmap,
+// allocated here (m->bits, freed by the caller)
+int member_bits(tid_ctx *ctx, const int32_t *col, int64_t n, uint32_t lo, uint32_t hi, Members *m);
+// rows of `in` whose first column is a member, in order
+int compact_member(tid_ctx *ctx, const tid_set *in, int64_t n, const Members &m, tid_set *out);
 int compact_filter(tid_ctx *ctx, const tid_set *in, int64_t n, const Pred *preds, int n_preds, tid_set *out);
 // store triples (in store order) whose fixed_slot holds fixed_val (fixed_slot -1:
 // any) and whose key_slot term is in the key table (2^tbits slots, home slot =
