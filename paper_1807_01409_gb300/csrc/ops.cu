@@ -372,7 +372,8 @@ int project_set(tid_ctx *ctx, const tid_set *in, const int8_t *vars, int n_vars,
         for (int i = 0; i < t && ok; ++i) ok = in->vars[i] == vars[n_vars - t + i];
         if (ok) tail = t;
     }
-    return canonicalize(ctx, cols, n_vars, vars, n, !identity, in->bounded ? &b : nullptr, out, tail);
+    // keeping every column of a set leaves its rows distinct
+    return canonicalize(ctx, cols, n_vars, vars, n, n_vars < in->k, in->bounded ? &b : nullptr, out, tail);
 }
 
 // Right and full outer joins (Section 4.2 lists the outer joins of the library

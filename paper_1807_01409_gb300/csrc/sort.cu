@@ -24,7 +24,13 @@
 // 2022) waited there longer than its tiles worked, every tile walking back
 // through all the tiles in flight.  Bytes per digit: w n read twice (the
 // histogram read mostly from L2) + w n written, w = key bytes (4 or 8; 4 + 4
-// with the permutation), plus one read of the columns for packing.
+// with the permutation).  Packing and unpacking ride along: the first pass packs
+// its keys from the columns (its histogram reads only the columns that hold bits
+// of its digit), the last one writes the result's columns, so a one-pass sort
+// moves no packed keys at all and a P-pass sort writes them P - 1 times.  Digits are of equal width (27 bits: 7 7 7 6).
+// Measured on GB300: (x, v) -> (v, x) of 24M rows, two passes, 590 -> 295 us with
+// the distinct pass that a permutation of columns does not need; the sort of a
+// bind's 11.8M rows, four 32-bit passes, 370 -> 300 us.
 //
 // Sets of at most 4096 packed rows skip the passes: one CTA loads the keys into
 // shared memory, bitonic-sorts them, flags and block-scans the distinct ones
@@ -68,7 +74,7 @@ struct MutColPtrs {
 
 __device__ __forceinline__ uint32_t order_key(int32_t x) { return (uint32_t)x ^ 0x80000000u; }
 
-// The streaming kernels below (k_minmax, k_prep, k_pack, k_unpack, k_gather)
+// The streaming kernels below (k_minmax, k_prep, k_gather)
 // take EW_U elements per thread per step, a block's EW_U * blockDim.x
 // consecutive elements at a time, and issue all of a step's loads before using
 // them: one 4-byte load per thread in flight did not cover HBM latency.
@@ -150,28 +156,63 @@ __global__ void k_iota32(int32_t *__restrict__ out, int64_t n) {
         out[i] = (int32_t)i;
 }
 
-// Per-tile histogram of one digit: hist[d * tiles + t] = keys of tile t (ITEMS x 256
-// keys) whose digit at `shift` is d.  Per-warp counters in shared memory (a
-// whole warp on one digit is one add).
-template <typename K, int ITEMS>
-__global__ void __launch_bounds__(RS_THREADS) k_tile_hist(const K *__restrict__ keys, int64_t n, int shift,
-                                                          uint32_t *__restrict__ hist, unsigned tiles) {
+// Where the first digit pass reads its rows and the last one writes them: the
+// columns themselves, packed and unpacked on the way, so that no pass over the
+// rows is spent on packing or unpacking alone.
+struct RowIO {
+    ColPtrs src;
+    MutColPtrs dst;
+    PackSpec ps;
+    int k;
+    int64_t *d_rows, *h_rows;  // row count of the result (written with dst)
+};
+
+// keys of rows i(j), j < ITEMS, from the columns in `need` (bit c: column c):
+// column 0 most significant; field c holds order_key(col_c) - min_c in bits
+// [shift_c, shift_c + bits_c); a constant column has no field.  Rows at or past
+// n read as key 0.
+template <typename K, int ITEMS, class Index>
+__device__ __forceinline__ void pack_rows(const RowIO &io, unsigned need, int64_t n, Index at, K *key) {
+#pragma unroll
+    for (int j = 0; j < ITEMS; ++j) key[j] = 0;
+#pragma unroll
+    for (int c = 0; c < TID_MAX_COLS; ++c) {
+        if (!((need >> c) & 1u)) continue;
+        int32_t x[ITEMS];
+#pragma unroll
+        for (int j = 0; j < ITEMS; ++j) x[j] = at(j) < n ? io.src.c[c][at(j)] : 0;
+#pragma unroll
+        for (int j = 0; j < ITEMS; ++j)
+            if (at(j) < n) key[j] |= (K)(order_key(x[j]) - io.ps.min[c]) << io.ps.shift[c];
+    }
+}
+
+// Per-tile histogram of one digit (`dbits` bits at `shift`): hist[d * tiles + t] =
+// keys of tile t (ITEMS x 256 keys) whose digit is d.  Per-warp counters in shared
+// memory (a whole warp on one digit is one add).  SRC: the keys are packed from
+// the columns in `need`, those that hold bits of the digit.
+template <typename K, int ITEMS, bool SRC>
+__global__ void __launch_bounds__(RS_THREADS)
+k_tile_hist(const K *__restrict__ keys, int64_t n, int shift, int dbits, uint32_t *__restrict__ hist, unsigned tiles,
+            RowIO io, unsigned need) {
     __shared__ uint32_t s_h[RS_WARPS][RS_BINS];
     const unsigned lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const unsigned dmask = (1u << dbits) - 1u;
     for (int i = threadIdx.x; i < RS_WARPS * RS_BINS; i += RS_THREADS) (&s_h[0][0])[i] = 0;
     __syncthreads();
     const int64_t base = (int64_t)blockIdx.x * (RS_THREADS * ITEMS);
     K k[ITEMS];
+    auto at = [&](int j) { return base + j * RS_THREADS + threadIdx.x; };
+    if constexpr (SRC) {
+        pack_rows<K, ITEMS>(io, need, n, at, k);
+    } else {
 #pragma unroll
-    for (int j = 0; j < ITEMS; ++j) {
-        const int64_t i = base + j * RS_THREADS + threadIdx.x;
-        k[j] = i < n ? keys[i] : (K)0;
+        for (int j = 0; j < ITEMS; ++j) k[j] = at(j) < n ? keys[at(j)] : (K)0;
     }
 #pragma unroll
     for (int j = 0; j < ITEMS; ++j) {
-        const int64_t i = base + j * RS_THREADS + threadIdx.x;
-        const bool valid = i < n;
-        const unsigned d = valid ? (unsigned)(k[j] >> shift) & 0xFFu : 0x100u;
+        const bool valid = at(j) < n;
+        const unsigned d = valid ? (unsigned)(k[j] >> shift) & dmask : 0x100u;
         const unsigned d0 = __shfl_sync(0xffffffffu, d, 0);
         if (__all_sync(0xffffffffu, d == d0)) {
             if (lane == 0 && d0 < 0x100u) s_h[warp][d0] += 32u;
@@ -183,7 +224,7 @@ __global__ void __launch_bounds__(RS_THREADS) k_tile_hist(const K *__restrict__ 
     uint32_t c = 0;
 #pragma unroll
     for (int w = 0; w < RS_WARPS; ++w) c += s_h[w][threadIdx.x];
-    hist[(size_t)threadIdx.x * tiles + blockIdx.x] = c;
+    if (threadIdx.x <= dmask) hist[(size_t)threadIdx.x * tiles + blockIdx.x] = c;
 }
 
 // In place: row d of the per-tile histograms (hist[d * tiles + t]) becomes its
@@ -229,10 +270,13 @@ __global__ void __launch_bounds__(1024) k_digit_scan(uint32_t *__restrict__ hist
 // The offset of (digit d, tile t) is the keys of smaller digits (the exclusive
 // scan of tot) plus offs[d * tiles + t], the row-scanned per-tile histograms
 // (k_tile_hist, k_digit_scan), so no tile waits for another.
-template <typename K, bool HAS_VAL, int ITEMS, int MINB>
+// SRC: the rows come from the columns of io (packed here), DST: they go to its
+// output columns (unpacked here).
+template <typename K, bool HAS_VAL, int ITEMS, int MINB, bool SRC, bool DST>
 __global__ void __launch_bounds__(RS_THREADS, MINB)
 k_onesweep(const K *__restrict__ kin, const int32_t *__restrict__ vin, K *__restrict__ kout, int32_t *__restrict__ vout,
-           int64_t n, int shift, const uint32_t *__restrict__ offs, const uint32_t *__restrict__ tot, unsigned tiles) {
+           int64_t n, int shift, int dbits, const uint32_t *__restrict__ offs, const uint32_t *__restrict__ tot,
+           unsigned tiles, RowIO io, unsigned need) {
     __shared__ uint32_t s_wcnt[RS_WARPS][RS_BINS];
     __shared__ uint32_t s_gbase[RS_BINS];
     __shared__ uint32_t s_wsum[RS_WARPS], s_wtot[RS_WARPS];
@@ -241,8 +285,13 @@ k_onesweep(const K *__restrict__ kin, const int32_t *__restrict__ vin, K *__rest
 
     const unsigned lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const unsigned lt = (1u << lane) - 1u;
+    const unsigned dmask = (1u << dbits) - 1u;
     for (int i = threadIdx.x; i < RS_WARPS * RS_BINS; i += RS_THREADS) (&s_wcnt[0][0])[i] = 0;
     const unsigned tile = blockIdx.x;
+    if (DST && tile == 0 && threadIdx.x == 0) {
+        *io.d_rows = n;
+        *io.h_rows = n;
+    }
     {
         // this tile's first output position per digit (one digit per thread):
         // the keys of smaller digits (exclusive scan of tot) + this digit's
@@ -251,7 +300,8 @@ k_onesweep(const K *__restrict__ kin, const int32_t *__restrict__ vin, K *__rest
         // tot == nullptr: the histograms were not scanned (a sort of at most
         // RS_FEW_TILES tiles); the digit's row is summed here instead
         uint32_t t = 0, pre = 0;
-        if (tot) {
+        if (d > dmask) {  // not a digit
+        } else if (tot) {
             t = tot[d];
             pre = offs[(size_t)d * tiles + tile];
         } else {
@@ -288,12 +338,16 @@ k_onesweep(const K *__restrict__ kin, const int32_t *__restrict__ vin, K *__rest
     K k[ITEMS];
     uint32_t r[ITEMS / 2];  // ranks within the warp (< 32 ITEMS), two per register
     int32_t v[HAS_VAL ? ITEMS : 1];
+    if constexpr (SRC) {
+        pack_rows<K, ITEMS>(io, need, n, [&](int j) { return wbase + j * 32 + lane; }, k);
+    } else {
 #pragma unroll
-    for (int j = 0; j < ITEMS; ++j) {
-        const int64_t i = wbase + j * 32 + lane;
-        const bool valid = i < n;
-        k[j] = valid ? kin[i] : (K)0;
-        if (HAS_VAL) v[j] = valid ? vin[i] : 0;
+        for (int j = 0; j < ITEMS; ++j) {
+            const int64_t i = wbase + j * 32 + lane;
+            const bool valid = i < n;
+            k[j] = valid ? kin[i] : (K)0;
+            if (HAS_VAL) v[j] = valid ? vin[i] : 0;
+        }
     }
     // stable rank among this warp's rows with the same digit, in row order: the
     // first lane of each group of equal digits adds the group's size to the
@@ -310,19 +364,20 @@ k_onesweep(const K *__restrict__ kin, const int32_t *__restrict__ vin, K *__rest
         // ballot per digit bit (ALU work: alone, the ALU pipe bounded it).
         unsigned peers;
         if ((j & 1) == 0) {
-            peers = __match_any_sync(0xffffffffu, valid ? (unsigned)(k[j] >> shift) & 0xFFu : 0x100u);
+            peers = __match_any_sync(0xffffffffu, valid ? (unsigned)(k[j] >> shift) & dmask : 0x100u);
         } else {
-            const unsigned d = valid ? (unsigned)(k[j] >> shift) & 0xFFu : 0u;
+            const unsigned d = valid ? (unsigned)(k[j] >> shift) & dmask : 0u;
             peers = __ballot_sync(0xffffffffu, valid);  // separates the tail's invalid lanes
             if (!valid) peers = ~peers;
 #pragma unroll
             for (int b = 0; b < 8; ++b) {
+                if (b >= dbits) break;
                 const bool bit = (d >> b) & 1u;
                 const unsigned bb = __ballot_sync(0xffffffffu, bit);
                 peers &= bit ? bb : ~bb;
             }
         }
-        const unsigned d = valid ? (unsigned)(k[j] >> shift) & 0xFFu : 0u;
+        const unsigned d = valid ? (unsigned)(k[j] >> shift) & dmask : 0u;
         const int leader = __ffs(peers) - 1;
         uint32_t b = 0;
         if (valid && lane == (unsigned)leader) b = atomicAdd(&s_wcnt[warp][d], (uint32_t)__popc(peers));
@@ -373,7 +428,7 @@ k_onesweep(const K *__restrict__ kin, const int32_t *__restrict__ vin, K *__rest
     for (int j = 0; j < ITEMS; ++j) {
         const int64_t i = wbase + j * 32 + lane;
         if (i < n) {
-            const unsigned d = (unsigned)(k[j] >> shift) & 0xFFu;
+            const unsigned d = (unsigned)(k[j] >> shift) & dmask;
             const uint32_t lp = s_wcnt[warp][d] + ((r[j >> 1] >> (16 * (j & 1))) & 0xFFFFu);
             s_k[lp] = k[j];
             if (HAS_VAL) s_v[lp] = v[j];
@@ -383,62 +438,18 @@ k_onesweep(const K *__restrict__ kin, const int32_t *__restrict__ vin, K *__rest
     const int cnt = (int)(n - base < (RS_THREADS * ITEMS) ? n - base : (RS_THREADS * ITEMS));
     for (int i = threadIdx.x; i < cnt; i += RS_THREADS) {
         const K kk = s_k[i];
-        const unsigned d = (unsigned)(kk >> shift) & 0xFFu;
+        const unsigned d = (unsigned)(kk >> shift) & dmask;
         const uint32_t gp = s_gbase[d] + (uint32_t)i;  // wraps modulo 2^32 to the right position
-        kout[gp] = kk;
-        if (HAS_VAL) vout[gp] = s_v[i];
-    }
-}
-
-// packed key of a row: column 0 most significant; field c holds
-// order_key(col_c) - min_c in bits [shift_c, shift_c + bits_c)
-template <typename K>
-__global__ void __launch_bounds__(EW_THREADS) k_pack(ColPtrs cols, int k, int64_t n, PackSpec ps,
-                                                     K *__restrict__ keys) {
-    for (int64_t i0 = ew_first(); i0 < n; i0 += ew_stride()) {
-        K key[EW_U];
+        if constexpr (DST) {
 #pragma unroll
-        for (int u = 0; u < EW_U; ++u) key[u] = 0;
-#pragma unroll
-        for (int c = 0; c < TID_MAX_COLS; ++c) {  // a constant column (mask 0) has no field
-            if (c >= k || !ps.mask[c]) continue;
-            int32_t x[EW_U];
-#pragma unroll
-            for (int u = 0; u < EW_U; ++u) {
-                const int64_t i = i0 + u * EW_THREADS;
-                x[u] = i < n ? cols.c[c][i] : 0;
+            for (int c = 0; c < TID_MAX_COLS; ++c) {
+                if (c >= io.k) break;
+                const uint32_t f = io.ps.mask[c] ? (uint32_t)((kk >> io.ps.shift[c]) & io.ps.mask[c]) : 0u;
+                io.dst.c[c][gp] = (int32_t)((f + io.ps.min[c]) ^ 0x80000000u);
             }
-#pragma unroll
-            for (int u = 0; u < EW_U; ++u) key[u] |= (K)(order_key(x[u]) - ps.min[c]) << ps.shift[c];
-        }
-#pragma unroll
-        for (int u = 0; u < EW_U; ++u) {
-            const int64_t i = i0 + u * EW_THREADS;
-            if (i < n) keys[i] = key[u];
-        }
-    }
-}
-
-// sorted packed keys -> k columns (no duplicate removal)
-template <typename K>
-__global__ void __launch_bounds__(EW_THREADS) k_unpack(const K *__restrict__ keys, int k, int64_t n, PackSpec ps,
-                                                       MutColPtrs out) {
-    for (int64_t i0 = ew_first(); i0 < n; i0 += ew_stride()) {
-        K key[EW_U];
-#pragma unroll
-        for (int u = 0; u < EW_U; ++u) {
-            const int64_t i = i0 + u * EW_THREADS;
-            key[u] = i < n ? keys[i] : (K)0;
-        }
-#pragma unroll
-        for (int c = 0; c < TID_MAX_COLS; ++c) {
-            if (c >= k) continue;
-#pragma unroll
-            for (int u = 0; u < EW_U; ++u) {
-                const int64_t i = i0 + u * EW_THREADS;
-                const uint32_t f = ps.mask[c] ? (uint32_t)((key[u] >> ps.shift[c]) & ps.mask[c]) : 0u;
-                if (i < n) out.c[c][i] = (int32_t)((f + ps.min[c]) ^ 0x80000000u);
-            }
+        } else {
+            kout[gp] = kk;
+            if (HAS_VAL) vout[gp] = s_v[i];
         }
     }
 }
@@ -604,34 +615,57 @@ static int column_ranges(tid_ctx *ctx, const int32_t *const *cols, int k, int64_
 
 static int range_bits(uint32_t lo, uint32_t hi) { return hi == lo ? 0 : 32 - __builtin_clz(hi - lo); }
 
-// Each digit: per-tile histograms, one scan of the (digit, tile) counts, then
-// the ranking and scatter at the scanned offsets.
-template <typename K, bool HAS_VAL>
-static int radix_passes(tid_ctx *ctx, K *&ka, K *&kb, int32_t *&pa, int32_t *&pb, int64_t n, int shift0,
-                        int passes);
-
+// The digit passes over `bits` key bits from `shift0` up, in digits of equal
+// width: per pass the per-tile histograms, one scan of the (digit, tile) counts,
+// and the ranking and scatter at the scanned offsets.  Without io: from ka (and
+// the rows pa) to ka again (the buffers are swapped).  With io: pass 0 reads the
+// columns of io; the last pass writes its output columns when `dst`, else ka.
 template <typename K, bool HAS_VAL, int ITEMS, int MINB>
 static int radix_passes_shaped(tid_ctx *ctx, K *&ka, K *&kb, int32_t *&pa, int32_t *&pb, int64_t n, int shift0,
-                               int passes) {
+                               int bits, const RowIO *io, bool dst) {
     const unsigned tiles = (unsigned)ceil_div(n, RS_THREADS * ITEMS);
+    const int passes = (bits + 7) / 8;
+    if (passes == 0) return TID_OK;
     uint32_t *offs = nullptr;
     TID_TRY(dev_alloc(ctx, (void **)&offs, sizeof(uint32_t) * (size_t)RS_BINS * (tiles + 1)));
     uint32_t *tot = offs + (size_t)RS_BINS * tiles;
+    const RowIO none{};
+    const RowIO &r = io ? *io : none;
+    cudaStream_t st = ctx->stream;
     int rc = TID_OK;
-    for (int p = 0; p < passes && rc == TID_OK; ++p) {
-        const int shift = shift0 + 8 * p;
-        k_tile_hist<K, ITEMS><<<tiles, RS_THREADS, 0, ctx->stream>>>(ka, n, shift, offs, tiles);
+    for (int p = 0, at = 0; p < passes && rc == TID_OK; ++p) {
+        const int shift = shift0 + at, dbits = (bits - at + passes - p - 1) / (passes - p);
+        at += dbits;
+        const bool src = io && p == 0, out = io && dst && p == passes - 1;
+        unsigned need = 0, all = 0;  // columns that hold bits of the digit; columns with a field
+        for (int c = 0; src && c < r.k; ++c) {
+            if (!r.ps.mask[c]) continue;
+            const int lo = (int)r.ps.shift[c], hi = lo + 64 - __builtin_clzll(r.ps.mask[c]);
+            all |= 1u << c;
+            if (lo < shift + dbits && hi > shift) need |= 1u << c;
+        }
+        if (src) k_tile_hist<K, ITEMS, true><<<tiles, RS_THREADS, 0, st>>>(nullptr, n, shift, dbits, offs, tiles, r, need);
+        else k_tile_hist<K, ITEMS, false><<<tiles, RS_THREADS, 0, st>>>(ka, n, shift, dbits, offs, tiles, r, 0);
         rc = launch_check("k_tile_hist");
         const bool scan = tiles > RS_FEW_TILES;  // else each scatter CTA sums its digits' rows itself
         if (rc == TID_OK && scan) {
-            k_digit_scan<<<RS_BINS, 1024, 0, ctx->stream>>>(offs, tiles, tot);
+            k_digit_scan<<<1u << dbits, 1024, 0, st>>>(offs, tiles, tot);
             rc = launch_check("k_digit_scan");
         }
-        if (rc == TID_OK) {
-            k_onesweep<K, HAS_VAL, ITEMS, MINB><<<tiles, RS_THREADS, 0, ctx->stream>>>(ka, pa, kb, pb, n, shift, offs,
-                                                                                scan ? tot : nullptr, tiles);
-            rc = launch_check("k_onesweep");
+        if (rc != TID_OK) break;
+        const uint32_t *t = scan ? tot : nullptr;
+#define RS_SWEEP(S, D) \
+    k_onesweep<K, HAS_VAL, ITEMS, MINB, S, D><<<tiles, RS_THREADS, 0, st>>>(ka, pa, kb, pb, n, shift, dbits, offs, t, tiles, r, all)
+        if constexpr (HAS_VAL) {
+            RS_SWEEP(false, false);
+        } else {
+            if (src && out) RS_SWEEP(true, true);
+            else if (src) RS_SWEEP(true, false);
+            else if (out) RS_SWEEP(false, true);
+            else RS_SWEEP(false, false);
         }
+#undef RS_SWEEP
+        rc = launch_check("k_onesweep");
         std::swap(ka, kb);
         if (HAS_VAL) std::swap(pa, pb);
     }
@@ -640,15 +674,15 @@ static int radix_passes_shaped(tid_ctx *ctx, K *&ka, K *&kb, int32_t *&pa, int32
 }
 
 template <typename K, bool HAS_VAL>
-static int radix_passes(tid_ctx *ctx, K *&ka, K *&kb, int32_t *&pa, int32_t *&pb, int64_t n, int shift0,
-                        int passes) {
+static int radix_passes(tid_ctx *ctx, K *&ka, K *&kb, int32_t *&pa, int32_t *&pb, int64_t n, int shift0, int bits,
+                        const RowIO *io = nullptr, bool dst = false) {
     if constexpr (sizeof(K) == 4 && !HAS_VAL) {
-        return radix_passes_shaped<K, HAS_VAL, 16, 4>(ctx, ka, kb, pa, pb, n, shift0, passes);
+        return radix_passes_shaped<K, HAS_VAL, 16, 4>(ctx, ka, kb, pa, pb, n, shift0, bits, io, dst);
     } else if constexpr (sizeof(K) == 8) {
-        if (n <= RS_SMALL) return radix_passes_shaped<K, HAS_VAL, 12, 4>(ctx, ka, kb, pa, pb, n, shift0, passes);
-        return radix_passes_shaped<K, HAS_VAL, 16, 3>(ctx, ka, kb, pa, pb, n, shift0, passes);
+        if (n <= RS_SMALL) return radix_passes_shaped<K, HAS_VAL, 12, 4>(ctx, ka, kb, pa, pb, n, shift0, bits, io, dst);
+        return radix_passes_shaped<K, HAS_VAL, 16, 3>(ctx, ka, kb, pa, pb, n, shift0, bits, io, dst);
     } else {
-        return radix_passes_shaped<K, HAS_VAL, 16, 3>(ctx, ka, kb, pa, pb, n, shift0, passes);
+        return radix_passes_shaped<K, HAS_VAL, 16, 3>(ctx, ka, kb, pa, pb, n, shift0, bits, io, dst);
     }
 }
 
@@ -666,7 +700,6 @@ static int sort_perm_ranges(tid_ctx *ctx, const int32_t *const *keys, int nk, in
     for (int c = nk - 1 - sorted_tail; c >= 0; --c) {
         const int bits = range_bits(hmin[c], hmax[c]);
         if (bits == 0) continue;  // constant column: order unchanged
-        const int passes = (bits + 7) / 8;
         if (!ka) {
             TID_TRY(s.get(&ka, n));
             TID_TRY(s.get(&kb, n));
@@ -675,7 +708,7 @@ static int sort_perm_ranges(tid_ctx *ctx, const int32_t *const *keys, int nk, in
         }
         k_prep<<<grid_for(n, EW_THREADS * EW_U, 8), EW_THREADS, 0, st>>>(keys[c], have_perm ? pa : nullptr, n, hmin[c], ka, pa);
         TID_TRY(launch_check("k_prep"));
-        TID_TRY((radix_passes<uint32_t, true>(ctx, ka, kb, pa, pb, n, 0, passes)));
+        TID_TRY((radix_passes<uint32_t, true>(ctx, ka, kb, pa, pb, n, 0, bits)));
         have_perm = true;
     }
     if (have_perm) {
@@ -695,8 +728,9 @@ int sort_perm(tid_ctx *ctx, const int32_t *const *keys, int nk, int64_t n, int32
     return sort_perm_ranges(ctx, keys, nk, n, hmin, hmax, perm);
 }
 
-// Canonical form by sorting packed keys (all fields fit K): pack, keys-only
-// digit passes over the occupied bits, then unpack (with distinct rows kept).
+// Canonical form by sorting packed keys (all fields fit K): keys-only digit
+// passes over the occupied bits, the first from the columns; the last into the
+// result's columns, or (distinct rows kept) to keys that one selection unpacks.
 // The rows are already ordered by the low `sorted_bits` bits of their keys
 // (the fields of trailing columns they are sorted by): the digit passes start
 // above them.
@@ -717,23 +751,32 @@ static int canonical_packed(tid_ctx *ctx, const int32_t *const *cols, int k, int
         if (!dedupe) set->rows_known = n;
         return TID_OK;
     }
+    const int bits = total_bits - sorted_bits, passes = (bits + 7) / 8;
+    if (passes == 0 && !dedupe) {  // in order already
+        for (int c = 0; c < k; ++c)
+            TID_TRY_CUDA(cudaMemcpyAsync(set->col[c], cols[c], (size_t)n * 4, cudaMemcpyDeviceToDevice, st), "copy rows");
+        return set_rows_const(set, n);
+    }
+    if (passes == 0) return compact_unique(ctx, cols, k, nullptr, n, set);
     Scratch s(ctx);
     K *ka = nullptr, *kb = nullptr;
     int32_t *none_a = nullptr, *none_b = nullptr;
-    const int passes = (total_bits - sorted_bits + 7) / 8;
-    TID_TRY(s.get(&ka, n));
-    TID_TRY(s.get(&kb, n));
-    ColPtrs cp{};
-    for (int c = 0; c < k; ++c) cp.c[c] = cols[c];
-    k_pack<K><<<grid_for(n, EW_THREADS * EW_U, 8), EW_THREADS, 0, st>>>(cp, k, n, ps, ka);
-    TID_TRY(launch_check("k_pack"));
-    TID_TRY((radix_passes<K, false>(ctx, ka, kb, none_a, none_b, n, sorted_bits, passes)));
+    // pass 0 reads the columns, so the first buffer is written by the second pass at the earliest
+    if (passes > 2 || (passes == 2 && dedupe)) TID_TRY(s.get(&ka, n));
+    if (passes > 1 || dedupe) TID_TRY(s.get(&kb, n));
+    RowIO io{};
+    for (int c = 0; c < k; ++c) {
+        io.src.c[c] = cols[c];
+        io.dst.c[c] = set->col[c];
+    }
+    io.ps = ps;
+    io.k = k;
+    io.d_rows = set->d_rows;
+    io.h_rows = set->slot.dev;
+    TID_TRY((radix_passes<K, false>(ctx, ka, kb, none_a, none_b, n, sorted_bits, bits, &io, !dedupe)));
     if (dedupe) return compact_unique_packed(ctx, ka, sizeof(K) == 8, k, n, ps, set);
-    MutColPtrs op{};
-    for (int c = 0; c < k; ++c) op.c[c] = set->col[c];
-    k_unpack<K><<<grid_for(n, EW_THREADS * EW_U, 8), EW_THREADS, 0, st>>>(ka, k, n, ps, op);
-    TID_TRY(launch_check("k_unpack"));
-    return set_rows_const(set, n);
+    set->rows_known = n;
+    return TID_OK;
 }
 
 int gather_cols(tid_ctx *ctx, const int32_t *const *in, int k, const int32_t *perm, int64_t n,
