@@ -301,9 +301,11 @@ int tid_filter(tid_ctx *ctx, const tid_set *in, const tid_pred *preds, int n_pre
  * side).  A pair joins when every shared column is equal and non-zero.
  * Output columns: L's, then R's non-shared ones in R's order (at most
  * TID_MAX_COLS).  No shared variable gives the cross product.  Algorithms:
- * sort-merge (sort both sides on the key, count matches per left row by
- * binary search, scan, write) or hash (group the smaller side by key in an
- * open-addressing table, probe with the other).  Output canonical.  The
+ * sort-merge (each left row finds its run of equal keys in the right side,
+ * which is sorted on the key first unless it leads with it) or hash (group the
+ * smaller side by key in an open-addressing table, probe with the other, sort
+ * the joined rows); TID_JOIN_AUTO takes the first when the right side leads
+ * with the shared variables.  Output canonical.  The
  * count phase is followed by one synchronisation to size the output; more
  * than 2^31-1 output rows is TID_ERR_CAPACITY.  algo is TID_JOIN_AUTO,
  * TID_JOIN_SORT_MERGE or TID_JOIN_HASH, optionally or-ed with TID_JOIN_LEFT,

@@ -13,9 +13,18 @@
 // by binary search over the scanned counts, so a key with millions of matches
 // is spread over as many threads (no per-row serial loops).
 //
-//  * sort-merge: both sides ordered by the key (free when the key columns are
-//    a prefix of a canonical set's column order; else a radix-sorted
-//    permutation); per left row, lower/upper bound in the right keys.
+//  * runs: the right side leads with the key columns, so a key's rows are one run
+//    of it, ordered by its other columns; each left row, whatever its order by
+//    the key, finds its run and is written with it, which is canonical order --
+//    no sort.  A run is found through a table over the range of the first key
+//    column (a bucket's first and one-past-last right row), then by binary
+//    search inside the bucket where it holds more than the one key.
+//  * members: when one side holds a single key column and nothing else, the
+//    join keeps the rows of the other side whose key is among its terms (one
+//    bit per term): a row selection, no search and no count read-back.
+//  * sort-merge (the right side does not lead with the key): both sides ordered
+//    by the key (a radix-sorted permutation where it is no prefix); per left
+//    row, lower/upper bound in the right keys.
 //  * hash: the smaller side is grouped by key in an open-addressing table
 //    (key -> [start, count) into a grouped row array, built with CAS inserts,
 //    a scan and a scatter); the other side probes it.  A table of at most
@@ -135,6 +144,85 @@ __device__ __forceinline__ void warp_bracket(const Cols &RK, const Cols &LK, int
 // per left row: [lo, hi) of equal keys in the sorted right keys
 constexpr uint32_t NO_MATCH = 0xFFFFFFFFu;  // left outer join: a left row written once, padded
 
+// Where the right rows of a first-key term lie: bucket (order(term) - lo) >> shift
+// holds rows [x, y) (x == y: none), for terms with order in [lo, lo + span].
+// At most one bucket per right row, so the table is no
+// larger than two columns of the right side and stays in L2 with it; IDs of a
+// graph are dense, and the shift is then 0.
+struct RunTable {
+    uint2 *bucket;  // null: none (search the whole right side)
+    uint32_t lo, span;
+    int shift;
+};
+
+__device__ __forceinline__ uint32_t sort_order(int32_t x) { return (uint32_t)x ^ 0x80000000u; }
+
+__global__ void __launch_bounds__(256) k_run_table(const int32_t *__restrict__ key, int64_t nr, RunTable t) {
+    constexpr int U = 4;
+    for (int64_t i0 = (int64_t)blockIdx.x * (256 * U) + threadIdx.x; i0 < nr; i0 += (int64_t)gridDim.x * (256 * U)) {
+        int32_t x[U], y[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int64_t i = min(i0 + u * 256, nr - 1);
+            x[u] = key[i];
+            y[u] = key[i > 0 ? i - 1 : 0];
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int64_t i = i0 + u * 256;
+            if (i >= nr) break;
+            const uint32_t dx = sort_order(x[u]) - t.lo, dy = sort_order(y[u]) - t.lo;
+            if (dx > t.span || dy > t.span) continue;  // outside the column's bounds: not a row of this column
+            const uint32_t b = dx >> t.shift, p = dy >> t.shift;
+            if (i == 0 || b != p) {
+                t.bucket[b].x = (uint32_t)i;
+                if (i > 0) t.bucket[p].y = (uint32_t)i;
+            }
+            if (i == nr - 1) t.bucket[b].y = (uint32_t)nr;
+        }
+    }
+}
+
+// cnt[l] right rows match left row l, from lo_out[l] on; exact: a bucket of the
+// table holds the rows of one key
+__global__ void __launch_bounds__(256) k_run_count(Cols LK, int64_t nl, Cols RK, int nk, bool left, RunTable t, bool exact,
+                                                   uint32_t *__restrict__ cnt, uint32_t *__restrict__ lo_out,
+                                                   unsigned long long *__restrict__ total) {
+    constexpr int U = 4;  // rows per thread whose table reads are in flight together
+    unsigned long long acc = 0;
+    for (int64_t l0 = (int64_t)blockIdx.x * (256 * U) + threadIdx.x; l0 < nl; l0 += (int64_t)gridDim.x * (256 * U)) {
+        uint2 b[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int64_t l = min(l0 + u * 256, nl - 1);
+            const int32_t x = LK.c[0][l];
+            const uint32_t d = sort_order(x) - t.lo;
+            b[u] = x != 0 && d <= t.span ? t.bucket[d >> t.shift] : make_uint2(0, 0);
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int64_t l = l0 + u * 256;
+            if (l >= nl) break;
+            uint32_t c = b[u].y - b[u].x, lo = b[u].x;
+            if (!exact && c) {
+                int64_t a = 0, a2 = 0;
+                if (!has_zero(LK, l, nk)) eq_range(RK, LK, l, nk, b[u].x, b[u].y, &a, &a2);
+                lo = (uint32_t)a;
+                c = (uint32_t)(a2 - a);
+            }
+            if (left && c == 0) {
+                c = 1;
+                lo = NO_MATCH;
+            }
+            cnt[l] = c;
+            lo_out[l] = lo;
+            acc += c;
+        }
+    }
+    block_add_u64(acc, total);  // once per warp: one address takes these atomics one at a time
+}
+
+// The same by binary search over all of the right keys; the left keys are sorted.
 __global__ void k_sm_count(Cols LK, int64_t nl, Cols RK, int64_t nr, int nk, bool left, uint32_t *__restrict__ cnt,
                            uint32_t *__restrict__ lo_out, unsigned long long *__restrict__ total) {
     unsigned long long acc = 0;
@@ -190,26 +278,13 @@ __device__ __forceinline__ int64_t jw_split(const uint32_t *__restrict__ off, in
     return lo;
 }
 
-__device__ __forceinline__ void join_row(const uint32_t *__restrict__ lo, const int32_t *__restrict__ lperm,
-                                         const int32_t *__restrict__ rmap, const int32_t *__restrict__ rperm,
-                                         const Cols &L, int kl, const Cols &Rrest, int nrest, const MCols &outL,
-                                         const MCols &outR, bool left_is_probe, int64_t l, uint32_t lol, int64_t k,
-                                         int64_t o) {
-    if (lol == NO_MATCH) {  // left outer join: the left row alone, right columns unbound
-        write_out(L, kl, Rrest, nrest, lperm ? lperm[l] : l, -1, outL, outR, o);
-        return;
-    }
-    const int64_t j = (int64_t)lol + k;
-    int64_t lr, rr;
-    if (left_is_probe) {
-        lr = lperm ? lperm[l] : l;
-        rr = rmap ? rmap[j] : j;
-        if (rperm) rr = rperm[rr];
-    } else {  // hash join built on the left: "l" walks right rows, j indexes grouped left rows
-        rr = l;
-        lr = rmap[j];
-    }
-    write_out(L, kl, Rrest, nrest, lr, rr, outL, outR, o);
+// split[t] = rows among the first t JW_TILE items, for every tile boundary (its own
+// launch: a search inside the write kernel was some twenty dependent loads at the
+// start of every CTA)
+__global__ void __launch_bounds__(256) k_join_split(const uint32_t *__restrict__ off, int64_t nl, int64_t total,
+                                                    int64_t tiles, uint32_t *__restrict__ split) {
+    const int64_t t = (int64_t)blockIdx.x * 256 + threadIdx.x;
+    if (t <= tiles) split[t] = (uint32_t)jw_split(off, nl, total, min(t * JW_TILE, nl + total));
 }
 
 __global__ void __launch_bounds__(JW_THREADS) k_join_write(const uint32_t *__restrict__ off, int64_t nl,
@@ -218,25 +293,28 @@ __global__ void __launch_bounds__(JW_THREADS) k_join_write(const uint32_t *__res
                                                            const int32_t *__restrict__ rmap,
                                                            const int32_t *__restrict__ rperm, int64_t total, Cols L,
                                                            int kl, Cols Rrest, int nrest, MCols outL, MCols outR,
-                                                           bool left_is_probe) {
-    __shared__ uint32_t s_off[JW_TILE + 1];  // off[rb .. r1 - 1]
-    __shared__ int64_t s_r[2];
+                                                           bool left_is_probe, const uint32_t *__restrict__ split) {
+    __shared__ uint32_t s_off[JW_TILE + 1], s_lo[JW_TILE + 1];  // of rows rb .. r1 - 1
     const int64_t d0 = (int64_t)blockIdx.x * JW_TILE, d1 = min(d0 + JW_TILE, nl + total);
-    if (threadIdx.x < 2) s_r[threadIdx.x] = jw_split(off, nl, total, threadIdx.x == 0 ? d0 : d1);
-    __syncthreads();
-    const int64_t r0 = s_r[0], r1 = s_r[1];
+    const int64_t r0 = split[blockIdx.x], r1 = split[blockIdx.x + 1];
     const int64_t o0 = d0 - r0, o1 = d1 - r1;
     if (o0 >= o1) return;  // only rows here
     // the output rows [o0, o1) belong to rows rb .. r1 - 1: row r0 - 1 precedes
     // output o0 in the merged order (off[r0 - 1] <= o0), row r1 follows o1 - 1
     const int64_t rb = r0 > 0 ? r0 - 1 : 0;
     const int nr = (int)(r1 - rb);
-    for (int i = threadIdx.x; i < nr; i += JW_THREADS) s_off[i] = off[rb + i];
+    for (int i = threadIdx.x; i < nr; i += JW_THREADS) {
+        s_off[i] = off[rb + i];
+        s_lo[i] = lo[rb + i];
+    }
     __syncthreads();
+    // every output row's left and right row first, then column by column, so
+    // that a column's reads are in flight together
+    int32_t lr[JW_ITEMS], rr[JW_ITEMS];
+    const int64_t last = o1 - 1;
 #pragma unroll
     for (int q = 0; q < JW_ITEMS; ++q) {
-        const int64_t o = o0 + q * JW_THREADS + threadIdx.x;
-        if (o >= o1) break;
+        const int64_t o = min(o0 + q * JW_THREADS + threadIdx.x, last);
         // last i with s_off[i] <= o.  First guess: rows of one match each
         // (the common case) put output o at row o - s_off[0] of the tile.
         int a = (int)min((int64_t)(nr - 1), o - (int64_t)s_off[0]);
@@ -249,8 +327,54 @@ __global__ void __launch_bounds__(JW_THREADS) k_join_write(const uint32_t *__res
                 else b = m;
             }
         }
-        const int64_t l = rb + a;
-        join_row(lo, lperm, rmap, rperm, L, kl, Rrest, nrest, outL, outR, left_is_probe, l, lo[l], o - s_off[a], o);
+        lr[q] = (int32_t)(rb + a);
+        // left outer join: a left row alone, right columns unbound (-1)
+        rr[q] = s_lo[a] == NO_MATCH ? -1 : (int32_t)(s_lo[a] + (uint32_t)(o - s_off[a]));
+    }
+    if (!left_is_probe) {  // hash join built on the left: the probe rows are right rows, rr indexes grouped left rows
+#pragma unroll
+        for (int q = 0; q < JW_ITEMS; ++q) {
+            const int32_t j = rmap[rr[q]];
+            rr[q] = lr[q];
+            lr[q] = j;
+        }
+    } else {
+        if (lperm) {
+#pragma unroll
+            for (int q = 0; q < JW_ITEMS; ++q) lr[q] = lperm[lr[q]];
+        }
+        if (rmap) {
+#pragma unroll
+            for (int q = 0; q < JW_ITEMS; ++q) rr[q] = rr[q] < 0 ? -1 : rmap[rr[q]];
+        }
+        if (rperm) {
+#pragma unroll
+            for (int q = 0; q < JW_ITEMS; ++q) rr[q] = rr[q] < 0 ? -1 : rperm[rr[q]];
+        }
+    }
+#pragma unroll
+    for (int c = 0; c < TID_MAX_COLS; ++c) {
+        if (c >= kl) break;
+        int32_t v[JW_ITEMS];
+#pragma unroll
+        for (int q = 0; q < JW_ITEMS; ++q) v[q] = L.c[c][lr[q]];
+#pragma unroll
+        for (int q = 0; q < JW_ITEMS; ++q) {
+            const int64_t o = o0 + q * JW_THREADS + threadIdx.x;
+            if (o < o1) outL.c[c][o] = v[q];
+        }
+    }
+#pragma unroll
+    for (int c = 0; c < TID_MAX_COLS; ++c) {
+        if (c >= nrest) break;
+        int32_t v[JW_ITEMS];
+#pragma unroll
+        for (int q = 0; q < JW_ITEMS; ++q) v[q] = rr[q] < 0 ? 0 : Rrest.c[c][rr[q]];
+#pragma unroll
+        for (int q = 0; q < JW_ITEMS; ++q) {
+            const int64_t o = o0 + q * JW_THREADS + threadIdx.x;
+            if (o < o1) outR.c[c][o] = v[q];
+        }
     }
 }
 
@@ -590,7 +714,11 @@ int join_sets(tid_ctx *ctx, const tid_set *L, const tid_set *R, int algo, tid_se
         lprefix = lprefix && lkey[i] == i;
         rprefix = rprefix && rkey[i] == i;
     }
-    if (algo == TID_JOIN_AUTO) algo = (nk == 0 || (lprefix && rprefix)) ? TID_JOIN_SORT_MERGE : TID_JOIN_HASH;
+    // runs (or members, or a merge of two sorted sides) need the right side alone
+    // to lead with the key; a sort of the joined rows is what the hash join costs
+    // (8M x 8M rows, 11.5M joined, on GB300: 2318 us by hash and sort, 280 us by
+    // runs, bound by the table lookups' and the right rows' random reads in L2)
+    if (algo == TID_JOIN_AUTO) algo = (nk == 0 || rprefix) ? TID_JOIN_SORT_MERGE : TID_JOIN_HASH;
     if (nk == 0 || left) algo = TID_JOIN_SORT_MERGE;  // cross product; left outer join
     if (!sorted_out && (algo != TID_JOIN_HASH || nk == 0 || left))
         return fail(TID_ERR_ARG, "join: unsorted output is for inner hash joins");
@@ -615,6 +743,31 @@ int join_sets(tid_ctx *ctx, const tid_set *L, const tid_set *R, int algo, tid_se
         *out = res;
         return TID_OK;
     };
+    if (algo == TID_JOIN_SORT_MERGE && !left && nk == 1 && lprefix && rprefix && (L->k == 1 || R->k == 1)) {
+        // members: Q's rows whose key is among B's terms.  Q is read once, so not
+        // when B is so small that its searches of Q cost less (the bits of B's
+        // range are cleared and set first: at most as many bytes as both sides).
+        // 0.5M keys against 8.2M rows: 127 us by k_merge_join (dependent searches),
+        // 70 us as a selection
+        const bool b_is_l = L->k == 1 && (R->k > 1 || nl <= nr);
+        const tid_set *B = b_is_l ? L : R, *Q = b_is_l ? R : L;
+        const int64_t nb = b_is_l ? nl : nr, nq = b_is_l ? nr : nl;
+        const uint64_t w = B->bounded ? (uint64_t)B->hi[0] - B->lo[0] + 1 : ~0ull;
+        if (w <= (uint64_t)(32 * (nl + nr)) && w <= 0xFFFFFFFFull && (!b_is_l || nq <= 64 * nb)) {
+            Members m{};
+            TID_TRY(member_bits(ctx, B->col[0], nb, B->lo[0], B->hi[0], &m));
+            tid_set *res = nullptr;
+            int rc = set_alloc(ctx, kout, ovars, nq, &res);
+            if (rc == TID_OK) rc = compact_member(ctx, Q, nq, m, res);
+            dev_free(ctx, (void *)m.bits);
+            if (rc == TID_OK) rc = set_ready(res);
+            if (rc != TID_OK) {
+                if (res) set_free(res);
+                return rc;
+            }
+            return finish(res);
+        }
+    }
     if (sorted_out && algo == TID_JOIN_SORT_MERGE && nk > 0 && lprefix && rprefix && (L->k == nk || R->k == nk)) {
         // single pass into a result sized by the bound on its rows
         const int64_t ub = (L->k == nk ? nr : nl) + (left && L->k == nk ? nl : 0);
@@ -661,15 +814,41 @@ int join_sets(tid_ctx *ctx, const tid_set *L, const tid_set *R, int algo, tid_se
     const int32_t *lperm = nullptr, *rperm = nullptr, *rmap = nullptr;
     int64_t n_probe = nl;
     bool left_is_probe = true;
-    // The rows come out already canonical (sorted, distinct) when both inputs
-    // lead with the shared variables in the same order: a sort-merge join walks
-    // L in its order and each left row's matches in R's order, so the output is
-    // ordered by L's columns, then by R's other columns; a hash join does the
-    // same when its build side holds only the key columns (at most one match
-    // per probe row, the output ordered as the probe side).  Then no output sort.
+    // The rows come out already canonical (sorted, distinct) when L is walked in its
+    // order and each left row's matches in R's, which lead with the shared
+    // variables: the output is ordered by L's columns, then by R's other columns.
+    // A hash join does the same when both inputs lead with the shared variables and
+    // its build side holds only these (at most one match per probe row, the
+    // output ordered as the probe side).  Then no output sort.
     bool canonical_out = false;
 
-    if (algo == TID_JOIN_SORT_MERGE) {
+    // a few left rows in key order search the right side faster than a table of it is built
+    const bool runs = algo == TID_JOIN_SORT_MERGE && nk > 0 && rprefix && !(lprefix && nl <= nr / 64);
+    if (runs) {
+        Cols LK{}, RK{};
+        for (int i = 0; i < nk; ++i) {
+            LK.c[i] = L->col[lkey[i]];
+            RK.c[i] = R->col[i];
+        }
+        RunTable t{};
+        t.lo = R->bounded ? R->lo[0] : 0u;
+        t.span = R->bounded ? R->hi[0] - R->lo[0] : 0xFFFFFFFFu;
+        while (((uint64_t)t.span >> t.shift) + 1 > (uint64_t)std::max<int64_t>(nr, 1024)) ++t.shift;
+        const size_t nb = (size_t)(t.span >> t.shift) + 1;
+        uint32_t *cnt = nullptr;
+        TID_TRY(s.get(&t.bucket, nb));
+        TID_TRY(s.get(&cnt, nl));
+        TID_TRY(s.get(&lo, nl));
+        TID_TRY(s.get(&off, nl));
+        TID_TRY_CUDA(cudaMemsetAsync(t.bucket, 0, nb * sizeof(uint2), st), "run table");
+        k_run_table<<<grid_for(nr, 1024, 8), 256, 0, st>>>(RK.c[0], nr, t);
+        TID_TRY(launch_check("k_run_table"));
+        k_run_count<<<grid_for(nl, 1024, 8), 256, 0, st>>>(LK, nl, RK, nk, left, t, nk == 1 && t.shift == 0, cnt, lo,
+                                                           d_total);
+        TID_TRY(launch_check("k_run_count"));
+        TID_TRY(scan_exclusive_u32(ctx, cnt, off, nl, nullptr));
+        canonical_out = true;
+    } else if (algo == TID_JOIN_SORT_MERGE) {
         Cols LK{}, RK{};
         // left keys in key order
         if (lprefix) {
@@ -759,6 +938,14 @@ int join_sets(tid_ctx *ctx, const tid_set *L, const tid_set *R, int algo, tid_se
     TID_TRY(read_u64(ctx, d_total, &total));
     if (total > (unsigned long long)INT32_MAX)
         return fail(TID_ERR_CAPACITY, "tid_join: %llu output rows exceed 2^31-1", total);
+    uint32_t *split = nullptr;
+    const int64_t jtiles = ceil_div(n_probe + (int64_t)total, (int64_t)JW_TILE);
+    if (total > 0) {
+        TID_TRY(s.get(&split, jtiles + 1));
+        k_join_split<<<(unsigned)ceil_div(jtiles + 1, (int64_t)256), 256, 0, st>>>(off, n_probe, (int64_t)total, jtiles,
+                                                                                  split);
+        TID_TRY(launch_check("k_join_split"));
+    }
     if (canonical_out) {  // write straight into the result set
         tid_set *res = nullptr;
         TID_TRY(set_alloc(ctx, kout, ovars, (int64_t)total, &res));
@@ -767,8 +954,9 @@ int join_sets(tid_ctx *ctx, const tid_set *L, const tid_set *R, int algo, tid_se
         for (int c = 0; c < nrest; ++c) oR.c[c] = res->col[L->k + c];
         int rc = TID_OK;
         if (total > 0) {
-            k_join_write<<<(unsigned)ceil_div(n_probe + (int64_t)total, JW_TILE), JW_THREADS, 0, st>>>(
-                off, n_probe, lo, lperm, rmap, rperm, (int64_t)total, Lall, L->k, Rrest, nrest, oL, oR, left_is_probe);
+            k_join_write<<<(unsigned)jtiles, JW_THREADS, 0, st>>>(
+                off, n_probe, lo, lperm, rmap, rperm, (int64_t)total, Lall, L->k, Rrest, nrest, oL, oR, left_is_probe,
+                split);
             rc = launch_check("k_join_write");
         }
         if (rc == TID_OK) rc = set_rows_const(res, (int64_t)total);
@@ -785,8 +973,9 @@ int join_sets(tid_ctx *ctx, const tid_set *L, const tid_set *R, int algo, tid_se
     for (int c = 0; c < L->k; ++c) oL.c[c] = oc.c[c];
     for (int c = 0; c < nrest; ++c) oR.c[c] = oc.c[L->k + c];
     if (total > 0) {
-        k_join_write<<<(unsigned)ceil_div(n_probe + (int64_t)total, JW_TILE), JW_THREADS, 0, st>>>(
-            off, n_probe, lo, lperm, rmap, rperm, (int64_t)total, Lall, L->k, Rrest, nrest, oL, oR, left_is_probe);
+        k_join_write<<<(unsigned)jtiles, JW_THREADS, 0, st>>>(
+            off, n_probe, lo, lperm, rmap, rperm, (int64_t)total, Lall, L->k, Rrest, nrest, oL, oR, left_is_probe,
+                split);
         TID_TRY(launch_check("k_join_write"));
     }
     const int32_t *ocols[TID_MAX_COLS];

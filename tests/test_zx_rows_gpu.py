@@ -1,0 +1,134 @@
+"""Row selection and joins at the edges of their kernels, against the CPU oracle,
+bit-exact: selections around the step, range and kernel-choice boundaries, with
+every comparison at the ends of int32; joins whose right side leads with the key
+(runs found through a table over the key range, dense or spread over int32, one
+and two key columns, skewed, unbound keys) and joins with a set of keys only."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+from paper_1807_01409_gb300 import binding as tb
+
+pytestmark = pytest.mark.gpu
+LOWEST, HIGHEST = -2**31, 2**31 - 1
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    from paper_1807_01409_gb300 import build
+    build.build()
+    c = tb.tid_ctx_create(0, None)
+    yield c
+    tb.tid_ctx_destroy(c)
+
+
+def _rows(h):
+    try:
+        return tb.tid_set_to_host(h).copy()
+    finally:
+        tb.tid_set_free(h)
+
+
+def _set(ctx, s):
+    return tb.tid_set_from_host(ctx, s.rows, s.vars)
+
+
+# k_sel_mark / k_sel_expand from 2^18 rows up (steps of 1024, ranges of 8 or 32 steps), k_compact below
+SELECT_ROWS = [1, 2047, 2**18 - 1, 2**18, 2**18 + 1, 2**18 + 8 * 1024 + 1023, 1_300_003]
+PREDS = [("lt", 500, 0), ("ge", 999, 0), ("ne", 7, 0), ("eq", 7, 0), ("lt", LOWEST, 0), ("gt", HIGHEST, 0),
+         ("le", HIGHEST, 0), ("ge", LOWEST, 0), ("range", 10, 9), ("range", 990, HIGHEST)]
+
+
+@pytest.mark.parametrize("n", SELECT_ROWS)
+@pytest.mark.parametrize("k", [1, 2, 4])
+def test_filter_edges(ctx, orc, n, k):
+    rng = np.random.default_rng(n + k)
+    cols = [np.arange(1, n + 1)] + [rng.integers(0, 1000, n) for _ in range(k - 1)]
+    s = orc.TupleSet(tuple(range(k)), np.stack(cols, 1).astype(np.int32))
+    h = _set(ctx, s)
+    for cmp_, a, b in PREDS:
+        want = orc.filter(s, k - 1, cmp_, a, b).rows
+        got = _rows(tb.tid_filter(ctx, h, [(k - 1, cmp_, a, b)]))
+        assert np.array_equal(got, want), (cmp_, a, b)
+    if k > 1:  # two predicates, and a distinct prefix of a reordered set
+        got = _rows(tb.tid_filter(ctx, h, [(k - 1, "gt", 100, 0), (0, "le", n // 2 + 1, 0)]))
+        want = orc.filter(orc.filter(s, k - 1, "gt", 100, 0), 0, "le", n // 2 + 1, 0).rows
+        assert np.array_equal(got, want)
+        got = _rows(tb.tid_project(ctx, h, (k - 1,)))
+        assert np.array_equal(got, orc.project(s, (k - 1,)).rows)
+        got = _rows(tb.tid_project(ctx, h, tuple(range(k))[::-1]))
+        assert np.array_equal(got, orc.project(s, tuple(range(k))[::-1]).rows)
+    tb.tid_set_free(h)
+
+
+@pytest.mark.parametrize("n", [2**18 - 1, 2**18 + 5, 700_001])
+@pytest.mark.parametrize("shift", [0, 1])
+def test_bind_tests_edges(ctx, orc, n, shift):
+    """One tested slot (its values stashed), two tested slots, a repeated variable; borrowed columns
+    16-byte aligned or not."""
+    rng = np.random.default_rng(n + shift)
+    full = [rng.integers(1, 60_000, n + shift).astype(np.int32), rng.integers(1, 4, n + shift).astype(np.int32),
+            rng.integers(1, 50, n + shift).astype(np.int32)]
+    keep = np.unique(np.stack([c[shift:] for c in full], 1), axis=0, return_index=True)[1]
+    keep = rng.permutation(keep)
+    S, P, O = (np.ascontiguousarray(c[shift:][keep]) for c in full)
+    dev = [torch.from_numpy(np.concatenate([np.zeros(shift, np.int32), c])).cuda()[shift:] for c in (S, P, O)]
+    st = tb.tid_load(ctx, *dev, copy=0)
+    for key, var, preds in [((0, 2, 0), (0, -1, 1), [(1, "range", 10, 20)]), ((0, 2, 0), (0, -1, 1), [(0, "lt", 90, 0)]),
+                            ((0, 0, 0), (0, 1, 2), [(2, "ge", 10, 0), (0, "gt", 100, 0)]),
+                            ((0, 0, 0), (0, 1, 0), []), ((0, 0, 0), (0, 1, 2), [(1, "eq", 3, 0)])]:
+        idx = tb.tid_match(ctx, st, key)
+        want = orc.bind(S, P, O, key, var, orc.match(S, P, O, key))
+        for v, c, a, b in preds:
+            want = orc.filter(want, v, c, a, b)
+        got = _rows(tb.tid_bind(ctx, st, tb.make_pattern(*key, var=var), idx, preds))
+        assert np.array_equal(got, want.rows), (key, var, preds)
+        tb.tid_set_free(idx)
+    tb.tid_store_free(st)
+
+
+def _random_set(orc, rng, vars_, n, ids):
+    r = np.stack([ids(rng, n) for _ in vars_], 1).astype(np.int32)
+    return orc.TupleSet(vars_, orc.canonical(r))
+
+
+IDS = {
+    "dense": lambda rng, n: rng.integers(0, max(2, n // 2), n),           # 0: unbound rows among them
+    "clusters": lambda rng, n: rng.integers(0, max(2, n // 3), n) + (rng.integers(0, 2, n) << 30),
+    "wide": lambda rng, n: rng.integers(LOWEST, HIGHEST, n) // 7919 * 7919,
+    "skew": lambda rng, n: np.where(rng.random(n) < 0.02, 5, rng.integers(1, 4 * n + 2, n)),
+}
+JOINS = [((0, 1), (0, 2)), ((1, 0), (0, 2)), ((0, 1, 2), (1, 3)), ((2, 0, 1), (0, 1, 3)), ((0,), (0, 2)), ((0, 1), (0,)),
+         ((0,), (0,)), ((1, 0), (0,))]
+
+
+@pytest.mark.parametrize("ids", sorted(IDS))
+@pytest.mark.parametrize("shape", range(len(JOINS)))
+@pytest.mark.parametrize("size", [(3, 1), (1, 1025), (4000, 4097), (50_000, 7000), (300, 30_000)])
+def test_joins_on_a_leading_key(ctx, orc, ids, shape, size):
+    lv, rv = JOINS[shape]
+    rng = np.random.default_rng([shape, *size, len(ids)])
+    L = _random_set(orc, rng, lv, size[0], IDS[ids])
+    R = _random_set(orc, rng, rv, size[1], IDS[ids])
+    hl, hr = _set(ctx, L), _set(ctx, R)
+    want = orc.join(L, R, method="sortmerge")
+    for algo in ("auto", "sort_merge"):
+        got = _rows(tb.tid_join(ctx, hl, hr, algo))
+        assert np.array_equal(got, want.rows), algo
+    assert np.array_equal(_rows(tb.tid_join(ctx, hl, hr, "left")), orc.left_join(L, R).rows)
+    tb.tid_set_free(hl)
+    tb.tid_set_free(hr)
+
+
+def test_member_join_large(ctx, orc):
+    """Keys only against 2^18 rows and more: the selection's two-launch form."""
+    rng = np.random.default_rng(5)
+    R = _random_set(orc, rng, (0, 2), 400_000, IDS["dense"])
+    L = orc.TupleSet((0,), orc.canonical(rng.integers(0, 200_000, (60_000, 1)).astype(np.int32)))
+    hl, hr = _set(ctx, L), _set(ctx, R)
+    want = orc.join(L, R, method="sortmerge")
+    assert np.array_equal(_rows(tb.tid_join(ctx, hl, hr)), want.rows)
+    assert np.array_equal(_rows(tb.tid_join(ctx, hr, hl)), orc.join(R, L, method="sortmerge").rows)
+    tb.tid_set_free(hl)
+    tb.tid_set_free(hr)
