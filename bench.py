@@ -80,7 +80,7 @@ def _peaks():
     return 6800.0, "fallback"
 
 
-K1_REGION = ("// ---- k1_scan: dynamic steps", "int launch_scan(")  # the kernel, its grid and launch
+K1_REGION = ("// ---- k1_scan: mark and expand", "int launch_scan(")  # the kernels, their grids and launches
 
 
 def _kernel_region_sha1(kernel_src):

@@ -358,6 +358,7 @@ extern "C" int tid_ctx_destroy(tid_ctx *ctx) {
         sweep_pending(ctx, true);
     }
     if (ctx->lb_status) cudaFreeAsync(ctx->lb_status, ctx->stream);
+    if (ctx->sel_done) cudaFreeAsync(ctx->sel_done, ctx->stream);
     cudaStreamSynchronize(ctx->stream);
     for (auto *h : ctx->slabs_host) cudaFreeHost(h);
     if (ctx->err_host) cudaFreeHost(ctx->err_host);

@@ -27,6 +27,7 @@
 
 #include "lookback.cuh"
 #include "ops.cuh"
+#include "select.cuh"
 
 namespace tid {
 
@@ -469,17 +470,12 @@ k_compact(Row row, int64_t n, int k_out, OutCols out, int64_t cap, int64_t *__re
 
 // ---- mark and expand (long inputs) -------------------------------------------------
 //
-// k_sel_mark: a warp tests a step of 1024 rows, writes the step's 32 keep words
-// (bit b of word w: row 1024 j + 32 w + b) and its count, and adds the count to
-// the total of the range of steps that holds it; the last CTA to finish turns
-// the totals into the ranges' first output rows.  k_sel_expand: a CTA owns one
-// range; each of its warps scans the range's step counts and takes every eighth
-// step, so its warps never wait for each other.  A step that keeps many rows is
-// read word by word (lane l the word's row l: coalesced loads and stores); of
-// one that keeps few, the positions go to shared memory first and only the kept
-// rows are read, all lanes at work.  The test's columns are read twice, every
-// other value once, and no CTA waits for another: in the one-launch form a tile
-// waits for its predecessors' counts longer than its own work takes.
+// k_sel_mark and k_sel_expand: mark and expand (select.cuh) of rows.  A step that
+// keeps many rows is read word by word (lane l the word's row l: coalesced loads
+// and stores); of one that keeps few, the positions go to shared memory first and
+// only the kept rows are read, all lanes at work.  The test's columns are read
+// twice, every other value once; in the one-launch form a tile waits for its
+// predecessors' counts longer than its own work takes.
 // Bound: memory latency of the expansion's dependent loads (ncu: 57 % of DRAM
 // throughput binding 23.6M triples, long-scoreboard stalls).  Measured on GB300
 // (kernels, before -> after this form): FILTER of 24M two-column rows, half kept,
@@ -490,27 +486,15 @@ k_compact(Row row, int64_t n, int k_out, OutCols out, int64_t cap, int64_t *__re
 // filter against 32 us; one large range per resident CTA with block scans took
 // 97 us to expand against 83 us.
 
-constexpr int SEL_THREADS = 256;
-constexpr int SEL_WARPS = SEL_THREADS / 32;
-constexpr int SEL_STEP = 1024;         // rows per step
-constexpr unsigned SEL_DENSE = 256;    // kept rows from which a step is read word by word
 constexpr int64_t SEL_MIN_ROWS = (int64_t)1 << 18;  // below this, the single-pass kernel
-
-struct SelScratch {
-    uint32_t *bits;           // 32 keep words per step
-    uint32_t *cnt;            // kept rows per step
-    unsigned *done;           // CTAs of k_sel_mark that have finished
-    unsigned *tot;            // kept rows per range
-    unsigned long long *off;  // first output row per range
-    unsigned steps, per, ranges;  // range b owns steps [b per, (b + 1) per), per <= 32
-};
 
 template <class Row>
 __global__ void __launch_bounds__(SEL_THREADS)
 k_sel_mark(Row row, uint32_t n, SelScratch sc, int64_t *__restrict__ d_rows, int64_t *__restrict__ h_rows) {
     const unsigned lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const unsigned sub = lane & 7u;
-    for (unsigned step = blockIdx.x * SEL_WARPS + warp; step < sc.steps; step += gridDim.x * SEL_WARPS) {
+    const unsigned r0 = blockIdx.x * sc.per, r1 = min(r0 + sc.per, sc.steps);
+    unsigned kept = 0;
+    for (unsigned step = r0 + warp; step < r1; step += SEL_WARPS) {
         const uint32_t base = step * SEL_STEP + lane * 4;  // < 2^32: n < 2^31
         unsigned m[8];
         if ((step + 1) * SEL_STEP <= n) {
@@ -528,59 +512,13 @@ k_sel_mark(Row row, uint32_t n, SelScratch sc, int64_t *__restrict__ d_rows, int
                     if (q == g) m[q] = k4;
             }
         }
-        // lanes 8k .. 8k + 7 together hold word 4 g + k; lane 8k + g keeps it
-        uint32_t word = 0;
-#pragma unroll
-        for (int g = 0; g < 8; ++g) {
-            uint32_t v = m[g] << (4 * sub);
-            v |= __shfl_xor_sync(0xffffffffu, v, 1);
-            v |= __shfl_xor_sync(0xffffffffu, v, 2);
-            v |= __shfl_xor_sync(0xffffffffu, v, 4);
-            if (sub == (unsigned)g) word = v;
-        }
-        sc.bits[(size_t)step * 32 + sub * 4 + (lane >> 3)] = word;
+        const uint32_t word = sel_word(m);
+        sc.bits[(size_t)step * 32 + sel_word_index()] = word;
         const unsigned c = __reduce_add_sync(0xffffffffu, __popc(word));
-        if (lane == 0) {
-            sc.cnt[step] = c;
-            if (c) atomicAdd(sc.tot + step / sc.per, c);
-        }
+        if (lane == 0) sc.cnt[step] = c;
+        kept += c;
     }
-    // the last CTA: exclusive scan of the ranges' totals
-    __shared__ unsigned s_last;
-    __shared__ unsigned long long s_w[SEL_WARPS];
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        __threadfence();
-        s_last = atomicAdd(sc.done, 1u) == gridDim.x - 1;
-        __threadfence();
-    }
-    __syncthreads();
-    if (!s_last) return;
-    unsigned long long carry = 0;
-    for (unsigned b0 = 0; b0 < sc.ranges; b0 += SEL_THREADS) {
-        const unsigned b = b0 + threadIdx.x;
-        const unsigned long long c = b < sc.ranges ? __ldcg(sc.tot + b) : 0u;
-        unsigned long long x = c;
-#pragma unroll
-        for (int d = 1; d < 32; d <<= 1) {
-            const unsigned long long y = __shfl_up_sync(0xffffffffu, x, d);
-            if ((int)lane >= d) x += y;
-        }
-        if (lane == 31) s_w[warp] = x;
-        __syncthreads();
-        unsigned long long wb = 0, all = 0;
-        for (int w = 0; w < SEL_WARPS; ++w) {
-            if (w < (int)warp) wb += s_w[w];
-            all += s_w[w];
-        }
-        if (b < sc.ranges) sc.off[b] = carry + wb + x - c;
-        carry += all;
-        __syncthreads();  // s_w is rewritten by the next round
-    }
-    if (threadIdx.x == 0) {
-        *d_rows = (int64_t)carry;
-        *h_rows = (int64_t)carry;
-    }
+    sel_finish(sc, kept, d_rows, h_rows);
 }
 
 template <class Row, int K, bool BOUNDS>
@@ -609,32 +547,9 @@ k_sel_expand(Row row, int k_out, OutCols out, int64_t cap, SelScratch sc, uint32
         }
     };
     constexpr int UX = K == 1 ? 8 : 4;  // rows per lane read together
-    const unsigned r0 = blockIdx.x * sc.per, here = min(sc.per, sc.steps - r0);
-    const unsigned cnt = lane < here ? sc.cnt[r0 + lane] : 0u;
-    uint32_t next = warp < here ? sc.bits[(size_t)(r0 + warp) * 32 + lane] : 0u;
-    unsigned first = cnt;
-#pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
-        const unsigned y = __shfl_up_sync(0xffffffffu, first, d);
-        if ((int)lane >= d) first += y;
-    }
-    first -= cnt;  // of step r0 + lane
-    const unsigned long long o_range = sc.off[blockIdx.x];
-    for (unsigned li = warp; li < here; li += SEL_WARPS) {
-        const uint32_t word = next;
-        if (li + SEL_WARPS < here) next = sc.bits[(size_t)(r0 + li + SEL_WARPS) * 32 + lane];
-        const unsigned sn = __shfl_sync(0xffffffffu, cnt, li);
-        if (sn == 0) continue;
-        const unsigned long long o0 = o_range + __shfl_sync(0xffffffffu, first, li);
-        const unsigned pc = __popc(word);
-        unsigned xo = pc;
-#pragma unroll
-        for (int d = 1; d < 32; d <<= 1) {
-            const unsigned y = __shfl_up_sync(0xffffffffu, xo, d);
-            if ((int)lane >= d) xo += y;
-        }
-        xo -= pc;
-        const int64_t base = (int64_t)(r0 + li) * SEL_STEP;
+    uint16_t *stage = s_stage[warp];
+    sel_walk(sc, blockIdx.x, [&](unsigned step, uint32_t word, unsigned xo, unsigned sn, unsigned long long o0) {
+        const int64_t base = (int64_t)step * SEL_STEP;
         if (sn >= SEL_DENSE) {
 #pragma unroll 1
             for (int w0 = 0; w0 < 32; w0 += UX) {
@@ -652,13 +567,7 @@ k_sel_expand(Row row, int k_out, OutCols out, int64_t cap, SelScratch sc, uint32
                 }
             }
         } else {
-            uint16_t *stage = s_stage[warp];
-            uint32_t w = word;
-            while (w) {
-                stage[xo++] = (uint16_t)(lane * 32 + __ffs(w) - 1);
-                w &= w - 1;
-            }
-            __syncwarp();
+            sel_stage(word, xo, stage);
 #pragma unroll 1
             for (unsigned e0 = 0; e0 < sn; e0 += 32 * UX) {
                 int32_t v[UX][K];
@@ -673,9 +582,9 @@ k_sel_expand(Row row, int k_out, OutCols out, int64_t cap, SelScratch sc, uint32
                     if (e < sn) put(v[u], o0 + e);
                 }
             }
-            __syncwarp();
+            __syncwarp();  // the stage is rewritten by the next step
         }
-    }
+    });
     if (BOUNDS) merge_bounds<K>(mm, k_out, lo, hi);
 }
 
@@ -685,19 +594,6 @@ int expand_k(tid_ctx *ctx, const Row &row, int k_out, const OutCols &out, int64_
     if (mm) k_sel_expand<Row, K, true><<<sc.ranges, SEL_THREADS, 0, ctx->stream>>>(row, k_out, out, cap, sc, mm);
     else k_sel_expand<Row, K, false><<<sc.ranges, SEL_THREADS, 0, ctx->stream>>>(row, k_out, out, cap, sc, mm);
     return launch_check("k_sel_expand");
-}
-
-// grid of k_sel_mark: every CTA resident at once
-template <class Row>
-unsigned mark_grid() {
-    static unsigned cached = 0;
-    if (!cached) {
-        int v = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, k_sel_mark<Row>, SEL_THREADS, 0) != cudaSuccess || v <= 0)
-            v = 1;
-        cached = (unsigned)(v * sm_count());
-    }
-    return cached;
 }
 
 template <class Row>
@@ -723,35 +619,18 @@ int launch_compact(tid_ctx *ctx, Row row, int64_t n, int k_out, const OutCols &o
         k_compact<Row><<<tiles, CP_THREADS, smem, ctx->stream>>>(row, n, k_out, out, cap, d_rows, h_rows_dev, lb, mm);
         return launch_check("k_compact");
     }
-    SelScratch sc{};
-    sc.steps = (unsigned)ceil_div(n, (int64_t)SEL_STEP);
-    // a range is one step per warp, or four once that still gives every SM eight CTAs
-    sc.per = sc.steps >= (unsigned)sm_count() * 256 ? 32 : SEL_WARPS;
-    sc.ranges = (unsigned)ceil_div(sc.steps, (int64_t)sc.per);
-    const size_t bits_b = (size_t)sc.steps * 32 * 4, off_b = (size_t)sc.ranges * 8;
-    const size_t cnt_b = ((size_t)sc.steps * 4 + 255) / 256 * 256, tot_b = ((size_t)sc.ranges + 1) * 4;
     size_t stash_b = 0;
     if constexpr (std::is_same_v<Row, BindRow>) {
         if (row.n_eq == 0 && (row.test & (row.test - 1)) == 0) stash_b = (size_t)n * 4;
     }
-    void *blk = nullptr;
-    TID_TRY(dev_alloc(ctx, &blk, stash_b + bits_b + off_b + cnt_b + tot_b + 256));
+    SelScratch sc{};
+    void *blk = nullptr, *stash = nullptr;
+    TID_TRY(sel_scratch(ctx, n, 1, stash_b, &sc, &blk, &stash));
     if constexpr (std::is_same_v<Row, BindRow>) {
-        if (stash_b) row.stash = (int32_t *)((char *)blk + (bits_b + off_b + cnt_b + tot_b + 255) / 256 * 256);
+        if (stash_b) row.stash = (int32_t *)stash;
     }
-    sc.bits = (uint32_t *)blk;
-    sc.off = (unsigned long long *)((char *)blk + bits_b);
-    sc.cnt = (uint32_t *)((char *)blk + bits_b + off_b);
-    sc.done = (unsigned *)((char *)blk + bits_b + off_b + cnt_b);
-    sc.tot = sc.done + 1;
-    int rc = TID_OK;
-    cudaError_t e = cudaMemsetAsync(sc.done, 0, tot_b, ctx->stream);
-    if (e != cudaSuccess) rc = fail_cuda(e, "row selection totals");
-    if (rc == TID_OK) {
-        const unsigned grid = (unsigned)std::min<int64_t>(mark_grid<Row>(), ceil_div(sc.steps, (int64_t)SEL_WARPS));
-        k_sel_mark<Row><<<grid, SEL_THREADS, 0, ctx->stream>>>(row, (uint32_t)n, sc, d_rows, h_rows_dev);
-        rc = launch_check("k_sel_mark");
-    }
+    k_sel_mark<Row><<<sc.ranges, SEL_THREADS, 0, ctx->stream>>>(row, (uint32_t)n, sc, d_rows, h_rows_dev);
+    int rc = launch_check("k_sel_mark");
     if (rc == TID_OK) {
         if (k_out <= 1) rc = expand_k<Row, 1>(ctx, row, k_out, out, cap, sc, mm);
         else if (k_out == 2) rc = expand_k<Row, 2>(ctx, row, k_out, out, cap, sc, mm);
@@ -916,6 +795,37 @@ __global__ void __launch_bounds__(SC_THREADS) k_tile_sums(const uint32_t *__rest
 }
 
 }  // namespace
+
+int sel_scratch(tid_ctx *ctx, int64_t n, int lists, size_t extra, SelScratch *sc, void **block, void **extra_at) {
+    sc->steps = (unsigned)ceil_div(n, (int64_t)SEL_STEP);
+    // a range is one step per warp, or four once that still gives every SM eight CTAs
+    sc->per = sc->steps >= (unsigned)sm_count() * 256 ? 4 * SEL_WARPS : SEL_WARPS;
+    sc->ranges = (unsigned)ceil_div(sc->steps, (int64_t)sc->per);
+    auto pad = [](size_t b) { return (b + 255) / 256 * 256; };
+    const size_t bits_b = (size_t)sc->steps * 32 * 4 * lists, cnt_b = pad((size_t)sc->steps * 4 * lists);
+    const size_t off_b = pad((size_t)sc->ranges * 8 * lists), tot_b = pad((size_t)sc->ranges * 4 * lists);
+    if (!ctx->sel_done) {
+        void *d = nullptr;
+        TID_TRY(dev_alloc(ctx, &d, 256));
+        cudaError_t e = cudaMemsetAsync(d, 0, 256, ctx->stream);
+        if (e != cudaSuccess) {
+            dev_free(ctx, d);
+            return fail_cuda(e, "row selection");
+        }
+        ctx->sel_done = (unsigned *)d;
+    }
+    void *blk = nullptr;
+    TID_TRY(dev_alloc(ctx, &blk, bits_b + cnt_b + off_b + tot_b + extra));
+    char *p = (char *)blk;
+    sc->bits = (uint32_t *)p;
+    sc->cnt = (uint32_t *)(p += bits_b);
+    sc->off = (unsigned long long *)(p += cnt_b);
+    sc->tot = (uint32_t *)(p += off_b);
+    if (extra_at) *extra_at = p + tot_b;
+    sc->done = ctx->sel_done;
+    *block = blk;
+    return TID_OK;
+}
 
 int scan_exclusive_u32(tid_ctx *ctx, const uint32_t *in, uint32_t *out, int64_t n,
                        unsigned long long *total_dev) {

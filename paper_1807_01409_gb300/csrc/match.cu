@@ -7,21 +7,10 @@
 // columns once and writing each index once.  Only the columns a pattern binds
 // are read (template on the bound mask).
 //
-// k1_scan (tid_match): one cooperative launch in three phases, so that SMs that
-// stream faster also do more of the work.
-//  * phase A: warps draw runs of 12 1024-triple steps from one counter (the
-//    next run is drawn while the current one loads) and load them with 16-byte
-//    streaming
-//    loads, and write the step's 32-word hit bitmap (eight lanes merge their
-//    4-bit masks with three xor-shuffles) and its hit count to global memory;
-//    each step's count is also added (atomically) to the total of the CTA
-//    whose fixed range of steps holds it;
-//  * grid barrier; phase C: CTA c's offset is the sum of the totals of CTAs
-//    before it; it scans its steps' counts in shared memory and expands each
-//    step: a warp turns the step's 32 words into indices in a shared-memory
-//    stage (popc, warp prefix sum, set bits) and copies the stage out with
-//    coalesced stores.
-// Barrier waits are bounded (LB_SPIN_LIMIT polls, then TID_ERR_TIMEOUT).
+// k1_mark, k1_expand (tid_match): mark and expand (select.cuh).  k1_mark streams the
+// bound columns with 16-byte loads, a warp 1024 triples at a time, into one hit bit
+// per triple; k1_expand turns the hit bits into the ascending list.  Bound: HBM
+// bandwidth of the bound columns, from about 20M triples on; below, the launches.
 //
 // k1_match (tid_match_noalloc, whose scratch is a fixed array): every CTA owns
 // one contiguous chunk, streams it into a shared-memory bitmap, takes its
@@ -30,11 +19,12 @@
 // chunk) triples take several launches.
 //
 // Bytes per launch: 4 * (bound columns) * n read + 4 * hits written
-// (k1_scan: + n/8 bitmap written and read + 8 bytes per 1024 triples of counts).
+// (k1_mark, k1_expand: + n/8 bitmap written and read, mostly in L2).
 
 #include <algorithm>
 
 #include "lookback.cuh"
+#include "select.cuh"
 
 namespace tid {
 
@@ -51,37 +41,6 @@ constexpr int K1_STEP = K1_THREADS * 4 * K1_G;            // 8192 triples per st
 template <int MASK>
 constexpr int k1_bitmap_bytes() {
     return ((MASK & 1) + ((MASK >> 1) & 1) + ((MASK >> 2) & 1)) == 1 ? 48 * 1024 : 96 * 1024;
-}
-
-__device__ __forceinline__ int4 ld_stream_v4(const int32_t *p) {
-    int4 v;
-    asm("ld.global.nc.L1::no_allocate.L2::256B.v4.s32 {%0,%1,%2,%3}, [%4];"
-        : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
-        : "l"(p));
-    return v;
-}
-
-__device__ __forceinline__ int32_t ld_stream(const int32_t *p) {
-    int32_t v;
-    asm("ld.global.nc.L1::no_allocate.s32 %0, [%1];" : "=r"(v) : "l"(p));
-    return v;
-}
-
-// four consecutive elements e0..e0+3 of a column; elements at or past n read as 0
-template <bool VEC>
-__device__ __forceinline__ int4 load4(const int32_t *__restrict__ c, int64_t e0, int64_t n) {
-    if (VEC && e0 + 3 < n) return ld_stream_v4(c + e0);
-    int4 v = make_int4(0, 0, 0, 0);
-    if (e0 < n) v.x = ld_stream(c + e0);
-    if (e0 + 1 < n) v.y = ld_stream(c + e0 + 1);
-    if (e0 + 2 < n) v.z = ld_stream(c + e0 + 2);
-    if (e0 + 3 < n) v.w = ld_stream(c + e0 + 3);
-    return v;
-}
-
-__device__ __forceinline__ unsigned eq4(int4 v, int32_t k) {
-    return (unsigned)(v.x == k) | ((unsigned)(v.y == k) << 1) |
-           ((unsigned)(v.z == k) << 2) | ((unsigned)(v.w == k) << 3);
 }
 
 template <int MASK, bool VEC>
@@ -290,223 +249,6 @@ int run_mask(bool vec, cudaStream_t st, const int32_t *S, const int32_t *P, cons
                : run_segments<MASK, false>(st, S, P, O, n, ks, kp, ko, out, cap, d_rows, h_rows, sc);
 }
 
-// ---- k1_scan: dynamic steps, grid barriers, ordered expansion -------------------
-
-constexpr int K2S_STEP = 1024;                 // triples per warp step (32 lanes x 8 groups x 4)
-constexpr int K2S_WORDS = K2S_STEP / 32;       // bitmap words per step
-constexpr int K2S_CHUNK = K1_THREADS;          // steps scanned per round of phase C
-// Steps per draw: long enough that one counter serves all warps and the warps
-// stream one region of the store at a time (HBM pages), short enough that the
-// last draws end together (measured on GB300: 12 best among 1-48; 64 separate
-// counters over store partitions were slower).
-constexpr int K2S_DRAW = 12;
-constexpr int K2S_TICKET = 32;                 // step counter (own cache line in the control words)
-constexpr size_t K2S_CTL_BYTES = 256;
-
-struct ScanScratch {
-    uint32_t *bits;      // K2S_WORDS words per step
-    uint32_t *cnt;       // hits per step
-    unsigned *ctl;       // [1] grid barrier, [K2S_TICKET] step counter
-    unsigned *cta_tot;   // hits per CTA range (zeroed with the control words)
-    int *err;
-    int64_t steps;
-};
-
-template <int MASK, bool VEC>
-__global__ void __launch_bounds__(K1_THREADS)
-k1_scan(const int32_t *__restrict__ S, const int32_t *__restrict__ P, const int32_t *__restrict__ O, int64_t n,
-        int32_t ks, int32_t kp, int32_t ko, int32_t *__restrict__ out, int64_t cap, int64_t *__restrict__ d_rows,
-        int64_t *__restrict__ h_rows, ScanScratch sc) {
-    // step j covers triples [1024 j, 1024 j + 1024); lane l loads, in group g,
-    // triples 1024 j + 128 g + 4 l + (0..3), so lanes 8k..8k+7 hold word 4 g + k
-    static_assert(K1_G == 8, "bitmap layout assumes 8 load groups per step");
-    __shared__ uint32_t s_stage[K1_WARPS][K2S_STEP];
-    __shared__ uint32_t s_cnt[K2S_CHUNK], s_off[K2S_CHUNK];
-    __shared__ unsigned s_red[K1_WARPS];
-    __shared__ long long s_base;
-    const unsigned lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const unsigned sub = lane & 7u;
-
-    // CTA c owns steps [c per, (c + 1) per) in phase C
-    const int64_t per = (sc.steps + gridDim.x - 1) / gridDim.x;
-
-    // ---- phase A: runs of K2S_DRAW steps drawn from one counter
-    {
-        unsigned *ticket = sc.ctl + K2S_TICKET;
-        unsigned t = 0;  // first step of the current run
-        if (lane == 0) t = atomicAdd(ticket, (unsigned)K2S_DRAW);
-        t = __shfl_sync(0xffffffffu, t, 0);
-        unsigned k = 0;  // position in the run
-        while ((int64_t)(t + k) < sc.steps) {
-            const int64_t step = (int64_t)t + k;
-            unsigned nxt = 0;  // the next run, drawn while the last step of this one loads
-            if (lane == 0 && k + 1 == (unsigned)K2S_DRAW) nxt = atomicAdd(ticket, (unsigned)K2S_DRAW);
-            const int64_t base = step * K2S_STEP + lane * 4;
-            int4 vs[K1_G], vp[K1_G], vo[K1_G];
-            if (VEC && (step + 1) * K2S_STEP <= n) {
-#pragma unroll
-                for (int g = 0; g < K1_G; ++g) {
-                    if (MASK & 1) vs[g] = ld_stream_v4(S + base + g * 128);
-                    if (MASK & 2) vp[g] = ld_stream_v4(P + base + g * 128);
-                    if (MASK & 4) vo[g] = ld_stream_v4(O + base + g * 128);
-                }
-            } else {  // ragged last step (elements past n read as 0, which no bound key equals)
-#pragma unroll
-                for (int g = 0; g < K1_G; ++g) {
-                    if (MASK & 1) vs[g] = load4<VEC>(S, base + g * 128, n);
-                    if (MASK & 2) vp[g] = load4<VEC>(P, base + g * 128, n);
-                    if (MASK & 4) vo[g] = load4<VEC>(O, base + g * 128, n);
-                }
-            }
-            unsigned c = 0;
-            uint32_t *bw = sc.bits + (size_t)step * K2S_WORDS;
-#pragma unroll
-            for (int g = 0; g < K1_G; ++g) {
-                unsigned mm = 0xFu;
-                if (MASK & 1) mm &= eq4(vs[g], ks);
-                if (MASK & 2) mm &= eq4(vp[g], kp);
-                if (MASK & 4) mm &= eq4(vo[g], ko);
-                unsigned v = mm << (4 * sub);
-                v |= __shfl_xor_sync(0xffffffffu, v, 1);
-                v |= __shfl_xor_sync(0xffffffffu, v, 2);
-                v |= __shfl_xor_sync(0xffffffffu, v, 4);
-                if (sub == (unsigned)g) {
-                    __stcg(bw + g * 4 + (lane >> 3), v);
-                    c += __popc(v);
-                }
-            }
-#pragma unroll
-            for (int d = 16; d > 0; d >>= 1) c += __shfl_xor_sync(0xffffffffu, c, d);
-            if (lane == 0) {
-                __stcg(sc.cnt + step, c);
-                if (c) atomicAdd(sc.cta_tot + step / per, c);  // the total of the range that owns the step
-            }
-            if (++k == (unsigned)K2S_DRAW) {
-                t = __shfl_sync(0xffffffffu, nxt, 0);
-                k = 0;
-            }
-        }
-    }
-    if (!grid_barrier(sc.ctl + 1, gridDim.x, sc.err)) return;
-
-    const int64_t r0 = min((int64_t)blockIdx.x * per, sc.steps), r1 = min(r0 + per, sc.steps);
-    const unsigned mine = __ldcg(sc.cta_tot + blockIdx.x);
-
-    // ---- phase C: offset of this range, then ordered expansion
-    unsigned long long pre = 0, all = 0;
-    for (unsigned c = threadIdx.x; c < gridDim.x; c += K1_THREADS) {
-        const unsigned v = __ldcg(sc.cta_tot + c);
-        all += v;
-        if (c < blockIdx.x) pre += v;
-    }
-#pragma unroll
-    for (int d = 16; d > 0; d >>= 1) {
-        pre += __shfl_xor_sync(0xffffffffu, pre, d);
-        all += __shfl_xor_sync(0xffffffffu, all, d);
-    }
-    __shared__ unsigned long long s_pre[K1_WARPS], s_all[K1_WARPS];
-    if (lane == 0) {
-        s_pre[warp] = pre;
-        s_all[warp] = all;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        unsigned long long p = 0, a = 0;
-        for (int w = 0; w < K1_WARPS; ++w) {
-            p += s_pre[w];
-            a += s_all[w];
-        }
-        s_base = (long long)p;
-        if (blockIdx.x == 0) {
-            *d_rows = (int64_t)a;
-            *h_rows = (int64_t)a;
-        }
-    }
-    __syncthreads();
-    if (mine == 0) return;  // no hit in this range
-    long long run = s_base;
-    for (int64_t q0 = r0; q0 < r1; q0 += K2S_CHUNK) {
-        // block scan of this round's step counts
-        const int64_t j = q0 + threadIdx.x;
-        const unsigned c = j < r1 ? __ldcg(sc.cnt + j) : 0u;
-        unsigned x = c;
-#pragma unroll
-        for (int d = 1; d < 32; d <<= 1) {
-            const unsigned y = __shfl_up_sync(0xffffffffu, x, d);
-            if ((int)lane >= d) x += y;
-        }
-        if (lane == 31) s_red[warp] = x;
-        __syncthreads();
-        unsigned wb = 0, rt = 0;
-        for (int w = 0; w < K1_WARPS; ++w) {
-            if (w < (int)warp) wb += s_red[w];
-            rt += s_red[w];
-        }
-        s_cnt[threadIdx.x] = c;
-        s_off[threadIdx.x] = wb + x - c;
-        __syncthreads();
-        // warp w expands steps q0 + 32 w .. q0 + 32 w + 31
-        uint32_t *stage = s_stage[warp];
-        for (int i = 0; i < 32; ++i) {
-            const int li = (int)warp * 32 + i;
-            const int64_t step = q0 + li;
-            if (step >= r1) break;
-            const unsigned sc_n = s_cnt[li];
-            if (sc_n == 0) continue;
-            uint32_t word = __ldcg(sc.bits + (size_t)step * K2S_WORDS + lane);
-            const unsigned pc = __popc(word);
-            unsigned xo = pc;
-#pragma unroll
-            for (int d = 1; d < 32; d <<= 1) {
-                const unsigned y = __shfl_up_sync(0xffffffffu, xo, d);
-                if ((int)lane >= d) xo += y;
-            }
-            unsigned at = xo - pc;
-            const uint32_t wbase = (uint32_t)(step * K2S_STEP) + lane * 32;
-            while (word) {
-                const int b = __ffs(word) - 1;
-                stage[at++] = wbase + (uint32_t)b;
-                word &= word - 1;
-            }
-            __syncwarp();
-            const long long o0 = run + s_off[li];
-            for (unsigned e = lane; e < sc_n; e += 32) {
-                const long long pos = o0 + e;
-                if ((unsigned long long)pos < (unsigned long long)cap) out[pos] = (int32_t)stage[e];
-            }
-            __syncwarp();
-        }
-        run += rt;
-        __syncthreads();  // s_red, s_cnt, s_off are reused
-    }
-}
-
-template <int MASK, bool VEC>
-int scan_grid(unsigned *grid) {
-    static unsigned cached = 0;
-    if (!cached) {
-        int v = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, k1_scan<MASK, VEC>, K1_THREADS, 0) != cudaSuccess ||
-            v <= 0)
-            return fail(TID_ERR_CUDA, "k1_scan: no resident CTA");
-        cached = (unsigned)(v * sm_count());
-    }
-    *grid = cached;
-    return TID_OK;
-}
-
-template <int MASK, bool VEC>
-int run_scan(cudaStream_t st, const int32_t *S, const int32_t *P, const int32_t *O, int64_t n, int32_t ks,
-             int32_t kp, int32_t ko, int32_t *out, int64_t cap, int64_t *d_rows, int64_t *h_rows,
-             const ScanScratch &sc, unsigned grid) {
-    void *args[] = {(void *)&S, (void *)&P, (void *)&O, (void *)&n, (void *)&ks, (void *)&kp, (void *)&ko,
-                    (void *)&out, (void *)&cap, (void *)&d_rows, (void *)&h_rows, (void *)&sc};
-    TID_TRY_CUDA(cudaLaunchCooperativeKernel((const void *)k1_scan<MASK, VEC>, dim3(grid), dim3(K1_THREADS), args, 0,
-                                             st),
-                 "k1_scan");
-    return TID_OK;
-}
-
 }  // namespace
 
 // Status words one K1 launch needs at most (one per CTA of the largest grid).
@@ -552,34 +294,63 @@ int launch_match(cudaStream_t st, const int32_t *S, const int32_t *P, const int3
     }
 }
 
-// k1_scan with scratch from the context's pool (see tid_match).
+// ---- k1_scan: mark and expand ---------------------------------------------------
+
+namespace {
+
 template <int MASK, bool VEC>
-static int scan_with_scratch(tid_ctx *ctx, const int32_t *S, const int32_t *P, const int32_t *O, int64_t n,
-                             int32_t ks, int32_t kp, int32_t ko, int32_t *out, int64_t cap, int64_t *d_rows,
-                             int64_t *h_rows) {
-    cudaStream_t st = ctx->stream;
-    unsigned grid = 0;
-    TID_TRY((scan_grid<MASK, VEC>(&grid)));
-    const int64_t steps = ceil_div(n, (int64_t)K2S_STEP);
-    grid = (unsigned)std::min<int64_t>(grid, std::max<int64_t>(1, steps));
-    const size_t bits_b = (size_t)steps * K2S_WORDS * 4, cnt_b = ((size_t)steps * 4 + 255) / 256 * 256;
-    const size_t ctl_b = K2S_CTL_BYTES, tot_b = (size_t)grid * 4;  // control words: barriers and counters
+__global__ void __launch_bounds__(SEL_THREADS)
+k1_mark(const int32_t *__restrict__ S, const int32_t *__restrict__ P, const int32_t *__restrict__ O, int64_t n,
+        int32_t ks, int32_t kp, int32_t ko, SelScratch sc, int64_t *__restrict__ d_rows,
+        int64_t *__restrict__ h_rows) {
+    const unsigned lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const unsigned r0 = blockIdx.x * sc.per, r1 = min(r0 + sc.per, sc.steps);
+    unsigned kept = 0;
+    for (unsigned step = r0 + warp; step < r1; step += SEL_WARPS) {
+        int4 v[3][8];
+        load_step<MASK, VEC>(S, P, O, n, step, v);  // a triple past n reads as 0, which no bound key equals
+        unsigned m[8], any = 0;
+#pragma unroll
+        for (int g = 0; g < 8; ++g) {
+            m[g] = 0xFu;
+            if (MASK & 1) m[g] &= eq4(v[0][g], ks);
+            if (MASK & 2) m[g] &= eq4(v[1][g], kp);
+            if (MASK & 4) m[g] &= eq4(v[2][g], ko);
+            any |= m[g];
+        }
+        unsigned c = 0;
+        if (__any_sync(0xffffffffu, any)) {  // a step without a hit writes its count alone
+            const uint32_t word = sel_word(m);
+            __stcg(sc.bits + (size_t)step * 32 + sel_word_index(), word);
+            c = __reduce_add_sync(0xffffffffu, __popc(word));
+        }
+        if (lane == 0) __stcg(sc.cnt + step, c);
+        kept += c;
+    }
+    sel_finish(sc, kept, d_rows, h_rows);
+}
+
+__global__ void __launch_bounds__(SEL_THREADS) k1_expand(SelScratch sc, int32_t *__restrict__ out, int64_t cap) {
+    if (sc.tot[blockIdx.x]) sel_expand_index(sc, blockIdx.x, out, cap);
+}
+
+template <int MASK, bool VEC>
+int run_scan(tid_ctx *ctx, const int32_t *S, const int32_t *P, const int32_t *O, int64_t n, int32_t ks, int32_t kp,
+             int32_t ko, int32_t *out, int64_t cap, int64_t *d_rows, int64_t *h_rows) {
+    SelScratch sc{};
     void *blk = nullptr;
-    TID_TRY(dev_alloc(ctx, &blk, bits_b + cnt_b + ctl_b + tot_b));
-    ScanScratch sc{};
-    sc.bits = (uint32_t *)blk;
-    sc.cnt = (uint32_t *)((char *)blk + bits_b);
-    sc.ctl = (unsigned *)((char *)blk + bits_b + cnt_b);
-    sc.cta_tot = (unsigned *)((char *)blk + bits_b + cnt_b + ctl_b);
-    sc.err = ctx->err_dev;
-    sc.steps = steps;
-    int rc = TID_OK;
-    cudaError_t e = cudaMemsetAsync(sc.ctl, 0, ctl_b + tot_b, st);  // control words and range totals
-    if (e != cudaSuccess) rc = fail_cuda(e, "k1_scan control words");
-    if (rc == TID_OK) rc = run_scan<MASK, VEC>(st, S, P, O, n, ks, kp, ko, out, cap, d_rows, h_rows, sc, grid);
+    TID_TRY(sel_scratch(ctx, n, 1, 0, &sc, &blk, nullptr));
+    k1_mark<MASK, VEC><<<sc.ranges, SEL_THREADS, 0, ctx->stream>>>(S, P, O, n, ks, kp, ko, sc, d_rows, h_rows);
+    int rc = launch_check("k1_mark");
+    if (rc == TID_OK) {
+        k1_expand<<<sc.ranges, SEL_THREADS, 0, ctx->stream>>>(sc, out, cap);
+        rc = launch_check("k1_expand");
+    }
     dev_free(ctx, blk);
     return rc;
 }
+
+}  // namespace
 
 int launch_scan(tid_ctx *ctx, const int32_t *S, const int32_t *P, const int32_t *O, int64_t n, bool aligned16,
                 int32_t ks, int32_t kp, int32_t ko, int32_t *out, int64_t cap, int64_t *d_rows, int64_t *h_rows) {
@@ -588,15 +359,17 @@ int launch_scan(tid_ctx *ctx, const int32_t *S, const int32_t *P, const int32_t 
         LbScratch none{};
         return launch_match(ctx->stream, S, P, O, n, aligned16, ks, kp, ko, out, cap, d_rows, h_rows, none);
     }
-#define K1S_CALL(M, V) scan_with_scratch<M, V>(ctx, S, P, O, n, ks, kp, ko, out, cap, d_rows, h_rows)
+#define K1S_CALL(M) \
+    (aligned16 ? run_scan<M, true>(ctx, S, P, O, n, ks, kp, ko, out, cap, d_rows, h_rows) \
+               : run_scan<M, false>(ctx, S, P, O, n, ks, kp, ko, out, cap, d_rows, h_rows))
     switch (mask) {
-        case 1: return aligned16 ? K1S_CALL(1, true) : K1S_CALL(1, false);
-        case 2: return aligned16 ? K1S_CALL(2, true) : K1S_CALL(2, false);
-        case 3: return aligned16 ? K1S_CALL(3, true) : K1S_CALL(3, false);
-        case 4: return aligned16 ? K1S_CALL(4, true) : K1S_CALL(4, false);
-        case 5: return aligned16 ? K1S_CALL(5, true) : K1S_CALL(5, false);
-        case 6: return aligned16 ? K1S_CALL(6, true) : K1S_CALL(6, false);
-        default: return aligned16 ? K1S_CALL(7, true) : K1S_CALL(7, false);
+        case 1: return K1S_CALL(1);
+        case 2: return K1S_CALL(2);
+        case 3: return K1S_CALL(3);
+        case 4: return K1S_CALL(4);
+        case 5: return K1S_CALL(5);
+        case 6: return K1S_CALL(6);
+        default: return K1S_CALL(7);
     }
 #undef K1S_CALL
 }

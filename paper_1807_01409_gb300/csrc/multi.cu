@@ -4,47 +4,24 @@
 // subqueries: every triple is compared with each key and marked with the list
 // of subqueries it answers (a triple may answer several, as in the paper's
 // second union example).  Here the marks become one ascending index list per
-// pattern, built in the same pass, with the structure of K1:
-//  * each CTA streams one contiguous chunk per segment, loading the union of
-//    the patterns' bound columns once per step and testing every pattern on
-//    the loaded values (latency is hidden by resident warps rather than by
-//    holding a second step in registers, whose pattern loop is long); each pattern keeps a triple-ordered 1-bit-per-triple
-//    bitmap in shared memory (8 lanes merge 4-bit masks with three
-//    xor-shuffles), 48 KB in all when one column is loaded, 96 KB otherwise, so
-//    chunks shrink as patterns are added;
-//  * pattern j's chunk count is a popc over its bitmap; it has one look-back
-//    chain over (segment, chunk) in store order; warp w resolves the chains of
-//    patterns w and w + 8;
-//  * per pattern, each warp expands a contiguous run of bitmap words, 32 at a
-//    time: popc, a warp prefix sum, and each lane writes the indices of its set
-//    bits.
-// A launch walks all segments of the store (segment = resident CTAs x chunk).
-// Bytes per launch: 4 * |union of bound columns| * n read + 4 * sum of hits written.
+// pattern by mark and expand (select.cuh): k2_mark loads the union of the
+// patterns' bound columns once per step and tests every pattern on the loaded
+// values, leaving one hit bit per triple and pattern; k_scan_ranges scans each
+// pattern's range totals; k2_expand writes the lists.
+// Bytes per launch: 4 * |union of bound columns| * n read + 4 * sum of hits written
+// (+ n/8 per pattern of bitmap written and read, mostly in L2).  Measured on GB300,
+// three patterns over two columns of 200M triples, 32.3M hits: k2_mark 251 us
+// (6.4 TB/s), k_scan_ranges 12 us, k2_expand 102 us; before, chunks in shared memory
+// with one look-back chain per pattern took 483 us, and 88 us at 1M triples, where
+// they gave four CTAs work.
 
 #include <algorithm>
 
-#include "lookback.cuh"
+#include "select.cuh"
 
 namespace tid {
 
 namespace {
-
-constexpr int K2_THREADS = 256;
-constexpr int K2_WARPS = K2_THREADS / 32;
-constexpr int K2_G = 8;                          // 16-byte loads per column per thread per step
-constexpr int K2_STEP = K2_THREADS * 4 * K2_G;   // 8192 triples per step (256 bitmap words)
-
-// resident CTAs per SM the register budget is shaped for: loaded data is 32
-// registers per bound column
-template <int U>
-constexpr int k2_min_blocks() {
-    return ((U & 1) + ((U >> 1) & 1) + ((U >> 2) & 1)) == 1 ? 3 : (((U & 1) + ((U >> 1) & 1) + ((U >> 2) & 1)) == 2 ? 2 : 1);
-}
-
-template <int U>
-constexpr int k2_bitmap_bytes() {
-    return ((U & 1) + ((U >> 1) & 1) + ((U >> 2) & 1)) == 1 ? 48 * 1024 : 96 * 1024;
-}
 
 struct MultiArgs {
     int m;
@@ -55,232 +32,114 @@ struct MultiArgs {
     int64_t *h_rows[TID_MAX_MULTI];
 };
 
-__device__ __forceinline__ int4 ld_stream_v4(const int32_t *p) {
-    int4 v;
-    asm("ld.global.nc.L1::no_allocate.L2::256B.v4.s32 {%0,%1,%2,%3}, [%4];"
-        : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
-        : "l"(p));
-    return v;
-}
-
-__device__ __forceinline__ int32_t ld_stream(const int32_t *p) {
-    int32_t v;
-    asm("ld.global.nc.L1::no_allocate.s32 %0, [%1];" : "=r"(v) : "l"(p));
-    return v;
-}
-
-template <bool VEC>
-__device__ __forceinline__ int4 load4(const int32_t *__restrict__ c, int64_t e0, int64_t n) {
-    if (VEC && e0 + 3 < n) return ld_stream_v4(c + e0);
-    int4 v = make_int4(0, 0, 0, 0);
-    if (e0 < n) v.x = ld_stream(c + e0);
-    if (e0 + 1 < n) v.y = ld_stream(c + e0 + 1);
-    if (e0 + 2 < n) v.z = ld_stream(c + e0 + 2);
-    if (e0 + 3 < n) v.w = ld_stream(c + e0 + 3);
-    return v;
-}
-
-// 4-bit mask of lanes of v equal to k, or all ones if k is "?" (0)
-__device__ __forceinline__ unsigned eq4w(int4 v, int32_t k) {
-    if (k == 0) return 0xFu;
-    return (unsigned)(v.x == k) | ((unsigned)(v.y == k) << 1) | ((unsigned)(v.z == k) << 2) |
-           ((unsigned)(v.w == k) << 3);
+// list j's part of the scratch of several lists
+__device__ __forceinline__ SelScratch list_of(const SelScratch &all, int j) {
+    SelScratch sc = all;
+    sc.bits += (size_t)j * all.steps * 32;
+    sc.cnt += (size_t)j * all.steps;
+    sc.tot += (size_t)j * all.ranges;
+    sc.off += (size_t)j * all.ranges;
+    return sc;
 }
 
 template <int U, bool VEC>
-__global__ void __launch_bounds__(K2_THREADS, k2_min_blocks<U>())
-k2_match_multi(const int32_t *__restrict__ S, const int32_t *__restrict__ P, const int32_t *__restrict__ O,
-               int64_t n, int64_t chunk_len, int n_seg, MultiArgs args, Lookback lb) {
-    // pattern j's bitmap: words [j * wpp, (j+1) * wpp); bit b of word W is triple
-    // c0 + 32 W + b; step st, load group g, warp w, lanes 8k..8k+7 -> word
-    // st*256 + (g*8 + w)*4 + k (as in K1)
-    extern __shared__ uint32_t s_bits[];
-    __shared__ unsigned s_tile;
-    __shared__ unsigned s_wsum[K2_WARPS];
-    __shared__ long long s_prefix[TID_MAX_MULTI];
-
+__global__ void __launch_bounds__(SEL_THREADS)
+k2_mark(const int32_t *__restrict__ S, const int32_t *__restrict__ P, const int32_t *__restrict__ O, int64_t n,
+        const __grid_constant__ MultiArgs args, SelScratch sc) {
+    __shared__ unsigned s_kept[TID_MAX_MULTI][SEL_WARPS];
     const unsigned lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const unsigned sub = lane & 7u;
+    const unsigned r0 = blockIdx.x * sc.per, r1 = min(r0 + sc.per, sc.steps);
     const int m = args.m;
-    const unsigned G = lb.num_tiles;  // chunks per segment (= grid)
-    const int wpp = (int)(chunk_len / 32);
-    if (threadIdx.x == 0) s_tile = lb_ticket(lb);
-    __syncthreads();
-    const unsigned t = s_tile;
-    if (t >= G) return;
-    bool dead = false;
-    int4 vs[K2_G], vp[K2_G], vo[K2_G];
-    auto issue = [&](int64_t base) {
-        const int64_t t0 = base + threadIdx.x * 4;
-        if (VEC && base + K2_STEP <= n) {
+    for (int j = (int)lane; j < m; j += 32) s_kept[j][warp] = 0;
+    __syncwarp();
+    for (unsigned step = r0 + warp; step < r1; step += SEL_WARPS) {
+        int4 v[3][8];
+        load_step<U, VEC>(S, P, O, n, step, v);
+        // triples past n: a pattern binds at least one column of U or none at all
+        // (then it matches every triple of the store, and only those)
+        const int64_t left = n - ((int64_t)step * SEL_STEP + lane * 4);
+#pragma unroll 1
+        for (int j = 0; j < m; ++j) {
+            const int32_t ks = args.key[j][0], kp = args.key[j][1], ko = args.key[j][2];
+            unsigned k4[8], any = 0;
 #pragma unroll
-            for (int g = 0; g < K2_G; ++g) {
-                if (U & 1) vs[g] = ld_stream_v4(S + t0 + g * (K2_THREADS * 4));
-                if (U & 2) vp[g] = ld_stream_v4(P + t0 + g * (K2_THREADS * 4));
-                if (U & 4) vo[g] = ld_stream_v4(O + t0 + g * (K2_THREADS * 4));
+            for (int g = 0; g < 8; ++g) k4[g] = 0xFu;
+            if ((U & 1) && ks) {
+#pragma unroll
+                for (int g = 0; g < 8; ++g) k4[g] &= eq4(v[0][g], ks);
             }
-        } else {
+            if ((U & 2) && kp) {
 #pragma unroll
-            for (int g = 0; g < K2_G; ++g) {
-                const int64_t e0 = t0 + g * (K2_THREADS * 4);
-                if (U & 1) vs[g] = load4<VEC>(S, e0, n);
-                if (U & 2) vp[g] = load4<VEC>(P, e0, n);
-                if (U & 4) vo[g] = load4<VEC>(O, e0, n);
+                for (int g = 0; g < 8; ++g) k4[g] &= eq4(v[1][g], kp);
             }
-        }
-    };
-
-    for (int sg = 0; sg < n_seg; ++sg) {
-        const int64_t c0 = ((int64_t)sg * G + t) * chunk_len;
-        const int64_t c1 = min(c0 + chunk_len, n);
-        const int steps = (!dead && c1 > c0) ? (int)ceil_div(c1 - c0, K2_STEP) : 0;
-
-        // ---- stream the chunk: the loaded columns are tested against every pattern
-        if (steps > 0) issue(c0);
-        for (int st = 0; st < steps; ++st) {
-            const int64_t base = c0 + (int64_t)st * K2_STEP;
-            unsigned valid = 0xFFFFFFFFu;  // bit 4g+e: element of load group g is inside the chunk
-            if (base + K2_STEP > c1) {
-                valid = 0;
+            if ((U & 4) && ko) {
 #pragma unroll
-                for (int g = 0; g < K2_G; ++g) {
-                    const int64_t left = c1 - (base + g * (K2_THREADS * 4) + threadIdx.x * 4);
-                    const unsigned vm = left <= 0 ? 0u : (left >= 4 ? 0xFu : ((1u << left) - 1u));
-                    valid |= vm << (4 * g);
+                for (int g = 0; g < 8; ++g) k4[g] &= eq4(v[2][g], ko);
+            }
+            if ((ks | kp | ko) == 0 && (int64_t)(step + 1) * SEL_STEP > n) {
+#pragma unroll
+                for (int g = 0; g < 8; ++g) {
+                    const int64_t l = left - g * 128;
+                    k4[g] = l >= 4 ? 0xFu : (l <= 0 ? 0u : (1u << l) - 1u);
                 }
             }
-            for (int j = 0; j < m; ++j) {
-                const int32_t ks = args.key[j][0], kp = args.key[j][1], ko = args.key[j][2];
-                uint32_t *row = s_bits + (size_t)j * wpp + (size_t)st * K2_THREADS;
 #pragma unroll
-                for (int g = 0; g < K2_G; ++g) {
-                    unsigned mm = (valid >> (4 * g)) & 0xFu;
-                    if (U & 1) mm &= eq4w(vs[g], ks);
-                    if (U & 2) mm &= eq4w(vp[g], kp);
-                    if (U & 4) mm &= eq4w(vo[g], ko);
-                    unsigned v = mm << (4 * sub);
-                    v |= __shfl_xor_sync(0xffffffffu, v, 1);
-                    v |= __shfl_xor_sync(0xffffffffu, v, 2);
-                    v |= __shfl_xor_sync(0xffffffffu, v, 4);
-                    if (sub == (unsigned)g) row[(g * K2_WARPS + warp) * 4 + (lane >> 3)] = v;
-                }
+            for (int g = 0; g < 8; ++g) any |= k4[g];
+            unsigned c = 0;
+            if (__any_sync(0xffffffffu, any)) {  // a step without a hit writes its count alone
+                const uint32_t word = sel_word(k4);
+                __stcg(sc.bits + ((size_t)j * sc.steps + step) * 32 + sel_word_index(), word);
+                c = __reduce_add_sync(0xffffffffu, __popc(word));
             }
-            if (st + 1 < steps) issue(base + K2_STEP);  // registers are free once all patterns are tested
-        }
-        __syncthreads();
-
-        // ---- chunk offsets: chain of pattern j over (segment, chunk)
-        const int nwords = steps * K2_THREADS;
-        const unsigned idx = (unsigned)sg * G + t;
-        for (int j = (int)warp; j < m; j += K2_WARPS) {
-            const uint32_t *b = s_bits + (size_t)j * wpp;
-            unsigned tot = 0;
-            for (int i = (int)lane; i < nwords; i += 32) tot += __popc(b[i]);
-#pragma unroll
-            for (int d = 16; d > 0; d >>= 1) tot += __shfl_xor_sync(0xffffffffu, tot, d);
-            Lookback lj = lb;
-            lj.status = lb.status + (size_t)j * n_seg * G;
-            lj.num_tiles = (unsigned)n_seg * G;
-            long long excl = -1;
-            if (!dead) excl = lb_exclusive_prefix(lj, idx, tot);
-            else lb_abort(lj, idx);
             if (lane == 0) {
-                s_prefix[j] = excl;
-                if (idx == lj.num_tiles - 1 && excl >= 0) {
-                    *args.d_rows[j] = excl + tot;
-                    *args.h_rows[j] = excl + tot;
-                }
+                __stcg(sc.cnt + (size_t)j * sc.steps + step, c);
+                s_kept[j][warp] += c;
             }
         }
-        __syncthreads();
-        for (int j = 0; j < m; ++j) dead = dead || s_prefix[j] < 0;
-
-        // ---- expand: per pattern, warp w owns words [w0, w1), 32 at a time
-        if (!dead && steps > 0) {
-            const int per = (nwords / 32 + K2_WARPS - 1) / K2_WARPS * 32;
-            const int w0 = min(nwords, (int)warp * per), w1 = min(nwords, w0 + per);
-            for (int j = 0; j < m; ++j) {
-                const uint32_t *b = s_bits + (size_t)j * wpp;
-                unsigned wt = 0;
-                for (int i = w0 + (int)lane; i < w1; i += 32) wt += __popc(b[i]);
-#pragma unroll
-                for (int d = 16; d > 0; d >>= 1) wt += __shfl_xor_sync(0xffffffffu, wt, d);
-                __syncthreads();  // s_wsum is reused
-                if (lane == 0) s_wsum[warp] = wt;
-                __syncthreads();
-                long long run = s_prefix[j];
-                for (unsigned w = 0; w < warp; ++w) run += s_wsum[w];
-                int32_t *out = args.out[j];
-                const int64_t cap = args.cap[j];
-                for (int i0 = w0; i0 < w1; i0 += 32) {
-                    uint32_t word = b[i0 + lane];
-                    const unsigned c = __popc(word);
-                    unsigned x = c;
-#pragma unroll
-                    for (int d = 1; d < 32; d <<= 1) {
-                        const unsigned y = __shfl_up_sync(0xffffffffu, x, d);
-                        if ((int)lane >= d) x += y;
-                    }
-                    const unsigned batch = __shfl_sync(0xffffffffu, x, 31);
-                    if (batch == 0) continue;
-                    long long pos = run + (x - c);
-                    const int64_t wbase = c0 + (int64_t)(i0 + (int)lane) * 32;
-                    while (word) {
-                        const int bit = __ffs(word) - 1;
-                        if ((unsigned long long)pos < (unsigned long long)cap) out[pos] = (int32_t)(wbase + bit);
-                        ++pos;
-                        word &= word - 1;
-                    }
-                    run += batch;
-                }
-            }
-        }
-        __syncthreads();  // bitmaps are rewritten by the next segment
+    }
+    __syncthreads();
+    if ((int)threadIdx.x < m) {
+        unsigned t = 0;
+        for (int w = 0; w < SEL_WARPS; ++w) t += s_kept[threadIdx.x][w];
+        sc.tot[(size_t)threadIdx.x * sc.ranges + blockIdx.x] = t;
     }
 }
 
-template <int U, bool VEC>
-unsigned resident_k2() {
-    static unsigned cached = 0;
-    if (!cached) {
-        cudaFuncSetAttribute(k2_match_multi<U, VEC>, cudaFuncAttributeMaxDynamicSharedMemorySize, k2_bitmap_bytes<U>());
-        int v = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, k2_match_multi<U, VEC>, K2_THREADS, k2_bitmap_bytes<U>()) !=
-                cudaSuccess || v <= 0)
-            v = 1;
-        cached = (unsigned)(v * sm_count());
+// CTA j: the first output row of each of list j's ranges, and its row count
+__global__ void __launch_bounds__(SEL_THREADS) k_scan_ranges(const __grid_constant__ MultiArgs args, SelScratch all) {
+    const SelScratch sc = list_of(all, blockIdx.x);
+    const unsigned long long n = sel_scan_totals(sc.tot, sc.off, sc.ranges);
+    if (threadIdx.x == 0) {
+        *args.d_rows[blockIdx.x] = (int64_t)n;
+        *args.h_rows[blockIdx.x] = (int64_t)n;
     }
-    return cached;
 }
 
-// chunk length for m patterns: all m bitmaps fit the instance's bitmap bytes
-template <int U>
-int64_t k2_chunk_len(int m) {
-    const int64_t bits = (int64_t)k2_bitmap_bytes<U>() * 8 / m;
-    return std::max<int64_t>(K2_STEP, bits / K2_STEP * K2_STEP);
-}
-
-template <int U, bool VEC>
-int launch_u(tid_ctx *ctx, const int32_t *S, const int32_t *P, const int32_t *O, int64_t n, const MultiArgs &a) {
-    const unsigned gmax = resident_k2<U, VEC>();
-    int64_t chunk = k2_chunk_len<U>(a.m);
-    // fewer, longer chunks are never needed: shrink the grid for small stores
-    int64_t chunks = std::min<int64_t>(gmax, ceil_div(n, chunk));
-    if (chunks < (int64_t)gmax) chunk = ceil_div(ceil_div(n, chunks), K2_STEP) * K2_STEP;
-    chunks = std::min<int64_t>(chunks, ceil_div(n, chunk));
-    const int n_seg = (int)ceil_div(n, chunks * chunk);
-    Lookback lb{};
-    TID_TRY(lookback_scratch(ctx, (unsigned)(chunks * n_seg * a.m), &lb));
-    lb.num_tiles = (unsigned)chunks;
-    k2_match_multi<U, VEC><<<(unsigned)chunks, K2_THREADS, (size_t)(chunk / 8) * a.m, ctx->stream>>>(
-        S, P, O, n, chunk, n_seg, a, lb);
-    return launch_check("k2_match_multi");
+__global__ void __launch_bounds__(SEL_THREADS) k2_expand(const __grid_constant__ MultiArgs args, SelScratch all) {
+    const SelScratch sc = list_of(all, blockIdx.y);
+    if (sc.tot[blockIdx.x]) sel_expand_index(sc, blockIdx.x, args.out[blockIdx.y], args.cap[blockIdx.y]);
 }
 
 template <int U>
 int launch_vec(bool vec, tid_ctx *ctx, const int32_t *S, const int32_t *P, const int32_t *O, int64_t n,
                const MultiArgs &a) {
-    return vec ? launch_u<U, true>(ctx, S, P, O, n, a) : launch_u<U, false>(ctx, S, P, O, n, a);
+    SelScratch sc{};
+    void *blk = nullptr;
+    TID_TRY(sel_scratch(ctx, n, a.m, 0, &sc, &blk, nullptr));
+    cudaStream_t st = ctx->stream;
+    if (vec) k2_mark<U, true><<<sc.ranges, SEL_THREADS, 0, st>>>(S, P, O, n, a, sc);
+    else k2_mark<U, false><<<sc.ranges, SEL_THREADS, 0, st>>>(S, P, O, n, a, sc);
+    int rc = launch_check("k2_mark");
+    if (rc == TID_OK) {
+        k_scan_ranges<<<a.m, SEL_THREADS, 0, st>>>(a, sc);
+        rc = launch_check("k_scan_ranges");
+    }
+    if (rc == TID_OK) {
+        k2_expand<<<dim3(sc.ranges, a.m), SEL_THREADS, 0, st>>>(a, sc);
+        rc = launch_check("k2_expand");
+    }
+    dev_free(ctx, blk);
+    return rc;
 }
 
 }  // namespace

@@ -99,6 +99,7 @@ struct tid_ctx {
     size_t lb_cap = 0;           // status words allocated
     unsigned int *lb_ticket = nullptr;
     unsigned int epoch = 0;
+    unsigned int *sel_done = nullptr;  // finished CTAs of a row selection (select.cuh), 0 between launches
     // error word in mapped pinned memory (written by kernels, read by host)
     int *err_host = nullptr;
     int *err_dev = nullptr;

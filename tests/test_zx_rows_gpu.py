@@ -132,3 +132,31 @@ def test_member_join_large(ctx, orc):
     assert np.array_equal(_rows(tb.tid_join(ctx, hr, hl)), orc.join(R, L, method="sortmerge").rows)
     tb.tid_set_free(hl)
     tb.tid_set_free(hr)
+
+
+@pytest.mark.parametrize("n", [1, 1023, 1024, 1025, 8191, 8193, 300_001, 39_900_007])
+@pytest.mark.parametrize("shift", [0, 1])
+def test_search_edges(ctx, n, shift):
+    """Single and multi-pattern searches around the step and range boundaries (a range is 8 steps, from
+    39.8M triples on 32), columns 16-byte aligned or not, against torch.nonzero; ranges without a hit,
+    with few and with all."""
+    g = torch.Generator(device="cuda").manual_seed(n)
+    cols = [torch.randint(1, hi, (n + shift,), generator=g, device="cuda", dtype=torch.int32)[shift:]
+            for hi in (5, 400, 2_000_000)]
+    cols[1][n // 3: n // 2] = 7                       # a stretch where every triple matches
+    cols[2][n - 1] = 3_000_000                        # a single hit, the last triple
+    torch.cuda.synchronize()
+    st = tb.tid_load(ctx, *cols, copy=0)
+    keys = [(1, 0, 0), (0, 7, 0), (0, 0, 3_000_000), (2, 7, 0), (0, 0, 0), (4_000, 0, 0), (0, 9, 3_000_000)]
+    want = []
+    for k in keys:
+        hit = torch.ones(n, dtype=torch.bool, device="cuda")
+        for c, v in zip(cols, k):
+            if v:
+                hit &= c == v
+        want.append(torch.nonzero(hit)[:, 0].int().cpu().numpy())
+    for k, w in zip(keys, want):
+        assert np.array_equal(_rows(tb.tid_match(ctx, st, k))[:, 0], w), k
+    for h, k, w in zip(tb.tid_match_multi(ctx, st, keys), keys, want):
+        assert np.array_equal(_rows(h)[:, 0], w), k
+    tb.tid_store_free(st)
