@@ -22,7 +22,7 @@
 
 namespace tid {
 int bind_set(tid_ctx *ctx, const tid_store *st, const tid_pattern &pat, const tid_set *idx, const tid_pred *preds,
-             int n_preds, tid_set **out);
+             int n_preds, tid_set **out, const VarMember *mem = nullptr, int n_mem = 0);
 }  // namespace tid
 
 using namespace tid;

@@ -89,13 +89,19 @@ int pattern_vars(const tid_pattern &pat, int8_t *vars, int *k, bool *anonymous) 
 }
 
 int bind_set(tid_ctx *ctx, const tid_store *st, const tid_pattern &pat, const tid_set *idx, const tid_pred *preds,
-             int n_preds, tid_set **out) {
+             int n_preds, tid_set **out, const VarMember *mem, int n_mem) {
     int8_t vars[TID_MAX_COLS];
     int k = 0;
     bool anon = false;
     TID_TRY(pattern_vars(pat, vars, &k, &anon));
     Pred pr[MAX_PREDS];
     TID_TRY(make_preds(vars, k, preds, n_preds, pr, "tid_bind"));
+    BindMember bm[MAX_MEMBERS];
+    for (int q = 0; q < n_mem; ++q) {
+        bm[q].m = mem[q].m;
+        for (int c = 0; c < k; ++c)
+            if (vars[c] == mem[q].var) bm[q].col = c;
+    }
     int64_t n = 0;
     TID_TRY(set_rows_host(idx, &n));
     if (n == 0) return empty_set(ctx, k, vars, out);
@@ -108,7 +114,7 @@ int bind_set(tid_ctx *ctx, const tid_store *st, const tid_pattern &pat, const ti
         if (e == cudaSuccess) e = cudaMemsetAsync(mm + TID_MAX_COLS, 0, TID_MAX_COLS * sizeof(uint32_t), ctx->stream);
         if (e != cudaSuccess) rc = fail_cuda(e, "tid_bind");
     }
-    if (rc == TID_OK) rc = compact_bind(ctx, st, pat, idx->col[0], n, pr, n_preds, nullptr, 0, tmp, mm);
+    if (rc == TID_OK) rc = compact_bind(ctx, st, pat, idx->col[0], n, pr, n_preds, bm, n_mem, tmp, mm);
     uint32_t hb[2 * TID_MAX_COLS];
     if (rc == TID_OK) {
         cudaError_t e = cudaMemcpyAsync(hb, mm, sizeof hb, cudaMemcpyDeviceToHost, ctx->stream);
@@ -436,7 +442,7 @@ extern "C" int tid_bind(tid_ctx *ctx, const tid_store *st, tid_pattern pat, cons
     if (st->ctx != ctx) return fail(TID_ERR_ARG, "tid_bind: store belongs to another context");
     if (idx->k != 1 || idx->vars[0] != -1) return fail(TID_ERR_ARG, "tid_bind: idx must be an index set from tid_match");
     DeviceGuard g(ctx->device);
-    return bind_set(ctx, st, pat, idx, preds, n_preds, out);
+    return bind_set(ctx, st, pat, idx, preds, n_preds, out, nullptr, 0);
 }
 
 extern "C" int tid_filter(tid_ctx *ctx, const tid_set *in, const tid_pred *preds, int n_preds, tid_set **out) {

@@ -47,6 +47,11 @@ struct Bounds {
     uint32_t lo[TID_MAX_COLS], hi[TID_MAX_COLS];
 };
 
+struct VarMember {  // the same by variable
+    Members m;
+    int8_t var;
+};
+
 // exclusive scan of n uint32 (out may alias in); *total_dev receives the sum
 int scan_exclusive_u32(tid_ctx *ctx, const uint32_t *in, uint32_t *out, int64_t n,
                        unsigned long long *total_dev);

@@ -160,3 +160,54 @@ def test_search_edges(ctx, n, shift):
     for h, k, w in zip(tb.tid_match_multi(ctx, st, keys), keys, want):
         assert np.array_equal(_rows(h)[:, 0], w), k
     tb.tid_store_free(st)
+
+
+X, Y, Z, W = 0, 1, 2, 3
+
+
+def _plan_store(seed, n):
+    rng = np.random.default_rng(seed)
+    t = np.unique(np.stack([rng.integers(1, n // 6, n), rng.integers(1, 5, n) + (1 << 20), rng.integers(1, n // 6, n)], 1),
+                  axis=0)
+    t = t[rng.permutation(len(t))].astype(np.int32)
+    return [np.ascontiguousarray(t[:, c]) for c in range(3)]
+
+
+@pytest.mark.parametrize("algo", ["auto", "hash", "left", "right", "full"])
+@pytest.mark.parametrize("n", [3_000, 60_000, 1_200_000])
+def test_plan_extracts_what_a_join_needs(ctx, orc, algo, n):
+    """A small side reduces the extraction of a large MATCH (below and above the row selection's sizes), on
+    either input, through FILTERs, on one and two shared variables, with an empty small side; outer joins
+    keep their unmatched rows."""
+    from paper_1807_01409_gb300 import synth
+    S, P, O = _plan_store(n, n)
+    st = tb.tid_load(ctx, S, P, O)
+    p = 1 << 20
+    few = {"op": "match", "pattern": synth.Pattern(0, p + 1, int(O[P == p + 1][0]), var=(X, -1, -1))}
+    some = [{"op": "match", "pattern": synth.Pattern(0, p + 2, 0, var=(X, -1, Y))},
+            {"op": "filter", "input": 0, "var": X, "cmp": "le", "a": n // 600}]
+    many = {"op": "match", "pattern": synth.Pattern(0, p + 3, 0, var=(X, -1, Y))}
+    other = {"op": "match", "pattern": synth.Pattern(0, p + 4, 0, var=(Z, -1, X))}
+    none = {"op": "match", "pattern": synth.Pattern(0, p + 1, 1 << 29, var=(X, -1, -1))}
+    plans = []
+    for small in (few, none):
+        for big in (many, other):
+            plans += [[small, big, {"op": "join", "inputs": [0, 1], "algo": algo}],
+                      [small, big, {"op": "join", "inputs": [1, 0], "algo": algo}]]
+    plans += [some + [many, {"op": "join", "inputs": [1, 2], "algo": algo}],       # two shared variables
+              some + [many, {"op": "filter", "input": 2, "var": Y, "cmp": "ge", "a": 10},
+                      {"op": "join", "inputs": [3, 1], "algo": algo}],
+              [few, many, other, {"op": "join", "inputs": [0, 1], "algo": algo}, {"op": "join", "inputs": [3, 2], "algo": algo},
+               {"op": "project", "input": 4, "vars": [X, Z]}],
+              [few, many, {"op": "join", "inputs": [0, 1], "algo": algo}, {"op": "union", "inputs": [1, 2]}]]
+    if algo == "hash":  # an outer join is not a hash join; a chain through both inputs is
+        plans = plans[:-1]
+    for plan in plans:
+        got = _rows(tb.tid_exec(ctx, st, plan))
+        want = orc.execute(S, P, O, plan)
+        assert np.array_equal(got, want.rows), plan
+    bad = [few, many, {"op": "filter", "input": 1, "var": W, "cmp": "ge", "a": 1}, {"op": "join", "inputs": [0, 2]}]
+    with pytest.raises(tb.TidError) as e:  # a FILTER on a variable that its MATCH lacks is still refused
+        tb.tid_exec(ctx, st, bad)
+    assert e.value.code == tb.TID_ERR_ARG
+    tb.tid_store_free(st)
