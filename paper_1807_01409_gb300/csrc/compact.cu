@@ -548,7 +548,7 @@ k_sel_expand(Row row, int k_out, OutCols out, int64_t cap, SelScratch sc, uint32
     };
     constexpr int UX = K == 1 ? 8 : 4;  // rows per lane read together
     uint16_t *stage = s_stage[warp];
-    sel_walk(sc, blockIdx.x, [&](unsigned step, uint32_t word, unsigned xo, unsigned sn, unsigned long long o0) {
+    sel_walk(sc, blockIdx.x, warp, SEL_WARPS, [&](unsigned step, uint32_t word, unsigned xo, unsigned sn, unsigned long long o0) {
         const int64_t base = (int64_t)step * SEL_STEP;
         if (sn >= SEL_DENSE) {
 #pragma unroll 1
@@ -796,10 +796,11 @@ __global__ void __launch_bounds__(SC_THREADS) k_tile_sums(const uint32_t *__rest
 
 }  // namespace
 
-int sel_scratch(tid_ctx *ctx, int64_t n, int lists, size_t extra, SelScratch *sc, void **block, void **extra_at) {
+int sel_scratch(tid_ctx *ctx, int64_t n, int lists, size_t extra, SelScratch *sc, void **block, void **extra_at,
+                unsigned per) {
     sc->steps = (unsigned)ceil_div(n, (int64_t)SEL_STEP);
     // a range is one step per warp, or four once that still gives every SM eight CTAs
-    sc->per = sc->steps >= (unsigned)sm_count() * 256 ? 4 * SEL_WARPS : SEL_WARPS;
+    sc->per = per ? per : sc->steps >= (unsigned)sm_count() * 256 ? 4 * SEL_WARPS : SEL_WARPS;
     sc->ranges = (unsigned)ceil_div(sc->steps, (int64_t)sc->per);
     auto pad = [](size_t b) { return (b + 255) / 256 * 256; };
     const size_t bits_b = (size_t)sc->steps * 32 * 4 * lists, cnt_b = pad((size_t)sc->steps * 4 * lists);

@@ -6,20 +6,31 @@
 // each sorted in the union schema, so their union is a merge followed by
 // dropping adjacent duplicates -- no sort.  Merge path (Odeh, Green, Mwassi,
 // Shmueli and Birk, "Merge Path - Parallel Merging Made Simple", IPDPSW 2012):
-//  * k_merge_split: for every tile boundary d (a multiple of MG_TILE merged
-//    rows), the number of A rows among the first d merged rows, by binary
-//    search along the cross diagonal (A before B on equal rows);
-//  * k_merge_unique: a CTA loads its tile's A and B rows into shared memory,
-//    each thread merges 8 rows along its own diagonal, then rows equal to
-//    their predecessor in merged order are dropped and the kept rows written
-//    in order (ballot ranks, tile offset from the decoupled look-back).
-// Bytes: every input row read once, every distinct row written once (+ the
-// split search, O(tiles x log n) rows).
+//  * k_merge_split: for every tile boundary d, the number of A rows among the
+//    first d merged rows, by a search along the cross diagonal (A before B on
+//    equal rows), a warp per boundary testing 32 places at once;
+//  * rows whose columns fit 64 bits together (the usual case; a variable that one
+//    branch lacks takes one more value than the other holds, its 0, rather than
+//    the range from 0 to it): k_merge_mark packs a tile's rows as it loads them, so
+//    a row is one word of shared memory and a comparison one instruction; a thread
+//    merges 16 rows along its own diagonal and leaves two bits per merged row: from
+//    A or B, and different from its predecessor (mark of select.cuh);
+//    k_merge_expand writes the kept rows, reading A and B once more in order;
+//  * wider rows: k_merge_unique merges columns in shared memory, 8 rows per
+//    thread, tile offsets from the decoupled look-back.
+// Bytes: every input row read twice (the second time partly from L2), every
+// distinct row written once.  Measured on GB300, 23.6M (x, v) with 8.2M (x, y):
+// k_merge_split 26 -> 19 us (a warp per boundary instead of a thread), merging
+// 583 us by k_merge_unique, 416 us packed with a look-back (a tile waited for
+// its predecessors three times as long as it worked, at three CTAs per SM),
+// 162 us by k_merge_mark and 135 us by k_merge_expand.  Bound: the mark's
+// shared-memory steps; the expansion's reads.
 
 #include <algorithm>
 
 #include "lookback.cuh"
 #include "ops.cuh"
+#include "select.cuh"
 
 namespace tid {
 
@@ -50,18 +61,205 @@ __device__ __forceinline__ int cmp_pad(const PadCols &A, int64_t i, const PadCol
     return r;
 }
 
-__global__ void k_merge_split(PadCols A, int64_t na, PadCols B, int64_t nb, int nu, int64_t tiles,
-                              int64_t *__restrict__ split) {
-    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+// Warp t: split[t] for the boundary before tile t (t <= tiles).  A[mid] precedes
+// B[d - 1 - mid] for every mid below the answer and for none from it on.
+__global__ void __launch_bounds__(256) k_merge_split(PadCols A, int64_t na, PadCols B, int64_t nb, int nu, int64_t tiles,
+                                                     int tile_rows, int64_t *__restrict__ split) {
+    const int64_t t = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
     if (t > tiles) return;
-    const int64_t d = min(t * MG_TILE, na + nb);
+    const unsigned lane = threadIdx.x & 31;
+    const int64_t d = min(t * tile_rows, na + nb);
     int64_t lo = max((int64_t)0, d - nb), hi = min(d, na);
-    while (lo < hi) {  // A[mid] precedes B[d - 1 - mid]: at least mid + 1 A rows come first
-        const int64_t mid = (lo + hi) >> 1;
-        if (cmp_pad(A, mid, B, d - 1 - mid, nu) <= 0) lo = mid + 1;
+    while (lo < hi) {  // lane l tests the end of the l-th of 32 equal parts
+        const int64_t part = (hi - lo + 31) / 32, mid = lo + (lane + 1) * part - 1;
+        const bool below = mid < hi && cmp_pad(A, mid, B, d - 1 - mid, nu) <= 0;
+        const int full = __popc(__ballot_sync(0xffffffffu, below));  // parts wholly below the answer
+        lo += (int64_t)full * part;
+        hi = min(hi, lo + part - 1);
+    }
+    if (lane == 0) split[t] = min(lo, min(d, na));
+}
+
+typedef unsigned long long u64;
+
+constexpr int MP_THREADS = 256;
+constexpr int MP_ITEMS = 16;
+constexpr int MP_TILE = MP_THREADS * MP_ITEMS;  // merged rows per tile
+
+// One column's field of a packed row; zero: 0 is the field 0 and the values from
+// min + 1 (sort order) up follow it.
+__device__ __forceinline__ u64 pack_field(const MergePack &mp, int c, int32_t x) {
+    const uint32_t f = ((mp.zero >> c) & 1u) && x == 0 ? 0u : ((uint32_t)x ^ 0x80000000u) - mp.ps.min[c];
+    return (u64)f << mp.ps.shift[c];
+}
+__device__ __forceinline__ u64 pack_one(const MergePack &mp, const PadCols &A, int nu, int64_t i) {
+    u64 key = 0;
+#pragma unroll
+    for (int c = 0; c < TID_MAX_COLS; ++c)
+        if (c < nu && mp.ps.mask[c]) key |= pack_field(mp, c, pval(A, c, i));
+    return key;
+}
+
+// Merged rows: the selection's scratch, and per step the bits "from A" (32 words)
+// and the first A row.
+struct MergeBits {
+    SelScratch sc;
+    uint32_t *take;
+    uint32_t *first_a;
+};
+
+__global__ void __launch_bounds__(MP_THREADS, 4)
+k_merge_mark(PadCols A, int64_t na, PadCols B, int64_t nb, int nu, MergePack mp, const int64_t *__restrict__ split,
+             MergeBits mb, int64_t *__restrict__ d_rows, int64_t *__restrict__ h_rows) {
+    __shared__ u64 s_key[MP_TILE];
+    __shared__ u64 s_before;  // the merged row before the tile
+    __shared__ unsigned s_cnt[MP_THREADS / 32];
+    const unsigned lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t tile = blockIdx.x;
+    const int64_t d0 = tile * MP_TILE, d1 = min(d0 + MP_TILE, na + nb);
+    const int64_t a0 = split[tile], a1 = split[tile + 1], b0 = d0 - a0;
+    const int la = (int)(a1 - a0), len = (int)(d1 - d0);
+    {  // pack the tile's rows, A's first
+        u64 k[MP_ITEMS];
+#pragma unroll
+        for (int q = 0; q < MP_ITEMS; ++q) k[q] = 0;
+#pragma unroll
+        for (int c = 0; c < TID_MAX_COLS; ++c) {
+            if (c >= nu) break;
+            if (!mp.ps.mask[c]) continue;
+            int32_t x[MP_ITEMS];
+#pragma unroll
+            for (int q = 0; q < MP_ITEMS; ++q) {
+                const int r = q * MP_THREADS + threadIdx.x;
+                x[q] = 0;
+                if (r < la) {
+                    if (A.c[c]) x[q] = A.c[c][a0 + r];
+                } else if (r < len) {
+                    if (B.c[c]) x[q] = B.c[c][b0 + (r - la)];
+                }
+            }
+#pragma unroll
+            for (int q = 0; q < MP_ITEMS; ++q) k[q] |= pack_field(mp, c, x[q]);
+        }
+#pragma unroll
+        for (int q = 0; q < MP_ITEMS; ++q) {
+            const int r = q * MP_THREADS + threadIdx.x;
+            if (r < len) s_key[r] = k[q];
+        }
+    }
+    if (threadIdx.x == 0 && d0 > 0) {
+        u64 v = 0;
+        if (a0 > 0) v = pack_one(mp, A, nu, a0 - 1);
+        if (b0 > 0) v = max(v, pack_one(mp, B, nu, b0 - 1));
+        s_before = v;
+    }
+    __syncthreads();
+    // this thread's diagonal: local merged rows [dt, dt + 16)
+    const int dt = min((int)threadIdx.x * MP_ITEMS, len), lb_ = len - la;
+    int lo = max(0, dt - lb_), hi = min(dt, la);
+    while (lo < hi) {
+        const int mid = (lo + hi) >> 1;
+        if (s_key[mid] <= s_key[la + dt - 1 - mid]) lo = mid + 1;
         else hi = mid;
     }
-    split[t] = lo;
+    int i = lo, j = la + dt - lo;  // next A row, next B row
+    // the merged row before the diagonal: the larger of the two before it
+    u64 prev = 0;
+    bool has_prev = true;
+    if (i > 0) prev = s_key[i - 1];
+    if (j > la) prev = max(prev, s_key[j - 1]);
+    if (i == 0 && j == la) {  // the tile's first row
+        has_prev = d0 > 0;
+        prev = has_prev ? s_before : 0;
+    }
+    // step of this thread's rows: 64 threads each
+    const int64_t step = tile * (MP_TILE / SEL_STEP) + (threadIdx.x >> 6);
+    if ((threadIdx.x & 63) == 0 && step < mb.sc.steps) mb.first_a[step] = (uint32_t)(a0 + i);
+    u64 ka = i < la ? s_key[i] : 0, kb = j < len ? s_key[j] : 0;
+    unsigned keep = 0, take = 0;
+#pragma unroll
+    for (int e = 0; e < MP_ITEMS; ++e) {
+        if (dt + e >= len) break;
+        const bool take_a = j >= len || (i < la && ka <= kb);
+        const u64 v = take_a ? ka : kb;
+        if (!has_prev || v != prev) keep |= 1u << e;
+        has_prev = true;
+        prev = v;
+        if (take_a) {
+            take |= 1u << e;
+            ++i;
+            ka = i < la ? s_key[i] : 0;
+        } else {
+            ++j;
+            kb = j < len ? s_key[j] : 0;
+        }
+    }
+    // two threads' 16 rows are one word
+    const unsigned c = __reduce_add_sync(0xffffffffu, __popc(keep));
+    keep |= __shfl_down_sync(0xffffffffu, keep, 1) << 16;
+    take |= __shfl_down_sync(0xffffffffu, take, 1) << 16;
+    if (!(lane & 1) && step < mb.sc.steps) {
+        const size_t w = (size_t)step * 32 + ((threadIdx.x & 63) >> 1);
+        mb.sc.bits[w] = keep;
+        mb.take[w] = take;
+    }
+    if (lane == 0) s_cnt[warp] = c;
+    __syncthreads();
+    if ((threadIdx.x & 63) == 0 && step < mb.sc.steps) mb.sc.cnt[step] = s_cnt[warp] + s_cnt[warp + 1];
+    sel_finish(mb.sc, c, d_rows, h_rows);
+}
+
+template <int K>
+__global__ void __launch_bounds__(SEL_THREADS, K <= 3 ? 4 : 2)
+k_merge_expand(PadCols A, PadCols B, int nu, MergeBits mb, OutCols out, int64_t cap) {
+    const unsigned lane = threadIdx.x & 31, lt = (1u << lane) - 1u;
+    constexpr int UX = 4;  // rows per lane read together
+    // a range is four steps, one per warp: two ranges per CTA
+    const unsigned warp = threadIdx.x >> 5, per = MP_TILE / SEL_STEP;
+    const unsigned range = blockIdx.x * (SEL_WARPS / per) + warp / per;
+    if (range >= mb.sc.ranges) return;
+    sel_walk(mb.sc, range, warp % per, per, [&](unsigned step, uint32_t word, unsigned xo, unsigned, unsigned long long o0) {
+        const uint32_t take = mb.take[(size_t)step * 32 + lane];
+        const unsigned pc = __popc(take);
+        unsigned tx = pc;
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const unsigned y = __shfl_up_sync(0xffffffffu, tx, d);
+            if ((int)lane >= d) tx += y;
+        }
+        tx -= pc;
+        const uint32_t as = mb.first_a[step], bs = step * SEL_STEP - as;
+#pragma unroll 1
+        for (int w0 = 0; w0 < 32; w0 += UX) {
+            int32_t v[UX][K];
+            unsigned bw[UX];
+#pragma unroll
+            for (int u = 0; u < UX; ++u) {
+                const int w = w0 + u;
+                bw[u] = __shfl_sync(0xffffffffu, word, w);
+                const uint32_t tw = __shfl_sync(0xffffffffu, take, w), at = __shfl_sync(0xffffffffu, tx, w);
+                const bool from_a = (tw >> lane) & 1u;
+                const uint32_t r = from_a ? as + at + __popc(tw & lt) : bs + (w * 32 - at) + __popc(~tw & lt);
+                if ((bw[u] >> lane) & 1u) {
+#pragma unroll
+                    for (int c = 0; c < K; ++c) {
+                        if (c >= nu) break;
+                        const int32_t *p = from_a ? A.c[c] : B.c[c];
+                        v[u][c] = p ? p[r] : 0;
+                    }
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < UX; ++u) {
+                const unsigned long long pos = o0 + __shfl_sync(0xffffffffu, xo, w0 + u) + __popc(bw[u] & lt);
+                if (((bw[u] >> lane) & 1u) && pos < (unsigned long long)cap) {
+#pragma unroll
+                    for (int c = 0; c < K; ++c)
+                        if (c < nu) out.col[c][pos] = v[u][c];
+                }
+            }
+        }
+    });
 }
 
 // shared-memory rows: column c of local row r at s_rows[c * (MG_TILE + 1) + r];
@@ -193,10 +391,15 @@ struct Scratch {
 }  // namespace
 
 int merge_unique(tid_ctx *ctx, const int32_t *const *acols, int64_t na, const int32_t *const *bcols, int64_t nb,
-                 int nu, tid_set *out) {
+                 int nu, const MergePack *mp, tid_set *out) {
     if (nu < 1 || nu > TID_MAX_COLS) return fail(TID_ERR_ARG, "merge: %d columns", nu);
     cudaStream_t st = ctx->stream;
     if (na + nb == 0) return set_rows_const(out, 0);
+    if (nb == 0) {  // one sorted side with all its columns: its distinct rows
+        bool all = true;
+        for (int c = 0; c < nu; ++c) all = all && acols[c];
+        if (all) return compact_unique(ctx, acols, nu, nullptr, na, out);
+    }
     PadCols A{}, B{};
     for (int c = 0; c < nu; ++c) {
         A.c[c] = acols[c];
@@ -204,12 +407,33 @@ int merge_unique(tid_ctx *ctx, const int32_t *const *acols, int64_t na, const in
     }
     OutCols oc{};
     for (int c = 0; c < nu; ++c) oc.col[c] = out->col[c];
-    const int64_t tiles = ceil_div(na + nb, (int64_t)MG_TILE);
+    const int tile_rows = mp ? MP_TILE : MG_TILE;
+    const int64_t tiles = ceil_div(na + nb, (int64_t)tile_rows);
     Scratch s(ctx);
     TID_TRY(dev_alloc(ctx, &s.p, sizeof(int64_t) * (tiles + 1)));
     int64_t *split = (int64_t *)s.p;
-    k_merge_split<<<(unsigned)ceil_div(tiles + 1, 256), 256, 0, st>>>(A, na, B, nb, nu, tiles, split);
+    k_merge_split<<<(unsigned)ceil_div(tiles + 1, 8), 256, 0, st>>>(A, na, B, nb, nu, tiles, tile_rows, split);
     TID_TRY(launch_check("k_merge_split"));
+    if (mp) {
+        MergeBits mb{};
+        const size_t steps = (size_t)ceil_div(na + nb, (int64_t)SEL_STEP);
+        void *blk = nullptr, *extra = nullptr;
+        TID_TRY(sel_scratch(ctx, na + nb, 1, steps * 33 * 4, &mb.sc, &blk, &extra, MP_TILE / SEL_STEP));
+        mb.take = (uint32_t *)extra;
+        mb.first_a = mb.take + steps * 32;
+        k_merge_mark<<<(unsigned)tiles, MP_THREADS, 0, st>>>(A, na, B, nb, nu, *mp, split, mb, out->d_rows, out->slot.dev);
+        int rc = launch_check("k_merge_mark");
+        if (rc == TID_OK) {
+            const unsigned grid = (unsigned)ceil_div(mb.sc.ranges, (int64_t)(SEL_WARPS / (MP_TILE / SEL_STEP)));
+            if (nu <= 3) k_merge_expand<3><<<grid, SEL_THREADS, 0, st>>>(A, B, nu, mb, oc, out->cap);
+            else k_merge_expand<TID_MAX_COLS><<<grid, SEL_THREADS, 0, st>>>(A, B, nu, mb, oc, out->cap);
+            rc = launch_check("k_merge_expand");
+        }
+        dev_free(ctx, blk);
+        return rc;
+    }
+    Lookback lb{};
+    TID_TRY(lookback_scratch(ctx, (unsigned)tiles, &lb));
     const size_t smem = sizeof(int32_t) * nu * (MG_TILE + 1);
     static bool opted = false;
     if (!opted) {
@@ -218,8 +442,6 @@ int merge_unique(tid_ctx *ctx, const int32_t *const *acols, int64_t na, const in
                      "k_merge_unique smem");
         opted = true;
     }
-    Lookback lb{};
-    TID_TRY(lookback_scratch(ctx, (unsigned)tiles, &lb));
     k_merge_unique<<<(unsigned)tiles, MG_THREADS, smem, st>>>(A, na, B, nb, nu, split, oc, out->cap, out->d_rows,
                                                               out->slot.dev, lb);
     return launch_check("k_merge_unique");

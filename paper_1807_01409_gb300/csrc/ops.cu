@@ -159,7 +159,7 @@ int bind_set(tid_ctx *ctx, const tid_store *st, const tid_pattern &pat, const ti
         tid_set *o = nullptr;
         const int32_t *none[TID_MAX_COLS] = {nullptr};
         rc = set_alloc(ctx, k, vars, m, &o);
-        if (rc == TID_OK) rc = merge_unique(ctx, cols, m, none, 0, k, o);
+        if (rc == TID_OK) rc = merge_unique(ctx, cols, m, none, 0, k, nullptr, o);
         if (rc == TID_OK) rc = set_ready(o);
         if (rc == TID_OK) {
             o->bounded = m > 0;
@@ -260,6 +260,39 @@ int union_sets(tid_ctx *ctx, const tid_set *const *in, int k, tid_set **out) {
         }
     }
     if (ordered) {
+        // the rows as 64-bit words, if every field fits: a column's range over the
+        // inputs that have it, and 0 for those that lack it
+        MergePack mp{};
+        bool packed = known;
+        int bits = 0;
+        for (int u = nu - 1; u >= 0 && packed; --u) {
+            uint32_t lo = 0xFFFFFFFFu, hi = 0u;
+            bool absent = false;
+            for (int i = 0; i < k; ++i) {
+                if (rows[i] == 0) continue;
+                const int c = find_col(in[i], uv[u]);
+                if (c < 0) {
+                    absent = true;
+                    continue;
+                }
+                lo = std::min(lo, in[i]->lo[c]);
+                hi = std::max(hi, in[i]->hi[c]);
+            }
+            if (lo > hi) lo = hi = 0x80000000u;  // 0 in every row
+            if (absent && lo > 0x80000000u) {
+                mp.zero |= 1u << u;
+                lo -= 1;
+            } else if (absent) {
+                lo = std::min(lo, 0x80000000u);
+                hi = std::max(hi, 0x80000000u);
+            }
+            const int w = hi == lo ? 0 : 32 - __builtin_clz(hi - lo);
+            mp.ps.min[u] = lo;
+            mp.ps.shift[u] = (uint32_t)bits;
+            mp.ps.mask[u] = (1ull << w) - 1ull;
+            bits += w;
+            packed = bits <= 64;
+        }
         tid_set *cur = nullptr;  // union of the inputs merged so far (null: only in[0])
         int rc = TID_OK;
         for (int i = 1; i < k && rc == TID_OK; ++i) {
@@ -274,7 +307,7 @@ int union_sets(tid_ctx *ctx, const tid_set *const *in, int k, tid_set **out) {
             rc = set_rows_host(A, &na);
             tid_set *m = nullptr;
             if (rc == TID_OK) rc = set_alloc(ctx, nu, uv, na + rows[i], &m);
-            if (rc == TID_OK) rc = merge_unique(ctx, ac, na, bc, rows[i], nu, m);
+            if (rc == TID_OK) rc = merge_unique(ctx, ac, na, bc, rows[i], nu, packed ? &mp : nullptr, m);
             if (rc == TID_OK) rc = set_ready(m);
             if (cur) set_free(cur);
             cur = m;
@@ -287,7 +320,7 @@ int union_sets(tid_ctx *ctx, const tid_set *const *in, int k, tid_set **out) {
             const int32_t *ac[TID_MAX_COLS], *none[TID_MAX_COLS] = {nullptr};
             for (int u = 0; u < nu; ++u) ac[u] = in[0]->col[find_col(in[0], uv[u])];
             rc = set_alloc(ctx, nu, uv, rows[0], &cur);
-            if (rc == TID_OK) rc = merge_unique(ctx, ac, rows[0], none, 0, nu, cur);
+            if (rc == TID_OK) rc = merge_unique(ctx, ac, rows[0], none, 0, nu, nullptr, cur);
             if (rc == TID_OK) rc = set_ready(cur);
             if (rc != TID_OK) {
                 if (cur) set_free(cur);
@@ -355,7 +388,7 @@ int project_set(tid_ctx *ctx, const tid_set *in, const int8_t *vars, int n_vars,
         tid_set *o = nullptr;
         const int32_t *none[TID_MAX_COLS] = {nullptr};
         TID_TRY(set_alloc(ctx, n_vars, vars, n, &o));
-        int rc = merge_unique(ctx, cols, n, none, 0, n_vars, o);
+        int rc = merge_unique(ctx, cols, n, none, 0, n_vars, nullptr, o);
         if (rc == TID_OK) rc = set_ready(o);
         if (rc != TID_OK) {
             set_free(o);

@@ -41,6 +41,14 @@ struct PackSpec {
     unsigned long long mask[TID_MAX_COLS];
 };
 
+// The same for the rows of a union: where bit c of `zero` is set, column c's field
+// 0 stands for 0 (unbound, a branch without the variable) and its other values,
+// all above 0, start at min[c] + 1.
+struct MergePack {
+    PackSpec ps;
+    unsigned zero;
+};
+
 // Column value bounds in sort order (int32 ^ 0x80000000); any valid bounds
 // serve the packed sort, exact ones make its keys narrowest.
 struct Bounds {
@@ -109,9 +117,10 @@ int outer_join_sets(tid_ctx *ctx, const tid_set *L, const tid_set *R, int algo, 
 
 // merge (merge.cu): the distinct rows of two sets each sorted in the same nu
 // columns (acols / bcols, null = absent column, read as 0) into out (capacity
-// >= na + nb), in order; writes the row count
+// >= na + nb), in order; writes the row count; mp (or null): how every row of
+// both packs into 64 bits
 int merge_unique(tid_ctx *ctx, const int32_t *const *acols, int64_t na, const int32_t *const *bcols, int64_t nb,
-                 int nu, tid_set *out);
+                 int nu, const MergePack *mp, tid_set *out);
 
 // set operators (ops.cu)
 int filter_set(tid_ctx *ctx, const tid_set *in, const tid_pred *preds, int n_preds, tid_set **out);

@@ -32,7 +32,9 @@ struct SelScratch {           // of one list; list j of several follows at j * (
 // Scratch for `lists` selections over n rows from the context's pool (*block is
 // freed by the caller; `extra` further bytes at *extra_at).  The finished-CTA
 // counter is the context's: the last CTA of a mark kernel sets it back to 0.
-int sel_scratch(tid_ctx *ctx, int64_t n, int lists, size_t extra, SelScratch *sc, void **block, void **extra_at);
+// per: steps per range (0: chosen by n).
+int sel_scratch(tid_ctx *ctx, int64_t n, int lists, size_t extra, SelScratch *sc, void **block, void **extra_at,
+                unsigned per = 0);
 
 // 4-bit masks of a lane's rows (m[g], bits e: row 128 g + 4 lane + e of the step)
 // to the step's keep words: lane 8k + g returns word 4g + k.
@@ -109,11 +111,12 @@ __device__ __forceinline__ void sel_finish(const SelScratch &sc, unsigned kept, 
 }
 
 // Walks a range in an expand kernel: body(step, word, word_prefix, kept, first
-// row) for every step with kept rows, a warp taking every eighth step; lane l
-// holds keep word l and the kept rows of the words before it.
+// row) for every step with kept rows, the steps dealt out to `warps` warps, of
+// which this is number `warp`; lane l holds keep word l and the kept rows of the
+// words before it.
 template <class Body>
-__device__ __forceinline__ void sel_walk(const SelScratch &sc, unsigned range, Body body) {
-    const unsigned lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+__device__ __forceinline__ void sel_walk(const SelScratch &sc, unsigned range, unsigned warp, unsigned warps, Body body) {
+    const unsigned lane = threadIdx.x & 31;
     const unsigned r0 = range * sc.per, r1 = min(r0 + sc.per, sc.steps);
     unsigned long long run = sc.off[range];
     for (unsigned q0 = r0; q0 < r1; q0 += 32) {
@@ -128,9 +131,9 @@ __device__ __forceinline__ void sel_walk(const SelScratch &sc, unsigned range, B
         }
         const unsigned kept = __shfl_sync(0xffffffffu, first, 31);
         first -= cnt;  // of step q0 + lane
-        for (unsigned li = warp; li < here; li += SEL_WARPS) {
+        for (unsigned li = warp; li < here; li += warps) {
             const uint32_t word = next;
-            if (li + SEL_WARPS < here) next = sc.bits[(size_t)(q0 + li + SEL_WARPS) * 32 + lane];
+            if (li + warps < here) next = sc.bits[(size_t)(q0 + li + warps) * 32 + lane];
             const unsigned sn = __shfl_sync(0xffffffffu, cnt, li);
             if (sn == 0) continue;
             const unsigned long long o0 = run + __shfl_sync(0xffffffffu, first, li);
@@ -164,7 +167,7 @@ __device__ __forceinline__ void sel_expand_index(const SelScratch &sc, unsigned 
     __shared__ uint16_t s_stage[SEL_WARPS][SEL_DENSE];
     const unsigned lane = threadIdx.x & 31, lt = (1u << lane) - 1u;
     uint16_t *stage = s_stage[threadIdx.x >> 5];
-    sel_walk(sc, range, [&](unsigned step, uint32_t word, unsigned xo, unsigned sn, unsigned long long o0) {
+    sel_walk(sc, range, threadIdx.x >> 5, SEL_WARPS, [&](unsigned step, uint32_t word, unsigned xo, unsigned sn, unsigned long long o0) {
         const int32_t base = (int32_t)(step * SEL_STEP);
         if (sn >= SEL_DENSE) {
 #pragma unroll 8

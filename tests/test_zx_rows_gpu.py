@@ -211,3 +211,26 @@ def test_plan_extracts_what_a_join_needs(ctx, orc, algo, n):
         tb.tid_exec(ctx, st, bad)
     assert e.value.code == tb.TID_ERR_ARG
     tb.tid_store_free(st)
+
+
+UNIONS = [((0, 1), (0, 2)), ((0, 1), (0, 1)), ((0,), (0, 1, 2)), ((0, 1, 2), (0, 2)), ((0, 1), (0, 2), (0, 1, 3)), ((2,), (2,))]
+
+
+@pytest.mark.parametrize("ids", ["dense", "clusters", "wide", "literals", "one"])
+@pytest.mark.parametrize("shape", range(len(UNIONS)))
+@pytest.mark.parametrize("n", [1, 2048, 4095, 4097, 30_000])
+def test_union_merges(ctx, orc, ids, shape, n):
+    """Branches merged without a sort: rows of up to 64 bits packed (a branch without a variable adds its 0
+    to the other's values), wider ones by column; repeats across branches, tile boundaries, uneven sizes."""
+    rng = np.random.default_rng([n, shape, len(ids)])
+    fn = dict(IDS, literals=lambda r, m: (1 << 30) + r.integers(0, 5000, m), one=lambda r, m: np.full(m, 9))[ids]
+    sets = [_random_set(orc, rng, v, max(1, n >> i), fn) for i, v in enumerate(UNIONS[shape])]
+    if UNIONS[shape][0] == UNIONS[shape][1]:  # half of the second branch repeats the first
+        sets[1] = orc.TupleSet(sets[1].vars, orc.canonical(np.concatenate([sets[1].rows, sets[0].rows[::2]])))
+    hs = [_set(ctx, s) for s in sets]
+    got = tb.tid_union(ctx, hs)
+    want = orc.union(sets)
+    assert tb.tid_set_info(got)["vars"] == tuple(want.vars)
+    assert np.array_equal(_rows(got), want.rows)
+    for h in hs:
+        tb.tid_set_free(h)
