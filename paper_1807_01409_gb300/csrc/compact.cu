@@ -479,7 +479,7 @@ k_compact(Row row, int64_t n, int k_out, OutCols out, int64_t cap, int64_t *__re
 // Bound: memory latency of the expansion's dependent loads (ncu: 57 % of DRAM
 // throughput binding 23.6M triples, long-scoreboard stalls).  Measured on GB300
 // (kernels, before -> after this form): FILTER of 24M two-column rows, half kept,
-// 227 -> 115 us; bind of 23.6M triples of a 200M store with a range FILTER
+// 227 -> 83 us; bind of 23.6M triples of a 200M store with a range FILTER
 // 700 -> 400 us (the tested column is gathered once and stashed); before, per
 // 2048-row tile: a count and a write launch (filter), one look-back launch (bind).
 // A mark phase with 4-byte loads in place of 16-byte ones took 58 us on the

@@ -18,7 +18,10 @@ namespace tid {
 constexpr int SEL_THREADS = 256;
 constexpr int SEL_WARPS = SEL_THREADS / 32;
 constexpr int SEL_STEP = 1024;         // rows per step
-constexpr unsigned SEL_DENSE = 256;    // kept rows from which a step is written word by word
+// Kept rows from which a step is written word by word (32 rounds of its words); a
+// step that keeps fewer puts its positions in shared memory first, and its rounds
+// then have every lane at work (a third of the rows kept: 10 rounds for 32).
+constexpr unsigned SEL_DENSE = 640;
 
 struct SelScratch {           // of one list; list j of several follows at j * (steps, ranges)
     uint32_t *bits;           // 32 keep words per step (bit b of word w: row 1024 step + 32 w + b)
