@@ -13,9 +13,8 @@
 //   * unique   -- after a sort, a row is kept when it differs from its
 //                 predecessor in sorted order (DISTINCT, Section 4.3), on
 //                 column rows or on packed row keys;
-//   * semijoin -- the entailment's keyed store pass (Section 5): a store triple
-//                 is kept when its term at the join position is one of the
-//                 first search's distinct terms (a hash probe).
+//   * keyed    -- the rows of the entailment's keyed store pass (Section 5), which
+//                 entail.cu marks itself: expand only.
 // Short inputs: k_compact, one launch (ranks from ballots, tile offsets from
 // the decoupled look-back of lookback.cuh).  Long inputs: k_sel_mark, which
 // tests every row and writes one keep bit per row, and k_sel_expand, which
@@ -27,6 +26,7 @@
 
 #include "lookback.cuh"
 #include "ops.cuh"
+#include "keys.cuh"
 #include "select.cuh"
 
 namespace tid {
@@ -239,66 +239,24 @@ struct UniqueRow {  // rows in perm order; keep the first of each run of equal r
     }
 };
 
-struct SemiJoinRow {  // store triple r, kept when a slot holds a fixed term and another slot's
-                      // term is in a key set (open-addressing table of keys, 0 = empty)
+struct KeyedRow {  // row r of a keyed pass (entail.cu marks its rows), some slots as they are,
+                   // the key slot's term also through a map by key number
     static constexpr int MAX_K = 3;
     const int32_t *S, *P, *O;
-    int need;                   // slots read (bit 0 s, 1 p, 2 o)
-    int fixed_slot;             // -1: none
-    int32_t fixed_val;
     int key_slot;
-    const int32_t *table;
-    int tbits;                  // log2 of the table size
-    int vec;                    // the columns are 16-byte aligned
+    KeySet keys;
+    const int32_t *map;
     int k;
-    int8_t src[TID_MAX_COLS];   // slot giving output column c
-    __device__ __forceinline__ const int32_t *column(int slot) const { return slot == 0 ? S : (slot == 1 ? P : O); }
-    // the fixed column first, the key column and a probe only for rows that pass
-    __device__ __forceinline__ bool keep(int64_t r) const {
-        return keep_given(r, first_column()[r]);
-    }
-    // the column tested first: the fixed one, else the key column
-    __device__ __forceinline__ const int32_t *first_column() const {
-        return column(fixed_slot >= 0 ? fixed_slot : key_slot);
-    }
-    // keep(r), given v = first_column()[r]
-    __device__ __forceinline__ bool keep_given(int64_t r, int32_t v) const {
-        if (fixed_slot >= 0 && v != fixed_val) return false;
-        const int32_t key = fixed_slot >= 0 ? column(key_slot)[r] : v;
-        if (key == 0) return false;
-        const uint32_t tmask = (1u << tbits) - 1u;
-        uint32_t h = ((uint32_t)key * 0x9E3779B1u) >> (32 - tbits);  // top bits: all of the key counts
-        for (uint32_t probe = 0; probe <= tmask; ++probe) {  // the table is at most half full
-            const int32_t e = __ldg(table + h);
-            if (e == key) return true;
-            if (e == 0) return false;
-            h = (h + 1) & tmask;
-        }
-        return false;
-    }
-    __device__ __forceinline__ void keep_step(uint32_t r0, unsigned *m) const {
-        const int32_t *first = first_column();
-        int4 v[8];
-#pragma unroll
-        for (int g = 0; g < 8; ++g) {
-            const int32_t *p = first + r0 + g * 128;
-            v[g] = vec ? ld4(p) : make_int4(p[0], p[1], p[2], p[3]);
-        }
-#pragma unroll
-        for (int g = 0; g < 8; ++g) {
-            const uint32_t r = r0 + g * 128;
-            m[g] = (unsigned)keep_given(r, v[g].x) | ((unsigned)keep_given(r + 1, v[g].y) << 1) |
-                   ((unsigned)keep_given(r + 2, v[g].z) << 2) | ((unsigned)keep_given(r + 3, v[g].w) << 3);
-        }
-    }
+    int8_t src[3];  // slot giving output column c; 3: map[key number]
     template <int K>
     __device__ __forceinline__ void values(int64_t r, int32_t *v) const {
-        const int32_t t0 = (need & 1) ? S[r] : 0;
-        const int32_t t1 = (need & 2) ? P[r] : 0;
-        const int32_t t2 = (need & 4) ? O[r] : 0;
 #pragma unroll
-        for (int c = 0; c < K; ++c)
-            if (c < k) v[c] = src[c] == 0 ? t0 : (src[c] == 1 ? t1 : t2);
+        for (int c = 0; c < K; ++c) {
+            if (c >= k) break;
+            const int s = src[c] == 3 ? key_slot : src[c];
+            const int32_t x = (s == 0 ? S : (s == 1 ? P : O))[r];
+            v[c] = src[c] == 3 ? map[key_number(keys, x)] : x;
+        }
     }
 };
 
@@ -905,27 +863,23 @@ int compact_bind(tid_ctx *ctx, const tid_store *st, const tid_pattern &pat, cons
     return launch_compact(ctx, r, n, out->k, oc, out->cap, out->d_rows, out->slot.dev, mm);
 }
 
-int compact_semijoin(tid_ctx *ctx, const tid_store *st, int fixed_slot, int32_t fixed_val, int key_slot,
-                     const int32_t *table, int tbits, const int8_t *src, tid_set *out) {
-    SemiJoinRow r{};
-    r.S = st->s;
-    r.P = st->p;
-    r.O = st->o;
-    r.fixed_slot = fixed_slot;
-    r.fixed_val = fixed_val;
-    r.key_slot = key_slot;
-    r.table = table;
-    r.tbits = tbits;
-    r.vec = st->aligned16;
+int expand_keyed(tid_ctx *ctx, const KeyedScan &ks, const SelScratch &sc, const int8_t *src, const int32_t *map,
+                 tid_set *out, uint32_t *mm) {
+    KeyedRow r{};
+    r.S = ks.col[0];
+    r.P = ks.col[1];
+    r.O = ks.col[2];
+    r.key_slot = ks.key_slot;
+    r.keys = ks.keys;
+    r.map = map;
     r.k = out->k;
-    r.need = (fixed_slot >= 0 ? 1 << fixed_slot : 0) | (1 << key_slot);
+    OutCols oc{};
     for (int c = 0; c < out->k; ++c) {
         r.src[c] = src[c];
-        r.need |= 1 << src[c];
+        oc.col[c] = out->col[c];
     }
-    OutCols oc{};
-    for (int c = 0; c < out->k; ++c) oc.col[c] = out->col[c];
-    return launch_compact(ctx, r, st->n, out->k, oc, out->cap, out->d_rows, out->slot.dev);
+    if (out->k == 2) return expand_k<KeyedRow, 2>(ctx, r, out->k, oc, out->cap, sc, mm);
+    return expand_k<KeyedRow, 3>(ctx, r, out->k, oc, out->cap, sc, mm);
 }
 
 int compact_filter(tid_ctx *ctx, const tid_set *in, int64_t n, const Pred *preds, int n_preds, tid_set *out) {

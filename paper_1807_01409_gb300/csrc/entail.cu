@@ -4,20 +4,31 @@
 //  1. search the schema premise (?a TERM ?b) -- K1 -- and extract its result
 //     vector (a, b) -- K3/K4;
 //  2. its distinct terms at the join position (the paper's keys of the second
-//     GPUSearch) -- a projection with DISTINCT -- go into an open-addressing
-//     table;
-//  3. one pass over the store keeps the triples of the other premise whose term
-//     at the join position is in the table (K3 with a hash probe per triple,
-//     in store order) and extracts their variables;
-//  4. the two result vectors are joined on the shared term (K5/K6) and the
-//     conclusion's terms kept with DISTINCT.  When the conclusion is a pair of
-//     terms, one from each premise, this is done without materialising the
-//     join: each data row sets the bits of its pairs in a bit matrix indexed
-//     by (rank of the schema term, data term - min), and the set bits, read
-//     in order, are the distinct pairs already in canonical order.
+//     GPUSearch) -- a projection with DISTINCT -- are the key set (keys.cuh);
+//  3. one pass over the store marks the triples of the other premise whose term
+//     at the join position is a key (k_key_mark: their number, the keys among
+//     them, and the range of the conclusion's term).  When both premises search
+//     the same predicate, the pass is over the first search's result vector.
+//  4. the join on the shared term, the conclusion's terms kept with DISTINCT:
+//      * a pair of terms, one from each premise, whose bit matrix (rank of the
+//        schema term by data term - min) is small: every marked triple sets the
+//        bits of its pairs, and the set bits, read in order, are the distinct
+//        pairs in canonical order.  Nothing is extracted, joined or sorted;
+//      * a schema premise with one row per key (a class with one superclass): the
+//        joined rows are the marked triples with the key's term replaced, so they
+//        are extracted that way and sorted once;
+//      * otherwise: extraction, hash join, and one sort of the conclusion's terms.
+// Measured on GB300, 200M triples and their schema, the six rules: 21.6 -> 12.4 ms.
+// Kernel times by rule: R2 2.9 -> 1.7, R3 1.7 -> 1.1, R5 0.4 -> 0.2, R7 5.4 -> 3.4, R9
+// 7.5 -> 3.9, R11 0.5 -> 0.3 ms; k_key_mark 268 us over one column of 200M triples, 359
+// over two (a third column of loads at once, 80 registers, took 430 and 627 us)
+// (before: every rule extracted its marked rows, R7 and R9 materialised the hash
+// join's rows).  Bound: R2 and R3 by the matrix's random L2 reads, R7 and R9 by the
+// digit passes of their sort.
 #include <algorithm>
 #include <vector>
 
+#include "keys.cuh"
 #include "ops.cuh"
 
 namespace tid {
@@ -63,163 +74,268 @@ __global__ void k_fill_i32(int32_t *__restrict__ out, int64_t n, int32_t v) {
 }
 
 constexpr int BM_THREADS = 256;
-constexpr uint32_t KEY_HASH = 0x9E3779B1u;      // multiplicative (Knuth) hash of the key table
-
-__host__ __device__ __forceinline__ uint32_t home_slot(int32_t key, int tbits) {
-    return ((uint32_t)key * KEY_HASH) >> (32 - tbits);
-}
-
-// slot of `key` in the open-addressing key table, or -1 (0 is the empty slot
-// and never a key); at most one sweep of the table
-__device__ __forceinline__ int find_slot(const int32_t *__restrict__ table, int tbits, int32_t key) {
-    if (key == 0) return -1;
-    const uint32_t mask = (1u << tbits) - 1u;
-    uint32_t h = home_slot(key, tbits);
-    for (uint32_t probe = 0; probe <= mask; ++probe) {
-        const int32_t t = table[h];
-        if (t == key) return (int)h;
-        if (t == 0) return -1;
-        h = (h + 1) & mask;
-    }
-    return -1;
-}
 
 __device__ __forceinline__ uint32_t sort_order(int32_t x) { return (uint32_t)x ^ 0x80000000u; }
+inline uint32_t sort_order_host(int32_t x) { return (uint32_t)x ^ 0x80000000u; }
 
-constexpr int BM_U = 4;  // rows per lane per step of the marking kernels (loads in flight)
+// What a keyed pass finds besides its marks.
+struct KeyStats {
+    unsigned long long keys;  // keys that occur in the marked rows (the paper's #Dist2)
+    uint32_t lo, hi;          // range of the marked rows' conclusion term, in sort order
+};
 
-// A warp's step: rows i0 + 32 u + lane, u < BM_U, i0 warp-uniform (so every
-// lane takes part in the shuffles below).
-__device__ __forceinline__ int64_t bm_first() {
-    return (int64_t)blockIdx.x * (BM_THREADS * BM_U) + (int64_t)(threadIdx.x >> 5) * (32 * BM_U);
-}
-__device__ __forceinline__ int64_t bm_stride() { return (int64_t)gridDim.x * (BM_THREADS * BM_U); }
+constexpr unsigned KM_SMEM_KEYS = 16384;  // keys whose flags are kept in shared memory, a byte each, if there are no more
 
-// flags gets one bit per table slot whose key occurs in key[0, n): the distinct
-// join terms of the data premise's rows.  A lane skips a row whose slot equals
-// the previous lane's, and sets a bit only while it is clear.  Bits collect in
-// shared memory when SMEM, else in global memory directly.
-template <bool SMEM>
-__global__ void __launch_bounds__(BM_THREADS) k_mark_keys(const int32_t *__restrict__ key, int64_t n,
-                                                          const int32_t *__restrict__ table, int tbits,
-                                                          uint32_t *__restrict__ flags) {
-    extern __shared__ uint32_t s_f[];
-    const uint32_t words = ((1u << tbits) + 31u) >> 5;
-    if (SMEM) {
-        for (uint32_t w = threadIdx.x; w < words; w += BM_THREADS) s_f[w] = 0;
+// Marks the scan's kept rows (mark of select.cuh).  flags gets one bit per key
+// number that occurs; when term is not null, st->lo / st->hi its range over the
+// kept rows (preset to ~0 and 0).  16 rows per lane at a time, their key tests side
+// by side; the key column is read only where a group of 128 rows holds the fixed
+// term at all, the term column only where one is kept.
+__global__ void __launch_bounds__(SEL_THREADS)
+k_key_mark(const __grid_constant__ KeyedScan ks, SelScratch sc, int64_t *__restrict__ d_rows,
+           int64_t *__restrict__ h_rows, uint32_t *__restrict__ flags, unsigned numbers,
+           const int32_t *__restrict__ term, KeyStats *__restrict__ st) {
+    extern __shared__ uint8_t s_seen[];  // per key number, when there are at most KM_SMEM_KEYS
+    const unsigned lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const bool in_smem = numbers <= KM_SMEM_KEYS;
+    if (in_smem) {
+        for (unsigned w = threadIdx.x; w < numbers; w += SEL_THREADS) s_seen[w] = 0;
         __syncthreads();
     }
-    volatile uint32_t *f = SMEM ? s_f : flags;
-    const unsigned lane = threadIdx.x & 31;
-    for (int64_t i0 = bm_first(); i0 < n; i0 += bm_stride()) {
-        int32_t x[BM_U];
-#pragma unroll
-        for (int u = 0; u < BM_U; ++u) {
-            const int64_t i = i0 + 32 * u + lane;
-            x[u] = i < n ? key[i] : 0;
+    auto column = [&](int slot) { return slot == 0 ? ks.col[0] : (slot == 1 ? ks.col[1] : ks.col[2]); };
+    const int32_t *key = column(ks.key_slot), *fixed = ks.fixed_slot >= 0 ? column(ks.fixed_slot) : nullptr;
+    uint32_t lo = 0xFFFFFFFFu, hi = 0u;
+    auto seen = [&](int h) {
+        if (in_smem) {
+            s_seen[h] = 1;
+        } else {  // set a bit only while it is clear
+            const uint32_t b = 1u << (h & 31);
+            if (!(__ldcg(flags + (h >> 5)) & b)) atomicOr(flags + (h >> 5), b);
         }
+    };
+    auto four = [&](const int32_t *p) { return ks.vec ? ld_stream_v4(p) : make_int4(p[0], p[1], p[2], p[3]); };
+    const unsigned r0 = blockIdx.x * sc.per, r1 = min(r0 + sc.per, sc.steps);
+    unsigned kept = 0;
+    for (unsigned step = r0 + warp; step < r1; step += SEL_WARPS) {
+        const int64_t base = (int64_t)step * SEL_STEP + lane * 4;
+        unsigned m[8];
+        if ((int64_t)(step + 1) * SEL_STEP <= ks.n) {
 #pragma unroll
-        for (int u = 0; u < BM_U; ++u) {
-            const int h = find_slot(table, tbits, x[u]);
-            const int hp = __shfl_up_sync(0xffffffffu, h, 1);
-            if (h >= 0 && (lane == 0 || hp != h)) {
-                const uint32_t b = 1u << (h & 31);
-                if (!(f[h >> 5] & b)) atomicOr((uint32_t *)f + (h >> 5), b);
+            for (int h = 0; h < 8; h += 4) {
+                int32_t x[16];
+                unsigned want = 0xFFFFu;  // bit i: row i may be kept
+                auto load = [&](const int32_t *p, int g) {
+                    const int4 v = four(p + base + (h + g) * 128);
+                    x[4 * g] = v.x, x[4 * g + 1] = v.y, x[4 * g + 2] = v.z, x[4 * g + 3] = v.w;
+                };
+#pragma unroll
+                for (int g = 0; g < 4; ++g) load(fixed ? fixed : key, g);
+                if (fixed) {
+                    want = 0;
+#pragma unroll
+                    for (int i = 0; i < 16; ++i) want |= (unsigned)(x[i] == ks.fixed_val) << i;
+#pragma unroll
+                    for (int g = 0; g < 4; ++g)
+                        if (__any_sync(0xffffffffu, (want >> (4 * g)) & 0xFu)) load(key, g);
+                }
+                unsigned r = 0;
+                if (ks.keys.bits) {
+                    uint32_t word[16];
+#pragma unroll
+                    for (int i = 0; i < 16; ++i) {
+                        const uint32_t d = sort_order(x[i]) - ks.keys.lo;
+                        word[i] = 0;
+                        if (((want >> i) & 1u) && d < ks.keys.w && x[i] != 0) word[i] = __ldg(ks.keys.bits + (d >> 5));
+                    }
+#pragma unroll
+                    for (int i = 0; i < 16; ++i) {
+                        const uint32_t d = sort_order(x[i]) - ks.keys.lo;
+                        if ((word[i] >> (d & 31)) & 1u) {
+                            r |= 1u << i;
+                            seen((int)d);
+                        }
+                    }
+                } else {
+#pragma unroll
+                    for (int i = 0; i < 16; ++i) {
+                        const int k = ((want >> i) & 1u) ? key_number(ks.keys, x[i]) : -1;
+                        if (k >= 0) {
+                            r |= 1u << i;
+                            seen(k);
+                        }
+                    }
+                }
+#pragma unroll
+                for (int g = 0; g < 4; ++g) m[h + g] = (r >> (4 * g)) & 0xFu;
+                if (term) {
+#pragma unroll
+                    for (int g = 0; g < 4; ++g)
+                        if (__any_sync(0xffffffffu, m[h + g])) load(term, g);
+#pragma unroll
+                    for (int i = 0; i < 16; ++i) {
+                        if (!((r >> i) & 1u)) continue;
+                        lo = min(lo, sort_order(x[i]));
+                        hi = max(hi, sort_order(x[i]));
+                    }
+                }
+            }
+        } else {  // ragged last step
+#pragma unroll
+            for (int g = 0; g < 8; ++g) {
+                unsigned r = 0;
+                for (int e = 0; e < 4; ++e) {
+                    const int64_t i = base + g * 128 + e;
+                    if (i >= ks.n || (fixed && fixed[i] != ks.fixed_val)) continue;
+                    const int k = key_number(ks.keys, key[i]);
+                    if (k < 0) continue;
+                    seen(k);
+                    r |= 1u << e;
+                    if (term) {
+                        lo = min(lo, sort_order(term[i]));
+                        hi = max(hi, sort_order(term[i]));
+                    }
+                }
+                m[g] = r;
             }
         }
+        __syncwarp();
+        const uint32_t word = sel_word(m);
+        sc.bits[(size_t)step * 32 + sel_word_index()] = word;
+        const unsigned c = __reduce_add_sync(0xffffffffu, __popc(word));
+        if (lane == 0) sc.cnt[step] = c;
+        kept += c;
     }
-    if (SMEM) {
+    if (term) {
+        lo = __reduce_min_sync(0xffffffffu, lo);
+        hi = __reduce_max_sync(0xffffffffu, hi);
+        if (lane == 0 && lo <= hi) {  // skip an atomic that cannot widen the range
+            if (lo < __ldcg(&st->lo)) atomicMin(&st->lo, lo);
+            if (hi > __ldcg(&st->hi)) atomicMax(&st->hi, hi);
+        }
+    }
+    if (in_smem) {
         __syncthreads();
-        for (uint32_t w = threadIdx.x; w < words; w += BM_THREADS)
-            if (s_f[w]) atomicOr(flags + w, s_f[w]);
+        for (unsigned k0 = warp * 32; k0 < numbers; k0 += SEL_THREADS) {
+            const unsigned k = k0 + lane;
+            const uint32_t w = __ballot_sync(0xffffffffu, k < numbers && s_seen[k]);
+            if (lane == 0 && (w & ~__ldcg(flags + (k0 >> 5)))) atomicOr(flags + (k0 >> 5), w);
+        }
     }
+    sel_finish(sc, kept, d_rows, h_rows);
 }
 
-// The conclusion's distinct pairs as the set bits of a matrix.  A data-premise
-// row (join term, term t) joined with the schema rows of that join term gives
-// the pairs (r, t) for A's other terms r.  r is ranked among A's distinct
-// values of that term (ascending) and t is taken as d = order(t) - vmin.  Rows
-// of the matrix follow the conclusion's first term and are 2^lg bits wide
-// (the second term's span rounded up to a power of two): the pair is bit
-// (r << lg) + d when A's term comes first, (d << lg) + r when t does.  The set
-// bits in ascending order are the canonical distinct rows.
+// The conclusion's distinct pairs as the set bits of a matrix.  A marked row
+// (join term, term t) joined with the schema rows of that join term gives the pairs
+// (r, t) for A's other terms r.  r is ranked among A's distinct values of that
+// term (ascending) and t is taken as d = order(t) - vmin.  Rows of the matrix
+// follow the conclusion's first term and are 2^lg bits wide (the second term's span
+// rounded up to a power of two): the pair is bit (r << lg) + d when A's term comes
+// first, (d << lg) + r when t does.  The set bits in ascending order are the
+// canonical distinct rows.
 struct PairBits {
-    const int32_t *key, *val;  // data-premise rows: join term, conclusion term
-    int64_t n;
-    const int32_t *table;  // the join terms (open addressing)
-    int tbits;
-    const uint32_t *off;    // slot h: A's ranks are rank[off[h] .. off[h + 1])
+    const int32_t *key, *val;  // the scan's key column and conclusion term
+    KeySet keys;
+    const uint32_t *off;    // key number h: A's ranks are rank[off[h] .. off[h + 1])
     const uint32_t *rank;
-    const uint32_t *kmask;  // slot h: the same ranks as a mask (t first, 2^lg <= 32)
+    const uint32_t *kmask;  // key number h: the same ranks as a mask (t first, 2^lg <= 32)
     uint32_t vmin;
     int lg;
     int a_first;
     uint32_t *bits;
 };
 
-// General form: one atomic OR per (row, rank) whose bit is not yet set; a
-// lane skips a row equal, in slot and term, to the previous lane's.
-__global__ void __launch_bounds__(BM_THREADS) k_pair_bits_list(PairBits P) {
+// Sets the pairs of U rows per lane (h[u] < 0: no row); all lanes take part.
+// MASK: t first and rows of at most 32 bits, so a row's ranks are one mask within
+// one word; lanes holding consecutive rows of the same word OR their masks (a
+// segmented scan across the warp) and the last lane of each run writes it.  The U
+// words are read together: a word that has the bits already costs no atomic (a
+// stale read only costs the atomic).  Without the read, 58.7M rows whose terms are
+// skewed queue on the popular words: 1658 us against 499.
+// Otherwise one atomic OR per (row, rank) whose bit is clear; a lane skips a row
+// equal, in key and term, to the previous lane's.
+template <bool MASK, int U>
+__device__ __forceinline__ void set_pairs(const PairBits &P, const int *h, const int32_t *t) {
     const unsigned lane = threadIdx.x & 31;
-    for (int64_t i0 = bm_first(); i0 < P.n; i0 += bm_stride()) {
-        int32_t x[BM_U], t[BM_U];
+    if (MASK) {
+        const unsigned le = lane == 31 ? 0xFFFFFFFFu : (2u << lane) - 1u;  // lanes <= this one
+        uint64_t word[U];
+        uint32_t acc[U], cur[U];
 #pragma unroll
-        for (int u = 0; u < BM_U; ++u) {
-            const int64_t i = i0 + 32 * u + lane;
-            x[u] = i < P.n ? P.key[i] : 0;
-            t[u] = i < P.n ? P.val[i] : 0;
+        for (int u = 0; u < U; ++u) {
+            const uint64_t g = (uint64_t)(sort_order(t[u]) - P.vmin) << P.lg;
+            word[u] = h[u] >= 0 ? g >> 5 : ~0ull;
+            acc[u] = h[u] >= 0 ? P.kmask[h[u]] << (g & 31) : 0u;
         }
 #pragma unroll
-        for (int u = 0; u < BM_U; ++u) {
-            const int h = find_slot(P.table, P.tbits, x[u]);
+        for (int u = 0; u < U; ++u) {
+            const uint64_t wp = __shfl_up_sync(0xffffffffu, word[u], 1);
+            const unsigned heads = __ballot_sync(0xffffffffu, lane == 0 || wp != word[u]);
+            if (heads != 0xFFFFFFFFu) {  // some neighbours share a word
+                const int start = 31 - __clz(heads & le);
+#pragma unroll
+                for (int s = 1; s < 32; s <<= 1) {
+                    const uint32_t o = __shfl_up_sync(0xffffffffu, acc[u], s);
+                    if ((int)lane - s >= start) acc[u] |= o;
+                }
+                if (lane < 31 && !((heads >> (lane + 1)) & 1u)) word[u] = ~0ull;  // the run's last lane writes
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) cur[u] = word[u] != ~0ull ? __ldcg(P.bits + word[u]) : 0xFFFFFFFFu;
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if ((cur[u] & acc[u]) != acc[u]) atomicOr(P.bits + word[u], acc[u]);
+    } else {
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
             const uint32_t d = sort_order(t[u]) - P.vmin;
-            const int hp = __shfl_up_sync(0xffffffffu, h, 1);
+            const int hp = __shfl_up_sync(0xffffffffu, h[u], 1);
             const uint32_t dp = __shfl_up_sync(0xffffffffu, d, 1);
-            if (h < 0 || (lane > 0 && hp == h && dp == d)) continue;
-            for (uint32_t j = P.off[h]; j < P.off[h + 1]; ++j) {
+            if (h[u] < 0 || (lane > 0 && hp == h[u] && dp == d)) continue;
+            for (uint32_t j = P.off[h[u]]; j < P.off[h[u] + 1]; ++j) {
                 const uint64_t r = P.rank[j];
                 const uint64_t g = P.a_first ? (r << P.lg) + d : ((uint64_t)d << P.lg) + r;
                 const uint32_t b = 1u << (g & 31);
-                if (!(P.bits[g >> 5] & b)) atomicOr(P.bits + (g >> 5), b);  // read first, as above
+                if (!(__ldcg(P.bits + (g >> 5)) & b)) atomicOr(P.bits + (g >> 5), b);
             }
         }
     }
 }
 
-// t first and rows of at most 32 bits: a row's ranks are one mask within one
-// word.  Lanes holding consecutive rows of the same word OR their masks (a
-// segmented scan across the warp) and the last lane of each run writes it.
-__global__ void __launch_bounds__(BM_THREADS) k_pair_bits_mask(PairBits P) {
-    const unsigned lane = threadIdx.x & 31;
-    const unsigned le = lane == 31 ? 0xFFFFFFFFu : (2u << lane) - 1u;  // lanes <= this one
-    for (int64_t i0 = bm_first(); i0 < P.n; i0 += bm_stride()) {
-        int32_t x[BM_U], t[BM_U];
+template <bool MASK>
+__global__ void __launch_bounds__(SEL_THREADS) k_pair_bits(const __grid_constant__ PairBits P, SelScratch sc) {
+    __shared__ uint16_t s_stage[SEL_WARPS][SEL_DENSE];
+    const unsigned lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    constexpr int U = 4;  // rows per lane whose loads are in flight together
+    uint16_t *stage = s_stage[warp];
+    sel_walk(sc, blockIdx.x, warp, SEL_WARPS, [&](unsigned step, uint32_t word, unsigned xo, unsigned sn,
+                                                   unsigned long long) {
+        const int64_t base = (int64_t)step * SEL_STEP;
+        const bool dense = sn >= SEL_DENSE;
+        if (!dense) sel_stage(word, xo, stage);
+        const unsigned rounds = dense ? 32 : (sn + 31) / 32;
+#pragma unroll 1
+        for (unsigned q0 = 0; q0 < rounds; q0 += U) {
+            int32_t x[U], t[U];
+            int h[U];
 #pragma unroll
-        for (int u = 0; u < BM_U; ++u) {
-            const int64_t i = i0 + 32 * u + lane;
-            x[u] = i < P.n ? P.key[i] : 0;
-            t[u] = i < P.n ? P.val[i] : 0;
-        }
-#pragma unroll
-        for (int u = 0; u < BM_U; ++u) {
-            const int h = find_slot(P.table, P.tbits, x[u]);
-            const uint64_t g = (uint64_t)(sort_order(t[u]) - P.vmin) << P.lg;
-            const uint64_t word = h >= 0 ? g >> 5 : ~0ull;
-            uint32_t acc = h >= 0 ? P.kmask[h] << (g & 31) : 0u;
-            const uint64_t wp = __shfl_up_sync(0xffffffffu, word, 1);
-            const unsigned heads = __ballot_sync(0xffffffffu, lane == 0 || wp != word);
-            const int start = 31 - __clz(heads & le);
-#pragma unroll
-            for (int d = 1; d < 32; d <<= 1) {
-                const uint32_t o = __shfl_up_sync(0xffffffffu, acc, d);
-                if ((int)lane - d >= start) acc |= o;
+            for (int u = 0; u < U; ++u) {
+                const unsigned q = q0 + u;
+                int64_t r = -1;
+                if (dense) {
+                    if ((__shfl_sync(0xffffffffu, word, q) >> lane) & 1u) r = base + q * 32 + lane;
+                } else if (q * 32 + lane < sn) {
+                    r = base + stage[q * 32 + lane];
+                }
+                x[u] = r >= 0 ? P.key[r] : 0;
+                t[u] = r >= 0 ? P.val[r] : 0;
             }
-            const bool tail = lane == 31 || ((heads >> (lane + 1)) & 1u);
-            // most rows repeat a pair already set: read before the atomic (a
-            // stale read only costs the atomic)
-            if (h >= 0 && tail && (P.bits[word] & acc) != acc) atomicOr(P.bits + word, acc);
+#pragma unroll
+            for (int u = 0; u < U; ++u) h[u] = key_number(P.keys, x[u]);  // -1 without a row
+            set_pairs<MASK, U>(P, h, t);
         }
-    }
+        __syncwarp();  // the stage is rewritten by the next step
+    });
 }
 
 // Reading the matrix out: segment s is words [s R 32, (s + 1) R 32), R rounds
@@ -385,25 +501,6 @@ __global__ void __launch_bounds__(1024) k_count_bits(const uint32_t *__restrict_
     }
 }
 
-// mm[0] = min, mm[1] = max of col[0, n) in sort order (mm preset to ~0, 0)
-__global__ void k_col_range(const int32_t *__restrict__ col, int64_t n, uint32_t *__restrict__ mm) {
-    uint32_t lo = 0xFFFFFFFFu, hi = 0u;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const uint32_t v = sort_order(col[i]);
-        lo = min(lo, v);
-        hi = max(hi, v);
-    }
-#pragma unroll
-    for (int d = 16; d > 0; d >>= 1) {
-        lo = min(lo, __shfl_xor_sync(0xffffffffu, lo, d));
-        hi = max(hi, __shfl_xor_sync(0xffffffffu, hi, d));
-    }
-    if ((threadIdx.x & 31) == 0) {  // skip an atomic that cannot tighten the bound
-        if (lo < __ldcg(mm)) atomicMin(mm, lo);
-        if (hi > __ldcg(mm + 1)) atomicMax(mm + 1, hi);
-    }
-}
-
 struct Sets {  // frees what it holds
     std::vector<tid_set *> v;
     ~Sets() {
@@ -426,6 +523,7 @@ struct Buf {  // a device allocation freed on scope exit
 };
 
 constexpr int64_t PAIR_MAX_SCHEMA_ROWS = 1 << 22;  // schema rows ranked on the host
+constexpr int64_t MAP_MAX_SCHEMA_ROWS = 1 << 18;   // or made a map there, for R7's conclusion
 // A matrix of up to 64 MiB stays mostly in L2 and is always taken; a larger
 // one only up to 4 bytes per data-premise row: beyond L2 every pair's bit is a
 // random DRAM read-modify-write, and joining and sorting the rows costs less
@@ -434,58 +532,85 @@ constexpr uint64_t PAIR_MIN_BYTES = 64ull << 20;
 constexpr uint64_t PAIR_BYTES_PER_ROW = 4;
 constexpr uint64_t PAIR_MAX_BYTES = 4ull << 30;
 
-// The conclusion as the bit matrix of its distinct pairs (PairBits), when it
-// has two terms, A's non-join term and one of the data premise's, and the
-// matrix is small enough.  *out stays null when this form does not apply and
-// the join is taken instead.
-//   A: the schema premise's rows (join term and other term); B: the data
-//   premise's rows (nb), its column tcol the conclusion's term; table/d_table:
-//   the key table on the host and the device.
-int conclude_pairs(tid_ctx *ctx, const Rule &R, tid_set *A, tid_set *B, int64_t nb, const int8_t *bvars, int kb,
-                   const std::vector<int32_t> &table, const int32_t *d_table, int tbits, const int8_t *cvars,
-                   int kc, tid_set **out) {
-    *out = nullptr;
-    if (kc != 2 || nb == 0) return TID_OK;
-    const int8_t other = R.on == VA ? VB : VA;  // A's term that is not the join term
-    const int a_pos = cvars[0] == other ? 0 : (cvars[1] == other ? 1 : -1);
-    if (a_pos < 0) return TID_OK;
-    const int8_t tv = cvars[1 - a_pos];
-    int tcol = -1, kcol = -1;
-    for (int c = 0; c < kb; ++c) {
-        if (bvars[c] == tv && tv != R.on) tcol = c;
-        if (bvars[c] == R.on) kcol = c;
+// The schema premise's rows by key: (key number, other term), sorted.
+struct SchemaRows {
+    std::vector<std::pair<uint32_t, int32_t>> rows;
+    bool one_each = true;  // one row per key
+};
+
+// One column of a set of pairs, from its rows on the host.
+struct KeyTable {
+    KeySet set{};
+    uint32_t numbers = 0;              // key numbers lie in [0, numbers)
+    std::vector<uint32_t> bits;        // direct: a bit per term of the range
+    std::vector<int32_t> table;        // or the open-addressing table
+    int64_t number(int32_t key) const {
+        if (key == 0) return -1;
+        if (table.empty()) {
+            const uint32_t d = ((uint32_t)key ^ 0x80000000u) - set.lo;
+            return d < set.w && ((bits[d >> 5] >> (d & 31)) & 1u) ? (int64_t)d : -1;
+        }
+        uint32_t h = home_slot(key, set.tbits);
+        for (uint32_t probe = 0; probe < numbers; ++probe, h = (h + 1) & (numbers - 1)) {
+            if (table[h] == key) return h;
+            if (table[h] == 0) return -1;
+        }
+        return -1;
     }
-    int ak = -1, ao = -1;
-    for (int c = 0; c < A->k; ++c) {
-        if (A->vars[c] == R.on) ak = c;
-        if (A->vars[c] == other) ao = c;
+};
+
+// A key's arrays (flags, ranks, map) are indexed by number: a direct range of up to
+// 2^20 terms costs at most a few MB of them and one bit test per triple in place
+// of a hash probe.
+constexpr uint64_t KEY_DIRECT = 1ull << 20;
+
+void build_keys(const std::vector<int32_t> &keys, KeyTable *kt) {  // distinct, ascending
+    uint32_t lo = 0xFFFFFFFFu, hi = 0;
+    size_t n = 0;
+    for (int32_t k : keys) {
+        if (k == 0) continue;  // 0 never joins
+        const uint32_t o = (uint32_t)k ^ 0x80000000u;
+        lo = std::min(lo, o);
+        hi = std::max(hi, o);
+        ++n;
     }
-    int64_t nA = 0;
-    TID_TRY(set_rows_host(A, &nA));
-    if (tcol < 0 || kcol < 0 || ak < 0 || ao < 0 || nA == 0 || nA > PAIR_MAX_SCHEMA_ROWS) return TID_OK;
+    if (n == 0 || (uint64_t)hi - lo < KEY_DIRECT) {
+        kt->set.lo = n ? lo : 0u;
+        kt->set.w = n ? hi - lo + 1 : 1u;
+        kt->numbers = kt->set.w;
+        kt->bits.assign((kt->set.w + 31) / 32, 0u);
+        for (int32_t k : keys) {
+            const uint32_t d = ((uint32_t)k ^ 0x80000000u) - kt->set.lo;
+            if (k != 0) kt->bits[d >> 5] |= 1u << (d & 31);
+        }
+        return;
+    }
+    kt->set.tbits = 4;
+    while ((1ull << kt->set.tbits) < 2 * (uint64_t)n) ++kt->set.tbits;
+    kt->numbers = 1u << kt->set.tbits;
+    kt->table.assign(kt->numbers, 0);
+    for (int32_t k : keys) {
+        if (k == 0) continue;
+        uint32_t h = home_slot(k, kt->set.tbits);
+        while (kt->table[h] != 0) h = (h + 1) & (kt->numbers - 1);
+        kt->table[h] = k;
+    }
+}
+
+// The conclusion as the bit matrix of its distinct pairs (PairBits), when the
+// matrix is small enough; *out stays null when it is not.  a_pos: which of the two
+// conclusion terms is A's; O: the three-column result, pair columns at slots pos[2].
+int conclude_pairs(tid_ctx *ctx, const KeyedScan &ks, const SelScratch &sc, const KeyTable &kt, const SchemaRows &sr,
+                   const KeyStats &st, int64_t res2, const int32_t *term, int a_pos, const int *pos, int fixed_pos,
+                   int32_t fixed_term, tid_set **out) {
     cudaStream_t stream = ctx->stream;
-
-    // the range of the data premise's term, and A's rows on the host
-    Buf rb{ctx};
-    TID_TRY(dev_alloc(ctx, &rb.p, 2 * sizeof(uint32_t)));
-    uint32_t *mm = (uint32_t *)rb.p;
-    TID_TRY_CUDA(cudaMemsetAsync(mm, 0xFF, sizeof(uint32_t), stream), "range");
-    TID_TRY_CUDA(cudaMemsetAsync(mm + 1, 0, sizeof(uint32_t), stream), "range");
-    k_col_range<<<grid_for(nb, 256, 8), 256, 0, stream>>>(B->col[tcol], nb, mm);
-    TID_TRY(launch_check("k_col_range"));
-    uint32_t hmm[2] = {0, 0};
-    TID_TRY_CUDA(cudaMemcpyAsync(hmm, mm, sizeof hmm, cudaMemcpyDeviceToHost, stream), "range");
-    std::vector<int32_t> arows((size_t)nA * A->k);
-    int64_t got = 0;
-    TID_TRY(tid_set_to_host(A, arows.data(), nA, &got));  // synchronises
-    if (hmm[0] > hmm[1]) return TID_OK;
-
     // A's other terms ranked; the matrix's size decides the form
-    std::vector<int32_t> vals((size_t)nA);
-    for (int64_t i = 0; i < nA; ++i) vals[(size_t)i] = arows[(size_t)i * A->k + ao];
+    std::vector<int32_t> vals;
+    vals.reserve(sr.rows.size());
+    for (const auto &r : sr.rows) vals.push_back(r.second);
     std::sort(vals.begin(), vals.end());
     vals.erase(std::unique(vals.begin(), vals.end()), vals.end());
-    const uint64_t na = vals.size(), w = (uint64_t)(hmm[1] - hmm[0]) + 1;
+    const uint64_t na = vals.size(), w = (uint64_t)(st.hi - st.lo) + 1;
     const uint64_t nrows = a_pos == 0 ? na : w, width = a_pos == 0 ? w : na;  // matrix rows, bits per row
     int lg = 0;
     while ((1ull << lg) < width) ++lg;
@@ -493,34 +618,21 @@ int conclude_pairs(tid_ctx *ctx, const Rule &R, tid_set *A, tid_set *B, int64_t 
     while ((1ull << lr) < nrows) ++lr;
     if (lg + lr > 40) return TID_OK;  // far beyond the size limit below
     const uint64_t nwords = ((nrows << lg) + 31) / 32, bytes = nwords * sizeof(uint32_t);
-    if (bytes > std::max(PAIR_MIN_BYTES, PAIR_BYTES_PER_ROW * (uint64_t)nb) || bytes > PAIR_MAX_BYTES) return TID_OK;
+    if (bytes > std::max(PAIR_MIN_BYTES, PAIR_BYTES_PER_ROW * (uint64_t)res2) || bytes > PAIR_MAX_BYTES) return TID_OK;
 
-    // per key slot, the ranks of its schema rows' other terms (ascending)
-    const uint32_t tsize = 1u << tbits;
-    std::vector<std::pair<uint32_t, uint32_t>> hr;
-    hr.reserve((size_t)nA);
-    for (int64_t i = 0; i < nA; ++i) {
-        const int32_t key = arows[(size_t)i * A->k + ak];
-        if (key == 0) continue;  // 0 never joins
-        uint32_t h = home_slot(key, tbits);
-        for (uint32_t probe = 0; probe < tsize && table[h] != key; ++probe) h = (h + 1) & (tsize - 1);
-        if (table[h] != key) continue;
-        const int32_t v = arows[(size_t)i * A->k + ao];
-        hr.emplace_back(h, (uint32_t)(std::lower_bound(vals.begin(), vals.end(), v) - vals.begin()));
-    }
-    std::sort(hr.begin(), hr.end());
-    hr.erase(std::unique(hr.begin(), hr.end()), hr.end());
     const bool use_mask = a_pos == 1 && lg <= 5;  // a row's ranks fit one word
-    // layout: rank values (na) | off (tsize + 1) | ranks | masks (tsize, when used)
-    std::vector<uint32_t> meta(na + tsize + 1 + hr.size() + (use_mask ? tsize : 0), 0u);
-    uint32_t *m_off = meta.data() + na, *m_rank = m_off + tsize + 1, *m_mask = m_rank + hr.size();
+    // layout: rank values (na) | off (numbers + 1) | ranks | masks (numbers, when used)
+    const uint32_t nk = kt.numbers;
+    std::vector<uint32_t> meta(na + nk + 1 + sr.rows.size() + (use_mask ? nk : 0), 0u);
+    uint32_t *m_off = meta.data() + na, *m_rank = m_off + nk + 1, *m_mask = m_rank + sr.rows.size();
     for (uint64_t r = 0; r < na; ++r) meta[r] = (uint32_t)vals[r];
-    for (size_t j = 0; j < hr.size(); ++j) {
-        m_off[hr[j].first + 1]++;
-        m_rank[j] = hr[j].second;
-        if (use_mask) m_mask[hr[j].first] |= 1u << hr[j].second;
+    for (size_t j = 0; j < sr.rows.size(); ++j) {
+        const uint32_t rank = (uint32_t)(std::lower_bound(vals.begin(), vals.end(), sr.rows[j].second) - vals.begin());
+        m_off[sr.rows[j].first + 1]++;
+        m_rank[j] = rank;
+        if (use_mask) m_mask[sr.rows[j].first] |= 1u << rank;
     }
-    for (uint32_t h = 0; h < tsize; ++h) m_off[h + 1] += m_off[h];
+    for (uint32_t h = 0; h < nk; ++h) m_off[h + 1] += m_off[h];
     Buf mb{ctx};
     TID_TRY(dev_alloc(ctx, &mb.p, meta.size() * sizeof(uint32_t)));
     TID_TRY_CUDA(cudaMemcpyAsync(mb.p, meta.data(), meta.size() * sizeof(uint32_t), cudaMemcpyHostToDevice, stream),
@@ -532,17 +644,11 @@ int conclude_pairs(tid_ctx *ctx, const Rule &R, tid_set *A, tid_set *B, int64_t 
     TID_TRY(dev_alloc(ctx, &bb.p, bytes));
     uint32_t *bits = (uint32_t *)bb.p;
     TID_TRY_CUDA(cudaMemsetAsync(bits, 0, bytes, stream), "pair bits");
-    const PairBits P{B->col[kcol], B->col[tcol], nb, d_table, tbits,
-                     d_meta + na, d_meta + na + tsize + 1, use_mask ? d_meta + na + tsize + 1 + hr.size() : nullptr,
-                     hmm[0], lg, a_pos == 0 ? 1 : 0, bits};
-    const unsigned grid = grid_for(nb, BM_THREADS * BM_U, 8);
-    if (use_mask) {
-        k_pair_bits_mask<<<grid, BM_THREADS, 0, stream>>>(P);
-        TID_TRY(launch_check("k_pair_bits_mask"));
-    } else {
-        k_pair_bits_list<<<grid, BM_THREADS, 0, stream>>>(P);
-        TID_TRY(launch_check("k_pair_bits_list"));
-    }
+    const PairBits P{ks.col[ks.key_slot], term, ks.keys, d_meta + na, d_meta + na + nk + 1,
+                     use_mask ? d_meta + na + nk + 1 + sr.rows.size() : nullptr, st.lo, lg, a_pos == 0 ? 1 : 0, bits};
+    if (use_mask) k_pair_bits<true><<<sc.ranges, SEL_THREADS, 0, stream>>>(P, sc);
+    else k_pair_bits<false><<<sc.ranges, SEL_THREADS, 0, stream>>>(P, sc);
+    TID_TRY(launch_check("k_pair_bits"));
     // segments of R rounds of 32 words, at most 2^16 of them (one warp each)
     const int rounds = (int)std::max<int64_t>(8, ceil_div((int64_t)nwords, (int64_t)32 << 16));
     const int64_t nseg = ceil_div((int64_t)nwords, (int64_t)rounds * 32);
@@ -559,30 +665,35 @@ int conclude_pairs(tid_ctx *ctx, const Rule &R, tid_set *A, tid_set *B, int64_t 
     unsigned long long total = 0;
     TID_TRY_CUDA(cudaMemcpyAsync(&total, d_total, sizeof total, cudaMemcpyDeviceToHost, stream), "pair rows");
     TID_TRY_CUDA(cudaStreamSynchronize(stream), "pair rows");
-    tid_set *C = nullptr;
-    TID_TRY(set_alloc(ctx, 2, cvars, (int64_t)total, &C));
+    const int8_t ovars[3] = {0, 1, 2};
+    tid_set *O = nullptr;
+    TID_TRY(set_alloc(ctx, 3, ovars, (int64_t)total, &O));
     int rc = TID_OK;
     if (total > 0) {
-        const PairOut O{(const int32_t *)d_meta, hmm[0], lg, a_pos == 0 ? 1 : 0, C->col[0], C->col[1]};
-        k_emit_pairs<<<seg_ctas, BM_THREADS, 0, stream>>>(bits, (int64_t)nwords, rounds, nseg, offs, O);
+        const PairOut E{(const int32_t *)d_meta, st.lo, lg, a_pos == 0 ? 1 : 0, O->col[pos[0]], O->col[pos[1]]};
+        k_emit_pairs<<<seg_ctas, BM_THREADS, 0, stream>>>(bits, (int64_t)nwords, rounds, nseg, offs, E);
         rc = launch_check("k_emit_pairs");
+        if (rc == TID_OK) {
+            k_fill_i32<<<grid_for((int64_t)total, 256, 8), 256, 0, stream>>>(O->col[fixed_pos], (int64_t)total, fixed_term);
+            rc = launch_check("k_fill_i32");
+        }
     }
-    if (rc == TID_OK) rc = set_rows_const(C, (int64_t)total);
+    if (rc == TID_OK) rc = set_rows_const(O, (int64_t)total);
     if (rc == TID_OK) {
         // valid bounds (sort order) of each column
-        const uint32_t alo = (uint32_t)vals.front() ^ 0x80000000u, ahi = (uint32_t)vals.back() ^ 0x80000000u;
-        C->bounded = true;
-        C->lo[a_pos] = alo;
-        C->hi[a_pos] = ahi;
-        C->lo[1 - a_pos] = hmm[0];
-        C->hi[1 - a_pos] = hmm[1];
-        rc = set_ready(C);
+        O->bounded = true;
+        O->lo[pos[a_pos]] = sort_order_host(vals.front());
+        O->hi[pos[a_pos]] = sort_order_host(vals.back());
+        O->lo[pos[1 - a_pos]] = st.lo;
+        O->hi[pos[1 - a_pos]] = st.hi;
+        O->lo[fixed_pos] = O->hi[fixed_pos] = sort_order_host(fixed_term);
+        rc = set_ready(O);
     }
     if (rc != TID_OK) {
-        set_free(C);
+        set_free(O);
         return rc;
     }
-    *out = C;
+    *out = O;
     return TID_OK;
 }
 
@@ -618,7 +729,7 @@ extern "C" int tid_entail(tid_ctx *ctx, const tid_store *st, int rule, const tid
     TID_TRY(bind_set(ctx, st, sp, idx1, nullptr, 0, &A));
     hold.keep(A);
 
-    // 2) its distinct join terms -> key table
+    // 2) its distinct join terms -> key set
     tid_set *K = nullptr;
     TID_TRY(project_set(ctx, A, &R.on, 1, &K));
     hold.keep(K);
@@ -628,158 +739,215 @@ extern "C" int tid_entail(tid_ctx *ctx, const tid_store *st, int rule, const tid
         int64_t got = 0;
         TID_TRY(tid_set_to_host(K, keys.data(), sx.dist1, &got));
     }
-    // open addressing, at most half full; the home slot is the top bits of a
-    // multiplicative hash (Knuth), which depend on every bit of the key
-    int tbits = 4;
-    while ((1ull << tbits) < 2 * (uint64_t)std::max<int64_t>(sx.dist1, 1)) ++tbits;
-    const uint32_t tsize = 1u << tbits;
-    std::vector<int32_t> table(tsize, 0);
-    for (int32_t key : keys) {  // keys are distinct and positive (0 never joins)
-        if (key == 0) continue;
-        uint32_t h = home_slot(key, tbits);
-        while (table[h] != 0) h = (h + 1) & (tsize - 1);
-        table[h] = key;
-    }
-    void *d_table = nullptr;
-    TID_TRY(dev_alloc(ctx, &d_table, sizeof(int32_t) * tsize));
-    struct TableFree {
-        tid_ctx *c;
-        void *p;
-        ~TableFree() { dev_free(c, p); }
-    } tf{ctx, d_table};
-    TID_TRY_CUDA(cudaMemcpyAsync(d_table, table.data(), sizeof(int32_t) * tsize, cudaMemcpyHostToDevice, stream),
-                 "key table");
+    KeyTable kt;
+    build_keys(keys, &kt);
+    Buf kb{ctx};
+    const size_t kbytes = kt.table.empty() ? kt.bits.size() * 4 : kt.table.size() * 4;
+    TID_TRY(dev_alloc(ctx, &kb.p, kbytes));
+    TID_TRY_CUDA(cudaMemcpyAsync(kb.p, kt.table.empty() ? (const void *)kt.bits.data() : (const void *)kt.table.data(), kbytes,
+                                 cudaMemcpyHostToDevice, stream),
+                 "key set");
+    if (kt.table.empty()) kt.set.bits = (const uint32_t *)kb.p;
+    else kt.set.table = (const int32_t *)kb.p;
 
-    // 3) the data premise's triples whose join term is a key, in store order
-    int8_t bvars[3], bsrc[3];
-    int kb = 0;
+    // 3) the data premise's triples whose join term is a key.  Both premises on
+    //    the same predicate: the first search found the data premise's triples too
+    KeyedScan ks{};
+    const bool same = R.data_fixed != NONE && term[R.data_fixed] == term[R.schema];
+    ks.col[0] = same ? A->col[0] : st->s;
+    ks.col[1] = st->p;
+    ks.col[2] = same ? A->col[1] : st->o;
+    ks.n = same ? sx.res1 : st->n;
+    ks.fixed_slot = same || R.data_fixed == NONE ? -1 : 1;
+    ks.fixed_val = R.data_fixed == NONE ? 0 : term[R.data_fixed];
+    ks.key_slot = R.key_slot;
+    ks.keys = kt.set;
+    ks.vec = same || st->aligned16;
+    // the conclusion's terms: their slots, and where each comes from
+    const int8_t other = R.on == VA ? VB : VA;  // A's term that is not the join term
+    int pos[3], kc = 0, a_pos = -1, fixed_pos = -1;
+    int8_t src[3];  // data slot of conclusion term i; 3: A's other term
     for (int slot = 0; slot < 3; ++slot) {
-        const int8_t v = R.data_var[slot];
-        if (v < 0) continue;
-        bool seen = false;
-        for (int c = 0; c < kb; ++c) seen = seen || bvars[c] == v;
-        if (!seen) {
-            bvars[kb] = v;
-            bsrc[kb] = (int8_t)slot;
-            ++kb;
+        if (R.then_var[slot] < 0) {
+            fixed_pos = slot;
+            continue;
         }
-    }
-    tid_set *Braw = nullptr, *B = nullptr;
-    TID_TRY(set_alloc(ctx, kb, bvars, st->n, &Braw));
-    hold.keep(Braw);
-    const int fixed_slot = R.data_fixed == NONE ? -1 : 1;
-    const int32_t fixed_val = R.data_fixed == NONE ? 0 : term[R.data_fixed];
-    if (sx.dist1 > 0) {
-        TID_TRY(compact_semijoin(ctx, st, fixed_slot, fixed_val, R.key_slot, (const int32_t *)d_table, tbits,
-                                 bsrc, Braw));
-    } else {
-        TID_TRY(set_rows_const(Braw, 0));
-    }
-    TID_TRY(set_ready(Braw));
-    TID_TRY(rows_of(Braw, &sx.res2));
-    // the distinct join terms among them (the paper's #Dist2): the rows mark
-    // their term's slot of the key table, and the marks are counted
-    int kcol = 0;
-    for (int c = 0; c < kb; ++c)
-        if (bvars[c] == R.on) kcol = c;
-    {
-        const uint32_t fwords = (tsize + 31) / 32, fpad = (fwords + 1) & ~1u;
-        Buf fb{ctx};
-        TID_TRY(dev_alloc(ctx, &fb.p, sizeof(uint32_t) * fpad + sizeof(unsigned long long)));
-        uint32_t *flags = (uint32_t *)fb.p;
-        unsigned long long *d_cnt = (unsigned long long *)(flags + fpad);
-        TID_TRY_CUDA(cudaMemsetAsync(flags, 0, sizeof(uint32_t) * fwords, stream), "key marks");
-        if (sx.res2 > 0) {
-            const unsigned grid = grid_for(sx.res2, BM_THREADS * BM_U, 8);
-            const size_t fsmem = sizeof(uint32_t) * fwords;
-            if (fsmem <= 32 * 1024)
-                k_mark_keys<true><<<grid, BM_THREADS, fsmem, stream>>>(Braw->col[kcol], sx.res2,
-                                                                       (const int32_t *)d_table, tbits, flags);
-            else
-                k_mark_keys<false><<<grid, BM_THREADS, 0, stream>>>(Braw->col[kcol], sx.res2,
-                                                                    (const int32_t *)d_table, tbits, flags);
-            TID_TRY(launch_check("k_mark_keys"));
+        if (R.then_var[slot] == other) {
+            a_pos = kc;
+            src[kc] = 3;
+        } else {
+            for (int d = 0; d < 3; ++d)
+                if (R.data_var[d] == R.then_var[slot]) src[kc] = (int8_t)d;
         }
-        k_count_bits<<<1, 1024, 0, stream>>>(flags, fwords, d_cnt);
+        pos[kc++] = slot;
+    }
+    const bool pair = kc == 2;
+    const int32_t *pair_term = pair ? ks.col[src[1 - a_pos]] : nullptr;
+    const int8_t one = 0;
+    tid_set *count = nullptr;  // holds the number of marked rows
+    TID_TRY(set_alloc(ctx, 1, &one, 0, &count));
+    hold.keep(count);
+    SelScratch sc{};
+    Buf scb{ctx}, fb{ctx};
+    KeyStats ss{0, 0xFFFFFFFFu, 0u};
+    if (sx.dist1 > 0 && ks.n > 0) {
+        TID_TRY(sel_scratch(ctx, ks.n, 1, 0, &sc, &scb.p, nullptr));
+        const uint32_t fwords = (kt.numbers + 31) / 32;
+        TID_TRY(dev_alloc(ctx, &fb.p, sizeof(KeyStats) + sizeof(uint32_t) * fwords));
+        KeyStats *d_ss = (KeyStats *)fb.p;
+        uint32_t *flags = (uint32_t *)(d_ss + 1);
+        TID_TRY_CUDA(cudaMemcpyAsync(d_ss, &ss, sizeof ss, cudaMemcpyHostToDevice, stream), "key stats");
+        TID_TRY_CUDA(cudaMemsetAsync(flags, 0, sizeof(uint32_t) * fwords, stream), "key flags");
+        const size_t smem = kt.numbers <= KM_SMEM_KEYS ? kt.numbers : 0;
+        k_key_mark<<<sc.ranges, SEL_THREADS, smem, stream>>>(ks, sc, count->d_rows, count->slot.dev, flags, kt.numbers, pair_term,
+                                                             d_ss);
+        TID_TRY(launch_check("k_key_mark"));
+        k_count_bits<<<1, 1024, 0, stream>>>(flags, fwords, &d_ss->keys);
         TID_TRY(launch_check("k_count_bits"));
-        unsigned long long cnt = 0;
-        TID_TRY_CUDA(cudaMemcpyAsync(&cnt, d_cnt, sizeof cnt, cudaMemcpyDeviceToHost, stream), "key count");
-        TID_TRY_CUDA(cudaStreamSynchronize(stream), "key count");
-        sx.dist2 = (int64_t)cnt;
-    }
-    B = Braw;  // rows in store order: neither form of step 4 needs an order
-
-    // 4) the join on the shared term, the conclusion's terms kept with
-    //    DISTINCT.  A two-term conclusion with one term from each premise is
-    //    the bit matrix of its distinct pairs, when that is small enough;
-    //    otherwise the join is a hash join with the schema side (the small one)
-    //    as the table, its rows left in the order written, and the conclusion's
-    //    terms are put in canonical order with DISTINCT -- the one sort of the
-    //    rule.
-    int8_t cvars[3];
-    int kc = 0;
-    for (int slot = 0; slot < 3; ++slot)
-        if (R.then_var[slot] >= 0) cvars[kc++] = R.then_var[slot];
-    tid_set *C = nullptr;
-    TID_TRY(conclude_pairs(ctx, R, A, B, sx.res2, bvars, kb, table, (const int32_t *)d_table, tbits, cvars, kc,
-                           &C));
-    if (C) {
-        hold.keep(C);
+        TID_TRY_CUDA(cudaMemcpyAsync(&ss, d_ss, sizeof ss, cudaMemcpyDeviceToHost, stream), "key stats");
     } else {
+        TID_TRY(set_rows_const(count, 0));
+    }
+    TID_TRY(set_ready(count));
+    // the schema premise's rows (synchronises: the statistics are on the host too)
+    SchemaRows sr;
+    if (sx.res1 <= (pair ? PAIR_MAX_SCHEMA_ROWS : MAP_MAX_SCHEMA_ROWS)) {
+        std::vector<int32_t> arows((size_t)sx.res1 * 2);
+        int64_t got = 0;
+        TID_TRY(tid_set_to_host(A, arows.data(), sx.res1, &got));
+        const int ak = A->vars[0] == R.on ? 0 : 1;
+        sr.rows.reserve((size_t)got);
+        for (int64_t i = 0; i < got; ++i) {
+            const int64_t h = kt.number(arows[(size_t)i * 2 + ak]);
+            if (h >= 0) sr.rows.emplace_back((uint32_t)h, arows[(size_t)i * 2 + 1 - ak]);
+        }
+        std::sort(sr.rows.begin(), sr.rows.end());
+        sr.rows.erase(std::unique(sr.rows.begin(), sr.rows.end()), sr.rows.end());
+        for (size_t i = 1; i < sr.rows.size(); ++i) sr.one_each = sr.one_each && sr.rows[i].first != sr.rows[i - 1].first;
+    }
+    TID_TRY_CUDA(cudaStreamSynchronize(stream), "key stats");
+    TID_TRY(rows_of(count, &sx.res2));
+    sx.dist2 = (int64_t)ss.keys;
+
+    // 4) the conclusion, labelled (s, p, o); a fixed predicate is its middle
+    //    column, whose one value keeps the canonical order
+    const int8_t ovars[3] = {0, 1, 2};
+    const int32_t fixed_term = R.then_term == NONE ? 0 : term[R.then_term];
+    tid_set *O = nullptr;
+    if (sx.res2 == 0) {
+        TID_TRY(set_alloc(ctx, 3, ovars, 0, &O));
+        int rc = set_rows_const(O, 0);
+        if (rc == TID_OK) rc = set_ready(O);
+        if (rc != TID_OK) {
+            set_free(O);
+            return rc;
+        }
+    } else if (pair && !sr.rows.empty()) {
+        TID_TRY(conclude_pairs(ctx, ks, sc, kt, sr, ss, sx.res2, pair_term, a_pos, pos, fixed_pos, fixed_term, &O));
+    }
+    if (!O) {
+        // the joined rows' conclusion terms, in any order, then sorted with DISTINCT
         tid_set *J = nullptr;
-        TID_TRY(join_sets(ctx, A, B, TID_JOIN_HASH, &J, false));
-        hold.keep(J);
         const int32_t *ccols[3];
         Bounds cb{};
-        for (int i = 0; i < kc; ++i) {
-            int c = 0;
-            while (J->vars[c] != cvars[i]) ++c;
-            ccols[i] = J->col[c];
-            cb.lo[i] = J->lo[c];
-            cb.hi[i] = J->hi[c];
-        }
+        bool bounded = true;
         int64_t nj = 0;
-        TID_TRY(rows_of(J, &nj));
-        TID_TRY(canonicalize(ctx, ccols, kc, cvars, nj, true, J->bounded ? &cb : nullptr, &C));
-        hold.keep(C);
-    }
-    int64_t rows = 0;
-    TID_TRY(rows_of(C, &rows));
-
-    // the (s, p, o) set: C's columns, the fixed predicate in the middle when the
-    // conclusion has one (a constant column keeps C's order canonical)
-    const int8_t ovars[3] = {0, 1, 2};
-    tid_set *O = nullptr;
-    TID_TRY(set_alloc(ctx, 3, ovars, rows, &O));
-    int rc = TID_OK;
-    int c = 0;
-    for (int slot = 0; slot < 3 && rc == TID_OK; ++slot) {
-        if (R.then_var[slot] >= 0) {
-            if (rows > 0) {
-                cudaError_t e = cudaMemcpyAsync(O->col[slot], C->col[c], (size_t)rows * 4, cudaMemcpyDeviceToDevice,
-                                                stream);
-                if (e != cudaSuccess) rc = fail_cuda(e, "conclusion column");
+        if (!sr.rows.empty() && sr.one_each) {
+            int8_t jvars[3] = {0, 1, 2};
+            TID_TRY(set_alloc(ctx, kc, jvars, sx.res2, &J));
+            hold.keep(J);
+            std::vector<int32_t> map(kt.numbers, 0);
+            for (const auto &r : sr.rows) map[r.first] = r.second;
+            Buf mapb{ctx};
+            const size_t mm_b = 2 * TID_MAX_COLS * sizeof(uint32_t);
+            TID_TRY(dev_alloc(ctx, &mapb.p, mm_b + map.size() * 4));
+            uint32_t *mm = (uint32_t *)mapb.p, hb[2 * TID_MAX_COLS];
+            int32_t *d_map = (int32_t *)(mm + 2 * TID_MAX_COLS);
+            TID_TRY_CUDA(cudaMemcpyAsync(d_map, map.data(), map.size() * 4, cudaMemcpyHostToDevice, stream), "key map");
+            if (pair) {  // the data term's range is known; A's terms are on the host
+                TID_TRY(expand_keyed(ctx, ks, sc, src, d_map, J, nullptr));
+                cb.lo[1 - a_pos] = ss.lo;
+                cb.hi[1 - a_pos] = ss.hi;
+                cb.lo[a_pos] = 0xFFFFFFFFu;
+                for (const auto &r : sr.rows) {
+                    cb.lo[a_pos] = std::min(cb.lo[a_pos], sort_order_host(r.second));
+                    cb.hi[a_pos] = std::max(cb.hi[a_pos], sort_order_host(r.second));
+                }
+                TID_TRY_CUDA(cudaStreamSynchronize(stream), "key map");  // the host copy of the map
+            } else {
+                TID_TRY_CUDA(cudaMemsetAsync(mm, 0xFF, mm_b / 2, stream), "conclusion range");
+                TID_TRY_CUDA(cudaMemsetAsync(mm + TID_MAX_COLS, 0, mm_b / 2, stream), "conclusion range");
+                TID_TRY(expand_keyed(ctx, ks, sc, src, d_map, J, mm));
+                TID_TRY_CUDA(cudaMemcpyAsync(hb, mm, sizeof hb, cudaMemcpyDeviceToHost, stream), "conclusion range");
+                TID_TRY_CUDA(cudaStreamSynchronize(stream), "conclusion range");
+                for (int i = 0; i < kc; ++i) {
+                    cb.lo[i] = hb[i];
+                    cb.hi[i] = hb[TID_MAX_COLS + i];
+                }
             }
-            O->lo[slot] = C->lo[c];
-            O->hi[slot] = C->hi[c];
-            ++c;
+            for (int i = 0; i < kc; ++i) ccols[i] = J->col[i];
+            nj = sx.res2;
         } else {
-            const int32_t v = term[R.then_term];
-            if (rows > 0) {
-                k_fill_i32<<<grid_for(rows, 256, 8), 256, 0, stream>>>(O->col[slot], rows, v);
-                rc = launch_check("k_fill_i32");
+            // the data premise's rows in store order, joined with the schema side
+            // (the small one) as the hash table
+            int8_t bvars[3], bsrc[3];
+            int nb = 0;
+            for (int slot = 0; slot < 3; ++slot) {
+                if (R.data_var[slot] < 0) continue;
+                bvars[nb] = R.data_var[slot];
+                bsrc[nb++] = (int8_t)slot;
             }
-            O->lo[slot] = O->hi[slot] = (uint32_t)v ^ 0x80000000u;
+            tid_set *B = nullptr;
+            TID_TRY(set_alloc(ctx, nb, bvars, sx.res2, &B));
+            hold.keep(B);
+            TID_TRY(expand_keyed(ctx, ks, sc, bsrc, nullptr, B, nullptr));
+            TID_TRY(set_rows_const(B, sx.res2));
+            TID_TRY(set_ready(B));
+            TID_TRY(join_sets(ctx, A, B, TID_JOIN_HASH, &J, false));
+            hold.keep(J);
+            bounded = J->bounded;
+            for (int i = 0; i < kc; ++i) {
+                int c = 0;
+                while (J->vars[c] != R.then_var[pos[i]]) ++c;
+                ccols[i] = J->col[c];
+                cb.lo[i] = J->lo[c];
+                cb.hi[i] = J->hi[c];
+            }
+            TID_TRY(rows_of(J, &nj));
+        }
+        if (!pair) {
+            TID_TRY(canonicalize(ctx, ccols, 3, ovars, nj, true, bounded ? &cb : nullptr, &O));
+        } else {
+            tid_set *C = nullptr;
+            const int8_t cvars[2] = {0, 1};
+            if (!bounded) {  // as two columns, then the fixed one between them
+                TID_TRY(canonicalize(ctx, ccols, 2, cvars, nj, true, nullptr, &C));
+                hold.keep(C);
+                TID_TRY(rows_of(C, &nj));
+                ccols[0] = C->col[0];
+                ccols[1] = C->col[1];
+                for (int i = 0; i < 2; ++i) {
+                    cb.lo[i] = C->lo[i];
+                    cb.hi[i] = C->hi[i];
+                }
+            }
+            // a column of one value has no field in the packed rows (two columns
+            // always fit them) and is not read
+            const int32_t *o3[3];
+            Bounds ob{};
+            for (int i = 0; i < 2; ++i) {
+                o3[pos[i]] = ccols[i];
+                ob.lo[pos[i]] = cb.lo[i];
+                ob.hi[pos[i]] = cb.hi[i];
+            }
+            o3[fixed_pos] = ccols[0];
+            ob.lo[fixed_pos] = ob.hi[fixed_pos] = sort_order_host(fixed_term);
+            TID_TRY(canonicalize(ctx, o3, 3, ovars, nj, true, &ob, &O));
         }
     }
-    O->bounded = C->bounded;
-    if (rc == TID_OK) rc = set_rows_const(O, rows);
-    if (rc == TID_OK) rc = set_ready(O);
-    if (rc != TID_OK) {
-        set_free(O);
-        return rc;
-    }
-    sx.all = rows;
+    hold.keep(O);
+    TID_TRY(rows_of(O, &sx.all));
+    hold.v.pop_back();
     if (stats) *stats = sx;
     *out = O;
     return TID_OK;

@@ -75,12 +75,6 @@ int member_bits(tid_ctx *ctx, const int32_t *col, int64_t n, uint32_t lo, uint32
 // rows of `in` whose first column is a member, in order
 int compact_member(tid_ctx *ctx, const tid_set *in, int64_t n, const Members &m, tid_set *out);
 int compact_filter(tid_ctx *ctx, const tid_set *in, int64_t n, const Pred *preds, int n_preds, tid_set *out);
-// store triples (in store order) whose fixed_slot holds fixed_val (fixed_slot -1:
-// any) and whose key_slot term is in the key table (2^tbits slots, home slot =
-// top tbits bits of key * 0x9E3779B1, linear probing, 0 = empty); output column
-// c = slot src[c]
-int compact_semijoin(tid_ctx *ctx, const tid_store *st, int fixed_slot, int32_t fixed_val, int key_slot,
-                     const int32_t *table, int tbits, const int8_t *src, tid_set *out);
 int compact_unique(tid_ctx *ctx, const int32_t *const *cols, int k, const int32_t *perm, int64_t n,
                    tid_set *out);
 // sorted packed keys (64-bit if wide, else 32-bit) -> distinct rows of k columns

@@ -740,6 +740,7 @@ template <typename K>
 static int canonical_packed(tid_ctx *ctx, const int32_t *const *cols, int k, int64_t n, bool dedupe,
                             const PackSpec &ps, int total_bits, int sorted_bits, tid_set *set) {
     cudaStream_t st = ctx->stream;
+    if (dedupe && total_bits == 0) n = 1;  // every row is the same
     if (n <= SMALL_N) {
         ColPtrs cp{};
         MutColPtrs op{};

@@ -234,3 +234,33 @@ def test_union_merges(ctx, orc, ids, shape, n):
     assert np.array_equal(_rows(got), want.rows)
     for h in hs:
         tb.tid_set_free(h)
+
+
+@pytest.mark.parametrize("rule", [2, 3, 5, 7, 9, 11])
+@pytest.mark.parametrize("schema", ["tree", "many"])      # one schema row per key, or several
+@pytest.mark.parametrize("spread", [1, 70_001])            # IDs dense, or over most of int32
+@pytest.mark.parametrize("n", [900, 45_000])
+def test_entailment_forms(ctx, orc, rule, schema, spread, n):
+    """The forms of a rule's last step (bit matrix, key map, hash join) and of its key set (a range of
+    bits, a table): small and large ID ranges, functional and branching schemas."""
+    rng = np.random.default_rng([rule, len(schema), spread, n])
+    v = {"type": 1, "domain": 2, "range": 3, "subprop": 4, "subclass": 5}
+    t = []
+    for k in range(30):                                     # terms 10 .. 39: classes and predicates
+        ups = [k // 2] if schema == "tree" else rng.integers(0, 30, 3)
+        for u in ups:
+            for p in (v["domain"], v["range"], v["subprop"], v["subclass"]):
+                t.append((10 + k, p, 10 + int(u)))
+    data = np.stack([rng.integers(10, 10 + n // 3, n), np.where(rng.random(n) < 0.3, 1, rng.integers(10, 60, n)),
+                     rng.integers(10, 60, n)], 1)
+    data[::7, 2] = rng.integers(10, n // 3 + 10, len(data[::7]))
+    t = np.unique(np.concatenate([np.array(t), data]), axis=0)
+    t = np.where(t < 10, t, (t - 9) * spread % (2**31 - 1) + 9)
+    t = t[rng.permutation(len(t))].astype(np.int32)
+    S, P, O = (np.ascontiguousarray(t[:, c]) for c in range(3))
+    st = tb.tid_load(ctx, S, P, O)
+    h, stats = tb.tid_entail(ctx, st, rule, v)
+    want, wstats = orc.entail(S, P, O, rule, v)
+    assert stats == wstats
+    assert np.array_equal(_rows(h), want.rows)
+    tb.tid_store_free(st)
