@@ -75,22 +75,86 @@ DeviceGuard::~DeviceGuard() {
 // ---------------------------------------------------------------------------
 // memory
 // ---------------------------------------------------------------------------
+// Class c holds blocks of (4 + c % 4) / 4 * 256 << (c / 4) bytes.
+static size_t class_bytes(int c) { return ((size_t)64 << (c / 4)) * (4 + c % 4); }
+static int block_class(size_t *bytes) {  // *bytes is rounded up to the class
+    int c = 0;
+    while (class_bytes(c) < *bytes) ++c;
+    *bytes = class_bytes(c);
+    return c;
+}
+
+// Gives the held blocks back to the pool; false if there are none.
+static bool drop_blocks(tid_ctx *ctx) {
+    std::lock_guard<std::mutex> lk(ctx->blocks_mu);
+    BlockCache &b = ctx->blocks;
+    bool any = false;
+    for (auto &f : b.free_blocks) {
+        for (void *p : f) {
+            b.class_of.erase(p);
+            cudaFreeAsync(p, ctx->stream);
+            any = true;
+        }
+        f.clear();
+    }
+    b.held = 0;
+    return any;
+}
+
 int dev_alloc(tid_ctx *ctx, void **p, size_t bytes) {
     *p = nullptr;
     const int64_t fa = ctx->fail_after.load(std::memory_order_relaxed);
     if (fa >= 0 && ctx->allocs.fetch_add(1, std::memory_order_relaxed) >= fa)
         return fail(TID_ERR_OOM, "device allocation refused (injected failure)");
     if (bytes == 0) bytes = 256;
+    // (a capture's allocations belong to its graph)
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    int cls = -1;
+    if (bytes <= BlockCache::MAX_BLOCK && cudaStreamIsCapturing(ctx->stream, &cap) == cudaSuccess &&
+        cap == cudaStreamCaptureStatusNone)
+        cls = block_class(&bytes);
+    if (cls >= 0) {
+        std::lock_guard<std::mutex> lk(ctx->blocks_mu);
+        auto &f = ctx->blocks.free_blocks[cls];
+        if (!f.empty()) {
+            *p = f.back();
+            f.pop_back();
+            ctx->blocks.held -= bytes;
+            return TID_OK;
+        }
+    }
     cudaError_t e = cudaMallocFromPoolAsync(p, bytes, ctx->pool, ctx->stream);
+    if (e == cudaErrorMemoryAllocation && drop_blocks(ctx)) {
+        cudaGetLastError();
+        e = cudaMallocFromPoolAsync(p, bytes, ctx->pool, ctx->stream);
+    }
     if (e != cudaSuccess) {
         *p = nullptr;
         return fail_cuda(e, "device allocation");
+    }
+    if (cls >= 0) {
+        std::lock_guard<std::mutex> lk(ctx->blocks_mu);
+        ctx->blocks.class_of[*p] = cls;
     }
     return TID_OK;
 }
 
 void dev_free(tid_ctx *ctx, void *p) {
-    if (p) cudaFreeAsync(p, ctx->stream);
+    if (!p) return;
+    {
+        std::lock_guard<std::mutex> lk(ctx->blocks_mu);
+        auto it = ctx->blocks.class_of.find(p);
+        if (it != ctx->blocks.class_of.end()) {
+            const size_t bytes = class_bytes(it->second);
+            if (ctx->blocks.held + bytes <= BlockCache::MAX_HELD) {
+                ctx->blocks.free_blocks[it->second].push_back(p);
+                ctx->blocks.held += bytes;
+                return;
+            }
+            ctx->blocks.class_of.erase(it);
+        }
+    }
+    cudaFreeAsync(p, ctx->stream);
 }
 
 // The context's look-back scratch, grown on demand to >= `words` status words
@@ -145,23 +209,41 @@ int lookback_scratch(tid_ctx *ctx, unsigned int num_tiles, Lookback *lb) {
 // ---------------------------------------------------------------------------
 static constexpr int SLAB_SLOTS = 4096;
 
+static void recycle(tid_ctx *ctx, const PendingSlot &p) {
+    if (ctx->free_events.size() < MAX_FREE_EVENTS) ctx->free_events.push_back(p.ev);
+    else cudaEventDestroy(p.ev);
+    ctx->free_slots.push_back({p.slot.slab, p.slot.index});
+}
+
 static void sweep_pending(tid_ctx *ctx, bool wait) {
     auto &pend = ctx->pending;
     size_t w = 0;
     for (size_t i = 0; i < pend.size(); ++i) {
         cudaError_t q = wait ? cudaEventSynchronize(pend[i].ev) : cudaEventQuery(pend[i].ev);
-        if (q == cudaSuccess || q != cudaErrorNotReady) {
-            cudaEventDestroy(pend[i].ev);
-            ctx->free_slots.push_back({pend[i].slot.slab, pend[i].slot.index});
-        } else {
-            pend[w++] = pend[i];
-        }
+        if (q == cudaSuccess || q != cudaErrorNotReady) recycle(ctx, pend[i]);
+        else pend[w++] = pend[i];
     }
+    if (w) cudaGetLastError();  // "not ready" is no failure of a later launch
     pend.resize(w);
+}
+
+// The oldest pending slots whose producers are done, a few at a time (a program
+// that frees sets far ahead of the GPU has thousands pending).
+static void sweep_oldest(tid_ctx *ctx) {
+    auto &pend = ctx->pending;
+    for (int i = 0; i < 4 && !pend.empty(); ++i) {
+        if (cudaEventQuery(pend.front().ev) == cudaErrorNotReady) {
+            cudaGetLastError();  // "not ready" is no failure of a later launch
+            break;
+        }
+        recycle(ctx, pend.front());
+        pend.pop_front();
+    }
 }
 
 static int slot_acquire(tid_ctx *ctx, Slot *s) {
     std::lock_guard<std::mutex> lk(ctx->mu);
+    if (ctx->free_events.empty()) sweep_oldest(ctx);
     if (ctx->free_slots.empty()) sweep_pending(ctx, false);
     if (ctx->free_slots.empty()) {
         void *h = nullptr;
@@ -214,7 +296,15 @@ int set_alloc(tid_ctx *ctx, int k, const int8_t *vars, int64_t cap, tid_set **ou
     s->d_rows = (int64_t *)((char *)s->block + colb * k);
     rc = slot_acquire(ctx, &s->slot);
     if (rc == TID_OK) {
-        cudaError_t e = cudaEventCreateWithFlags(&s->ready, cudaEventDisableTiming);
+        cudaError_t e = cudaSuccess;
+        {
+            std::lock_guard<std::mutex> lk(ctx->mu);
+            if (!ctx->free_events.empty()) {
+                s->ready = ctx->free_events.back();
+                ctx->free_events.pop_back();
+            }
+        }
+        if (!s->ready) e = cudaEventCreateWithFlags(&s->ready, cudaEventDisableTiming);
         if (e != cudaSuccess) {
             s->ready = nullptr;
             rc = fail_cuda(e, "event");
@@ -357,8 +447,10 @@ extern "C" int tid_ctx_destroy(tid_ctx *ctx) {
         std::lock_guard<std::mutex> lk(ctx->mu);
         sweep_pending(ctx, true);
     }
-    if (ctx->lb_status) cudaFreeAsync(ctx->lb_status, ctx->stream);
-    if (ctx->sel_done) cudaFreeAsync(ctx->sel_done, ctx->stream);
+    if (ctx->lb_status) dev_free(ctx, ctx->lb_status);
+    if (ctx->sel_done) dev_free(ctx, ctx->sel_done);
+    drop_blocks(ctx);
+    for (cudaEvent_t ev : ctx->free_events) cudaEventDestroy(ev);
     cudaStreamSynchronize(ctx->stream);
     for (auto *h : ctx->slabs_host) cudaFreeHost(h);
     if (ctx->err_host) cudaFreeHost(ctx->err_host);

@@ -7,8 +7,10 @@
 #include <nvtx3/nvToolsExt.h>
 
 #include <atomic>
+#include <deque>
 #include <mutex>
 #include <string>
+#include <unordered_map>
 #include <vector>
 
 #include "tid.h"
@@ -82,6 +84,21 @@ struct PendingSlot {  // a freed set's slot, reusable once its producer event co
     cudaEvent_t ev;
 };
 
+// Device blocks a context has freed and hands out again without a driver call (a
+// plan on a small store makes some thirty small allocations per operator chain).
+// Everything a context does is ordered on its one stream, so a block may be
+// reused by the next launch.  Sizes are rounded up to a class (four per power of
+// two); larger blocks, and blocks freed while `bytes` are held, go back to the pool.
+constexpr size_t MAX_FREE_EVENTS = 1024;
+
+struct BlockCache {
+    static constexpr size_t MAX_BLOCK = (size_t)64 << 20, MAX_HELD = (size_t)256 << 20;
+    static constexpr int CLASSES = 4 * 18 + 1;  // 256 B << 18 = 64 MB
+    std::vector<void *> free_blocks[CLASSES];
+    std::unordered_map<void *, int> class_of;  // blocks of a class, in use or held
+    size_t held = 0;
+};
+
 struct SharedBlock {  // device allocations shared by several sets (freed with the last)
     void *ptr[2] = {nullptr, nullptr};
     int refs = 0;
@@ -107,8 +124,11 @@ struct tid_ctx {
     std::vector<int64_t *> slabs_host;
     std::vector<int64_t *> slabs_dev;
     std::vector<std::pair<int, int>> free_slots;
-    std::vector<tid::PendingSlot> pending;
+    std::deque<tid::PendingSlot> pending;
+    std::vector<cudaEvent_t> free_events;  // of freed sets (at most MAX_FREE_EVENTS)
     std::mutex mu;
+    tid::BlockCache blocks;
+    std::mutex blocks_mu;
     // the batched search's last plan on this context (tid_batch_tuning)
     int batch_shape = -1, batch_keys = 0, batch_subs = 0;
     // testing aid (tid_ctx_inject_alloc_failure): allocations left before they fail
