@@ -91,7 +91,7 @@ static bool drop_blocks(tid_ctx *ctx) {
     bool any = false;
     for (auto &f : b.free_blocks) {
         for (void *p : f) {
-            b.class_of.erase(p);
+            b.known.erase(p);
             cudaFreeAsync(p, ctx->stream);
             any = true;
         }
@@ -119,6 +119,7 @@ int dev_alloc(tid_ctx *ctx, void **p, size_t bytes) {
         if (!f.empty()) {
             *p = f.back();
             f.pop_back();
+            ctx->blocks.known[*p].held = false;
             ctx->blocks.held -= bytes;
             return TID_OK;
         }
@@ -134,7 +135,7 @@ int dev_alloc(tid_ctx *ctx, void **p, size_t bytes) {
     }
     if (cls >= 0) {
         std::lock_guard<std::mutex> lk(ctx->blocks_mu);
-        ctx->blocks.class_of[*p] = cls;
+        ctx->blocks.known[*p] = {cls, false};
     }
     return TID_OK;
 }
@@ -143,15 +144,17 @@ void dev_free(tid_ctx *ctx, void *p) {
     if (!p) return;
     {
         std::lock_guard<std::mutex> lk(ctx->blocks_mu);
-        auto it = ctx->blocks.class_of.find(p);
-        if (it != ctx->blocks.class_of.end()) {
-            const size_t bytes = class_bytes(it->second);
+        auto it = ctx->blocks.known.find(p);
+        if (it != ctx->blocks.known.end()) {
+            if (it->second.held) return;  // freed already: never in the list twice
+            const size_t bytes = class_bytes(it->second.cls);
             if (ctx->blocks.held + bytes <= BlockCache::MAX_HELD) {
-                ctx->blocks.free_blocks[it->second].push_back(p);
+                ctx->blocks.free_blocks[it->second.cls].push_back(p);
+                it->second.held = true;
                 ctx->blocks.held += bytes;
                 return;
             }
-            ctx->blocks.class_of.erase(it);
+            ctx->blocks.known.erase(it);
         }
     }
     cudaFreeAsync(p, ctx->stream);
