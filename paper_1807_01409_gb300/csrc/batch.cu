@@ -270,20 +270,25 @@ __global__ void __launch_bounds__(KB_THREADS) k_batch(BatchArgs a) {
         for (int k = lane; k < a.kids; k += 32) row[k] = cnt[k];
 }
 
-// QUEUE shape: only the (triple, mask) pairs the prefilter admits are looked
-// up.  For each 32-triple slot, lane l lists the masks its triple may answer;
-// an exclusive scan over the lanes' counts gives each lane its place in a
-// per-warp queue of (lane, mask) bytes, lane-major, so for any one mask the
-// queue is in triple order.  The warp then looks the queue up 32 entries at a
-// time -- an entry's triple values and mixed columns come from its lane by
-// shuffle -- and counts or writes the hits as the direct shape does (lanes with
-// the same key id grouped by match_any, ranked in queue order, hence in triple
-// order).  Lookups per triple follow the prefilter's candidates instead of the
-// number of masks present; UNROLL slots are loaded per iteration.
+// QUEUE shape: only the (triple, mask) pairs the prefilter admits are looked up.
+// For each 32-triple slot and each mask that some lane may answer, the lanes'
+// candidates join a per-warp queue in lane order (a ballot places them), with the
+// triple's values, so for any one mask the queue is in triple order.  Whenever 32
+// wait, the warp looks them up, all lanes at work -- whatever slots they came
+// from -- and counts or writes the hits as the direct shape does (lanes with the
+// same key id grouped by match_any, ranked in queue order, hence in triple order).
+// A slot without a candidate costs its loads, three prefilter reads and one warp
+// reduction.  UNROLL slots are loaded per iteration.
+// Measured on GB300, 512 queries (all shapes) on 200M triples: a count pass 1477 ->
+// 848 us against the form that queued and looked up every slot by itself (a
+// five-step scan per slot, lookups with a few lanes at work).  Bound: instruction
+// issue of the prefilter.
+constexpr int KB_RING = 64;  // queue entries: under 32 wait when a mask adds up to 32
+
 template <int U, bool WRITE, int UNROLL>
 __global__ void __launch_bounds__(KB_THREADS) k_batch_q(BatchArgs a) {
     extern __shared__ __align__(16) unsigned char kb_smem[];
-    __shared__ uint8_t s_queue[KB_WARPS][32 * 7];
+    __shared__ int4 s_queue[KB_WARPS][KB_RING];  // (offset in the slice << 3) | mask, s, p, o
     __shared__ uint32_t s_msk[8];
     Entry *s_tab = (Entry *)kb_smem;
     uint16_t *s_disp = (uint16_t *)(s_tab + a.ns);
@@ -301,10 +306,45 @@ __global__ void __launch_bounds__(KB_THREADS) k_batch_q(BatchArgs a) {
     for (int k = lane; k < a.kids; k += 32)
         cnt[k] = WRITE ? row[k] + (a.abs32 ? (uint32_t)a.off[k] : 0u) : 0u;
     __syncthreads();
-    uint8_t *queue = s_queue[warp];
+    int4 *queue = s_queue[warp];
+    unsigned head = 0, tail = 0;  // entries [head, tail) wait
     const int64_t lo = gw * a.slice, hi = min(lo + a.slice, a.n);
+    auto look_up = [&](unsigned waiting) {  // the first min(waiting, 32) entries
+        const bool on = lane < waiting;
+        const int4 e = on ? queue[(head + lane) & (KB_RING - 1)] : make_int4(0, 0, 0, 0);
+        const int m = e.x & 7;
+        int k = -1;
+        if (on) {
+            const uint32_t ms = (U & 1) ? kb_colmix(a.hp, 0, (uint32_t)e.y) : 0u;
+            const uint32_t mp = (U & 2) ? kb_colmix(a.hp, 1, (uint32_t)e.z) : 0u;
+            const uint32_t mo = (U & 4) ? kb_colmix(a.hp, 2, (uint32_t)e.w) : 0u;
+            uint32_t h = s_msk[m];
+            if (m & 1) h ^= ms;
+            if (m & 2) h ^= kb_rotl(mp, 11);
+            if (m & 4) h ^= kb_rotl(mo, 22);
+            const uint32_t d = s_disp[kb_bucket(h, a.nb)];
+            const Entry en = s_tab[kb_slot(a.hp, h, d, a.ns)];
+            const bool hit = (en.mask_kid >> 28) == m && (!(m & 1) || en.s == e.y) && (!(m & 2) || en.p == e.z) &&
+                             (!(m & 4) || en.o == e.w);
+            k = hit ? (en.mask_kid & 0x0FFFFFFF) : -1;
+        }
+        if (__any_sync(0xffffffffu, k >= 0)) {
+            const unsigned peers = __match_any_sync(0xffffffffu, k);
+            if (k >= 0) {
+                const uint32_t cc = cnt[k];
+                if (WRITE) {
+                    const uint32_t r = cc + __popc(peers & lt);
+                    a.arena[a.abs32 ? (int64_t)r : a.off[k] + r] = (int32_t)(lo + ((uint32_t)e.x >> 3));
+                }
+                __syncwarp(peers);
+                if (lane == (unsigned)(__ffs(peers) - 1)) cnt[k] = cc + __popc(peers);
+            }
+        }
+        __syncwarp();
+    };
     for (int64_t b0 = lo; b0 < hi; b0 += 32 * UNROLL) {
         int32_t vs[UNROLL], vp[UNROLL], vo[UNROLL];
+        uint32_t cand[UNROLL];
 #pragma unroll
         for (int u = 0; u < UNROLL; ++u) {
             const int64_t i = b0 + u * 32 + lane;
@@ -315,7 +355,6 @@ __global__ void __launch_bounds__(KB_THREADS) k_batch_q(BatchArgs a) {
         }
 #pragma unroll
         for (int u = 0; u < UNROLL; ++u) {
-            const int64_t i = b0 + u * 32 + lane;
             const uint32_t v3[3] = {(uint32_t)vs[u], (uint32_t)vp[u], (uint32_t)vo[u]};
             uint32_t e3[3] = {0u, 0u, 0u};
 #pragma unroll
@@ -324,87 +363,66 @@ __global__ void __launch_bounds__(KB_THREADS) k_batch_q(BatchArgs a) {
                 const uint32_t f = kb_fentry(a.hp, c, v3[c]);
                 e3[c] = (s_filt[c * KB_FILTER_WORDS + (f >> 3)] >> ((f & 7u) * 4u)) & 0xFu;
             }
-            const uint32_t cand = i < hi ? kb_candidates(e3[0], e3[1], e3[2]) & 0xFEu : 0u;
-            const unsigned c = __popc(cand);
-            unsigned x = c;
+            cand[u] = b0 + u * 32 + lane < hi ? kb_candidates(e3[0], e3[1], e3[2]) & 0xFEu : 0u;
+        }
 #pragma unroll
-            for (int d = 1; d < 32; d <<= 1) {
-                const unsigned y = __shfl_up_sync(0xffffffffu, x, d);
-                if ((int)lane >= d) x += y;
-            }
-            const unsigned tot = __shfl_sync(0xffffffffu, x, 31);
-            if (tot == 0) continue;
-            unsigned at = x - c;
-            for (uint32_t cm = cand; cm; cm &= cm - 1) queue[at++] = (uint8_t)((lane << 3) | (__ffs(cm) - 1));
-            const uint32_t ms = (U & 1) ? kb_colmix(a.hp, 0, v3[0]) : 0u;
-            const uint32_t mp = (U & 2) ? kb_colmix(a.hp, 1, v3[1]) : 0u;
-            const uint32_t mo = (U & 4) ? kb_colmix(a.hp, 2, v3[2]) : 0u;
-            __syncwarp();
-            for (unsigned r0 = 0; r0 < tot; r0 += 32) {
-                const unsigned e = r0 + lane;
-                const unsigned qe = e < tot ? queue[e] : 0u;
-                const int src = (int)(qe >> 3), m = (int)(qe & 7u);
-                const int32_t ts = (U & 1) ? __shfl_sync(0xffffffffu, vs[u], src) : 0;
-                const int32_t tp = (U & 2) ? __shfl_sync(0xffffffffu, vp[u], src) : 0;
-                const int32_t to = (U & 4) ? __shfl_sync(0xffffffffu, vo[u], src) : 0;
-                const uint32_t hs = (U & 1) ? __shfl_sync(0xffffffffu, ms, src) : 0u;
-                const uint32_t hq = (U & 2) ? __shfl_sync(0xffffffffu, mp, src) : 0u;
-                const uint32_t ho = (U & 4) ? __shfl_sync(0xffffffffu, mo, src) : 0u;
-                int k = -1;
-                if (m != 0) {
-                    uint32_t h = s_msk[m];
-                    if (m & 1) h ^= hs;
-                    if (m & 2) h ^= kb_rotl(hq, 11);
-                    if (m & 4) h ^= kb_rotl(ho, 22);
-                    const uint32_t d = s_disp[kb_bucket(h, a.nb)];
-                    const Entry en = s_tab[kb_slot(a.hp, h, d, a.ns)];
-                    const bool hit = (en.mask_kid >> 28) == m && (!(m & 1) || en.s == ts) &&
-                                     (!(m & 2) || en.p == tp) && (!(m & 4) || en.o == to);
-                    k = hit ? (en.mask_kid & 0x0FFFFFFF) : -1;
-                }
-                if (!__any_sync(0xffffffffu, k >= 0)) continue;
-                const unsigned peers = __match_any_sync(0xffffffffu, k);
-                if (k >= 0) {
-                    const uint32_t cc = cnt[k];
-                    if (WRITE) {
-                        const uint32_t r = cc + __popc(peers & lt);
-                        a.arena[a.abs32 ? (int64_t)r : a.off[k] + r] = (int32_t)(b0 + u * 32 + src);
-                    }
-                    __syncwarp(peers);
-                    if (lane == (unsigned)(__ffs(peers) - 1)) cnt[k] = cc + __popc(peers);
-                }
+        for (int u = 0; u < UNROLL; ++u) {
+            for (uint32_t any = __reduce_or_sync(0xffffffffu, cand[u]); any; any &= any - 1) {
+                const int m = __ffs(any) - 1;
+                const bool mine = (cand[u] >> m) & 1u;
+                const unsigned b = __ballot_sync(0xffffffffu, mine);
+                if (mine)
+                    queue[(tail + __popc(b & lt)) & (KB_RING - 1)] =
+                        make_int4((int)(((uint32_t)(b0 - lo) + u * 32 + lane) << 3 | (uint32_t)m), vs[u], vp[u], vo[u]);
+                tail += __popc(b);
                 __syncwarp();
+                if (tail - head >= 32) {
+                    look_up(32);
+                    head += 32;
+                }
             }
-            __syncwarp();  // the next slot rewrites the queue
         }
     }
+    if (tail != head) look_up(tail - head);
     __syncwarp();
     if (!WRITE)
         for (int k = lane; k < a.kids; k += 32) row[k] = cnt[k];
 }
 
 // counts[w][k] -> exclusive prefix over w for each k; rows[k] = total of k.
-// Block: 32 key ids (lanes) x 8 ranges of warps (the block's warps).
-__global__ void __launch_bounds__(256) k_batch_scan(uint32_t *counts, int64_t GW, int kids, int64_t *rows) {
-    __shared__ uint32_t s_sum[8][32];
+// Block: 32 key ids (lanes) x KS_PARTS ranges of warps (the block's warps: the sums
+// of a key's thousands of counts are many short chains, 512 keys 239 -> 32 us
+// against eight ranges).
+constexpr int KS_PARTS = 32;
+__global__ void __launch_bounds__(32 * KS_PARTS) k_batch_scan(uint32_t *counts, int64_t GW, int kids, int64_t *rows) {
+    __shared__ uint32_t s_sum[KS_PARTS][32];
     const unsigned lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int k = blockIdx.x * 32 + lane;
-    const int64_t per = (GW + 7) / 8;
+    const int64_t per = (GW + KS_PARTS - 1) / KS_PARTS;
     const int64_t b = min((int64_t)w * per, GW), e = min(b + per, GW);
     uint32_t sum = 0;
-    if (k < kids)
+    if (k < kids) {
+#pragma unroll 16
         for (int64_t g = b; g < e; ++g) sum += counts[g * kids + k];
+    }
     s_sum[w][lane] = sum;
     __syncthreads();
     uint32_t run = 0;
     for (unsigned v = 0; v < w; ++v) run += s_sum[v][lane];
     if (k < kids) {
-        for (int64_t g = b; g < e; ++g) {
-            const uint32_t c = counts[g * kids + k];
-            counts[g * kids + k] = run;
-            run += c;
+        constexpr int Q = 8;  // counts read ahead of the writes
+        for (int64_t g = b; g < e; g += Q) {
+            uint32_t c[Q];
+#pragma unroll
+            for (int q = 0; q < Q; ++q) c[q] = g + q < e ? counts[(g + q) * kids + k] : 0u;
+#pragma unroll
+            for (int q = 0; q < Q; ++q) {
+                if (g + q >= e) break;
+                counts[(g + q) * kids + k] = run;
+                run += c[q];
+            }
         }
-        if (w == 7) rows[k] = run;
+        if (w == KS_PARTS - 1) rows[k] = run;
     }
 }
 
@@ -848,7 +866,7 @@ int run_batch(tid_ctx *ctx, const tid_store *st, const std::vector<SubPlan> &pla
         if ((rc = upload_plan(ctx, s, sp, x.GW, &x.up)) != TID_OK) return give_up(rc);
         x.a = batch_args(st, sp, x.up, slice_of(st->n, x.GW, shape));
         if ((rc = pass_of(sp.U, shape, stream, false, x.grid, x.smem, x.a)) != TID_OK) return give_up(rc);
-        k_batch_scan<<<(unsigned)ceil_div(kids, 32), 256, 0, stream>>>(x.up.counts, x.GW, kids,
+        k_batch_scan<<<(unsigned)ceil_div(kids, 32), 32 * KS_PARTS, 0, stream>>>(x.up.counts, x.GW, kids,
                                                                        (int64_t *)x.sb->ptr[0]);
         if ((rc = launch_check("k_batch_scan")) != TID_OK) return give_up(rc);
         x.tot.resize(kids);
