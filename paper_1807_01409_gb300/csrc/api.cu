@@ -347,12 +347,22 @@ int set_ready(tid_set *set) {
     return TID_OK;
 }
 
+cudaError_t reset_bounds(tid_ctx *ctx) {
+    // 16 words of bounds, then the finished-CTA counter
+    const size_t least = TID_MAX_COLS * sizeof(uint32_t);
+    cudaError_t e = cudaMemsetAsync(ctx->bounds_dev, 0xFF, least, ctx->stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(ctx->bounds_dev + TID_MAX_COLS, 0, 256 - least, ctx->stream);
+    return e;
+}
+
 int check_ctx_error(tid_ctx *ctx) {
     int e = *(volatile int *)ctx->err_host;
     if (e != 0) {
         *(volatile int *)ctx->err_host = 0;
-        // a launch that gave up may leave the ticket counter off zero
+        // a launch that gave up may leave the ticket counter off zero, and the
+        // bounds with some of its CTAs' values
         if (ctx->lb_ticket) cudaMemsetAsync(ctx->lb_ticket, 0, sizeof(unsigned int), ctx->stream);
+        if (ctx->bounds_dev) reset_bounds(ctx);
         if (e == TID_ERR_TIMEOUT) return fail(TID_ERR_TIMEOUT, "an in-kernel wait gave up");
         return fail(e, "kernel reported error %d", e);
     }
@@ -419,6 +429,8 @@ extern "C" int tid_ctx_create(int device, void *cuda_stream, tid_ctx **out) {
         void *d = nullptr;
         e = cudaHostGetDevicePointer(&d, h, 0);
         c->err_dev = (int *)d;
+        c->bounds_host = (uint32_t *)h + 16;  // a line of its own behind the error word
+        c->bounds_map = (uint32_t *)d + 16;
     }
     if (e != cudaSuccess) {
         int rc = fail_cuda(e, "tid_ctx_create");
@@ -452,6 +464,7 @@ extern "C" int tid_ctx_destroy(tid_ctx *ctx) {
     }
     if (ctx->lb_status) dev_free(ctx, ctx->lb_status);
     if (ctx->sel_done) dev_free(ctx, ctx->sel_done);
+    if (ctx->bounds_dev) dev_free(ctx, ctx->bounds_dev);
     drop_blocks(ctx);
     for (cudaEvent_t ev : ctx->free_events) cudaEventDestroy(ev);
     cudaStreamSynchronize(ctx->stream);

@@ -302,28 +302,38 @@ struct PackedUniqueRow {  // sorted packed keys; keep the first of each run of e
     }
 };
 
-// bounds (sort order) of the values a thread wrote, merged per warp into mm
+// bounds (sort order) of the values a thread wrote, merged per warp into mm.acc;
+// the last CTA moves the result to the host (all threads of every CTA call this)
 template <int K>
-__device__ __forceinline__ void merge_bounds(uint32_t *mm, int k_out, const uint32_t *lo, const uint32_t *hi) {
+__device__ __forceinline__ void merge_bounds(const BoundsOut &mm, int k_out, const uint32_t *lo, const uint32_t *hi) {
     const unsigned lane = threadIdx.x & 31;
 #pragma unroll
     for (int c = 0; c < K; ++c) {
         if (c < k_out) {
-            uint32_t a = lo[c], b = hi[c];
-#pragma unroll
-            for (int d = 16; d > 0; d >>= 1) {
-                a = min(a, __shfl_xor_sync(0xffffffffu, a, d));
-                b = max(b, __shfl_xor_sync(0xffffffffu, b, d));
-            }
+            const uint32_t a = __reduce_min_sync(0xffffffffu, lo[c]), b = __reduce_max_sync(0xffffffffu, hi[c]);
             // the bounds only tighten, so a warp that cannot improve the
             // current one (read from L2; a stale read only costs an atomic)
             // skips its atomic: many warps otherwise queue on one address
             if (lane == 0 && a <= b) {
-                if (a < __ldcg(mm + c)) atomicMin(mm + c, a);
-                if (b > __ldcg(mm + TID_MAX_COLS + c)) atomicMax(mm + TID_MAX_COLS + c, b);
+                if (a < __ldcg(mm.acc + c)) atomicMin(mm.acc + c, a);
+                if (b > __ldcg(mm.acc + TID_MAX_COLS + c)) atomicMax(mm.acc + TID_MAX_COLS + c, b);
             }
         }
     }
+    __shared__ unsigned s_end;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        s_end = atomicAdd(mm.done, 1u) == gridDim.x - 1;
+        __threadfence();
+    }
+    __syncthreads();
+    if (!s_end) return;
+    if (threadIdx.x < 2 * TID_MAX_COLS) {
+        mm.host[threadIdx.x] = __ldcg(mm.acc + threadIdx.x);
+        mm.acc[threadIdx.x] = threadIdx.x < TID_MAX_COLS ? 0xFFFFFFFFu : 0u;
+    }
+    if (threadIdx.x == 0) *mm.done = 0;
 }
 
 // ---- single-pass compaction (small inputs) ----------------------------------------
@@ -335,7 +345,7 @@ __device__ __forceinline__ void merge_bounds(uint32_t *mm, int k_out, const uint
 template <class Row>
 __global__ void __launch_bounds__(CP_THREADS)
 k_compact(Row row, int64_t n, int k_out, OutCols out, int64_t cap, int64_t *__restrict__ d_rows,
-          int64_t *__restrict__ h_rows, Lookback lb, uint32_t *__restrict__ mm) {
+          int64_t *__restrict__ h_rows, Lookback lb, BoundsOut mm) {
     extern __shared__ int32_t s_vals[];  // column c of staged row i at s_vals[c * CP_TILE + i]
     __shared__ unsigned s_tile, s_total;
     __shared__ unsigned s_off[CP_ITEMS * CP_WARPS];
@@ -423,7 +433,7 @@ k_compact(Row row, int64_t n, int k_out, OutCols out, int64_t cap, int64_t *__re
             }
         }
     }
-    if (mm) merge_bounds<TID_MAX_COLS>(mm, k_out, lo, hi);  // column bounds of the kept rows
+    if (mm.acc) merge_bounds<TID_MAX_COLS>(mm, k_out, lo, hi);  // column bounds of the kept rows
 }
 
 // ---- mark and expand (long inputs) -------------------------------------------------
@@ -444,7 +454,10 @@ k_compact(Row row, int64_t n, int k_out, OutCols out, int64_t cap, int64_t *__re
 // filter against 32 us; one large range per resident CTA with block scans took
 // 97 us to expand against 83 us.
 
-constexpr int64_t SEL_MIN_ROWS = (int64_t)1 << 18;  // below this, the single-pass kernel
+// Below this, the single-pass kernel: its tiles of 2048 rows test eight rows per
+// thread one after another, so it pays while the input is a few tiles (binding
+// 20K to 250K matched triples with a test: 22 us in one launch, @@ us in two).
+constexpr int64_t SEL_MIN_ROWS = (int64_t)1 << 13;
 
 template <class Row>
 __global__ void __launch_bounds__(SEL_THREADS)
@@ -481,7 +494,7 @@ k_sel_mark(Row row, uint32_t n, SelScratch sc, int64_t *__restrict__ d_rows, int
 
 template <class Row, int K, bool BOUNDS>
 __global__ void __launch_bounds__(SEL_THREADS, K == 2 ? 5 : (K <= 3 ? 4 : 2))
-k_sel_expand(Row row, int k_out, OutCols out, int64_t cap, SelScratch sc, uint32_t *__restrict__ mm) {
+k_sel_expand(Row row, int k_out, OutCols out, int64_t cap, SelScratch sc, BoundsOut mm) {
     __shared__ uint16_t s_stage[SEL_WARPS][SEL_DENSE];
     const unsigned lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const unsigned lt = (1u << lane) - 1u;
@@ -548,15 +561,15 @@ k_sel_expand(Row row, int k_out, OutCols out, int64_t cap, SelScratch sc, uint32
 
 template <class Row, int K>
 int expand_k(tid_ctx *ctx, const Row &row, int k_out, const OutCols &out, int64_t cap, const SelScratch &sc,
-             uint32_t *mm) {
-    if (mm) k_sel_expand<Row, K, true><<<sc.ranges, SEL_THREADS, 0, ctx->stream>>>(row, k_out, out, cap, sc, mm);
+             const BoundsOut &mm) {
+    if (mm.acc) k_sel_expand<Row, K, true><<<sc.ranges, SEL_THREADS, 0, ctx->stream>>>(row, k_out, out, cap, sc, mm);
     else k_sel_expand<Row, K, false><<<sc.ranges, SEL_THREADS, 0, ctx->stream>>>(row, k_out, out, cap, sc, mm);
     return launch_check("k_sel_expand");
 }
 
 template <class Row>
 int launch_compact(tid_ctx *ctx, Row row, int64_t n, int k_out, const OutCols &out, int64_t cap,
-                   int64_t *d_rows, int64_t *h_rows_dev, uint32_t *mm = nullptr) {
+                   int64_t *d_rows, int64_t *h_rows_dev, const BoundsOut &mm = BoundsOut{}) {
     if (n == 0) {
         TID_TRY_CUDA(cudaMemsetAsync(d_rows, 0, sizeof(int64_t), ctx->stream), "memset rows");
         TID_TRY_CUDA(cudaMemsetAsync(h_rows_dev, 0, sizeof(int64_t), ctx->stream), "memset rows");
@@ -602,7 +615,7 @@ int launch_compact(tid_ctx *ctx, Row row, int64_t n, int k_out, const OutCols &o
 // Bind with nothing to test (no repeated variable, no predicate): every row is
 // kept in index order, so row r is written at r -- a plain gather, no
 // compaction -- with the column bounds of the output.
-__global__ void __launch_bounds__(256) k_bind_gather(BindRow row, int64_t n, OutCols out, uint32_t *__restrict__ mm,
+__global__ void __launch_bounds__(256) k_bind_gather(BindRow row, int64_t n, OutCols out, BoundsOut mm,
                                                      int64_t *__restrict__ d_rows, int64_t *__restrict__ h_rows) {
     constexpr int K = 3, U = 4;  // a pattern has at most three variables; rows per thread in flight
     uint32_t lo[K], hi[K];
@@ -631,7 +644,7 @@ __global__ void __launch_bounds__(256) k_bind_gather(BindRow row, int64_t n, Out
             }
         }
     }
-    if (mm) merge_bounds<K>(mm, row.k, lo, hi);
+    if (mm.acc) merge_bounds<K>(mm, row.k, lo, hi);
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         *d_rows = n;
         *h_rows = n;
@@ -754,6 +767,24 @@ __global__ void __launch_bounds__(SC_THREADS) k_tile_sums(const uint32_t *__rest
 
 }  // namespace
 
+int bounds_out(tid_ctx *ctx, BoundsOut *b) {
+    if (!ctx->bounds_dev) {
+        void *p = nullptr;
+        TID_TRY(dev_alloc(ctx, &p, 256));
+        ctx->bounds_dev = (uint32_t *)p;
+        cudaError_t e = reset_bounds(ctx);
+        if (e != cudaSuccess) {
+            ctx->bounds_dev = nullptr;
+            dev_free(ctx, p);
+            return fail_cuda(e, "bounds");
+        }
+    }
+    b->acc = ctx->bounds_dev;
+    b->done = ctx->bounds_dev + 2 * TID_MAX_COLS;
+    b->host = ctx->bounds_map;
+    return TID_OK;
+}
+
 int sel_scratch(tid_ctx *ctx, int64_t n, int lists, size_t extra, SelScratch *sc, void **block, void **extra_at,
                 unsigned per) {
     sc->steps = (unsigned)ceil_div(n, (int64_t)SEL_STEP);
@@ -816,7 +847,7 @@ int scan_exclusive_u32(tid_ctx *ctx, const uint32_t *in, uint32_t *out, int64_t 
 }
 
 int compact_bind(tid_ctx *ctx, const tid_store *st, const tid_pattern &pat, const int32_t *idx, int64_t n,
-                 const Pred *preds, int n_preds, const BindMember *mem, int n_mem, tid_set *out, uint32_t *mm) {
+                 const Pred *preds, int n_preds, const BindMember *mem, int n_mem, tid_set *out, const BoundsOut &mm) {
     BindRow r{};
     r.S = st->s;
     r.P = st->p;
@@ -864,7 +895,7 @@ int compact_bind(tid_ctx *ctx, const tid_store *st, const tid_pattern &pat, cons
 }
 
 int expand_keyed(tid_ctx *ctx, const KeyedScan &ks, const SelScratch &sc, const int8_t *src, const int32_t *map,
-                 tid_set *out, uint32_t *mm) {
+                 tid_set *out, const BoundsOut &mm) {
     KeyedRow r{};
     r.S = ks.col[0];
     r.P = ks.col[1];

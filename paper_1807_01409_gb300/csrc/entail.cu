@@ -859,13 +859,14 @@ extern "C" int tid_entail(tid_ctx *ctx, const tid_store *st, int rule, const tid
             std::vector<int32_t> map(kt.numbers, 0);
             for (const auto &r : sr.rows) map[r.first] = r.second;
             Buf mapb{ctx};
-            const size_t mm_b = 2 * TID_MAX_COLS * sizeof(uint32_t);
-            TID_TRY(dev_alloc(ctx, &mapb.p, mm_b + map.size() * 4));
-            uint32_t *mm = (uint32_t *)mapb.p, hb[2 * TID_MAX_COLS];
-            int32_t *d_map = (int32_t *)(mm + 2 * TID_MAX_COLS);
+            TID_TRY(dev_alloc(ctx, &mapb.p, map.size() * 4));
+            int32_t *d_map = (int32_t *)mapb.p;
             TID_TRY_CUDA(cudaMemcpyAsync(d_map, map.data(), map.size() * 4, cudaMemcpyHostToDevice, stream), "key map");
+            BoundsOut mm{};
+            if (!pair) TID_TRY(bounds_out(ctx, &mm));
+            TID_TRY(expand_keyed(ctx, ks, sc, src, d_map, J, mm));
+            TID_TRY_CUDA(cudaStreamSynchronize(stream), "conclusion range");  // (and the host copy of the map)
             if (pair) {  // the data term's range is known; A's terms are on the host
-                TID_TRY(expand_keyed(ctx, ks, sc, src, d_map, J, nullptr));
                 cb.lo[1 - a_pos] = ss.lo;
                 cb.hi[1 - a_pos] = ss.hi;
                 cb.lo[a_pos] = 0xFFFFFFFFu;
@@ -873,16 +874,10 @@ extern "C" int tid_entail(tid_ctx *ctx, const tid_store *st, int rule, const tid
                     cb.lo[a_pos] = std::min(cb.lo[a_pos], sort_order_host(r.second));
                     cb.hi[a_pos] = std::max(cb.hi[a_pos], sort_order_host(r.second));
                 }
-                TID_TRY_CUDA(cudaStreamSynchronize(stream), "key map");  // the host copy of the map
             } else {
-                TID_TRY_CUDA(cudaMemsetAsync(mm, 0xFF, mm_b / 2, stream), "conclusion range");
-                TID_TRY_CUDA(cudaMemsetAsync(mm + TID_MAX_COLS, 0, mm_b / 2, stream), "conclusion range");
-                TID_TRY(expand_keyed(ctx, ks, sc, src, d_map, J, mm));
-                TID_TRY_CUDA(cudaMemcpyAsync(hb, mm, sizeof hb, cudaMemcpyDeviceToHost, stream), "conclusion range");
-                TID_TRY_CUDA(cudaStreamSynchronize(stream), "conclusion range");
                 for (int i = 0; i < kc; ++i) {
-                    cb.lo[i] = hb[i];
-                    cb.hi[i] = hb[TID_MAX_COLS + i];
+                    cb.lo[i] = ((volatile uint32_t *)ctx->bounds_host)[i];
+                    cb.hi[i] = ((volatile uint32_t *)ctx->bounds_host)[TID_MAX_COLS + i];
                 }
             }
             for (int i = 0; i < kc; ++i) ccols[i] = J->col[i];
@@ -900,7 +895,7 @@ extern "C" int tid_entail(tid_ctx *ctx, const tid_store *st, int rule, const tid
             tid_set *B = nullptr;
             TID_TRY(set_alloc(ctx, nb, bvars, sx.res2, &B));
             hold.keep(B);
-            TID_TRY(expand_keyed(ctx, ks, sc, bsrc, nullptr, B, nullptr));
+            TID_TRY(expand_keyed(ctx, ks, sc, bsrc, nullptr, B, BoundsOut{}));
             TID_TRY(set_rows_const(B, sx.res2));
             TID_TRY(set_ready(B));
             TID_TRY(join_sets(ctx, A, B, TID_JOIN_HASH, &J, false));

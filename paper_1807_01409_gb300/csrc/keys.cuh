@@ -2,6 +2,7 @@
 // search asks of every triple whether its term is one of them, and which.
 #pragma once
 
+#include "ops.cuh"
 #include "select.cuh"
 
 namespace tid {
@@ -53,8 +54,8 @@ struct KeyedScan {
 };
 
 // The kept rows of a marked scan, in order, into out's columns: column c is slot
-// src[c], or (src[c] == 3) map[number of the row's key].  mm as in compact_bind.
+// src[c], or (src[c] == 3) map[number of the row's key].
 int expand_keyed(tid_ctx *ctx, const KeyedScan &ks, const SelScratch &sc, const int8_t *src, const int32_t *map,
-                 tid_set *out, uint32_t *mm);
+                 tid_set *out, const BoundsOut &mm);
 
 }  // namespace tid

@@ -107,22 +107,14 @@ int bind_set(tid_ctx *ctx, const tid_store *st, const tid_pattern &pat, const ti
     if (n == 0) return empty_set(ctx, k, vars, out);
     tid_set *tmp = nullptr;
     TID_TRY(set_alloc(ctx, k, vars, n, &tmp));
-    uint32_t *mm = nullptr;  // column bounds of the extracted rows, for the sort
-    int rc = dev_alloc(ctx, (void **)&mm, 2 * TID_MAX_COLS * sizeof(uint32_t));
-    if (rc == TID_OK) {
-        cudaError_t e = cudaMemsetAsync(mm, 0xFF, TID_MAX_COLS * sizeof(uint32_t), ctx->stream);
-        if (e == cudaSuccess) e = cudaMemsetAsync(mm + TID_MAX_COLS, 0, TID_MAX_COLS * sizeof(uint32_t), ctx->stream);
-        if (e != cudaSuccess) rc = fail_cuda(e, "tid_bind");
-    }
+    BoundsOut mm{};  // column bounds of the extracted rows, for the sort
+    int rc = bounds_out(ctx, &mm);
     if (rc == TID_OK) rc = compact_bind(ctx, st, pat, idx->col[0], n, pr, n_preds, bm, n_mem, tmp, mm);
-    uint32_t hb[2 * TID_MAX_COLS];
-    if (rc == TID_OK) {
-        cudaError_t e = cudaMemcpyAsync(hb, mm, sizeof hb, cudaMemcpyDeviceToHost, ctx->stream);
-        if (e != cudaSuccess) rc = fail_cuda(e, "tid_bind bounds");
-    }
     if (rc == TID_OK) rc = set_ready(tmp);
     int64_t m = 0;
-    if (rc == TID_OK) rc = set_rows_host(tmp, &m);
+    if (rc == TID_OK) rc = set_rows_host(tmp, &m);  // waits: the bounds are on the host too
+    uint32_t hb[2 * TID_MAX_COLS];
+    for (int c = 0; c < 2 * TID_MAX_COLS; ++c) hb[c] = ((volatile uint32_t *)ctx->bounds_host)[c];
     const int32_t *cols[TID_MAX_COLS];
     Bounds b{};
     for (int c = 0; c < k; ++c) {
@@ -151,7 +143,6 @@ int bind_set(tid_ctx *ctx, const tid_store *st, const tid_pattern &pat, const ti
             tmp->lo[c] = b.lo[c];
             tmp->hi[c] = b.hi[c];
         }
-        if (mm) dev_free(ctx, mm);
         *out = tmp;
         return TID_OK;
     }
@@ -175,7 +166,6 @@ int bind_set(tid_ctx *ctx, const tid_store *st, const tid_pattern &pat, const ti
         // distinct triples give distinct rows unless a "?" slot is anonymous
         rc = canonicalize(ctx, cols, k, vars, m, anon, &b, out);
     }
-    if (mm) dev_free(ctx, mm);
     set_free(tmp);
     return rc;
 }

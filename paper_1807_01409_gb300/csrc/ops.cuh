@@ -55,6 +55,21 @@ struct Bounds {
     uint32_t lo[TID_MAX_COLS], hi[TID_MAX_COLS];
 };
 
+// Where a kernel that writes a set's rows leaves their columns' bounds (sort order):
+// word c the least, word 8 + c the largest value of column c.  Every CTA merges its
+// rows' into `acc` (least values start at ~0, largest at 0); the last one of the grid
+// moves acc to `host` (mapped memory) and makes it neutral again, so an extraction
+// needs no launch to preset its bounds and no copy to read them: they are on the host
+// with its row count.
+struct BoundsOut {
+    uint32_t *acc = nullptr;  // null: not wanted
+    unsigned *done = nullptr;
+    uint32_t *host = nullptr;
+};
+// the context's one; read by the caller, once the kernel's set is ready, from
+// ctx->bounds_host before the next extraction
+int bounds_out(tid_ctx *ctx, BoundsOut *b);
+
 struct VarMember {  // the same by variable
     Members m;
     int8_t var;
@@ -65,10 +80,9 @@ int scan_exclusive_u32(tid_ctx *ctx, const uint32_t *in, uint32_t *out, int64_t 
                        unsigned long long *total_dev);
 
 // row selections (compact.cu); `out` must have capacity >= n
-// bind; if mm is not null, mm[c] / mm[8 + c] receive (atomic min / max) the
-// sort-order bounds of output column c over the kept rows (caller presets them)
+// bind, with the bounds of the kept rows
 int compact_bind(tid_ctx *ctx, const tid_store *st, const tid_pattern &pat, const int32_t *idx, int64_t n,
-                 const Pred *preds, int n_preds, const BindMember *mem, int n_mem, tid_set *out, uint32_t *mm);
+                 const Pred *preds, int n_preds, const BindMember *mem, int n_mem, tid_set *out, const BoundsOut &mm);
 // the terms of col[0, n) in [lo, hi] (sort order, hi - lo < 2^32 - 1) as a bitmap,
 // allocated here (m->bits, freed by the caller)
 int member_bits(tid_ctx *ctx, const int32_t *col, int64_t n, uint32_t lo, uint32_t hi, Members *m);

@@ -123,6 +123,9 @@ struct tid_ctx {
     unsigned int *lb_ticket = nullptr;
     unsigned int epoch = 0;
     unsigned int *sel_done = nullptr;  // finished CTAs of a row selection (select.cuh), 0 between launches
+    // column bounds of an extraction: a kernel's CTAs merge theirs in bounds_dev (16
+    // words, neutral between launches), its last CTA moves them to mapped host memory
+    uint32_t *bounds_dev = nullptr, *bounds_host = nullptr, *bounds_map = nullptr;
     // error word in mapped pinned memory (written by kernels, read by host)
     int *err_host = nullptr;
     int *err_dev = nullptr;
@@ -202,6 +205,7 @@ void set_free(tid_set *set);      // tid_set_free without clearing the error mes
 // A one-column set labelled -1 viewing `col` (rows known on the host, count in
 // *d_rows on the device) inside sb's allocations; takes one reference on sb.
 int set_view(tid_ctx *ctx, tid::SharedBlock *sb, int32_t *col, int64_t *d_rows, int64_t rows, tid_set **out);
+cudaError_t reset_bounds(tid_ctx *ctx);  // bounds_dev to neutral values
 int check_ctx_error(tid_ctx *ctx); // reads and clears the kernel error word
 bool store_spo_sorted(const tid_store *st);  // triples in (s, p, o) order (waits for the load's check)
 int launch_check(const char *what);

@@ -34,8 +34,8 @@ def _set(ctx, s):
     return tb.tid_set_from_host(ctx, s.rows, s.vars)
 
 
-# k_sel_mark / k_sel_expand from 2^18 rows up (steps of 1024, ranges of 8 or 32 steps), k_compact below
-SELECT_ROWS = [1, 2047, 2**18 - 1, 2**18, 2**18 + 1, 2**18 + 8 * 1024 + 1023, 1_300_003]
+# k_sel_mark / k_sel_expand from 2^13 rows up (steps of 1024, ranges of 8 or 32 steps), k_compact below
+SELECT_ROWS = [1, 2047, 2**13 - 1, 2**13, 2**13 + 1, 20_001, 2**18 - 1, 2**18, 2**18 + 1, 2**18 + 8 * 1024 + 1023, 1_300_003]
 PREDS = [("lt", 500, 0), ("ge", 999, 0), ("ne", 7, 0), ("eq", 7, 0), ("lt", LOWEST, 0), ("gt", HIGHEST, 0),
          ("le", HIGHEST, 0), ("ge", LOWEST, 0), ("range", 10, 9), ("range", 990, HIGHEST)]
 
@@ -62,7 +62,7 @@ def test_filter_edges(ctx, orc, n, k):
     tb.tid_set_free(h)
 
 
-@pytest.mark.parametrize("n", [2**18 - 1, 2**18 + 5, 700_001])
+@pytest.mark.parametrize("n", [5000, 40_000, 2**18 - 1, 2**18 + 5, 700_001])
 @pytest.mark.parametrize("shift", [0, 1])
 def test_bind_tests_edges(ctx, orc, n, shift):
     """One tested slot (its values stashed), two tested slots, a repeated variable; borrowed columns
