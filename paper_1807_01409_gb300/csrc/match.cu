@@ -331,7 +331,7 @@ k1_mark(const int32_t *__restrict__ S, const int32_t *__restrict__ P, const int3
 }
 
 __global__ void __launch_bounds__(SEL_THREADS) k1_expand(SelScratch sc, int32_t *__restrict__ out, int64_t cap) {
-    if (sc.tot[blockIdx.x]) sel_expand_index(sc, blockIdx.x, out, cap);
+    sel_expand_index(sc, out, cap);
 }
 
 template <int MASK, bool VEC>
@@ -343,7 +343,7 @@ int run_scan(tid_ctx *ctx, const int32_t *S, const int32_t *P, const int32_t *O,
     k1_mark<MASK, VEC><<<sc.ranges, SEL_THREADS, 0, ctx->stream>>>(S, P, O, n, ks, kp, ko, sc, d_rows, h_rows);
     int rc = launch_check("k1_mark");
     if (rc == TID_OK) {
-        k1_expand<<<sc.ranges, SEL_THREADS, 0, ctx->stream>>>(sc, out, cap);
+        k1_expand<<<sel_index_grid(sc), SEL_THREADS, 0, ctx->stream>>>(sc, out, cap);
         rc = launch_check("k1_expand");
     }
     dev_free(ctx, blk);

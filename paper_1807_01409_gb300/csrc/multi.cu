@@ -11,7 +11,7 @@
 // Bytes per launch: 4 * |union of bound columns| * n read + 4 * sum of hits written
 // (+ n/8 per pattern of bitmap written and read, mostly in L2).  Measured on GB300,
 // three patterns over two columns of 200M triples, 32.3M hits: k2_mark 251 us
-// (6.4 TB/s), k_scan_ranges 12 us, k2_expand 102 us; before, chunks in shared memory
+// (6.4 TB/s), k_scan_ranges 12 us, k2_expand 95 us; before, chunks in shared memory
 // with one look-back chain per pattern took 483 us, and 88 us at 1M triples, where
 // they gave four CTAs work.
 
@@ -117,7 +117,7 @@ __global__ void __launch_bounds__(SEL_THREADS) k_scan_ranges(const __grid_consta
 
 __global__ void __launch_bounds__(SEL_THREADS) k2_expand(const __grid_constant__ MultiArgs args, SelScratch all) {
     const SelScratch sc = list_of(all, blockIdx.y);
-    if (sc.tot[blockIdx.x]) sel_expand_index(sc, blockIdx.x, args.out[blockIdx.y], args.cap[blockIdx.y]);
+    sel_expand_index(sc, args.out[blockIdx.y], args.cap[blockIdx.y]);
 }
 
 template <int U>
@@ -135,7 +135,7 @@ int launch_vec(bool vec, tid_ctx *ctx, const int32_t *S, const int32_t *P, const
         rc = launch_check("k_scan_ranges");
     }
     if (rc == TID_OK) {
-        k2_expand<<<dim3(sc.ranges, a.m), SEL_THREADS, 0, st>>>(a, sc);
+        k2_expand<<<dim3(sel_index_grid(sc), a.m), SEL_THREADS, 0, st>>>(a, sc);
         rc = launch_check("k2_expand");
     }
     dev_free(ctx, blk);

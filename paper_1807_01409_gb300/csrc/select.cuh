@@ -125,7 +125,9 @@ __device__ __forceinline__ void sel_walk(const SelScratch &sc, unsigned range, u
     for (unsigned q0 = r0; q0 < r1; q0 += 32) {
         const unsigned here = min(32u, r1 - q0);
         const unsigned cnt = lane < here ? sc.cnt[q0 + lane] : 0u;
-        uint32_t next = warp < here ? sc.bits[(size_t)(q0 + warp) * 32 + lane] : 0u;
+        // this warp's steps that have kept rows, and the first one's words
+        unsigned todo = __ballot_sync(0xffffffffu, cnt != 0 && lane % warps == warp);
+        uint32_t next = todo ? sc.bits[(size_t)(q0 + __ffs(todo) - 1) * 32 + lane] : 0u;
         unsigned first = cnt;
 #pragma unroll
         for (int d = 1; d < 32; d <<= 1) {
@@ -134,11 +136,12 @@ __device__ __forceinline__ void sel_walk(const SelScratch &sc, unsigned range, u
         }
         const unsigned kept = __shfl_sync(0xffffffffu, first, 31);
         first -= cnt;  // of step q0 + lane
-        for (unsigned li = warp; li < here; li += warps) {
+        while (todo) {
+            const unsigned li = __ffs(todo) - 1;
+            todo &= todo - 1;
             const uint32_t word = next;
-            if (li + warps < here) next = sc.bits[(size_t)(q0 + li + warps) * 32 + lane];
+            if (todo) next = sc.bits[(size_t)(q0 + __ffs(todo) - 1) * 32 + lane];
             const unsigned sn = __shfl_sync(0xffffffffu, cnt, li);
-            if (sn == 0) continue;
             const unsigned long long o0 = run + __shfl_sync(0xffffffffu, first, li);
             const unsigned pc = __popc(word);
             unsigned xo = pc;
@@ -166,11 +169,19 @@ __device__ __forceinline__ void sel_stage(uint32_t word, unsigned at, uint16_t *
 
 // ---- expand of a search: the kept rows' numbers -------------------------------
 
-__device__ __forceinline__ void sel_expand_index(const SelScratch &sc, unsigned range, int32_t *out, int64_t cap) {
+// A long range (32 steps) is two warps', so that the thousands of ranges of a large
+// store, most of them without a hit, are few CTAs (one warp left too few in flight
+// where hits are many: 23.6M of 200M triples 67 us, two 58).  A short one is a CTA's.
+constexpr unsigned SEL_RANGE_WARPS = 2;
+__device__ __forceinline__ void sel_expand_index(const SelScratch &sc, int32_t *out, int64_t cap) {
     __shared__ uint16_t s_stage[SEL_WARPS][SEL_DENSE];
     const unsigned lane = threadIdx.x & 31, lt = (1u << lane) - 1u;
     uint16_t *stage = s_stage[threadIdx.x >> 5];
-    sel_walk(sc, range, threadIdx.x >> 5, SEL_WARPS, [&](unsigned step, uint32_t word, unsigned xo, unsigned sn, unsigned long long o0) {
+    const bool long_range = sc.per > SEL_WARPS;
+    const unsigned warp = threadIdx.x >> 5, warps = long_range ? SEL_RANGE_WARPS : SEL_WARPS;
+    const unsigned range = blockIdx.x * (SEL_WARPS / warps) + warp / warps;
+    if (range >= sc.ranges || sc.tot[range] == 0) return;
+    sel_walk(sc, range, warp % warps, warps, [&](unsigned step, uint32_t word, unsigned xo, unsigned sn, unsigned long long o0) {
         const int32_t base = (int32_t)(step * SEL_STEP);
         if (sn >= SEL_DENSE) {
 #pragma unroll 8
@@ -186,6 +197,11 @@ __device__ __forceinline__ void sel_expand_index(const SelScratch &sc, unsigned 
             __syncwarp();  // the stage is rewritten by the next step
         }
     });
+}
+
+inline unsigned sel_index_grid(const SelScratch &sc) {
+    constexpr unsigned in_cta = SEL_WARPS / SEL_RANGE_WARPS;
+    return sc.per > SEL_WARPS ? (sc.ranges + in_cta - 1) / in_cta : sc.ranges;
 }
 
 // ---- streaming loads of store columns ------------------------------------------
