@@ -61,14 +61,11 @@ __device__ __forceinline__ int cmp_pad(const PadCols &A, int64_t i, const PadCol
     return r;
 }
 
-// Warp t: split[t] for the boundary before tile t (t <= tiles).  A[mid] precedes
+// A rows among the first d merged rows (a warp's search): A[mid] precedes
 // B[d - 1 - mid] for every mid below the answer and for none from it on.
-__global__ void __launch_bounds__(256) k_merge_split(PadCols A, int64_t na, PadCols B, int64_t nb, int nu, int64_t tiles,
-                                                     int tile_rows, int64_t *__restrict__ split) {
-    const int64_t t = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
-    if (t > tiles) return;
+__device__ __forceinline__ int64_t warp_split(const PadCols &A, int64_t na, const PadCols &B, int64_t nb, int nu,
+                                              int64_t d) {
     const unsigned lane = threadIdx.x & 31;
-    const int64_t d = min(t * tile_rows, na + nb);
     int64_t lo = max((int64_t)0, d - nb), hi = min(d, na);
     while (lo < hi) {  // lane l tests the end of the l-th of 32 equal parts
         const int64_t part = (hi - lo + 31) / 32, mid = lo + (lane + 1) * part - 1;
@@ -77,14 +74,27 @@ __global__ void __launch_bounds__(256) k_merge_split(PadCols A, int64_t na, PadC
         lo += (int64_t)full * part;
         hi = min(hi, lo + part - 1);
     }
-    if (lane == 0) split[t] = min(lo, min(d, na));
+    return min(lo, min(d, na));
+}
+
+// Warp t: split[t] for the boundary before tile t (t <= tiles)
+__global__ void __launch_bounds__(256) k_merge_split(PadCols A, int64_t na, PadCols B, int64_t nb, int nu, int64_t tiles,
+                                                     int tile_rows, int64_t *__restrict__ split) {
+    const int64_t t = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
+    if (t > tiles) return;
+    const int64_t s = warp_split(A, na, B, nb, nu, min(t * tile_rows, na + nb));
+    if ((threadIdx.x & 31) == 0) split[t] = s;
 }
 
 typedef unsigned long long u64;
 
 constexpr int MP_THREADS = 256;
-constexpr int MP_ITEMS = 16;
-constexpr int MP_TILE = MP_THREADS * MP_ITEMS;  // merged rows per tile
+// Merged rows per thread: 16, or 4 where 16 would leave SMs without a tile (a tile's
+// time is then its chain of loads, search and merge steps).
+template <int ITEMS>
+constexpr int mp_tile() {
+    return MP_THREADS * ITEMS;
+}
 
 // One column's field of a packed row; zero: 0 is the field 0 and the values from
 // min + 1 (sort order) up follow it.
@@ -108,16 +118,28 @@ struct MergeBits {
     uint32_t *first_a;
 };
 
+template <int MP_ITEMS>
 __global__ void __launch_bounds__(MP_THREADS, 4)
 k_merge_mark(PadCols A, int64_t na, PadCols B, int64_t nb, int nu, MergePack mp, const int64_t *__restrict__ split,
              MergeBits mb, int64_t *__restrict__ d_rows, int64_t *__restrict__ h_rows) {
+    constexpr int MP_TILE = mp_tile<MP_ITEMS>();
+    constexpr int STEP_THREADS = SEL_STEP / MP_ITEMS;  // threads whose rows make a step
+    constexpr int WORD_THREADS = 32 / MP_ITEMS;        // and a word
     __shared__ u64 s_key[MP_TILE];
     __shared__ u64 s_before;  // the merged row before the tile
+    __shared__ int64_t s_split[2];
     __shared__ unsigned s_cnt[MP_THREADS / 32];
     const unsigned lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t tile = blockIdx.x;
     const int64_t d0 = tile * MP_TILE, d1 = min(d0 + MP_TILE, na + nb);
-    const int64_t a0 = split[tile], a1 = split[tile + 1], b0 = d0 - a0;
+    if (!split) {  // a few tiles: their own searches cost less than a launch for them
+        if (warp < 2) {
+            const int64_t s = warp_split(A, na, B, nb, nu, warp == 0 ? d0 : d1);
+            if (lane == 0) s_split[warp] = s;
+        }
+        __syncthreads();
+    }
+    const int64_t a0 = split ? split[tile] : s_split[0], a1 = split ? split[tile + 1] : s_split[1], b0 = d0 - a0;
     const int la = (int)(a1 - a0), len = (int)(d1 - d0);
     {  // pack the tile's rows, A's first
         u64 k[MP_ITEMS];
@@ -154,7 +176,7 @@ k_merge_mark(PadCols A, int64_t na, PadCols B, int64_t nb, int nu, MergePack mp,
         s_before = v;
     }
     __syncthreads();
-    // this thread's diagonal: local merged rows [dt, dt + 16)
+    // this thread's diagonal: local merged rows [dt, dt + MP_ITEMS)
     const int dt = min((int)threadIdx.x * MP_ITEMS, len), lb_ = len - la;
     int lo = max(0, dt - lb_), hi = min(dt, la);
     while (lo < hi) {
@@ -172,9 +194,8 @@ k_merge_mark(PadCols A, int64_t na, PadCols B, int64_t nb, int nu, MergePack mp,
         has_prev = d0 > 0;
         prev = has_prev ? s_before : 0;
     }
-    // step of this thread's rows: 64 threads each
-    const int64_t step = tile * (MP_TILE / SEL_STEP) + (threadIdx.x >> 6);
-    if ((threadIdx.x & 63) == 0 && step < mb.sc.steps) mb.first_a[step] = (uint32_t)(a0 + i);
+    const int64_t step = tile * (MP_TILE / SEL_STEP) + threadIdx.x / STEP_THREADS;
+    if (threadIdx.x % STEP_THREADS == 0 && step < mb.sc.steps) mb.first_a[step] = (uint32_t)(a0 + i);
     u64 ka = i < la ? s_key[i] : 0, kb = j < len ? s_key[j] : 0;
     unsigned keep = 0, take = 0;
 #pragma unroll
@@ -194,18 +215,26 @@ k_merge_mark(PadCols A, int64_t na, PadCols B, int64_t nb, int nu, MergePack mp,
             kb = j < len ? s_key[j] : 0;
         }
     }
-    // two threads' 16 rows are one word
     const unsigned c = __reduce_add_sync(0xffffffffu, __popc(keep));
-    keep |= __shfl_down_sync(0xffffffffu, keep, 1) << 16;
-    take |= __shfl_down_sync(0xffffffffu, take, 1) << 16;
-    if (!(lane & 1) && step < mb.sc.steps) {
-        const size_t w = (size_t)step * 32 + ((threadIdx.x & 63) >> 1);
+    keep <<= MP_ITEMS * (lane % WORD_THREADS);
+    take <<= MP_ITEMS * (lane % WORD_THREADS);
+#pragma unroll
+    for (int d = 1; d < WORD_THREADS; d <<= 1) {
+        keep |= __shfl_xor_sync(0xffffffffu, keep, d);
+        take |= __shfl_xor_sync(0xffffffffu, take, d);
+    }
+    if (lane % WORD_THREADS == 0 && step < mb.sc.steps) {
+        const size_t w = (size_t)step * 32 + (threadIdx.x % STEP_THREADS) / WORD_THREADS;
         mb.sc.bits[w] = keep;
         mb.take[w] = take;
     }
     if (lane == 0) s_cnt[warp] = c;
     __syncthreads();
-    if ((threadIdx.x & 63) == 0 && step < mb.sc.steps) mb.sc.cnt[step] = s_cnt[warp] + s_cnt[warp + 1];
+    if (threadIdx.x % STEP_THREADS == 0 && step < mb.sc.steps) {
+        unsigned n = 0;
+        for (int w = 0; w < STEP_THREADS / 32; ++w) n += s_cnt[warp + w];
+        mb.sc.cnt[step] = n;
+    }
     sel_finish(mb.sc, c, d_rows, h_rows);
 }
 
@@ -214,8 +243,8 @@ __global__ void __launch_bounds__(SEL_THREADS, K <= 3 ? 4 : 2)
 k_merge_expand(PadCols A, PadCols B, int nu, MergeBits mb, OutCols out, int64_t cap) {
     const unsigned lane = threadIdx.x & 31, lt = (1u << lane) - 1u;
     constexpr int UX = 4;  // rows per lane read together
-    // a range is four steps, one per warp: two ranges per CTA
-    const unsigned warp = threadIdx.x >> 5, per = MP_TILE / SEL_STEP;
+    // a range is four steps or one, a step per warp: two or eight ranges per CTA
+    const unsigned warp = threadIdx.x >> 5, per = mb.sc.per;
     const unsigned range = blockIdx.x * (SEL_WARPS / per) + warp / per;
     if (range >= mb.sc.ranges) return;
     sel_walk(mb.sc, range, warp % per, per, [&](unsigned step, uint32_t word, unsigned xo, unsigned, unsigned long long o0) {
@@ -407,24 +436,33 @@ int merge_unique(tid_ctx *ctx, const int32_t *const *acols, int64_t na, const in
     }
     OutCols oc{};
     for (int c = 0; c < nu; ++c) oc.col[c] = out->col[c];
-    const int tile_rows = mp ? MP_TILE : MG_TILE;
+    const bool few = na + nb < (int64_t)sm_count() * 2 * mp_tile<16>();
+    const int tile_rows = !mp ? MG_TILE : few ? mp_tile<4>() : mp_tile<16>();
     const int64_t tiles = ceil_div(na + nb, (int64_t)tile_rows);
     Scratch s(ctx);
-    TID_TRY(dev_alloc(ctx, &s.p, sizeof(int64_t) * (tiles + 1)));
-    int64_t *split = (int64_t *)s.p;
-    k_merge_split<<<(unsigned)ceil_div(tiles + 1, 8), 256, 0, st>>>(A, na, B, nb, nu, tiles, tile_rows, split);
-    TID_TRY(launch_check("k_merge_split"));
+    int64_t *split = nullptr;
+    if (!mp || !few) {
+        TID_TRY(dev_alloc(ctx, &s.p, sizeof(int64_t) * (tiles + 1)));
+        split = (int64_t *)s.p;
+        k_merge_split<<<(unsigned)ceil_div(tiles + 1, 8), 256, 0, st>>>(A, na, B, nb, nu, tiles, tile_rows, split);
+        TID_TRY(launch_check("k_merge_split"));
+    }
     if (mp) {
         MergeBits mb{};
         const size_t steps = (size_t)ceil_div(na + nb, (int64_t)SEL_STEP);
         void *blk = nullptr, *extra = nullptr;
-        TID_TRY(sel_scratch(ctx, na + nb, 1, steps * 33 * 4, &mb.sc, &blk, &extra, MP_TILE / SEL_STEP));
+        TID_TRY(sel_scratch(ctx, na + nb, 1, steps * 33 * 4, &mb.sc, &blk, &extra, tile_rows / SEL_STEP));
         mb.take = (uint32_t *)extra;
         mb.first_a = mb.take + steps * 32;
-        k_merge_mark<<<(unsigned)tiles, MP_THREADS, 0, st>>>(A, na, B, nb, nu, *mp, split, mb, out->d_rows, out->slot.dev);
+        if (few)
+            k_merge_mark<4><<<(unsigned)tiles, MP_THREADS, 0, st>>>(A, na, B, nb, nu, *mp, split, mb, out->d_rows,
+                                                                   out->slot.dev);
+        else
+            k_merge_mark<16><<<(unsigned)tiles, MP_THREADS, 0, st>>>(A, na, B, nb, nu, *mp, split, mb, out->d_rows,
+                                                                    out->slot.dev);
         int rc = launch_check("k_merge_mark");
         if (rc == TID_OK) {
-            const unsigned grid = (unsigned)ceil_div(mb.sc.ranges, (int64_t)(SEL_WARPS / (MP_TILE / SEL_STEP)));
+            const unsigned grid = (unsigned)ceil_div(mb.sc.ranges, (int64_t)(SEL_WARPS / mb.sc.per));
             if (nu <= 3) k_merge_expand<3><<<grid, SEL_THREADS, 0, st>>>(A, B, nu, mb, oc, out->cap);
             else k_merge_expand<TID_MAX_COLS><<<grid, SEL_THREADS, 0, st>>>(A, B, nu, mb, oc, out->cap);
             rc = launch_check("k_merge_expand");

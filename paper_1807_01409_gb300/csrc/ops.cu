@@ -283,6 +283,32 @@ int union_sets(tid_ctx *ctx, const tid_set *const *in, int k, tid_set **out) {
             bits += w;
             packed = bits <= 64;
         }
+        if (packed && total > 0 && total <= SMALL_UNION_ROWS && k <= SMALL_UNION_INPUTS) {
+            // sorted and deduplicated by one CTA, one launch in place of two per pair
+            // of inputs (the plans of a 200K-triple store 1.89 -> 1.73 ms; at 4000
+            // rows the sort takes 4 us longer than the merge)
+            const int32_t *cols[SMALL_UNION_INPUTS][TID_MAX_COLS] = {};
+            for (int i = 0; i < k; ++i)
+                for (int u = 0; u < nu; ++u) {
+                    const int c = find_col(in[i], uv[u]);
+                    cols[i][u] = c >= 0 ? in[i]->col[c] : nullptr;
+                }
+            tid_set *o = nullptr;
+            TID_TRY(set_alloc(ctx, nu, uv, total, &o));
+            int rc = small_union(ctx, cols, rows.data(), k, nu, mp, o);
+            if (rc == TID_OK) rc = set_ready(o);
+            if (rc != TID_OK) {
+                set_free(o);
+                return rc;
+            }
+            o->bounded = true;
+            for (int u = 0; u < nu; ++u) {
+                o->lo[u] = b.lo[u];
+                o->hi[u] = b.hi[u];
+            }
+            *out = o;
+            return TID_OK;
+        }
         tid_set *cur = nullptr;  // union of the inputs merged so far (null: only in[0])
         int rc = TID_OK;
         for (int i = 1; i < k && rc == TID_OK; ++i) {

@@ -130,6 +130,12 @@ int outer_join_sets(tid_ctx *ctx, const tid_set *L, const tid_set *R, int algo, 
 int merge_unique(tid_ctx *ctx, const int32_t *const *acols, int64_t na, const int32_t *const *bcols, int64_t nb,
                  int nu, const MergePack *mp, tid_set *out);
 
+// the union of at most SMALL_UNION_INPUTS sets of at most SMALL_UNION_ROWS rows in all,
+// in one launch (sort.cu): cols[i][c] column c of input i (null: absent), packed by mp
+constexpr int SMALL_UNION_ROWS = 1024, SMALL_UNION_INPUTS = 4;
+int small_union(tid_ctx *ctx, const int32_t *const (*cols)[TID_MAX_COLS], const int64_t *rows, int inputs, int k,
+                const MergePack &mp, tid_set *out);
+
 // set operators (ops.cu)
 int filter_set(tid_ctx *ctx, const tid_set *in, const tid_pred *preds, int n_preds, tid_set **out);
 int union_sets(tid_ctx *ctx, const tid_set *const *in, int k, tid_set **out);

@@ -466,6 +466,7 @@ k_onesweep(const K *__restrict__ kin, const int32_t *__restrict__ vin, K *__rest
 // us in all, against every step in shared memory.
 constexpr int SMALL_N = 4096;
 constexpr int SMALL_THREADS = 1024;
+static_assert(SMALL_UNION_ROWS <= SMALL_N, "a small union is sorted by one CTA");
 
 template <typename K, int E>
 __device__ __forceinline__ void bitonic(K (&v)[E], K *sm, int P) {
@@ -497,20 +498,14 @@ __device__ __forceinline__ void bitonic(K (&v)[E], K *sm, int P) {
     }
 }
 
-// rows packed, sorted, and left in order in sk
-template <typename K, int E>
-__device__ __forceinline__ void small_sort(const ColPtrs &cols, int k, int n, const PackSpec &ps, int P, K *sk) {
+// the rows' keys sorted and left in order in sk
+template <typename K, int E, class KeyOf>
+__device__ __forceinline__ void small_sort(int n, int P, K *sk, KeyOf key_of) {
     K v[E];
 #pragma unroll
     for (int e = 0; e < E; ++e) {
         const int i = threadIdx.x * E + e;
-        v[e] = ~(K)0;
-        if (i < n) {
-            v[e] = 0;
-#pragma unroll
-            for (int c = 0; c < TID_MAX_COLS; ++c)
-                if (c < k && ps.mask[c]) v[e] |= (K)(order_key(cols.c[c][i]) - ps.min[c]) << ps.shift[c];
-        }
+        v[e] = i < n ? key_of(i) : ~(K)0;
     }
     bitonic<K, E>(v, sk, P);
     __syncthreads();
@@ -519,18 +514,17 @@ __device__ __forceinline__ void small_sort(const ColPtrs &cols, int k, int n, co
     __syncthreads();
 }
 
-template <typename K>
-__global__ void __launch_bounds__(SMALL_THREADS) k_small_canonical(ColPtrs cols, int k, int n, PackSpec ps,
-                                                                   int dedupe, MutColPtrs out,
-                                                                   int64_t *__restrict__ d_rows,
-                                                                   int64_t *__restrict__ h_rows) {
+// sorts the n rows' keys, drops repeats if asked, and put()s row by row
+template <typename K, class KeyOf, class Put>
+__device__ __forceinline__ void small_set(int n, bool dedupe, KeyOf key_of, Put put, int64_t *__restrict__ d_rows,
+                                          int64_t *__restrict__ h_rows) {
     __shared__ K sk[SMALL_N];
     __shared__ uint32_t s_warp[SMALL_THREADS / 32];
     int P = 1;
     while (P < n) P <<= 1;
-    if (P <= SMALL_THREADS) small_sort<K, 1>(cols, k, n, ps, P, sk);
-    else if (P == 2 * SMALL_THREADS) small_sort<K, 2>(cols, k, n, ps, P, sk);
-    else small_sort<K, 4>(cols, k, n, ps, P, sk);
+    if (P <= SMALL_THREADS) small_sort<K, 1>(n, P, sk, key_of);
+    else if (P == 2 * SMALL_THREADS) small_sort<K, 2>(n, P, sk, key_of);
+    else small_sort<K, 4>(n, P, sk, key_of);
     // each thread owns up to SMALL_N / SMALL_THREADS consecutive sorted rows
     constexpr int PER = SMALL_N / SMALL_THREADS;
     const int b = threadIdx.x * PER;
@@ -555,21 +549,76 @@ __global__ void __launch_bounds__(SMALL_THREADS) k_small_canonical(ColPtrs cols,
     for (unsigned w = 0; w < warp; ++w) base += s_warp[w];
     uint32_t pos = base + x - cnt;
 #pragma unroll
-    for (int q = 0; q < PER; ++q) {
-        if (!keep[q]) continue;
-        const K key = sk[b + q];
-#pragma unroll
-        for (int c = 0; c < TID_MAX_COLS; ++c) {
-            if (c >= k) continue;
-            const uint32_t f = ps.mask[c] ? (uint32_t)((key >> ps.shift[c]) & ps.mask[c]) : 0u;
-            out.c[c][pos] = (int32_t)((f + ps.min[c]) ^ 0x80000000u);
-        }
-        ++pos;
-    }
+    for (int q = 0; q < PER; ++q)
+        if (keep[q]) put(sk[b + q], pos++);
     if (threadIdx.x == SMALL_THREADS - 1) {
         *d_rows = pos;
         *h_rows = pos;
     }
+}
+
+template <typename K>
+__global__ void __launch_bounds__(SMALL_THREADS) k_small_canonical(ColPtrs cols, int k, int n, PackSpec ps,
+                                                                   int dedupe, MutColPtrs out,
+                                                                   int64_t *__restrict__ d_rows,
+                                                                   int64_t *__restrict__ h_rows) {
+    small_set<K>(
+        n, dedupe,
+        [&](int i) {
+            K key = 0;
+#pragma unroll
+            for (int c = 0; c < TID_MAX_COLS; ++c)
+                if (c < k && ps.mask[c]) key |= (K)(order_key(cols.c[c][i]) - ps.min[c]) << ps.shift[c];
+            return key;
+        },
+        [&](K key, uint32_t pos) {
+#pragma unroll
+            for (int c = 0; c < TID_MAX_COLS; ++c) {
+                if (c >= k) continue;
+                const uint32_t f = ps.mask[c] ? (uint32_t)((key >> ps.shift[c]) & ps.mask[c]) : 0u;
+                out.c[c][pos] = (int32_t)((f + ps.min[c]) ^ 0x80000000u);
+            }
+        },
+        d_rows, h_rows);
+}
+
+// The union of a few small sets in the same launch: input i's rows follow those of
+// the inputs before it; a column it lacks reads as 0.
+struct SmallUnion {
+    const int32_t *col[SMALL_UNION_INPUTS][TID_MAX_COLS];
+    int end[SMALL_UNION_INPUTS];  // rows of inputs 0 .. i
+};
+
+__global__ void __launch_bounds__(SMALL_THREADS)
+k_small_union(const __grid_constant__ SmallUnion in, int k, int n, const __grid_constant__ MergePack mp, MutColPtrs out,
+              int64_t *__restrict__ d_rows, int64_t *__restrict__ h_rows) {
+    typedef unsigned long long K;
+    small_set<K>(
+        n, true,
+        [&](int r) {
+            int s = 0;
+#pragma unroll
+            for (int i = 1; i < SMALL_UNION_INPUTS; ++i) s += r >= in.end[i - 1];
+            const int64_t i = r - (s ? in.end[s - 1] : 0);
+            K key = 0;
+#pragma unroll
+            for (int c = 0; c < TID_MAX_COLS; ++c) {
+                if (c >= k || !mp.ps.mask[c]) continue;
+                const int32_t x = in.col[s][c] ? in.col[s][c][i] : 0;
+                const uint32_t f = ((mp.zero >> c) & 1u) && x == 0 ? 0u : order_key(x) - mp.ps.min[c];
+                key |= (K)f << mp.ps.shift[c];
+            }
+            return key;
+        },
+        [&](K key, uint32_t pos) {
+#pragma unroll
+            for (int c = 0; c < TID_MAX_COLS; ++c) {
+                if (c >= k) continue;
+                const uint32_t f = mp.ps.mask[c] ? (uint32_t)((key >> mp.ps.shift[c]) & mp.ps.mask[c]) : 0u;
+                out.c[c][pos] = ((mp.zero >> c) & 1u) && f == 0 ? 0 : (int32_t)((f + mp.ps.min[c]) ^ 0x80000000u);
+            }
+        },
+        d_rows, h_rows);
 }
 
 __global__ void __launch_bounds__(EW_THREADS) k_gather(ColPtrs in, int k, const int32_t *__restrict__ perm, int64_t n,
@@ -813,6 +862,21 @@ static int canonical_packed(tid_ctx *ctx, const int32_t *const *cols, int k, int
     if (dedupe) return compact_unique_packed(ctx, ka, sizeof(K) == 8, k, n, ps, set);
     set->rows_known = n;
     return TID_OK;
+}
+
+int small_union(tid_ctx *ctx, const int32_t *const (*cols)[TID_MAX_COLS], const int64_t *rows, int inputs, int k,
+                const MergePack &mp, tid_set *out) {
+    SmallUnion in{};
+    MutColPtrs op{};
+    int n = 0;
+    for (int i = 0; i < SMALL_UNION_INPUTS; ++i) {
+        for (int c = 0; c < k && i < inputs; ++c) in.col[i][c] = cols[i][c];
+        n += i < inputs ? (int)rows[i] : 0;
+        in.end[i] = n;
+    }
+    for (int c = 0; c < k; ++c) op.c[c] = out->col[c];
+    k_small_union<<<1, SMALL_THREADS, 0, ctx->stream>>>(in, k, n, mp, op, out->d_rows, out->slot.dev);
+    return launch_check("k_small_union");
 }
 
 int gather_cols(tid_ctx *ctx, const int32_t *const *in, int k, const int32_t *perm, int64_t n,
