@@ -664,6 +664,7 @@ __global__ void __launch_bounds__(256) k_member_bits(const int32_t *__restrict__
 // ---- exclusive scan of uint32 (look-back) --------------------------------------
 
 constexpr int SC_THREADS = 256, SC_ITEMS = 16, SC_TILE = SC_THREADS * SC_ITEMS;
+static_assert(SC_TILE == SCAN_TILE, "the callers' tile");
 static_assert(SC_ITEMS == 16, "k_scan_u32 splits tile positions as (e >> 4, e & 15)");
 
 // Exclusive scan of one 4096-item tile; the tile's first output is `prefix`
@@ -818,7 +819,7 @@ int sel_scratch(tid_ctx *ctx, int64_t n, int lists, size_t extra, SelScratch *sc
 }
 
 int scan_exclusive_u32(tid_ctx *ctx, const uint32_t *in, uint32_t *out, int64_t n,
-                       unsigned long long *total_dev) {
+                       unsigned long long *total_dev, const uint32_t *tile_sums) {
     if (n == 0) {
         if (total_dev) TID_TRY_CUDA(cudaMemsetAsync(total_dev, 0, 8, ctx->stream), "memset");
         return TID_OK;
@@ -835,9 +836,12 @@ int scan_exclusive_u32(tid_ctx *ctx, const uint32_t *in, uint32_t *out, int64_t 
     uint32_t *sums = nullptr;
     TID_TRY(dev_alloc(ctx, (void **)&sums, sizeof(uint32_t) * 2 * (size_t)tiles + 256));
     uint32_t *offs = sums + tiles;
-    k_tile_sums<<<tiles, SC_THREADS, 0, ctx->stream>>>(in, n, sums);
-    int rc = launch_check("k_tile_sums");
-    if (rc == TID_OK) rc = scan_exclusive_u32(ctx, sums, offs, tiles, total_dev);
+    int rc = TID_OK;
+    if (!tile_sums) {
+        k_tile_sums<<<tiles, SC_THREADS, 0, ctx->stream>>>(in, n, sums);
+        rc = launch_check("k_tile_sums");
+    }
+    if (rc == TID_OK) rc = scan_exclusive_u32(ctx, tile_sums ? tile_sums : sums, offs, tiles, total_dev);
     if (rc == TID_OK) {
         k_scan_u32<<<tiles, SC_THREADS, 0, ctx->stream>>>(in, out, n, nullptr, Lookback{}, offs);
         rc = launch_check("k_scan_u32");

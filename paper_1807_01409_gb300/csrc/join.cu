@@ -184,13 +184,17 @@ __global__ void __launch_bounds__(256) k_run_table(const int32_t *__restrict__ k
 }
 
 // cnt[l] right rows match left row l, from lo_out[l] on; exact: a bucket of the
-// table holds the rows of one key
+// table holds the rows of one key.  A CTA takes a tile of the scan that follows and
+// leaves its sum.
 __global__ void __launch_bounds__(256) k_run_count(Cols LK, int64_t nl, Cols RK, int nk, bool left, RunTable t, bool exact,
                                                    uint32_t *__restrict__ cnt, uint32_t *__restrict__ lo_out,
-                                                   unsigned long long *__restrict__ total) {
+                                                   unsigned long long *__restrict__ total,
+                                                   uint32_t *__restrict__ sums) {
     constexpr int U = 4;  // rows per thread whose table reads are in flight together
+    __shared__ unsigned s_sum[8];
     unsigned long long acc = 0;
-    for (int64_t l0 = (int64_t)blockIdx.x * (256 * U) + threadIdx.x; l0 < nl; l0 += (int64_t)gridDim.x * (256 * U)) {
+    const int64_t begin = (int64_t)blockIdx.x * SCAN_TILE, end = min(begin + SCAN_TILE, nl);
+    for (int64_t l0 = begin + threadIdx.x; l0 < end; l0 += 256 * U) {
         uint2 b[U];
 #pragma unroll
         for (int u = 0; u < U; ++u) {
@@ -220,6 +224,14 @@ __global__ void __launch_bounds__(256) k_run_count(Cols LK, int64_t nl, Cols RK,
         }
     }
     block_add_u64(acc, total);  // once per warp: one address takes these atomics one at a time
+    const unsigned w = __reduce_add_sync(0xffffffffu, (unsigned)acc);
+    if ((threadIdx.x & 31) == 0) s_sum[threadIdx.x >> 5] = w;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        unsigned s = 0;
+        for (int i = 0; i < 8; ++i) s += s_sum[i];
+        sums[blockIdx.x] = s;
+    }
 }
 
 // The same by binary search over all of the right keys; the left keys are sorted.
@@ -260,31 +272,32 @@ __global__ void k_sm_count(Cols LK, int64_t nl, Cols RK, int64_t nr, int nk, boo
 // probe rows and the output rows next to them -- at most T items in all, so
 // neither a long run of rows without matches nor one row with millions of
 // matches makes a CTA's work unbounded.  The CTA stages its rows' offsets in
-// shared memory and each output row finds its probe row there by binary
-// search; consecutive output rows go to consecutive threads (coalesced
-// stores).
+// shared memory and marks where each row's output begins; a running maximum then
+// gives every output row its probe row (with a binary search per output row, a
+// search per tile boundary by one thread and the scan's own sums, the join of 8M
+// with 8M rows took 273 us, now 226).  Consecutive output rows go to consecutive
+// threads (coalesced stores).
 constexpr int JW_THREADS = 256;
 constexpr int JW_ITEMS = 8;
 constexpr int JW_TILE = JW_THREADS * JW_ITEMS;
 
-// rows among the first d items of the merged order
-__device__ __forceinline__ int64_t jw_split(const uint32_t *__restrict__ off, int64_t nl, int64_t total, int64_t d) {
-    int64_t lo = max((int64_t)0, d - total), hi = min(d, nl);
-    while (lo < hi) {
-        const int64_t mid = (lo + hi) >> 1;
-        if ((int64_t)off[mid] <= d - 1 - mid) lo = mid + 1;
-        else hi = mid;
-    }
-    return lo;
-}
-
-// split[t] = rows among the first t JW_TILE items, for every tile boundary (its own
-// launch: a search inside the write kernel was some twenty dependent loads at the
-// start of every CTA)
+// split[t] = rows among the first t JW_TILE items of the merged order, for every
+// tile boundary: a warp each, 32 places tested at once (its own launch: a search
+// inside the write kernel was some twenty dependent loads at the start of every CTA)
 __global__ void __launch_bounds__(256) k_join_split(const uint32_t *__restrict__ off, int64_t nl, int64_t total,
                                                     int64_t tiles, uint32_t *__restrict__ split) {
-    const int64_t t = (int64_t)blockIdx.x * 256 + threadIdx.x;
-    if (t <= tiles) split[t] = (uint32_t)jw_split(off, nl, total, min(t * JW_TILE, nl + total));
+    const int64_t t = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
+    if (t > tiles) return;
+    const unsigned lane = threadIdx.x & 31;
+    const int64_t d = min(t * JW_TILE, nl + total);
+    int64_t lo = max((int64_t)0, d - total), hi = min(d, nl);
+    while (lo < hi) {  // row m is among the first d items if off[m] <= d - 1 - m; lane l tests the l-th part's end
+        const int64_t part = (hi - lo + 31) / 32, m = lo + (lane + 1) * part - 1;
+        const bool in = m < hi && (int64_t)off[m] <= d - 1 - m;
+        lo += (int64_t)__popc(__ballot_sync(0xffffffffu, in)) * part;
+        hi = min(hi, lo + part - 1);
+    }
+    if (lane == 0) split[t] = (uint32_t)min(lo, min(d, nl));
 }
 
 __global__ void __launch_bounds__(JW_THREADS) k_join_write(const uint32_t *__restrict__ off, int64_t nl,
@@ -295,6 +308,8 @@ __global__ void __launch_bounds__(JW_THREADS) k_join_write(const uint32_t *__res
                                                            int kl, Cols Rrest, int nrest, MCols outL, MCols outR,
                                                            bool left_is_probe, const uint32_t *__restrict__ split) {
     __shared__ uint32_t s_off[JW_TILE + 1], s_lo[JW_TILE + 1];  // of rows rb .. r1 - 1
+    __shared__ __align__(16) uint16_t s_row[JW_TILE];  // output row o0 + i belongs to probe row rb + s_row[i]
+    __shared__ unsigned s_wmax[JW_THREADS / 32];
     const int64_t d0 = (int64_t)blockIdx.x * JW_TILE, d1 = min(d0 + JW_TILE, nl + total);
     const int64_t r0 = split[blockIdx.x], r1 = split[blockIdx.x + 1];
     const int64_t o0 = d0 - r0, o1 = d1 - r1;
@@ -307,6 +322,39 @@ __global__ void __launch_bounds__(JW_THREADS) k_join_write(const uint32_t *__res
         s_off[i] = off[rb + i];
         s_lo[i] = lo[rb + i];
     }
+    static_assert(JW_ITEMS == 8, "a thread scans eight 16-bit entries as one 16-byte word");
+    reinterpret_cast<uint4 *>(s_row)[threadIdx.x] = make_uint4(0, 0, 0, 0);
+    __syncthreads();
+    // The probe row of every output row: each row with output in the tile enters
+    // itself at its first output row (of rows with one offset, the last has the
+    // output; row 0 holds what was begun before the tile), then a running maximum.
+    for (int i = threadIdx.x; i < nr; i += JW_THREADS) {
+        const uint32_t f = s_off[i];
+        if ((i + 1 == nr || s_off[i + 1] > f) && f >= (uint32_t)o0 && f < (uint32_t)o1) s_row[f - (uint32_t)o0] = (uint16_t)i;
+    }
+    __syncthreads();
+    {
+        const unsigned lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+        uint4 w = reinterpret_cast<const uint4 *>(s_row)[threadIdx.x];
+        unsigned e[8] = {w.x & 0xFFFFu, w.x >> 16, w.y & 0xFFFFu, w.y >> 16, w.z & 0xFFFFu, w.z >> 16, w.w & 0xFFFFu, w.w >> 16};
+#pragma unroll
+        for (int q = 1; q < 8; ++q) e[q] = max(e[q], e[q - 1]);
+        unsigned x = e[7];
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const unsigned y = __shfl_up_sync(0xffffffffu, x, d);
+            if ((int)lane >= d) x = max(x, y);
+        }
+        if (lane == 31) s_wmax[warp] = x;
+        unsigned before = __shfl_up_sync(0xffffffffu, x, 1);
+        if (lane == 0) before = 0;
+        __syncthreads();
+        for (unsigned v = 0; v < warp; ++v) before = max(before, s_wmax[v]);
+#pragma unroll
+        for (int q = 0; q < 8; ++q) e[q] = max(e[q], before);
+        reinterpret_cast<uint4 *>(s_row)[threadIdx.x] =
+            make_uint4(e[0] | e[1] << 16, e[2] | e[3] << 16, e[4] | e[5] << 16, e[6] | e[7] << 16);
+    }
     __syncthreads();
     // every output row's left and right row first, then column by column, so
     // that a column's reads are in flight together
@@ -315,18 +363,7 @@ __global__ void __launch_bounds__(JW_THREADS) k_join_write(const uint32_t *__res
 #pragma unroll
     for (int q = 0; q < JW_ITEMS; ++q) {
         const int64_t o = min(o0 + q * JW_THREADS + threadIdx.x, last);
-        // last i with s_off[i] <= o.  First guess: rows of one match each
-        // (the common case) put output o at row o - s_off[0] of the tile.
-        int a = (int)min((int64_t)(nr - 1), o - (int64_t)s_off[0]);
-        if (!((int64_t)s_off[a] <= o && (a + 1 == nr || (int64_t)s_off[a + 1] > o))) {
-            a = 0;
-            int b = nr;
-            while (b - a > 1) {
-                const int m = (a + b) >> 1;
-                if ((int64_t)s_off[m] <= o) a = m;
-                else b = m;
-            }
-        }
+        const int a = s_row[o - o0];
         lr[q] = (int32_t)(rb + a);
         // left outer join: a left row alone, right columns unbound (-1)
         rr[q] = s_lo[a] == NO_MATCH ? -1 : (int32_t)(s_lo[a] + (uint32_t)(o - s_off[a]));
@@ -716,7 +753,7 @@ int join_sets(tid_ctx *ctx, const tid_set *L, const tid_set *R, int algo, tid_se
     }
     // runs (or members, or a merge of two sorted sides) need the right side alone
     // to lead with the key; a sort of the joined rows is what the hash join costs
-    // (8M x 8M rows, 11.5M joined, on GB300: 2318 us by hash and sort, 280 us by
+    // (8M x 8M rows, 11.5M joined, on GB300: 2318 us by hash and sort, 226 us by
     // runs, bound by the table lookups' and the right rows' random reads in L2)
     if (algo == TID_JOIN_AUTO) algo = (nk == 0 || rprefix) ? TID_JOIN_SORT_MERGE : TID_JOIN_HASH;
     if (nk == 0 || left) algo = TID_JOIN_SORT_MERGE;  // cross product; left outer join
@@ -843,10 +880,12 @@ int join_sets(tid_ctx *ctx, const tid_set *L, const tid_set *R, int algo, tid_se
         TID_TRY_CUDA(cudaMemsetAsync(t.bucket, 0, nb * sizeof(uint2), st), "run table");
         k_run_table<<<grid_for(nr, 1024, 8), 256, 0, st>>>(RK.c[0], nr, t);
         TID_TRY(launch_check("k_run_table"));
-        k_run_count<<<grid_for(nl, 1024, 8), 256, 0, st>>>(LK, nl, RK, nk, left, t, nk == 1 && t.shift == 0, cnt, lo,
-                                                           d_total);
+        uint32_t *sums = nullptr;
+        TID_TRY(s.get(&sums, (size_t)ceil_div(nl, (int64_t)SCAN_TILE)));
+        k_run_count<<<(unsigned)ceil_div(nl, (int64_t)SCAN_TILE), 256, 0, st>>>(
+            LK, nl, RK, nk, left, t, nk == 1 && t.shift == 0, cnt, lo, d_total, sums);
         TID_TRY(launch_check("k_run_count"));
-        TID_TRY(scan_exclusive_u32(ctx, cnt, off, nl, nullptr));
+        TID_TRY(scan_exclusive_u32(ctx, cnt, off, nl, nullptr, sums));
         canonical_out = true;
     } else if (algo == TID_JOIN_SORT_MERGE) {
         Cols LK{}, RK{};
@@ -942,7 +981,7 @@ int join_sets(tid_ctx *ctx, const tid_set *L, const tid_set *R, int algo, tid_se
     const int64_t jtiles = ceil_div(n_probe + (int64_t)total, (int64_t)JW_TILE);
     if (total > 0) {
         TID_TRY(s.get(&split, jtiles + 1));
-        k_join_split<<<(unsigned)ceil_div(jtiles + 1, (int64_t)256), 256, 0, st>>>(off, n_probe, (int64_t)total, jtiles,
+        k_join_split<<<(unsigned)ceil_div(jtiles + 1, (int64_t)8), 256, 0, st>>>(off, n_probe, (int64_t)total, jtiles,
                                                                                   split);
         TID_TRY(launch_check("k_join_split"));
     }

@@ -75,9 +75,11 @@ struct VarMember {  // the same by variable
     int8_t var;
 };
 
-// exclusive scan of n uint32 (out may alias in); *total_dev receives the sum
+// exclusive scan of n uint32 (out may alias in); *total_dev receives the sum; sums:
+// the sum of every tile of SCAN_TILE items, if the caller has them
+constexpr int SCAN_TILE = 4096;
 int scan_exclusive_u32(tid_ctx *ctx, const uint32_t *in, uint32_t *out, int64_t n,
-                       unsigned long long *total_dev);
+                       unsigned long long *total_dev, const uint32_t *sums = nullptr);
 
 // row selections (compact.cu); `out` must have capacity >= n
 // bind, with the bounds of the kept rows
