@@ -369,15 +369,23 @@ int check_ctx_error(tid_ctx *ctx) {
     return TID_OK;
 }
 
-// rows x k row-major from k columns
-__global__ void k_interleave(const int32_t *const *cols, int k, const int64_t *d_rows, int32_t *out) {
-    const int64_t n = *d_rows;
-    const int64_t total = n * k;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t r = i / k;
-        const int c = (int)(i - r * k);
-        out[i] = cols[c][r];
+struct SetCols {
+    const int32_t *c[TID_MAX_COLS];
+};
+
+// n rows x k row-major from k columns: a thread writes one row, its loads in flight
+// together (the columns come as arguments: a copy of their addresses to the device
+// and a division per value cost more than the rows of a small set)
+template <int K>
+__global__ void __launch_bounds__(256) k_interleave(SetCols cols, int k, int64_t n, int32_t *__restrict__ out) {
+    for (int64_t r = (int64_t)blockIdx.x * 256 + threadIdx.x; r < n; r += (int64_t)gridDim.x * 256) {
+        int32_t v[K];
+#pragma unroll
+        for (int c = 0; c < K; ++c)
+            if (c < k) v[c] = cols.c[c][r];
+#pragma unroll
+        for (int c = 0; c < K; ++c)
+            if (c < k) out[r * k + c] = v[c];
     }
 }
 
@@ -682,15 +690,13 @@ extern "C" int tid_set_to_host(tid_set *set, int32_t *buf, int64_t cap_rows, int
         TID_TRY_CUDA(cudaMemcpyAsync(buf, set->col[0], bytes, cudaMemcpyDeviceToHost, ctx->stream), "copy set");
     } else {
         void *tmp = nullptr;
-        TID_TRY(dev_alloc(ctx, &tmp, align_up(bytes, 256) + sizeof(int32_t *) * TID_MAX_COLS));
-        int32_t **dcols = (int32_t **)((char *)tmp + align_up(bytes, 256));
-        cudaError_t e = cudaMemcpyAsync(dcols, set->col, sizeof(int32_t *) * set->k, cudaMemcpyHostToDevice, ctx->stream);
-        if (e == cudaSuccess) {
-            const int64_t blocks = ceil_div(rows * set->k, 256);
-            k_interleave<<<grid_for(blocks, 1), 256, 0, ctx->stream>>>(
-                dcols, set->k, set->d_rows, (int32_t *)tmp);
-            e = cudaGetLastError();
-        }
+        TID_TRY(dev_alloc(ctx, &tmp, bytes));
+        SetCols sc{};
+        for (int c = 0; c < set->k; ++c) sc.c[c] = set->col[c];
+        const unsigned grid = grid_for(rows, 256);
+        if (set->k <= 3) k_interleave<3><<<grid, 256, 0, ctx->stream>>>(sc, set->k, rows, (int32_t *)tmp);
+        else k_interleave<TID_MAX_COLS><<<grid, 256, 0, ctx->stream>>>(sc, set->k, rows, (int32_t *)tmp);
+        cudaError_t e = cudaGetLastError();
         if (e == cudaSuccess) e = cudaMemcpyAsync(buf, tmp, bytes, cudaMemcpyDeviceToHost, ctx->stream);
         dev_free(ctx, tmp);
         if (e != cudaSuccess) return fail_cuda(e, "copy set");

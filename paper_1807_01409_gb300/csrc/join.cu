@@ -306,13 +306,18 @@ __global__ void __launch_bounds__(JW_THREADS) k_join_write(const uint32_t *__res
                                                            const int32_t *__restrict__ rmap,
                                                            const int32_t *__restrict__ rperm, int64_t total, Cols L,
                                                            int kl, Cols Rrest, int nrest, MCols outL, MCols outR,
-                                                           bool left_is_probe, const uint32_t *__restrict__ split) {
+                                                           bool left_is_probe, const uint32_t *__restrict__ split,
+                                                           int64_t *__restrict__ d_rows, int64_t *__restrict__ h_rows) {
     __shared__ uint32_t s_off[JW_TILE + 1], s_lo[JW_TILE + 1];  // of rows rb .. r1 - 1
     __shared__ __align__(16) uint16_t s_row[JW_TILE];  // output row o0 + i belongs to probe row rb + s_row[i]
     __shared__ unsigned s_wmax[JW_THREADS / 32];
     const int64_t d0 = (int64_t)blockIdx.x * JW_TILE, d1 = min(d0 + JW_TILE, nl + total);
     const int64_t r0 = split[blockIdx.x], r1 = split[blockIdx.x + 1];
     const int64_t o0 = d0 - r0, o1 = d1 - r1;
+    if (d_rows && blockIdx.x == 0 && threadIdx.x == 0) {  // the result's row count
+        *d_rows = total;
+        *h_rows = total;
+    }
     if (o0 >= o1) return;  // only rows here
     // the output rows [o0, o1) belong to rows rb .. r1 - 1: row r0 - 1 precedes
     // output o0 in the merged order (off[r0 - 1] <= o0), row r1 follows o1 - 1
@@ -995,10 +1000,11 @@ int join_sets(tid_ctx *ctx, const tid_set *L, const tid_set *R, int algo, tid_se
         if (total > 0) {
             k_join_write<<<(unsigned)jtiles, JW_THREADS, 0, st>>>(
                 off, n_probe, lo, lperm, rmap, rperm, (int64_t)total, Lall, L->k, Rrest, nrest, oL, oR, left_is_probe,
-                split);
+                split, res->d_rows, res->slot.dev);
             rc = launch_check("k_join_write");
         }
-        if (rc == TID_OK) rc = set_rows_const(res, (int64_t)total);
+        if (rc == TID_OK && total == 0) rc = set_rows_const(res, 0);
+        res->rows_known = (int64_t)total;
         if (rc == TID_OK) rc = set_ready(res);
         if (rc != TID_OK) {
             set_free(res);
@@ -1014,7 +1020,7 @@ int join_sets(tid_ctx *ctx, const tid_set *L, const tid_set *R, int algo, tid_se
     if (total > 0) {
         k_join_write<<<(unsigned)jtiles, JW_THREADS, 0, st>>>(
             off, n_probe, lo, lperm, rmap, rperm, (int64_t)total, Lall, L->k, Rrest, nrest, oL, oR, left_is_probe,
-                split);
+                split, nullptr, nullptr);
         TID_TRY(launch_check("k_join_write"));
     }
     const int32_t *ocols[TID_MAX_COLS];
