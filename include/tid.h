@@ -194,7 +194,7 @@ int tid_batch_table_check(const tid_pattern *pats, int q, uint32_t seed, int *at
  * shape (TID_BATCH_DIRECT: every present mask looked up for every triple;
  * TID_BATCH_DIRECT_SKIP: the same, skipping masks no lane of a warp may answer;
  * TID_BATCH_QUEUE4 / TID_BATCH_QUEUE8: only the prefilter's candidates looked
- * up, 4 or 8 slots of 32 triples in flight), the keys per sub-batch and the
+ * up, queued across slots of 32 triples or slot by slot), the keys per sub-batch and the
  * number of sub-batches; -1, 0, 0 before any such call.  Any pointer may be
  * NULL.  The choice is timed on the first call for each (GPU, store size, masks
  * read, log2 of the distinct keys) and kept for the process. */
@@ -320,7 +320,8 @@ int tid_join(tid_ctx *ctx, const tid_set *L, const tid_set *R, int algo, tid_set
 int tid_union(tid_ctx *ctx, const tid_set *const *in, int k, tid_set **out);
 
 /* SELECT the n_vars listed variables (in that order) with DISTINCT
- * (Section 4.3).  Output canonical. */
+ * (Section 4.3).  Output canonical.  Listing every variable of `in` only
+ * reorders its columns: a set's rows stay distinct. */
 int tid_project(tid_ctx *ctx, const tid_set *in, const int8_t *vars, int n_vars, tid_set **out);
 
 /* A set from `rows` x `cols` int32 in host memory (row-major), labelled with

@@ -270,7 +270,7 @@ __global__ void __launch_bounds__(KB_THREADS) k_batch(BatchArgs a) {
         for (int k = lane; k < a.kids; k += 32) row[k] = cnt[k];
 }
 
-// QUEUE shape: only the (triple, mask) pairs the prefilter admits are looked up.
+// QUEUE4 shape: only the (triple, mask) pairs the prefilter admits are looked up.
 // For each 32-triple slot and each mask that some lane may answer, the lanes'
 // candidates join a per-warp queue in lane order (a ballot places them), with the
 // triple's values, so for any one mask the queue is in triple order.  Whenever 32
@@ -389,6 +389,117 @@ __global__ void __launch_bounds__(KB_THREADS) k_batch_q(BatchArgs a) {
         for (int k = lane; k < a.kids; k += 32) row[k] = cnt[k];
 }
 
+// QUEUE8 shape: the same, slot by slot: lane l lists the masks its triple may answer,
+// an exclusive scan over the lanes' counts gives each lane its place in a queue of
+// (lane, mask) bytes, lane-major, and the queue is looked up 32 entries at a time, an
+// entry's values and mixed columns fetched from its lane by shuffle.  It costs a scan
+// per slot but nothing per mask, and its 2 KB queue leaves room for two CTAs per SM at
+// 1920 keys, where the 8 KB ring of the queue across slots leaves one: 4096 queries of
+// up to 10^7 results on 500M triples take 25.8 ms by it (two sub-batches of 1920 keys)
+// and 27.0 by the other (three of 1152).  The autotuner picks.
+template <int U, bool WRITE, int UNROLL>
+__global__ void __launch_bounds__(KB_THREADS) k_batch_slot(BatchArgs a) {
+    extern __shared__ __align__(16) unsigned char kb_smem[];
+    __shared__ uint8_t s_queue[KB_WARPS][32 * 7];
+    __shared__ uint32_t s_msk[8];
+    Entry *s_tab = (Entry *)kb_smem;
+    uint16_t *s_disp = (uint16_t *)(s_tab + a.ns);
+    uint32_t *s_filt = (uint32_t *)(kb_smem + sizeof(Entry) * a.ns + kb_disp_bytes(a.nb));
+    uint32_t *s_cnt = s_filt + 3 * KB_FILTER_WORDS;
+    const unsigned lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const unsigned lt = (1u << lane) - 1u;
+    for (uint32_t i = threadIdx.x; i < a.ns; i += KB_THREADS) s_tab[i] = a.table[i];
+    for (uint32_t i = threadIdx.x; i < a.nb; i += KB_THREADS) s_disp[i] = a.disp[i];
+    for (uint32_t i = threadIdx.x; i < 3 * KB_FILTER_WORDS; i += KB_THREADS) s_filt[i] = a.filter[i];
+    if (threadIdx.x < 8) s_msk[threadIdx.x] = a.hp.msk[threadIdx.x];
+    const int64_t gw = (int64_t)blockIdx.x * KB_WARPS + warp;
+    uint32_t *cnt = s_cnt + warp * a.kids;
+    uint32_t *row = a.counts + gw * a.kids;
+    for (int k = lane; k < a.kids; k += 32)
+        cnt[k] = WRITE ? row[k] + (a.abs32 ? (uint32_t)a.off[k] : 0u) : 0u;
+    __syncthreads();
+    uint8_t *queue = s_queue[warp];
+    const int64_t lo = gw * a.slice, hi = min(lo + a.slice, a.n);
+    for (int64_t b0 = lo; b0 < hi; b0 += 32 * UNROLL) {
+        int32_t vs[UNROLL], vp[UNROLL], vo[UNROLL];
+#pragma unroll
+        for (int u = 0; u < UNROLL; ++u) {
+            const int64_t i = b0 + u * 32 + lane;
+            const bool in = i < hi;
+            vs[u] = (U & 1) && in ? __ldcs(a.S + i) : 0;
+            vp[u] = (U & 2) && in ? __ldcs(a.P + i) : 0;
+            vo[u] = (U & 4) && in ? __ldcs(a.O + i) : 0;
+        }
+#pragma unroll
+        for (int u = 0; u < UNROLL; ++u) {
+            const int64_t i = b0 + u * 32 + lane;
+            const uint32_t v3[3] = {(uint32_t)vs[u], (uint32_t)vp[u], (uint32_t)vo[u]};
+            uint32_t e3[3] = {0u, 0u, 0u};
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                if (!(U & (1 << c))) continue;
+                const uint32_t f = kb_fentry(a.hp, c, v3[c]);
+                e3[c] = (s_filt[c * KB_FILTER_WORDS + (f >> 3)] >> ((f & 7u) * 4u)) & 0xFu;
+            }
+            const uint32_t cand = i < hi ? kb_candidates(e3[0], e3[1], e3[2]) & 0xFEu : 0u;
+            const unsigned c = __popc(cand);
+            unsigned x = c;
+#pragma unroll
+            for (int d = 1; d < 32; d <<= 1) {
+                const unsigned y = __shfl_up_sync(0xffffffffu, x, d);
+                if ((int)lane >= d) x += y;
+            }
+            const unsigned tot = __shfl_sync(0xffffffffu, x, 31);
+            if (tot == 0) continue;
+            unsigned at = x - c;
+            for (uint32_t cm = cand; cm; cm &= cm - 1) queue[at++] = (uint8_t)((lane << 3) | (__ffs(cm) - 1));
+            const uint32_t ms = (U & 1) ? kb_colmix(a.hp, 0, v3[0]) : 0u;
+            const uint32_t mp = (U & 2) ? kb_colmix(a.hp, 1, v3[1]) : 0u;
+            const uint32_t mo = (U & 4) ? kb_colmix(a.hp, 2, v3[2]) : 0u;
+            __syncwarp();
+            for (unsigned r0 = 0; r0 < tot; r0 += 32) {
+                const unsigned e = r0 + lane;
+                const unsigned qe = e < tot ? queue[e] : 0u;
+                const int src = (int)(qe >> 3), m = (int)(qe & 7u);
+                const int32_t ts = (U & 1) ? __shfl_sync(0xffffffffu, vs[u], src) : 0;
+                const int32_t tp = (U & 2) ? __shfl_sync(0xffffffffu, vp[u], src) : 0;
+                const int32_t to = (U & 4) ? __shfl_sync(0xffffffffu, vo[u], src) : 0;
+                const uint32_t hs = (U & 1) ? __shfl_sync(0xffffffffu, ms, src) : 0u;
+                const uint32_t hq = (U & 2) ? __shfl_sync(0xffffffffu, mp, src) : 0u;
+                const uint32_t ho = (U & 4) ? __shfl_sync(0xffffffffu, mo, src) : 0u;
+                int k = -1;
+                if (m != 0) {
+                    uint32_t h = s_msk[m];
+                    if (m & 1) h ^= hs;
+                    if (m & 2) h ^= kb_rotl(hq, 11);
+                    if (m & 4) h ^= kb_rotl(ho, 22);
+                    const uint32_t d = s_disp[kb_bucket(h, a.nb)];
+                    const Entry en = s_tab[kb_slot(a.hp, h, d, a.ns)];
+                    const bool hit = (en.mask_kid >> 28) == m && (!(m & 1) || en.s == ts) &&
+                                     (!(m & 2) || en.p == tp) && (!(m & 4) || en.o == to);
+                    k = hit ? (en.mask_kid & 0x0FFFFFFF) : -1;
+                }
+                if (!__any_sync(0xffffffffu, k >= 0)) continue;
+                const unsigned peers = __match_any_sync(0xffffffffu, k);
+                if (k >= 0) {
+                    const uint32_t cc = cnt[k];
+                    if (WRITE) {
+                        const uint32_t r = cc + __popc(peers & lt);
+                        a.arena[a.abs32 ? (int64_t)r : a.off[k] + r] = (int32_t)(b0 + u * 32 + src);
+                    }
+                    __syncwarp(peers);
+                    if (lane == (unsigned)(__ffs(peers) - 1)) cnt[k] = cc + __popc(peers);
+                }
+                __syncwarp();
+            }
+            __syncwarp();  // the next slot rewrites the queue
+        }
+    }
+    __syncwarp();
+    if (!WRITE)
+        for (int k = lane; k < a.kids; k += 32) row[k] = cnt[k];
+}
+
 // counts[w][k] -> exclusive prefix over w for each k; rows[k] = total of k.
 // Block: 32 key ids (lanes) x KS_PARTS ranges of warps (the block's warps: the sums
 // of a key's thousands of counts are many short chains, 512 keys 239 -> 32 us
@@ -439,8 +550,8 @@ template <int U, bool WRITE, int SH>
 void *kernel_of() {
     if (SH == SH_DIRECT) return (void *)k_batch<U, WRITE, false>;
     if (SH == SH_DIRECT_SKIP) return (void *)k_batch<U, WRITE, true>;
-    if (SH == SH_QUEUE4) return (void *)k_batch_q<U, WRITE, 4>;
-    return (void *)k_batch_q<U, WRITE, 8>;
+    if (SH == SH_QUEUE4) return (void *)k_batch_q<U, WRITE, 8>;
+    return (void *)k_batch_slot<U, WRITE, 8>;
 }
 
 // resident CTAs of both passes of a shape with `smem` bytes of dynamic shared memory
@@ -501,8 +612,6 @@ int grid_of(int U, int shape, size_t smem, unsigned *grid) { KB_DISPATCH(shape, 
 int pass_of(int U, int shape, cudaStream_t st, bool write, unsigned grid, size_t smem, const BatchArgs &a) {
     KB_DISPATCH(shape, U, run_pass, st, write, grid, smem, a)
 }
-
-int slots_of(int shape) { return shape == SH_QUEUE4 ? 4 : 8; }  // 32-triple slots per iteration
 
 using Key = std::tuple<int, int32_t, int32_t, int32_t>;  // mask, s, p, o (0 where unbound)
 
@@ -714,8 +823,8 @@ BatchArgs batch_args(const tid_store *st, const SubPlan &sp, const Uploaded &u, 
 }
 
 // triples per warp slice: the store split evenly over GW warps, in whole iterations
-int64_t slice_of(int64_t n, int64_t GW, int shape) {
-    const int64_t gran = 32 * slots_of(shape);
+int64_t slice_of(int64_t n, int64_t GW) {
+    const int64_t gran = 32 * KB_UNROLL;
     return std::max<int64_t>(gran, ceil_div(ceil_div(n, GW), gran) * gran);
 }
 
@@ -723,8 +832,8 @@ int64_t slice_of(int64_t n, int64_t GW, int shape) {
 //
 // Chooses, per (GPU, store size, masks read, log2 of the distinct keys), the
 // kernel shape (direct lookups of every present mask, with or without warp
-// skips of masks no lane may answer; or the candidate queue with 4 or 8 slots
-// in flight) and the sub-batch size (1920 keys: two CTAs per SM; 1152: three).
+// skips of masks no lane may answer; or the candidate queue, across slots or slot
+// by slot) and the sub-batch size (1920 keys: two CTAs per SM; 1152: three).
 // Each candidate's count pass is timed on a prefix of the store (2^25 triples;
 // CUDA events, best of two) with a table of the batch's first keys, and the
 // candidate with the least (sub-batches x pass time) is kept for the process.
@@ -797,7 +906,7 @@ int tune_batch(tid_ctx *ctx, const tid_store *st, const std::vector<Key> &keys, 
                 Scratch sc(ctx);
                 Uploaded up;
                 TID_TRY(upload_plan(ctx, sc, sp, GW, &up));
-                BatchArgs a = batch_args(&pre, sp, up, slice_of(pre.n, GW, shape));
+                BatchArgs a = batch_args(&pre, sp, up, slice_of(pre.n, GW));
                 float t = 1e30f;
                 for (int rep = 0; rep < 2; ++rep) {
                     TID_TRY_CUDA(cudaEventRecord(ev[0], stream), "tuner timing");
@@ -864,7 +973,7 @@ int run_batch(tid_ctx *ctx, const tid_store *st, const std::vector<SubPlan> &pla
         // the row counts live as long as the lists: both are the sets' shared block
         if ((rc = dev_alloc(ctx, &x.sb->ptr[0], sizeof(int64_t) * kids)) != TID_OK) return give_up(rc);
         if ((rc = upload_plan(ctx, s, sp, x.GW, &x.up)) != TID_OK) return give_up(rc);
-        x.a = batch_args(st, sp, x.up, slice_of(st->n, x.GW, shape));
+        x.a = batch_args(st, sp, x.up, slice_of(st->n, x.GW));
         if ((rc = pass_of(sp.U, shape, stream, false, x.grid, x.smem, x.a)) != TID_OK) return give_up(rc);
         k_batch_scan<<<(unsigned)ceil_div(kids, 32), 32 * KS_PARTS, 0, stream>>>(x.up.counts, x.GW, kids,
                                                                        (int64_t *)x.sb->ptr[0]);
