@@ -101,6 +101,12 @@ static bool drop_blocks(tid_ctx *ctx) {
     return any;
 }
 
+// True while a graph is captured from the context's stream.
+bool capturing(const tid_ctx *ctx) {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    return cudaStreamIsCapturing(ctx->stream, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone;
+}
+
 int dev_alloc(tid_ctx *ctx, void **p, size_t bytes) {
     *p = nullptr;
     const int64_t fa = ctx->fail_after.load(std::memory_order_relaxed);
@@ -108,11 +114,8 @@ int dev_alloc(tid_ctx *ctx, void **p, size_t bytes) {
         return fail(TID_ERR_OOM, "device allocation refused (injected failure)");
     if (bytes == 0) bytes = 256;
     // (a capture's allocations belong to its graph)
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     int cls = -1;
-    if (bytes <= BlockCache::MAX_BLOCK && cudaStreamIsCapturing(ctx->stream, &cap) == cudaSuccess &&
-        cap == cudaStreamCaptureStatusNone)
-        cls = block_class(&bytes);
+    if (bytes <= BlockCache::MAX_BLOCK && !capturing(ctx)) cls = block_class(&bytes);
     if (cls >= 0) {
         std::lock_guard<std::mutex> lk(ctx->blocks_mu);
         auto &f = ctx->blocks.free_blocks[cls];
@@ -218,27 +221,41 @@ static void recycle(tid_ctx *ctx, const PendingSlot &p) {
     ctx->free_slots.push_back({p.slot.slab, p.slot.index});
 }
 
-static void sweep_pending(tid_ctx *ctx, bool wait) {
+// While a graph is captured in the default (global) mode, by this thread or by
+// another, a query of an event is refused and ends that capture; in relaxed mode, the
+// calling thread's own affair, it is allowed for events recorded outside a capture.
+struct RelaxedCapture {
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+    ~RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+};
+
+// The producer is known to be done: any other answer of the query (not ready, refused,
+// a failed context) leaves the slot to it.
+static bool producer_done(cudaEvent_t ev) {
+    if (cudaEventQuery(ev) == cudaSuccess) return true;
+    cudaGetLastError();  // no failure of a later launch
+    return false;
+}
+
+static void sweep_pending(tid_ctx *ctx) {
+    RelaxedCapture mode;
     auto &pend = ctx->pending;
     size_t w = 0;
     for (size_t i = 0; i < pend.size(); ++i) {
-        cudaError_t q = wait ? cudaEventSynchronize(pend[i].ev) : cudaEventQuery(pend[i].ev);
-        if (q == cudaSuccess || q != cudaErrorNotReady) recycle(ctx, pend[i]);
+        if (producer_done(pend[i].ev)) recycle(ctx, pend[i]);
         else pend[w++] = pend[i];
     }
-    if (w) cudaGetLastError();  // "not ready" is no failure of a later launch
     pend.resize(w);
 }
 
 // The oldest pending slots whose producers are done, a few at a time (a program
 // that frees sets far ahead of the GPU has thousands pending).
 static void sweep_oldest(tid_ctx *ctx) {
+    RelaxedCapture mode;
     auto &pend = ctx->pending;
     for (int i = 0; i < 4 && !pend.empty(); ++i) {
-        if (cudaEventQuery(pend.front().ev) == cudaErrorNotReady) {
-            cudaGetLastError();  // "not ready" is no failure of a later launch
-            break;
-        }
+        if (!producer_done(pend.front().ev)) break;
         recycle(ctx, pend.front());
         pend.pop_front();
     }
@@ -247,7 +264,7 @@ static void sweep_oldest(tid_ctx *ctx) {
 static int slot_acquire(tid_ctx *ctx, Slot *s) {
     std::lock_guard<std::mutex> lk(ctx->mu);
     if (ctx->free_events.empty()) sweep_oldest(ctx);
-    if (ctx->free_slots.empty()) sweep_pending(ctx, false);
+    if (ctx->free_slots.empty()) sweep_pending(ctx);
     if (ctx->free_slots.empty()) {
         void *h = nullptr;
         TID_TRY_CUDA(cudaHostAlloc(&h, SLAB_SLOTS * sizeof(int64_t), cudaHostAllocMapped),
@@ -288,6 +305,7 @@ int set_alloc(tid_ctx *ctx, int k, const int8_t *vars, int64_t cap, tid_set **ou
     s->k = k;
     for (int c = 0; c < k; ++c) s->vars[c] = vars[c];
     s->cap = cap;
+    s->in_graph = capturing(ctx);
     const size_t colb = align_up((size_t)cap * sizeof(int32_t), 256);
     const size_t bytes = colb * (size_t)k + 256;
     int rc = dev_alloc(ctx, &s->block, bytes);
@@ -468,7 +486,8 @@ extern "C" int tid_ctx_destroy(tid_ctx *ctx) {
     cudaStreamSynchronize(ctx->stream);
     {
         std::lock_guard<std::mutex> lk(ctx->mu);
-        sweep_pending(ctx, true);
+        for (const PendingSlot &p : ctx->pending) cudaEventDestroy(p.ev);
+        ctx->pending.clear();
     }
     if (ctx->lb_status) dev_free(ctx, ctx->lb_status);
     if (ctx->sel_done) dev_free(ctx, ctx->sel_done);
@@ -727,7 +746,10 @@ void set_free(tid_set *set) {
     }
     if (set->slot.slab >= 0) {
         std::lock_guard<std::mutex> lk(ctx->mu);
-        if (set->ready) {
+        if (set->in_graph) {
+            // every run of the graph writes the slot, for as long as the program
+            // keeps the graph: it is never handed out again (nor is the event)
+        } else if (set->ready) {
             // the producer may still be writing the slot: recycle it once done
             ctx->pending.push_back({set->slot, set->ready});
             set->ready = nullptr;

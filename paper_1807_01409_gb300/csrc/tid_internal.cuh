@@ -168,6 +168,7 @@ struct tid_set {
     int64_t *d_rows = nullptr;   // device row count
     tid::Slot slot;              // host mirror of the row count
     cudaEvent_t ready = nullptr; // recorded after the producing work
+    bool in_graph = false;       // made under capture: a graph's work produces it
     int64_t rows_known = -1;
     void *block = nullptr;       // allocation holding the columns and d_rows
     tid::SharedBlock *shared = nullptr;  // or: a view into allocations shared with other sets
@@ -194,6 +195,7 @@ struct DeviceGuard {
     explicit DeviceGuard(int dev);
     ~DeviceGuard();
 };
+bool capturing(const tid_ctx *ctx);  // a graph is captured from the context's stream
 int dev_alloc(tid_ctx *ctx, void **p, size_t bytes);
 void dev_free(tid_ctx *ctx, void *p);
 int lookback_scratch(tid_ctx *ctx, unsigned int num_tiles, Lookback *lb);

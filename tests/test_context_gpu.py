@@ -1,0 +1,103 @@
+"""What a context keeps between calls, against the CPU oracle, bit-exact: searches
+captured in a CUDA graph before and beside the context's other work."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+from paper_1807_01409_gb300 import binding as tb
+
+pytestmark = pytest.mark.gpu
+
+
+class _Dev:
+    def __init__(self, ptr, n, typestr):
+        self.__cuda_array_interface__ = {"shape": (n,), "typestr": typestr, "data": (ptr, False), "version": 2}
+
+
+def _read(h):
+    """A set's rows by its device pointers (a captured set's row count is the graph's to write)."""
+    info = tb.tid_set_info(h)
+    n = int(torch.as_tensor(_Dev(info["dev_rows"], 1, "<i8"), device="cuda").item())
+    if n == 0:
+        return np.zeros((0, info["cols"]), np.int32)
+    return np.stack([torch.as_tensor(_Dev(p, n, "<i4"), device="cuda").cpu().numpy() for p in info["dev_cols"]], 1)
+
+
+def _rows(h):
+    try:
+        return tb.tid_set_to_host(h).copy()
+    finally:
+        tb.tid_set_free(h)
+
+
+class _Program:
+    """A context on a torch stream, with a store."""
+
+    def __init__(self, n=300_000, seed=3):
+        from paper_1807_01409_gb300 import build
+        build.build()
+        rng = np.random.default_rng(seed)
+        self.cols = [rng.integers(1, hi, n).astype(np.int32) for hi in (5_000, 4, 900)]
+        self.stream = torch.cuda.Stream()
+        self.ctx = tb.tid_ctx_create(0, self.stream.cuda_stream)
+        self.store = tb.tid_load(self.ctx, *self.cols)
+        tb.tid_ctx_sync(self.ctx)
+
+    def close(self):
+        torch.cuda.synchronize()
+        tb.tid_store_free(self.store)
+        tb.tid_ctx_destroy(self.ctx)
+
+    def captured(self, call):
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=self.stream):
+            out = call()
+        return g, out
+
+
+@pytest.fixture()
+def prog():
+    p = _Program()
+    yield p
+    p.close()
+
+
+def test_capture_after_sets_were_freed(prog, orc):
+    """A program that made and freed sets captures a search (sets freed but not reused yet are at hand),
+    and goes on: the graph and the context answer, and no error is left for the next context."""
+    keys = [(0, 2, 0), (17, 0, 0), (0, 1, 5)]
+    want = [orc.match(*prog.cols, k) for k in keys]
+    for k, w in zip(keys, want):
+        assert np.array_equal(_rows(tb.tid_match(prog.ctx, prog.store, k))[:, 0], w)
+    freed = [tb.tid_match(prog.ctx, prog.store, k) for k in keys * 5]
+    for h in freed:
+        tb.tid_set_free(h)
+    held = [tb.tid_match(prog.ctx, prog.store, keys[0]) for _ in range(20)]  # (no freed event left)
+    tb.tid_set_free(held.pop())
+    g, hs = prog.captured(lambda: [tb.tid_match(prog.ctx, prog.store, k) for k in keys])
+    g.replay()
+    torch.cuda.synchronize()
+    for h, w in zip(hs, want):
+        assert np.array_equal(_read(h)[:, 0], w)
+        tb.tid_set_free(h)
+    for h in held:
+        assert np.array_equal(_rows(h)[:, 0], want[0])
+    second = _Program(20_000)
+    assert np.array_equal(_rows(tb.tid_match(second.ctx, second.store, keys[0]))[:, 0], orc.match(*second.cols, keys[0]))
+    second.close()
+
+
+def test_a_captured_set_keeps_its_row_count(prog, orc):
+    """A graph writes the row counts of its sets at every run, also of those that were freed: no later
+    set may be counted where it writes."""
+    few, many = (17, 0, 0), (0, 2, 0)
+    want = orc.match(*prog.cols, few)
+    _rows(tb.tid_match(prog.ctx, prog.store, few))
+    g, _ = prog.captured(lambda: [tb.tid_set_free(tb.tid_match(prog.ctx, prog.store, many)) for _ in range(3)])
+    later = [tb.tid_match(prog.ctx, prog.store, few) for _ in range(40)]
+    tb.tid_ctx_sync(prog.ctx)
+    g.replay()
+    torch.cuda.synchronize()
+    for h in later:
+        assert np.array_equal(_rows(h)[:, 0], want)
