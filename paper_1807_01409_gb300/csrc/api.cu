@@ -163,29 +163,67 @@ void dev_free(tid_ctx *ctx, void *p) {
     cudaFreeAsync(p, ctx->stream);
 }
 
+// What a context keeps on the device between calls, neutral between launches: the
+// finished-CTA counter of the row selections, the bounds of an extraction, the
+// look-back's ticket and first status words.  One block, made with the context: an
+// allocation made while a graph is captured is the graph's, unmapped until the
+// graph runs, so it must not stay behind in the context.  (Called again by the
+// first call that needs it only if the context itself was created under capture.)
+int keep_scratch(tid_ctx *ctx) {
+    std::lock_guard<std::mutex> lk(ctx->mu);
+    if (ctx->kept) return TID_OK;
+    constexpr size_t LB_FIRST = 1024;
+    const size_t bytes = 3 * 256 + LB_FIRST * sizeof(unsigned long long);
+    void *p = nullptr;
+    TID_TRY(dev_alloc(ctx, &p, bytes));
+    cudaError_t e = cudaMemsetAsync(p, 0, bytes, ctx->stream);
+    if (e == cudaSuccess) {
+        ctx->bounds_dev = (uint32_t *)((char *)p + 256);
+        e = reset_bounds(ctx);
+    }
+    if (e != cudaSuccess) {
+        ctx->bounds_dev = nullptr;
+        dev_free(ctx, p);
+        return fail_cuda(e, "context scratch");
+    }
+    ctx->sel_done = (unsigned *)p;
+    ctx->lb_ticket = (unsigned *)((char *)p + 512);
+    ctx->lb_status = (unsigned long long *)((char *)p + 768);
+    ctx->lb_cap = LB_FIRST;
+    ctx->kept = p;
+    return TID_OK;
+}
+
 // The context's look-back scratch, grown on demand to >= `words` status words
 // (new words are zeroed, i.e. "not ready" for every epoch) plus a ticket
-// counter that is 0 between launches.
+// counter that is 0 between launches.  An array that a larger one replaces stays
+// until the context goes: launches recorded in a graph have its address.  Under
+// capture a larger array is the graph's, for this launch alone.
 int ctx_scratch(tid_ctx *ctx, size_t words, LbScratch *sc) {
+    const bool grows = words > ctx->lb_cap, in_graph = (grows || !ctx->kept) && capturing(ctx);
+    if (!ctx->kept && !in_graph) TID_TRY(keep_scratch(ctx));
+    sc->err = ctx->err_dev;
+    sc->epoch = &ctx->epoch;
     if (words > ctx->lb_cap) {
         size_t want = 1024;
         while (want < words) want *= 2;
-        if (ctx->lb_status) dev_free(ctx, ctx->lb_status);
-        ctx->lb_status = nullptr;
-        ctx->lb_cap = 0;
         void *p = nullptr;
         TID_TRY(dev_alloc(ctx, &p, want * sizeof(unsigned long long) + 256));
         TID_TRY_CUDA(cudaMemsetAsync(p, 0, want * sizeof(unsigned long long) + 256, ctx->stream),
                      "clear look-back scratch");
-        ctx->lb_status = (unsigned long long *)p;
-        ctx->lb_ticket = (unsigned int *)((char *)p + want * sizeof(unsigned long long));
+        sc->status = (unsigned long long *)p;
+        sc->ticket = (unsigned int *)((char *)p + want * sizeof(unsigned long long));
+        sc->cap = want;
+        if (in_graph) return TID_OK;
+        ctx->lb_grown[ctx->n_grown++] = p;
+        ctx->lb_status = sc->status;
+        ctx->lb_ticket = sc->ticket;
         ctx->lb_cap = want;
+        return TID_OK;
     }
     sc->status = ctx->lb_status;
     sc->cap = ctx->lb_cap;
     sc->ticket = ctx->lb_ticket;
-    sc->err = ctx->err_dev;
-    sc->epoch = &ctx->epoch;
     return TID_OK;
 }
 
@@ -458,8 +496,9 @@ extern "C" int tid_ctx_create(int device, void *cuda_stream, tid_ctx **out) {
         c->bounds_host = (uint32_t *)h + 16;  // a line of its own behind the error word
         c->bounds_map = (uint32_t *)d + 16;
     }
-    if (e != cudaSuccess) {
-        int rc = fail_cuda(e, "tid_ctx_create");
+    int rc = e == cudaSuccess ? TID_OK : fail_cuda(e, "tid_ctx_create");
+    if (rc == TID_OK && !capturing(c)) rc = keep_scratch(c);
+    if (rc != TID_OK) {
         if (c->err_host) cudaFreeHost(c->err_host);
         if (c->pool) cudaMemPoolDestroy(c->pool);
         if (c->own_stream && c->stream) cudaStreamDestroy(c->stream);
@@ -489,9 +528,8 @@ extern "C" int tid_ctx_destroy(tid_ctx *ctx) {
         for (const PendingSlot &p : ctx->pending) cudaEventDestroy(p.ev);
         ctx->pending.clear();
     }
-    if (ctx->lb_status) dev_free(ctx, ctx->lb_status);
-    if (ctx->sel_done) dev_free(ctx, ctx->sel_done);
-    if (ctx->bounds_dev) dev_free(ctx, ctx->bounds_dev);
+    dev_free(ctx, ctx->kept);
+    for (int i = 0; i < ctx->n_grown; ++i) dev_free(ctx, ctx->lb_grown[i]);
     drop_blocks(ctx);
     for (cudaEvent_t ev : ctx->free_events) cudaEventDestroy(ev);
     cudaStreamSynchronize(ctx->stream);

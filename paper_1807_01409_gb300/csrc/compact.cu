@@ -769,17 +769,7 @@ __global__ void __launch_bounds__(SC_THREADS) k_tile_sums(const uint32_t *__rest
 }  // namespace
 
 int bounds_out(tid_ctx *ctx, BoundsOut *b) {
-    if (!ctx->bounds_dev) {
-        void *p = nullptr;
-        TID_TRY(dev_alloc(ctx, &p, 256));
-        ctx->bounds_dev = (uint32_t *)p;
-        cudaError_t e = reset_bounds(ctx);
-        if (e != cudaSuccess) {
-            ctx->bounds_dev = nullptr;
-            dev_free(ctx, p);
-            return fail_cuda(e, "bounds");
-        }
-    }
+    if (!ctx->kept) TID_TRY(keep_scratch(ctx));
     b->acc = ctx->bounds_dev;
     b->done = ctx->bounds_dev + 2 * TID_MAX_COLS;
     b->host = ctx->bounds_map;
@@ -795,25 +785,28 @@ int sel_scratch(tid_ctx *ctx, int64_t n, int lists, size_t extra, SelScratch *sc
     auto pad = [](size_t b) { return (b + 255) / 256 * 256; };
     const size_t bits_b = (size_t)sc->steps * 32 * 4 * lists, cnt_b = pad((size_t)sc->steps * 4 * lists);
     const size_t off_b = pad((size_t)sc->ranges * 8 * lists), tot_b = pad((size_t)sc->ranges * 4 * lists);
-    if (!ctx->sel_done) {
-        void *d = nullptr;
-        TID_TRY(dev_alloc(ctx, &d, 256));
-        cudaError_t e = cudaMemsetAsync(d, 0, 256, ctx->stream);
-        if (e != cudaSuccess) {
-            dev_free(ctx, d);
-            return fail_cuda(e, "row selection");
-        }
-        ctx->sel_done = (unsigned *)d;
-    }
+    // a graph counts in its own word: it may run beside the context's later work
+    const bool in_graph = capturing(ctx);
+    if (!in_graph && !ctx->kept) TID_TRY(keep_scratch(ctx));
+    const size_t extra_b = pad(extra);
     void *blk = nullptr;
-    TID_TRY(dev_alloc(ctx, &blk, bits_b + cnt_b + off_b + tot_b + extra));
+    TID_TRY(dev_alloc(ctx, &blk, bits_b + cnt_b + off_b + tot_b + extra_b + (in_graph ? 256 : 0)));
     char *p = (char *)blk;
     sc->bits = (uint32_t *)p;
     sc->cnt = (uint32_t *)(p += bits_b);
     sc->off = (unsigned long long *)(p += cnt_b);
     sc->tot = (uint32_t *)(p += off_b);
-    if (extra_at) *extra_at = p + tot_b;
+    p += tot_b;
+    if (extra_at) *extra_at = p;
     sc->done = ctx->sel_done;
+    if (in_graph) {
+        sc->done = (unsigned *)(p + extra_b);
+        cudaError_t e = cudaMemsetAsync(sc->done, 0, sizeof(unsigned), ctx->stream);
+        if (e != cudaSuccess) {
+            dev_free(ctx, blk);
+            return fail_cuda(e, "row selection");
+        }
+    }
     *block = blk;
     return TID_OK;
 }

@@ -34,7 +34,8 @@ struct SelScratch {           // of one list; list j of several follows at j * (
 
 // Scratch for `lists` selections over n rows from the context's pool (*block is
 // freed by the caller; `extra` further bytes at *extra_at).  The finished-CTA
-// counter is the context's: the last CTA of a mark kernel sets it back to 0.
+// counter is the context's (under capture the graph's own): the last CTA of a mark
+// kernel sets it back to 0.
 // per: steps per range (0: chosen by n).
 int sel_scratch(tid_ctx *ctx, int64_t n, int lists, size_t extra, SelScratch *sc, void **block, void **extra_at,
                 unsigned per = 0);

@@ -117,11 +117,14 @@ struct tid_ctx {
     cudaStream_t stream = nullptr;
     bool own_stream = false;
     cudaMemPool_t pool = nullptr;
+    void *kept = nullptr;        // the block behind the scratch below (keep_scratch)
     // look-back scratch
     unsigned long long *lb_status = nullptr;
     size_t lb_cap = 0;           // status words allocated
     unsigned int *lb_ticket = nullptr;
     unsigned int epoch = 0;
+    void *lb_grown[32] = {nullptr};  // arrays allocated since, each twice the one before
+    int n_grown = 0;
     unsigned int *sel_done = nullptr;  // finished CTAs of a row selection (select.cuh), 0 between launches
     // column bounds of an extraction: a kernel's CTAs merge theirs in bounds_dev (16
     // words, neutral between launches), its last CTA moves them to mapped host memory
@@ -196,6 +199,7 @@ struct DeviceGuard {
     ~DeviceGuard();
 };
 bool capturing(const tid_ctx *ctx);  // a graph is captured from the context's stream
+int keep_scratch(tid_ctx *ctx);      // the scratch a context keeps between calls
 int dev_alloc(tid_ctx *ctx, void **p, size_t bytes);
 void dev_free(tid_ctx *ctx, void *p);
 int lookback_scratch(tid_ctx *ctx, unsigned int num_tiles, Lookback *lb);

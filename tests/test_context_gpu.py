@@ -101,3 +101,26 @@ def test_a_captured_set_keeps_its_row_count(prog, orc):
     torch.cuda.synchronize()
     for h in later:
         assert np.array_equal(_rows(h)[:, 0], want)
+
+
+def test_capture_before_any_search(prog, orc):
+    """The context's first search is captured: the context answers before the graph has run, and the
+    graph before, after and beside the context's own work, on another stream."""
+    keys = [(0, 2, 0), (17, 0, 0), (0, 1, 5)]
+    want = [orc.match(*prog.cols, k) for k in keys]
+    first = tb.tid_match(prog.ctx, prog.store, (0, 0, 0))  # (no search: every position)
+    g, hs = prog.captured(lambda: [tb.tid_match(prog.ctx, prog.store, keys[0])]
+                          + tb.tid_match_multi(prog.ctx, prog.store, keys[1:]))
+    for k, w in zip(keys, want):
+        assert np.array_equal(_rows(tb.tid_match(prog.ctx, prog.store, k))[:, 0], w), k
+    other = torch.cuda.Stream()
+    for _ in range(20):
+        with torch.cuda.stream(other):
+            g.replay()
+        for h, w in [(tb.tid_match(prog.ctx, prog.store, k), w) for k, w in zip(keys, want)]:
+            assert np.array_equal(_rows(h)[:, 0], w)
+    torch.cuda.synchronize()
+    for h, w in zip(hs, want):
+        assert np.array_equal(_read(h)[:, 0], w)
+        tb.tid_set_free(h)
+    tb.tid_set_free(first)
