@@ -22,6 +22,10 @@
  *  - Every call is ordered on the context's CUDA stream.  Calls that need a
  *    result size on the host (tid_join, tid_set_rows, tid_set_to_host, the
  *    plan executor) synchronise with that stream; the others do not.
+ *  - Calls on one context may come from several threads; what they queue is
+ *    ordered on the one stream.  A set or store is freed only when no call of
+ *    another thread is using it, and a wait that gave up is reported to the
+ *    thread that next looks.
  *  - Status: every call returns TID_OK or one of the TID_ERR_* codes below,
  *    and sets a thread-local message readable with tid_last_error().  No call
  *    aborts the process and no kernel traps: waits inside kernels give up

@@ -243,13 +243,14 @@ int make_lookback(const LbScratch &sc, unsigned int num_tiles, Lookback *lb) {
 }
 
 int lookback_scratch(tid_ctx *ctx, unsigned int num_tiles, Lookback *lb) {
+    std::lock_guard<std::mutex> lk(ctx->lb_mu);
     LbScratch sc{};
     TID_TRY(ctx_scratch(ctx, num_tiles, &sc));
     return make_lookback(sc, num_tiles, lb);
 }
 
 // ---------------------------------------------------------------------------
-// row-count slots (mapped pinned host memory)
+// row-count and bounds slots (mapped pinned host memory)
 // ---------------------------------------------------------------------------
 static constexpr int SLAB_SLOTS = 4096;
 
@@ -305,7 +306,7 @@ static int slot_acquire(tid_ctx *ctx, Slot *s) {
     if (ctx->free_slots.empty()) sweep_pending(ctx);
     if (ctx->free_slots.empty()) {
         void *h = nullptr;
-        TID_TRY_CUDA(cudaHostAlloc(&h, SLAB_SLOTS * sizeof(int64_t), cudaHostAllocMapped),
+        TID_TRY_CUDA(cudaHostAlloc(&h, SLAB_SLOTS * sizeof(SlotWords), cudaHostAllocMapped),
                      "pinned slot slab");
         void *d = nullptr;
         cudaError_t e = cudaHostGetDevicePointer(&d, h, 0);
@@ -314,17 +315,17 @@ static int slot_acquire(tid_ctx *ctx, Slot *s) {
             return fail_cuda(e, "mapped slot slab");
         }
         const int slab = (int)ctx->slabs_host.size();
-        ctx->slabs_host.push_back((int64_t *)h);
-        ctx->slabs_dev.push_back((int64_t *)d);
+        ctx->slabs_host.push_back((SlotWords *)h);
+        ctx->slabs_dev.push_back((SlotWords *)d);
         for (int i = SLAB_SLOTS - 1; i >= 0; --i) ctx->free_slots.push_back({slab, i});
     }
     auto si = ctx->free_slots.back();
     ctx->free_slots.pop_back();
     s->slab = si.first;
     s->index = si.second;
-    s->host = ctx->slabs_host[si.first] + si.second;
-    s->dev = ctx->slabs_dev[si.first] + si.second;
-    *(volatile int64_t *)s->host = -1;
+    s->words = ctx->slabs_host[si.first] + si.second;
+    s->dev = &ctx->slabs_dev[si.first][si.second].rows;
+    *(volatile int64_t *)&s->words->rows = -1;
     return TID_OK;
 }
 
@@ -493,8 +494,6 @@ extern "C" int tid_ctx_create(int device, void *cuda_stream, tid_ctx **out) {
         void *d = nullptr;
         e = cudaHostGetDevicePointer(&d, h, 0);
         c->err_dev = (int *)d;
-        c->bounds_host = (uint32_t *)h + 16;  // a line of its own behind the error word
-        c->bounds_map = (uint32_t *)d + 16;
     }
     int rc = e == cudaSuccess ? TID_OK : fail_cuda(e, "tid_ctx_create");
     if (rc == TID_OK && !capturing(c)) rc = keep_scratch(c);
@@ -701,7 +700,7 @@ int set_rows_host(tid_set *set, int64_t *rows) {
         DeviceGuard g(set->ctx->device);
         TID_TRY_CUDA(cudaEventSynchronize(set->ready), "wait for set");
         TID_TRY(check_ctx_error(set->ctx));
-        const int64_t r = *(volatile int64_t *)set->slot.host;
+        const int64_t r = *(volatile int64_t *)&set->slot.words->rows;
         if (r < 0) return fail(TID_ERR_CUDA, "row count was not produced");
         set->rows_known = r;
     }

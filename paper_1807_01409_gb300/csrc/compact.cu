@@ -21,6 +21,8 @@
 // reads the kept rows' values and writes them in order; no CTA of either waits
 // for another.
 
+#include <stddef.h>
+
 #include <algorithm>
 #include <type_traits>
 
@@ -303,7 +305,7 @@ struct PackedUniqueRow {  // sorted packed keys; keep the first of each run of e
 };
 
 // bounds (sort order) of the values a thread wrote, merged per warp into mm.acc;
-// the last CTA moves the result to the host (all threads of every CTA call this)
+// the last CTA moves the result to the set's slot (all threads of every CTA call this)
 template <int K>
 __device__ __forceinline__ void merge_bounds(const BoundsOut &mm, int k_out, const uint32_t *lo, const uint32_t *hi) {
     const unsigned lane = threadIdx.x & 31;
@@ -330,7 +332,8 @@ __device__ __forceinline__ void merge_bounds(const BoundsOut &mm, int k_out, con
     __syncthreads();
     if (!s_end) return;
     if (threadIdx.x < 2 * TID_MAX_COLS) {
-        mm.host[threadIdx.x] = __ldcg(mm.acc + threadIdx.x);
+        const unsigned c = threadIdx.x % TID_MAX_COLS;
+        if (c < BOUND_COLS) mm.host[threadIdx.x / TID_MAX_COLS * BOUND_COLS + c] = __ldcg(mm.acc + threadIdx.x);
         mm.acc[threadIdx.x] = threadIdx.x < TID_MAX_COLS ? 0xFFFFFFFFu : 0u;
     }
     if (threadIdx.x == 0) *mm.done = 0;
@@ -768,12 +771,23 @@ __global__ void __launch_bounds__(SC_THREADS) k_tile_sums(const uint32_t *__rest
 
 }  // namespace
 
-int bounds_out(tid_ctx *ctx, BoundsOut *b) {
+int bounds_out(tid_set *set, BoundsOut *b) {
+    tid_ctx *ctx = set->ctx;
+    if (set->k > BOUND_COLS) return fail(TID_ERR_ARG, "bounds of %d columns", set->k);
     if (!ctx->kept) TID_TRY(keep_scratch(ctx));
     b->acc = ctx->bounds_dev;
     b->done = ctx->bounds_dev + 2 * TID_MAX_COLS;
-    b->host = ctx->bounds_map;
+    b->host = (uint32_t *)(set->slot.dev + 1);
+    static_assert(offsetof(SlotWords, bounds) == sizeof(int64_t), "the bounds follow the row count");
     return TID_OK;
+}
+
+void read_bounds(const tid_set *set, int k, uint32_t *lo, uint32_t *hi) {
+    const volatile uint32_t *w = set->slot.words->bounds;
+    for (int c = 0; c < k; ++c) {
+        lo[c] = w[c];
+        hi[c] = w[BOUND_COLS + c];
+    }
 }
 
 int sel_scratch(tid_ctx *ctx, int64_t n, int lists, size_t extra, SelScratch *sc, void **block, void **extra_at,

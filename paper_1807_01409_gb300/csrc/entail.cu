@@ -863,7 +863,7 @@ extern "C" int tid_entail(tid_ctx *ctx, const tid_store *st, int rule, const tid
             int32_t *d_map = (int32_t *)mapb.p;
             TID_TRY_CUDA(cudaMemcpyAsync(d_map, map.data(), map.size() * 4, cudaMemcpyHostToDevice, stream), "key map");
             BoundsOut mm{};
-            if (!pair) TID_TRY(bounds_out(ctx, &mm));
+            if (!pair) TID_TRY(bounds_out(J, &mm));
             TID_TRY(expand_keyed(ctx, ks, sc, src, d_map, J, mm));
             TID_TRY_CUDA(cudaStreamSynchronize(stream), "conclusion range");  // (and the host copy of the map)
             if (pair) {  // the data term's range is known; A's terms are on the host
@@ -875,10 +875,7 @@ extern "C" int tid_entail(tid_ctx *ctx, const tid_store *st, int rule, const tid
                     cb.hi[a_pos] = std::max(cb.hi[a_pos], sort_order_host(r.second));
                 }
             } else {
-                for (int i = 0; i < kc; ++i) {
-                    cb.lo[i] = ((volatile uint32_t *)ctx->bounds_host)[i];
-                    cb.hi[i] = ((volatile uint32_t *)ctx->bounds_host)[TID_MAX_COLS + i];
-                }
+                read_bounds(J, kc, cb.lo, cb.hi);
             }
             for (int i = 0; i < kc; ++i) ccols[i] = J->col[i];
             nj = sx.res2;

@@ -108,20 +108,15 @@ int bind_set(tid_ctx *ctx, const tid_store *st, const tid_pattern &pat, const ti
     tid_set *tmp = nullptr;
     TID_TRY(set_alloc(ctx, k, vars, n, &tmp));
     BoundsOut mm{};  // column bounds of the extracted rows, for the sort
-    int rc = bounds_out(ctx, &mm);
+    int rc = bounds_out(tmp, &mm);
     if (rc == TID_OK) rc = compact_bind(ctx, st, pat, idx->col[0], n, pr, n_preds, bm, n_mem, tmp, mm);
     if (rc == TID_OK) rc = set_ready(tmp);
     int64_t m = 0;
     if (rc == TID_OK) rc = set_rows_host(tmp, &m);  // waits: the bounds are on the host too
-    uint32_t hb[2 * TID_MAX_COLS];
-    for (int c = 0; c < 2 * TID_MAX_COLS; ++c) hb[c] = ((volatile uint32_t *)ctx->bounds_host)[c];
     const int32_t *cols[TID_MAX_COLS];
     Bounds b{};
-    for (int c = 0; c < k; ++c) {
-        cols[c] = tmp->col[c];
-        b.lo[c] = hb[c];
-        b.hi[c] = hb[TID_MAX_COLS + c];
-    }
+    for (int c = 0; c < k; ++c) cols[c] = tmp->col[c];
+    read_bounds(tmp, k, b.lo, b.hi);
     // In a store sorted by (s, p, o) the hits, in index order, are sorted by
     // their variable slots in slot order (the bound slots are constant) when
     // no anonymous slot comes before a variable -- the set's canonical order.

@@ -55,20 +55,21 @@ struct Bounds {
     uint32_t lo[TID_MAX_COLS], hi[TID_MAX_COLS];
 };
 
-// Where a kernel that writes a set's rows leaves their columns' bounds (sort order):
-// word c the least, word 8 + c the largest value of column c.  Every CTA merges its
-// rows' into `acc` (least values start at ~0, largest at 0); the last one of the grid
-// moves acc to `host` (mapped memory) and makes it neutral again, so an extraction
-// needs no launch to preset its bounds and no copy to read them: they are on the host
-// with its row count.
+// Where a kernel that writes a set's rows leaves their columns' bounds (sort order;
+// at most BOUND_COLS columns).  Every CTA merges its rows' into `acc` (word c the
+// least, word 8 + c the largest value of column c; least values start at ~0, largest
+// at 0); the last one of the grid moves them to the set's slot and makes acc neutral
+// again, so an extraction needs no launch to preset its bounds and no copy to read
+// them: they are on the host with its row count, beside it, and no other extraction
+// of the context, queued by another thread meanwhile, writes there.
 struct BoundsOut {
     uint32_t *acc = nullptr;  // null: not wanted
     unsigned *done = nullptr;
     uint32_t *host = nullptr;
 };
-// the context's one; read by the caller, once the kernel's set is ready, from
-// ctx->bounds_host before the next extraction
-int bounds_out(tid_ctx *ctx, BoundsOut *b);
+int bounds_out(tid_set *set, BoundsOut *b);
+// bounds of set's columns [0, k), once the kernel that leaves them is done
+void read_bounds(const tid_set *set, int k, uint32_t *lo, uint32_t *hi);
 
 struct VarMember {  // the same by variable
     Members m;

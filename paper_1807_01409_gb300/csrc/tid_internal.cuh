@@ -73,9 +73,16 @@ constexpr unsigned LB_SPIN_LIMIT = 1u << 21;  // polls before a wait gives up
 // ---------------------------------------------------------------------------
 // objects behind the opaque handles
 // ---------------------------------------------------------------------------
-struct Slot {  // one int64 in mapped pinned host memory
-    int64_t *host = nullptr;
-    int64_t *dev = nullptr;
+// What the kernel that writes a set's rows leaves in mapped pinned host memory: their
+// number, and of an extraction the bounds of its columns (sort order).
+constexpr int BOUND_COLS = 3;
+struct SlotWords {
+    int64_t rows;
+    uint32_t bounds[2 * BOUND_COLS];  // word c the least, word BOUND_COLS + c the largest value of column c
+};
+struct Slot {
+    SlotWords *words = nullptr;
+    int64_t *dev = nullptr;  // device address of words->rows
     int slab = -1, index = -1;
 };
 
@@ -126,15 +133,15 @@ struct tid_ctx {
     void *lb_grown[32] = {nullptr};  // arrays allocated since, each twice the one before
     int n_grown = 0;
     unsigned int *sel_done = nullptr;  // finished CTAs of a row selection (select.cuh), 0 between launches
-    // column bounds of an extraction: a kernel's CTAs merge theirs in bounds_dev (16
-    // words, neutral between launches), its last CTA moves them to mapped host memory
-    uint32_t *bounds_dev = nullptr, *bounds_host = nullptr, *bounds_map = nullptr;
+    // column bounds of an extraction: a kernel's CTAs merge theirs here (16 words,
+    // neutral between launches), its last CTA moves them to the set's slot
+    uint32_t *bounds_dev = nullptr;
+    std::mutex lb_mu;            // look-back scratch and epoch
     // error word in mapped pinned memory (written by kernels, read by host)
     int *err_host = nullptr;
     int *err_dev = nullptr;
-    // mapped pinned slabs for row counts
-    std::vector<int64_t *> slabs_host;
-    std::vector<int64_t *> slabs_dev;
+    // mapped pinned slabs of slots
+    std::vector<tid::SlotWords *> slabs_host, slabs_dev;
     std::vector<std::pair<int, int>> free_slots;
     std::deque<tid::PendingSlot> pending;
     std::vector<cudaEvent_t> free_events;  // of freed sets (at most MAX_FREE_EVENTS)

@@ -1,5 +1,8 @@
 """What a context keeps between calls, against the CPU oracle, bit-exact: searches
-captured in a CUDA graph before and beside the context's other work."""
+captured in a CUDA graph before and beside the context's other work, and two
+threads on one context."""
+import threading
+
 import numpy as np
 import pytest
 
@@ -38,7 +41,9 @@ class _Program:
         from paper_1807_01409_gb300 import build
         build.build()
         rng = np.random.default_rng(seed)
-        self.cols = [rng.integers(1, hi, n).astype(np.int32) for hi in (5_000, 4, 900)]
+        t = np.unique(np.stack([rng.integers(1, hi, n) for hi in (5_000, 4, 900)], 1), axis=0)
+        t = t[rng.permutation(len(t))].astype(np.int32)
+        self.cols = [np.ascontiguousarray(t[:, c]) for c in range(3)]
         self.stream = torch.cuda.Stream()
         self.ctx = tb.tid_ctx_create(0, self.stream.cuda_stream)
         self.store = tb.tid_load(self.ctx, *self.cols)
@@ -124,3 +129,42 @@ def test_capture_before_any_search(prog, orc):
         assert np.array_equal(_read(h)[:, 0], w)
         tb.tid_set_free(h)
     tb.tid_set_free(first)
+
+
+def test_two_threads_on_one_context(orc):
+    """Extractions and joins of two threads interleave on one context: every thread gets its own column
+    bounds (values of one thread's columns lie far outside the other's) and look-back words."""
+    p = _Program(260_000, seed=8)
+    wide = [np.random.default_rng(9).permutation(np.arange(60_000, dtype=np.int32) * 35_000 + 1) for _ in range(2)]
+    other = [wide[0], np.full(60_000, 2, np.int32), wide[1]]
+    stores = [(p.store, p.cols), (tb.tid_load(p.ctx, *other), other)]
+    errors = []
+
+    def worker(store, cols):
+        try:
+            pat = tb.make_pattern(0, 2, 0, var=(0, -1, 1))
+            subj = tb.make_pattern(0, 2, 0, var=(0, -1, -1))
+            idx = orc.match(*cols, (0, 2, 0))
+            want, keys = (orc.bind(*cols, (0, 2, 0), v, idx) for v in ((0, -1, 1), (0, -1, -1)))
+            first = orc.filter(want, 0, "le", int(want.rows[len(want.rows) // 50, 0]))
+            pair = orc.join(first, keys, method="sortmerge")
+            for _ in range(40):
+                h = tb.tid_match(p.ctx, store, pat)
+                b, k = tb.tid_bind(p.ctx, store, pat, h), tb.tid_bind(p.ctx, store, subj, h)
+                f = tb.tid_filter(p.ctx, b, [(0, "le", int(want.rows[len(want.rows) // 50, 0]), 0)])
+                j = tb.tid_join(p.ctx, f, k)
+                for s, w in ((b, want), (k, keys), (f, first), (j, pair)):
+                    if not np.array_equal(_rows(s), w.rows):
+                        errors.append((len(cols[0]), w.vars, w.n))
+                tb.tid_set_free(h)
+        except Exception as e:  # reported below
+            errors.append(repr(e))
+
+    ths = [threading.Thread(target=worker, args=a) for a in stores]
+    for t in ths:
+        t.start()
+    for t in ths:
+        t.join()
+    tb.tid_store_free(stores[1][0])
+    p.close()
+    assert not errors, errors[:5]
