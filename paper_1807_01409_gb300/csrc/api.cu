@@ -75,30 +75,9 @@ DeviceGuard::~DeviceGuard() {
 // ---------------------------------------------------------------------------
 // memory
 // ---------------------------------------------------------------------------
-// Class c holds blocks of (4 + c % 4) / 4 * 256 << (c / 4) bytes.
-static size_t class_bytes(int c) { return ((size_t)64 << (c / 4)) * (4 + c % 4); }
-static int block_class(size_t *bytes) {  // *bytes is rounded up to the class
-    int c = 0;
-    while (class_bytes(c) < *bytes) ++c;
-    *bytes = class_bytes(c);
-    return c;
-}
-
 // Gives the held blocks back to the pool; false if there are none.
 static bool drop_blocks(tid_ctx *ctx) {
-    std::lock_guard<std::mutex> lk(ctx->blocks_mu);
-    BlockCache &b = ctx->blocks;
-    bool any = false;
-    for (auto &f : b.free_blocks) {
-        for (void *p : f) {
-            b.known.erase(p);
-            cudaFreeAsync(p, ctx->stream);
-            any = true;
-        }
-        f.clear();
-    }
-    b.held = 0;
-    return any;
+    return ctx->blocks.drop([&](void *p) { cudaFreeAsync(p, ctx->stream); });
 }
 
 // True while a graph is captured from the context's stream.
@@ -115,17 +94,10 @@ int dev_alloc(tid_ctx *ctx, void **p, size_t bytes) {
     if (bytes == 0) bytes = 256;
     // (a capture's allocations belong to its graph)
     int cls = -1;
-    if (bytes <= BlockCache::MAX_BLOCK && !capturing(ctx)) cls = block_class(&bytes);
-    if (cls >= 0) {
-        std::lock_guard<std::mutex> lk(ctx->blocks_mu);
-        auto &f = ctx->blocks.free_blocks[cls];
-        if (!f.empty()) {
-            *p = f.back();
-            f.pop_back();
-            ctx->blocks.known[*p].held = false;
-            ctx->blocks.held -= bytes;
-            return TID_OK;
-        }
+    if (bytes <= BlockCache::MAX_BLOCK && !capturing(ctx)) {
+        cls = BlockCache::class_of(bytes);
+        bytes = BlockCache::class_bytes(cls);
+        if ((*p = ctx->blocks.take(cls))) return TID_OK;
     }
     cudaError_t e = cudaMallocFromPoolAsync(p, bytes, ctx->pool, ctx->stream);
     if (e == cudaErrorMemoryAllocation && drop_blocks(ctx)) {
@@ -136,31 +108,17 @@ int dev_alloc(tid_ctx *ctx, void **p, size_t bytes) {
         *p = nullptr;
         return fail_cuda(e, "device allocation");
     }
-    if (cls >= 0) {
-        std::lock_guard<std::mutex> lk(ctx->blocks_mu);
-        ctx->blocks.known[*p] = {cls, false};
-    }
+    if (cls >= 0) ctx->blocks.add(*p, cls);
     return TID_OK;
 }
 
 void dev_free(tid_ctx *ctx, void *p) {
     if (!p) return;
-    {
-        std::lock_guard<std::mutex> lk(ctx->blocks_mu);
-        auto it = ctx->blocks.known.find(p);
-        if (it != ctx->blocks.known.end()) {
-            if (it->second.held) return;  // freed already: never in the list twice
-            const size_t bytes = class_bytes(it->second.cls);
-            if (ctx->blocks.held + bytes <= BlockCache::MAX_HELD) {
-                ctx->blocks.free_blocks[it->second.cls].push_back(p);
-                it->second.held = true;
-                ctx->blocks.held += bytes;
-                return;
-            }
-            ctx->blocks.known.erase(it);
-        }
+    switch (ctx->blocks.put(p)) {
+        case BlockCache::KEPT: break;
+        case BlockCache::POOL: cudaFreeAsync(p, ctx->stream); break;
+        case BlockCache::TWICE: ctx->freed_twice.store(true); break;
     }
-    cudaFreeAsync(p, ctx->stream);
 }
 
 // What a context keeps on the device between calls, neutral between launches: the
@@ -413,6 +371,7 @@ cudaError_t reset_bounds(tid_ctx *ctx) {
 }
 
 int check_ctx_error(tid_ctx *ctx) {
+    if (ctx->freed_twice.exchange(false)) return fail(TID_ERR_CUDA, "a device block was freed twice");
     int e = *(volatile int *)ctx->err_host;
     if (e != 0) {
         *(volatile int *)ctx->err_host = 0;

@@ -10,9 +10,9 @@
 #include <deque>
 #include <mutex>
 #include <string>
-#include <unordered_map>
 #include <vector>
 
+#include "blocks.cuh"
 #include "tid.h"
 
 namespace tid {
@@ -93,25 +93,6 @@ struct PendingSlot {  // a freed set's slot, reusable once its producer event co
 
 constexpr size_t MAX_FREE_EVENTS = 1024;
 
-// Device blocks a context has freed and hands out again without a driver call (a
-// plan on a small store makes some thirty small allocations per operator chain).
-// Everything a context does is ordered on its one stream, so a block may be
-// reused by the next launch.  Sizes are rounded up to a class (four per power of
-// two); larger blocks, and blocks freed while MAX_HELD bytes are held, go back to
-// the pool.  Measured on GB300, with the freed sets' events kept as well: a lookup in
-// a 1M-triple store 41.5 -> 36.0 us, eight plans on it 2.53 -> 2.38 ms.
-struct BlockCache {
-    static constexpr size_t MAX_BLOCK = (size_t)64 << 20, MAX_HELD = (size_t)256 << 20;
-    static constexpr int CLASSES = 4 * 18 + 1;  // 256 B << 18 = 64 MB
-    std::vector<void *> free_blocks[CLASSES];
-    struct Block {
-        int cls;
-        bool held;  // in free_blocks
-    };
-    std::unordered_map<void *, Block> known;  // blocks of a class, in use or held
-    size_t held = 0;
-};
-
 struct SharedBlock {  // device allocations shared by several sets (freed with the last)
     void *ptr[2] = {nullptr, nullptr};
     int refs = 0;
@@ -147,7 +128,7 @@ struct tid_ctx {
     std::vector<cudaEvent_t> free_events;  // of freed sets (at most MAX_FREE_EVENTS)
     std::mutex mu;
     tid::BlockCache blocks;
-    std::mutex blocks_mu;
+    std::atomic<bool> freed_twice{false};  // reported by the next check of the error word
     // the batched search's last plan on this context (tid_batch_tuning)
     int batch_shape = -1, batch_keys = 0, batch_subs = 0;
     // testing aid (tid_ctx_inject_alloc_failure): allocations left before they fail
