@@ -12,6 +12,7 @@
 #include <stddef.h>
 
 #include <mutex>
+#include <new>
 #include <unordered_map>
 
 namespace tid {
@@ -40,10 +41,14 @@ class BlockCache {
         return n->first;
     }
 
-    // A block from the pool, of class_bytes(cls), is in use.
-    void add(void *p, int cls) {
+    // A block from the pool, of class_bytes(cls), is in use.  Without host memory for
+    // the entry the block stays unknown and is freed to the pool.
+    void add(void *p, int cls) noexcept {
         std::lock_guard<std::mutex> lk(mu_);
-        known_[p] = Block{cls, USED, nullptr};
+        try {
+            known_[p] = Block{cls, USED, nullptr};
+        } catch (const std::bad_alloc &) {
+        }
     }
 
     // What becomes of a freed block: KEPT here; POOL, the caller's to give back; TWICE, freed

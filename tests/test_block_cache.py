@@ -1,5 +1,5 @@
 """The bookkeeping of a context's block cache (csrc/blocks.cuh), host code compiled
-with g++: classes, reuse, the limit on held bytes, and a block freed twice."""
+with g++: classes, reuse, the limit on held bytes, a block freed twice, and no host memory."""
 import os
 import subprocess
 
@@ -68,3 +68,23 @@ def test_a_block_freed_twice_is_reported(tmp_path):
     void *p = b.take(2), *q = b.take(2);
     CHECK(p && q && p != q && b.take(2) == nullptr);
     """)
+
+
+def test_no_host_memory_is_no_exception(tmp_path):
+    """Bookkeeping that finds no host memory does without: nothing is thrown through the C entries (a freed
+    block among them, also while an exception or an error path unwinds)."""
+    _run(tmp_path, r"""
+    static BlockCache b;
+    b.add(addr(0), 1);
+    refuse = true;
+    for (int i = 1; i < 1000; ++i) b.add(addr(i), 1);
+    for (int i = 1; i < 1000; ++i) CHECK(b.put(addr(i)) == BlockCache::POOL);   // unknown: the pool's
+    CHECK(b.put(addr(0)) == BlockCache::KEPT);
+    CHECK(b.take(1) == addr(0));
+    refuse = false;
+    """, head="""
+static bool refuse = false;
+void *operator new(size_t n) { if (refuse) throw std::bad_alloc(); return malloc(n); }
+void operator delete(void *p) noexcept { free(p); }
+void operator delete(void *p, size_t) noexcept { free(p); }
+""")
