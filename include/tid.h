@@ -394,7 +394,9 @@ int tid_set_to_host(tid_set *set, int32_t *buf, int64_t cap_rows, int64_t *rows_
 /* Free a set (NULL accepted).  Its memory is released stream-ordered on its
  * context's stream (work already queued there that reads it finishes first);
  * a set that views a shared allocation (tid_match_batch lists) releases it
- * with the last such set. */
+ * with the last such set.  While a CUDA graph is captured from the stream, the
+ * memory of a set made before the capture is set aside until the context is
+ * destroyed, as the graph may read it at every run. */
 int tid_set_free(tid_set *set);
 
 /* ------------------------------------------------------------------------ */

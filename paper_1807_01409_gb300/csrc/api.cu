@@ -76,8 +76,8 @@ DeviceGuard::~DeviceGuard() {
 // memory
 // ---------------------------------------------------------------------------
 // Gives the held blocks back to the pool; false if there are none.
-static bool drop_blocks(tid_ctx *ctx) {
-    return ctx->blocks.drop([&](void *p) { cudaFreeAsync(p, ctx->stream); });
+static bool drop_blocks(tid_ctx *ctx, bool all = false) {
+    return ctx->blocks.drop([&](void *p) { cudaFreeAsync(p, ctx->stream); }, all);
 }
 
 // True while a graph is captured from the context's stream.
@@ -92,9 +92,9 @@ int dev_alloc(tid_ctx *ctx, void **p, size_t bytes) {
     if (fa >= 0 && ctx->allocs.fetch_add(1, std::memory_order_relaxed) >= fa)
         return fail(TID_ERR_OOM, "device allocation refused (injected failure)");
     if (bytes == 0) bytes = 256;
-    // (a capture's allocations belong to its graph)
-    int cls = -1;
-    if (bytes <= BlockCache::MAX_BLOCK && !capturing(ctx)) {
+    const bool in_graph = capturing(ctx);  // then the allocation is the graph's
+    int cls = BlockCache::LARGE;
+    if (bytes <= BlockCache::MAX_BLOCK && !in_graph) {
         cls = BlockCache::class_of(bytes);
         bytes = BlockCache::class_bytes(cls);
         if ((*p = ctx->blocks.take(cls))) return TID_OK;
@@ -108,13 +108,13 @@ int dev_alloc(tid_ctx *ctx, void **p, size_t bytes) {
         *p = nullptr;
         return fail_cuda(e, "device allocation");
     }
-    if (cls >= 0) ctx->blocks.add(*p, cls);
+    if (!in_graph) ctx->blocks.add(*p, cls);
     return TID_OK;
 }
 
 void dev_free(tid_ctx *ctx, void *p) {
     if (!p) return;
-    switch (ctx->blocks.put(p)) {
+    switch (ctx->blocks.put(p, capturing(ctx))) {
         case BlockCache::KEPT: break;
         case BlockCache::POOL: cudaFreeAsync(p, ctx->stream); break;
         case BlockCache::TWICE: ctx->freed_twice.store(true); break;
@@ -488,7 +488,7 @@ extern "C" int tid_ctx_destroy(tid_ctx *ctx) {
     }
     dev_free(ctx, ctx->kept);
     for (int i = 0; i < ctx->n_grown; ++i) dev_free(ctx, ctx->lb_grown[i]);
-    drop_blocks(ctx);
+    drop_blocks(ctx, true);
     for (cudaEvent_t ev : ctx->free_events) cudaEventDestroy(ev);
     cudaStreamSynchronize(ctx->stream);
     for (auto *h : ctx->slabs_host) cudaFreeHost(h);

@@ -21,6 +21,7 @@ class BlockCache {
   public:
     static constexpr size_t MAX_BLOCK = (size_t)64 << 20, MAX_HELD = (size_t)256 << 20;
     static constexpr int CLASSES = 4 * 18 + 1;  // 256 B << 18 = 64 MB
+    static constexpr int LARGE = -1;
 
     // Class c holds blocks of (4 + c % 4) / 4 * 256 << (c / 4) bytes.
     static size_t class_bytes(int c) { return ((size_t)64 << (c / 4)) * (4 + c % 4); }
@@ -41,7 +42,7 @@ class BlockCache {
         return n->first;
     }
 
-    // A block from the pool, of class_bytes(cls), is in use.  Without host memory for
+    // A block from the pool, of class_bytes(cls), is in use (LARGE: above the classes).  Without host memory for
     // the entry the block stays unknown and is freed to the pool.
     void add(void *p, int cls) noexcept {
         std::lock_guard<std::mutex> lk(mu_);
@@ -53,14 +54,20 @@ class BlockCache {
 
     // What becomes of a freed block: KEPT here; POOL, the caller's to give back; TWICE, freed
     // though nobody has it (never held twice: two owners would share it).
+    // aside: freed while a graph is captured, which may read it at every run: not
+    // handed out again and not the pool's either, until the context goes.
     enum Freed { KEPT, POOL, TWICE };
-    Freed put(void *p) noexcept {  // allocates nothing: freeing cannot fail
+    Freed put(void *p, bool aside = false) noexcept {  // allocates nothing: freeing cannot fail
         std::lock_guard<std::mutex> lk(mu_);
         auto it = known_.find(p);
         if (it == known_.end()) return POOL;
         Block &b = it->second;
         if (b.state != USED) return TWICE;
-        const size_t bytes = class_bytes(b.cls);
+        if (aside) {
+            b.state = ASIDE;
+            return KEPT;
+        }
+        const size_t bytes = b.cls == LARGE ? MAX_HELD + 1 : class_bytes(b.cls);
         if (held_ + bytes > MAX_HELD) {
             known_.erase(it);
             return POOL;
@@ -72,13 +79,13 @@ class BlockCache {
         return KEPT;
     }
 
-    // Gives back(p) every held block; false if there are none.
+    // Gives back(p) every held block (all: those set aside too); false if there are none.
     template <class Back>
-    bool drop(Back back) {
+    bool drop(Back back, bool all = false) {
         std::lock_guard<std::mutex> lk(mu_);
         bool any = false;
         for (auto it = known_.begin(); it != known_.end();) {
-            if (it->second.state == HELD) {
+            if (it->second.state == HELD || (all && it->second.state == ASIDE)) {
                 back(it->first);
                 it = known_.erase(it);
                 any = true;
@@ -94,7 +101,7 @@ class BlockCache {
     size_t held() const { return held_; }
 
   private:
-    enum State { USED, HELD };
+    enum State { USED, HELD, ASIDE };
     struct Block;
     using Node = std::pair<void *const, Block>;  // an element of known_: stays where it is
     struct Block {

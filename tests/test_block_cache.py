@@ -1,5 +1,5 @@
 """The bookkeeping of a context's block cache (csrc/blocks.cuh), host code compiled
-with g++: classes, reuse, the limit on held bytes, a block freed twice, and no host memory."""
+with g++: classes, reuse, the limit on held bytes, a block freed twice, no host memory, and blocks freed while a graph is captured."""
 import os
 import subprocess
 
@@ -88,3 +88,21 @@ void *operator new(size_t n) { if (refuse) throw std::bad_alloc(); return malloc
 void operator delete(void *p) noexcept { free(p); }
 void operator delete(void *p, size_t) noexcept { free(p); }
 """)
+
+
+def test_blocks_freed_under_capture_are_set_aside(tmp_path):
+    _run(tmp_path, r"""
+    static BlockCache b;
+    b.add(addr(1), 2);
+    b.add(addr(2), 2);
+    b.add(addr(3), BlockCache::LARGE);
+    b.add(addr(4), BlockCache::LARGE);
+    CHECK(b.put(addr(1), true) == BlockCache::KEPT && b.take(2) == nullptr);
+    CHECK(b.put(addr(3), true) == BlockCache::KEPT && b.put(addr(3)) == BlockCache::TWICE);
+    CHECK(b.put(addr(9), true) == BlockCache::POOL);    // the graph's own
+    CHECK(b.put(addr(4)) == BlockCache::POOL && b.put(addr(4)) == BlockCache::POOL);
+    CHECK(b.put(addr(2)) == BlockCache::KEPT);
+    int given = 0;
+    CHECK(b.drop([&](void *) { ++given; }) && given == 1);
+    CHECK(b.drop([&](void *) { ++given; }, true) && given == 3);
+    """)

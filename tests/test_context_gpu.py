@@ -168,3 +168,26 @@ def test_two_threads_on_one_context(orc):
     tb.tid_store_free(stores[1][0])
     p.close()
     assert not errors, errors[:5]
+
+
+def test_a_set_freed_under_capture_outlives_the_graph(prog, orc):
+    """A graph that filters a set which is freed while it is captured: the set's memory is no other's,
+    however much the context allocates before the graph runs."""
+    key, pat = (0, 2, 0), tb.make_pattern(0, 2, 0, var=(0, -1, 1))
+    bound = orc.bind(*prog.cols, key, (0, -1, 1), orc.match(*prog.cols, key))
+    want = orc.filter(bound, 1, "le", 300).rows
+    idx = tb.tid_match(prog.ctx, prog.store, pat)
+    b = tb.tid_bind(prog.ctx, prog.store, pat, idx)
+    assert np.array_equal(_rows(tb.tid_filter(prog.ctx, b, [(1, "le", 300, 0)])), want)  # (its row count is known)
+
+    def call():
+        f = tb.tid_filter(prog.ctx, b, [(1, "le", 300, 0)])
+        tb.tid_set_free(b)
+        return f
+    g, f = prog.captured(call)
+    others = [tb.tid_set_from_host(prog.ctx, bound.rows + 7, (0, 1)) for _ in range(8)]
+    g.replay()
+    torch.cuda.synchronize()
+    assert np.array_equal(_read(f), want)
+    for h in others + [f, idx]:
+        tb.tid_set_free(h)
