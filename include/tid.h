@@ -324,8 +324,7 @@ int tid_join(tid_ctx *ctx, const tid_set *L, const tid_set *R, int algo, tid_set
 int tid_union(tid_ctx *ctx, const tid_set *const *in, int k, tid_set **out);
 
 /* SELECT the n_vars listed variables (in that order) with DISTINCT
- * (Section 4.3).  Output canonical.  Listing every variable of `in` only
- * reorders its columns: a set's rows stay distinct. */
+ * (Section 4.3).  Output canonical. */
 int tid_project(tid_ctx *ctx, const tid_set *in, const int8_t *vars, int n_vars, tid_set **out);
 
 /* A set from `rows` x `cols` int32 in host memory (row-major), labelled with

@@ -1,7 +1,7 @@
 // Row selection over tuple sets, and a device-wide exclusive scan.
 //
-// Three kernels serve the operators that keep a subset of rows in their
-// original order and write k output columns:
+// Serves the operators that keep a subset of rows in their original order and
+// write k output columns:
 //   * bind     -- from triple indices, the terms at a pattern's variable slots,
 //                 dropping rows whose repeated variable disagrees; the FILTER
 //                 predicates of the subquery are applied in the same pass
@@ -13,6 +13,7 @@
 //   * unique   -- after a sort, a row is kept when it differs from its
 //                 predecessor in sorted order (DISTINCT, Section 4.3), on
 //                 column rows or on packed row keys;
+//   * repeats  -- whether a sorted set repeats a row at all;
 //   * keyed    -- the rows of the entailment's keyed store pass (Section 5), which
 //                 entail.cu marks itself: expand only.
 // Short inputs: k_compact, one launch (ranks from ballots, tile offsets from
@@ -240,6 +241,74 @@ struct UniqueRow {  // rows in perm order; keep the first of each run of equal r
             if (c < k) v[c] = col[c][a];
     }
 };
+
+// Whether some row of a sorted set equals the one before it (1 or 0 as the "row
+// count" of a set): a reordering of all columns of a set whose rows are distinct
+// needs no DISTINCT.  A warp tests steps of 1024 rows, columns from the last to the
+// first, and leaves a step when no row of it can be a repeat any more: neighbours of a
+// sorted set differ in the last column, so mostly that one is read.  Bound: HBM (24M
+// rows of two columns: 23 us on GB300).
+struct SetCols {
+    const int32_t *col[TID_MAX_COLS];
+};
+constexpr int RP_THREADS = 256;
+__global__ void __launch_bounds__(RP_THREADS) k_repeats(SetCols in, int k, uint32_t n, unsigned steps, unsigned *acc,
+                                                        unsigned *done, int64_t *__restrict__ d_rows,
+                                                        int64_t *__restrict__ h_rows) {
+    const unsigned lane = threadIdx.x & 31;
+    const unsigned warps = gridDim.x * (RP_THREADS / 32);
+    unsigned found = 0;
+    for (unsigned step = blockIdx.x * (RP_THREADS / 32) + (threadIdx.x >> 5); step < steps; step += warps) {
+        const uint32_t r0 = step * SEL_STEP + lane * 4;  // < 2^32: n < 2^31
+        unsigned same[8], any = 1;
+#pragma unroll
+        for (int g = 0; g < 8; ++g) {  // rows past n, and the first row, equal no predecessor
+            const uint32_t r = r0 + g * 128;
+            same[g] = r + 4 <= n ? 0xFu : (r < n ? (1u << (n - r)) - 1u : 0u);
+            if (r == 0) same[g] &= ~1u;
+        }
+        const bool whole = (step + 1) * SEL_STEP <= n;
+#pragma unroll
+        for (int c = TID_MAX_COLS - 1; c >= 0; --c) {
+            if (c >= k || !any) continue;
+            const int32_t *p = in.col[c];
+            int4 x[8];
+            int32_t before[8];
+#pragma unroll
+            for (int g = 0; g < 8; ++g) {
+                const uint32_t r = r0 + g * 128;
+                if (whole) {
+                    x[g] = ld4(p + r);
+                } else {
+                    x[g] = make_int4(r < n ? p[r] : 0, r + 1 < n ? p[r + 1] : 0, r + 2 < n ? p[r + 2] : 0,
+                                     r + 3 < n ? p[r + 3] : 0);
+                }
+                before[g] = lane == 0 && r > 0 && r < n ? p[r - 1] : 0;
+            }
+            unsigned left = 0;
+#pragma unroll
+            for (int g = 0; g < 8; ++g) {
+                const int32_t up = __shfl_up_sync(0xffffffffu, x[g].w, 1);
+                const int32_t b = lane == 0 ? before[g] : up;
+                same[g] &= (unsigned)(x[g].x == b) | ((unsigned)(x[g].y == x[g].x) << 1) |
+                           ((unsigned)(x[g].z == x[g].y) << 2) | ((unsigned)(x[g].w == x[g].z) << 3);
+                left |= same[g];
+            }
+            any = __any_sync(0xffffffffu, left);
+        }
+        found |= any;
+    }
+    if (lane == 0 && found) atomicOr(acc, 1u);
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        if (atomicAdd(done, 1u) == gridDim.x - 1) {
+            __threadfence();
+            *d_rows = *h_rows = (int64_t)atomicExch(acc, 0u);
+            *done = 0;
+        }
+    }
+}
 
 struct KeyedRow {  // row r of a keyed pass (entail.cu marks its rows), some slots as they are,
                    // the key slot's term also through a map by key number
@@ -975,6 +1044,16 @@ int compact_unique(tid_ctx *ctx, const int32_t *const *cols, int k, const int32_
     OutCols oc{};
     for (int c = 0; c < out->k; ++c) oc.col[c] = out->col[c];
     return launch_compact(ctx, r, n, out->k, oc, out->cap, out->d_rows, out->slot.dev);
+}
+
+int find_repeats(tid_ctx *ctx, const tid_set *in, int64_t n, tid_set *flag) {
+    if (!ctx->kept) TID_TRY(keep_scratch(ctx));
+    SetCols sc{};
+    for (int c = 0; c < in->k; ++c) sc.col[c] = in->col[c];
+    const unsigned steps = (unsigned)ceil_div(n, (int64_t)SEL_STEP);
+    k_repeats<<<grid_for(steps, RP_THREADS / 32, 8), RP_THREADS, 0, ctx->stream>>>(
+        sc, in->k, (uint32_t)n, steps, ctx->sel_done + 1, ctx->sel_done, flag->d_rows, flag->slot.dev);
+    return launch_check("k_repeats");
 }
 
 int compact_unique_packed(tid_ctx *ctx, const void *keys, bool wide, int k, int64_t n, const PackSpec &ps,

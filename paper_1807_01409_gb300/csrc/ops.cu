@@ -371,6 +371,7 @@ int union_sets(tid_ctx *ctx, const tid_set *const *in, int k, tid_set **out) {
 }
 
 int project_set(tid_ctx *ctx, const tid_set *in, const int8_t *vars, int n_vars, tid_set **out) {
+    *out = nullptr;
     if (n_vars < 1 || n_vars > TID_MAX_COLS || !vars) return fail(TID_ERR_ARG, "tid_project: %d variables", n_vars);
     const int32_t *cols[TID_MAX_COLS];
     for (int i = 0; i < n_vars; ++i) {
@@ -422,8 +423,47 @@ int project_set(tid_ctx *ctx, const tid_set *in, const int8_t *vars, int n_vars,
         for (int i = 0; i < t && ok; ++i) ok = in->vars[i] == vars[n_vars - t + i];
         if (ok) tail = t;
     }
-    // keeping every column of a set leaves its rows distinct
-    return canonicalize(ctx, cols, n_vars, vars, n, n_vars < in->k, in->bounded ? &b : nullptr, out, tail);
+    // Keeping every column of a set leaves its rows distinct, and the sort needs no
+    // DISTINCT.  The rows may repeat all the same, where the store repeats triples, so a
+    // pass over the last columns looks for a repeat while the sort is queued behind it,
+    // and what it finds is dropped afterwards (24M rows of two columns, GB300: 562 us
+    // with DISTINCT, 447 with the look, 424 with neither).  Small sets drop repeats in
+    // their one launch; a graph cannot wait for the answer.
+    const bool all = n_vars == in->k, look = all && !identity && n > ONE_CTA_ROWS && !capturing(ctx);
+    tid_set *flag = nullptr;
+    int rc = TID_OK;
+    if (look) {
+        TID_TRY(set_alloc(ctx, 1, vars, 0, &flag));
+        rc = find_repeats(ctx, in, n, flag);
+        if (rc == TID_OK) rc = set_ready(flag);
+    }
+    if (rc == TID_OK)
+        rc = canonicalize(ctx, cols, n_vars, vars, n, !identity && !look, in->bounded ? &b : nullptr, out, tail);
+    int64_t repeats = 0;
+    if (rc == TID_OK && look) rc = set_rows_host(flag, &repeats);
+    set_free(flag);
+    if (rc == TID_OK && repeats) {
+        tid_set *sorted = *out, *o = nullptr;
+        rc = set_alloc(ctx, n_vars, vars, n, &o);
+        if (rc == TID_OK) rc = compact_unique(ctx, sorted->col, n_vars, nullptr, n, o);
+        if (rc == TID_OK) rc = set_ready(o);
+        if (rc == TID_OK) {
+            o->bounded = sorted->bounded;
+            for (int i = 0; i < n_vars; ++i) {
+                o->lo[i] = sorted->lo[i];
+                o->hi[i] = sorted->hi[i];
+            }
+            set_free(sorted);
+            *out = o;
+        } else if (o) {
+            set_free(o);
+        }
+    }
+    if (rc != TID_OK && *out) {
+        set_free(*out);
+        *out = nullptr;
+    }
+    return rc;
 }
 
 // Right and full outer joins (Section 4.2 lists the outer joins of the library

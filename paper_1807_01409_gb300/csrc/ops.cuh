@@ -94,6 +94,8 @@ int compact_member(tid_ctx *ctx, const tid_set *in, int64_t n, const Members &m,
 int compact_filter(tid_ctx *ctx, const tid_set *in, int64_t n, const Pred *preds, int n_preds, tid_set *out);
 int compact_unique(tid_ctx *ctx, const int32_t *const *cols, int k, const int32_t *perm, int64_t n,
                    tid_set *out);
+// flag's row count: 1 if some of the n > 0 sorted rows of `in` repeats, else 0
+int find_repeats(tid_ctx *ctx, const tid_set *in, int64_t n, tid_set *flag);
 // sorted packed keys (64-bit if wide, else 32-bit) -> distinct rows of k columns
 int compact_unique_packed(tid_ctx *ctx, const void *keys, bool wide, int k, int64_t n, const PackSpec &ps,
                           tid_set *out);
@@ -132,6 +134,9 @@ int outer_join_sets(tid_ctx *ctx, const tid_set *L, const tid_set *R, int algo, 
 // both packs into 64 bits
 int merge_unique(tid_ctx *ctx, const int32_t *const *acols, int64_t na, const int32_t *const *bcols, int64_t nb,
                  int nu, const MergePack *mp, tid_set *out);
+
+// rows that one CTA sorts (sort.cu), dropping repeats on the way
+constexpr int ONE_CTA_ROWS = 4096;
 
 // the union of at most SMALL_UNION_INPUTS sets of at most SMALL_UNION_ROWS rows in all,
 // in one launch (sort.cu): cols[i][c] column c of input i (null: absent), packed by mp

@@ -464,7 +464,7 @@ k_onesweep(const K *__restrict__ kin, const int32_t *__restrict__ vin, K *__rest
 // keys), the others exchange through shared memory.  Bound: the instructions of one SM.
 // Measured on GB300: the 20 small sets of eight plans on a 1M-triple store 245 -> 198
 // us in all, against every step in shared memory.
-constexpr int SMALL_N = 4096;
+constexpr int SMALL_N = ONE_CTA_ROWS;
 constexpr int SMALL_THREADS = 1024;
 static_assert(SMALL_UNION_ROWS <= SMALL_N, "a small union is sorted by one CTA");
 
