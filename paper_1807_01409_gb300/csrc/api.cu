@@ -500,11 +500,9 @@ extern "C" int tid_ctx_destroy(tid_ctx *ctx) {
 }
 
 namespace {
-// One CTA arrives at a barrier of two that no other CTA reaches: the library's
-// bounded wait gives up after `limit` polls and sets TID_ERR_TIMEOUT.
-__global__ void k_wait_for_nothing(unsigned *counter, int *err, unsigned limit) {
-    tid::grid_barrier(counter, 2u, err, limit);
-}
+// The second of two tiles, whose predecessor never reports: the look-back gives up
+// after `limit` polls and sets TID_ERR_TIMEOUT.
+__global__ void k_wait_for_tile(tid::Lookback lb, unsigned limit) { tid::lb_exclusive_prefix(lb, 1u, 1u, limit); }
 }  // namespace
 
 extern "C" int tid_ctx_test_bounded_wait(tid_ctx *ctx, int64_t polls) {
@@ -513,15 +511,10 @@ extern "C" int tid_ctx_test_bounded_wait(tid_ctx *ctx, int64_t polls) {
     if (polls < 1 || polls > (int64_t)LB_SPIN_LIMIT)
         return fail(TID_ERR_ARG, "tid_ctx_test_bounded_wait: polls = %lld", (long long)polls);
     DeviceGuard g(ctx->device);
-    void *counter = nullptr;
-    TID_TRY(dev_alloc(ctx, &counter, 256));
-    cudaError_t e = cudaMemsetAsync(counter, 0, sizeof(unsigned), ctx->stream);
-    if (e == cudaSuccess) {
-        k_wait_for_nothing<<<1, 32, 0, ctx->stream>>>((unsigned *)counter, ctx->err_dev, (unsigned)polls);
-        e = cudaGetLastError();
-    }
-    dev_free(ctx, counter);
-    if (e != cudaSuccess) return fail_cuda(e, "tid_ctx_test_bounded_wait");
+    Lookback lb{};
+    TID_TRY(lookback_scratch(ctx, 2, &lb));
+    k_wait_for_tile<<<1, 32, 0, ctx->stream>>>(lb, (unsigned)polls);
+    TID_TRY(launch_check("k_wait_for_tile"));
     return tid_ctx_sync(ctx);
 }
 

@@ -56,11 +56,12 @@ __device__ __forceinline__ void lb_abort(const Lookback &lb, unsigned tile) {
 // Called by all 32 lanes of ONE warp.  Publishes `total` for `tile` and
 // returns the tile's exclusive prefix (sum of the totals of tiles < tile), or
 // -1 if a wait gave up.  Each lane reads LB_DEPTH consecutive predecessors, so
-// one round trip to L2 inspects a window of 32 * LB_DEPTH tiles.
+// one round trip to L2 inspects a window of 32 * LB_DEPTH tiles.  `limit`: polls
+// before the wait gives up.
 constexpr int LB_DEPTH = 8;
 
-__device__ __forceinline__ long long lb_exclusive_prefix(const Lookback &lb, unsigned tile,
-                                                         unsigned total) {
+__device__ __forceinline__ long long lb_exclusive_prefix(const Lookback &lb, unsigned tile, unsigned total,
+                                                         unsigned limit = LB_SPIN_LIMIT) {
     const unsigned lane = threadIdx.x & 31;
     if (tile == 0) {
         if (lane == 0) lb_store(lb.status, lb_word(lb.epoch, LB_FLAG_PREFIX, total));
@@ -97,7 +98,7 @@ __device__ __forceinline__ long long lb_exclusive_prefix(const Lookback &lb, uns
         const unsigned upto = stop == 31 ? 0xffffffffu : ((2u << stop) - 1u);
         if (ab & upto) { gave_up = true; break; }
         if (nr & upto) {
-            if (++polls > LB_SPIN_LIMIT) {
+            if (++polls > limit) {
                 if (lane == 0) atomicExch(lb.err, TID_ERR_TIMEOUT);
                 gave_up = true;
                 break;
@@ -119,39 +120,6 @@ __device__ __forceinline__ long long lb_exclusive_prefix(const Lookback &lb, uns
     if (lane == 0)
         lb_store(lb.status + tile, lb_word(lb.epoch, LB_FLAG_PREFIX, (unsigned)(excl + total)));
     return excl;
-}
-
-// ---- grid barrier (cooperative launches only: every CTA is resident) --------
-
-__device__ __forceinline__ unsigned ld_acquire_u32(const unsigned *p) {
-    unsigned v;
-    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-    return v;
-}
-
-// All CTAs of a cooperative launch meet here; false if the wait gave up.
-__device__ __forceinline__ bool grid_barrier(unsigned *counter, unsigned expected, int *err,
-                                             unsigned limit = LB_SPIN_LIMIT) {
-    __shared__ int s_ok;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        __threadfence();
-        atomicAdd(counter, 1u);
-        int ok = 1;
-        unsigned polls = 0;
-        while (ld_acquire_u32(counter) < expected) {
-            if (++polls > limit) {
-                atomicExch(err, TID_ERR_TIMEOUT);
-                ok = 0;
-                break;
-            }
-            __nanosleep(100);
-        }
-        __threadfence();
-        s_ok = ok;
-    }
-    __syncthreads();
-    return s_ok != 0;
 }
 
 }  // namespace tid

@@ -191,3 +191,16 @@ def test_a_set_freed_under_capture_outlives_the_graph(prog, orc):
     assert np.array_equal(_read(f), want)
     for h in others + [f, idx]:
         tb.tid_set_free(h)
+
+
+def test_look_backs_answer_after_one_gave_up(prog, orc):
+    """The wait that is made to run out is an operator's own: it shares their status words, and a selection
+    that looks back answers right after it."""
+    rows = np.stack([np.arange(1, 8001), np.arange(8000) % 37], 1).astype(np.int32)  # four tiles
+    h = tb.tid_set_from_host(prog.ctx, rows, (0, 1))
+    want = orc.filter(orc.TupleSet((0, 1), rows), 1, "lt", 9).rows
+    for _ in range(3):
+        assert tb.tid_ctx_test_bounded_wait(prog.ctx, 50) == tb.TID_ERR_TIMEOUT
+        assert np.array_equal(_rows(tb.tid_filter(prog.ctx, h, [(1, "lt", 9, 0)])), want)
+    tb.tid_ctx_sync(prog.ctx)
+    tb.tid_set_free(h)
