@@ -208,6 +208,13 @@ int tid_batch_table_check(const tid_pattern *pats, int q, uint32_t seed, int *at
 #define TID_BATCH_QUEUE8      3
 int tid_batch_tuning(const tid_ctx *ctx, int32_t *shape, int32_t *keys_per_sub_batch, int32_t *sub_batches);
 
+/* Testing aid for tid_match_batch (the paper has no counterpart): the following
+ * calls on this context run in the kernel shape `shape` with at most `keys`
+ * (1 .. TID_BATCH_KEYS) distinct keys per sub-batch, whatever the autotuner
+ * would choose (which it leaves untouched); shape < 0 turns it off.  Results do
+ * not depend on it.  TID_ERR_ARG for an unknown shape or keys out of range. */
+int tid_ctx_test_batch_shape(tid_ctx *ctx, int32_t shape, int32_t keys);
+
 /* A variant of tid_match that allocates nothing, for callers that may not
  * allocate device memory when they scan (for example a server that gave all
  * free device memory to its own pool at start-up, or a latency-critical loop

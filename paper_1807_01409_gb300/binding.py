@@ -135,6 +135,7 @@ def lib():
         "tid_exec": (C.c_int, [_vp, _vp, C.POINTER(tid_plan_node), C.c_int, C.POINTER(_vp)]),
         "tid_plan_check": (C.c_int, [C.POINTER(tid_plan_node), C.c_int]),
         "tid_batch_tuning": (C.c_int, [_vp, C.POINTER(C.c_int32), C.POINTER(C.c_int32), C.POINTER(C.c_int32)]),
+        "tid_ctx_test_batch_shape": (C.c_int, [_vp, C.c_int32, C.c_int32]),
         "tid_batch_table_check": (C.c_int, [C.POINTER(tid_pattern), C.c_int, C.c_uint32, C.POINTER(C.c_int),
                                             C.POINTER(C.c_int)]),
         "tid_match_noalloc": (C.c_int, [C.c_int, _vp, _vp, _vp, _vp, C.c_int64, tid_pattern, _vp, C.c_int64,
@@ -370,6 +371,12 @@ def tid_batch_tuning(ctx):
     sh, keys, subs = C.c_int32(), C.c_int32(), C.c_int32()
     _check(lib().tid_batch_tuning(ctx, C.byref(sh), C.byref(keys), C.byref(subs)), "tid_batch_tuning")
     return {"shape": BATCH_SHAPES.get(sh.value, None), "keys_per_sub_batch": keys.value, "sub_batches": subs.value}
+
+
+def tid_ctx_test_batch_shape(ctx, shape, keys=TID_BATCH_KEYS):
+    """The following batches on ctx run in kernel shape `shape` (a key of BATCH_SHAPES; < 0: the autotuner's
+    choice again) with at most `keys` keys per sub-batch."""
+    _check(lib().tid_ctx_test_batch_shape(ctx, int(shape), int(keys)), "tid_ctx_test_batch_shape")
 
 
 def tid_batch_table_check(patterns, seed):

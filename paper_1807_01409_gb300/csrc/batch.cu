@@ -1065,7 +1065,9 @@ extern "C" int tid_match_batch(tid_ctx *ctx, const tid_store *st, const tid_patt
     int attempts = 0;
     Choice ch;
     bool tuned_now = false;
-    int rc = keys.empty() ? TID_OK : tune_batch(ctx, st, keys, &ch, &tuned_now);
+    int rc = TID_OK;
+    if (ctx->forced_shape >= 0) ch = Choice{ctx->forced_shape, ctx->forced_keys};
+    else if (!keys.empty()) rc = tune_batch(ctx, st, keys, &ch, &tuned_now);
     if (rc == TID_OK) rc = plan_batch(keys, ch.max_keys, KB_SEED, plans, first, &attempts);
     std::vector<tid_set *> by_kid(keys.size(), nullptr);
     if (rc == TID_OK && !plans.empty()) {
@@ -1151,6 +1153,16 @@ extern "C" int tid_batch_table_check(const tid_pattern *pats, int q, uint32_t se
     if (covered != keys.size()) return fail(TID_ERR_CAPACITY, "sub-batches hold %zu of %zu keys", covered, keys.size());
     if (attempts) *attempts = tries;
     if (sub_batches) *sub_batches = (int)plans.size();
+    return TID_OK;
+}
+
+extern "C" int tid_ctx_test_batch_shape(tid_ctx *ctx, int32_t shape, int32_t keys) {
+    clear_error();
+    if (!ctx) return fail(TID_ERR_ARG, "tid_ctx_test_batch_shape: null context");
+    if (shape >= SH_COUNT || (shape >= 0 && (keys < 1 || keys > KB_MAX_KIDS)))
+        return fail(TID_ERR_ARG, "tid_ctx_test_batch_shape: shape %d, %d keys", shape, keys);
+    ctx->forced_shape = shape < 0 ? -1 : shape;
+    ctx->forced_keys = keys;
     return TID_OK;
 }
 

@@ -131,6 +131,8 @@ struct tid_ctx {
     std::atomic<bool> freed_twice{false};  // reported by the next check of the error word
     // the batched search's last plan on this context (tid_batch_tuning)
     int batch_shape = -1, batch_keys = 0, batch_subs = 0;
+    // testing aid (tid_ctx_test_batch_shape): the shape every batch runs in, or -1
+    int forced_shape = -1, forced_keys = 0;
     // testing aid (tid_ctx_inject_alloc_failure): allocations left before they fail
     std::atomic<int64_t> fail_after{-1};
     std::atomic<int64_t> allocs{0};
