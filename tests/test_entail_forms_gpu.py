@@ -66,3 +66,30 @@ def test_a_joined_conclusion_is_sorted_once(ctx, orc):
         made[rule] = _allocations(ctx, lambda: tb.tid_set_free(tb.tid_entail(ctx, st, rule, VOCAB)[0]))
     assert made[9] <= made[7], made
     tb.tid_store_free(st)
+
+
+@pytest.mark.parametrize("keys", [16_000, 16_384, 16_385, 60_000])   # flags in shared memory up to 16384 key numbers
+@pytest.mark.parametrize("spread", [1, 30_011])                       # a range of bits; a table (32768 slots and more)
+@pytest.mark.parametrize("rule", [7, 9, 11])
+def test_many_keys(ctx, orc, keys, spread, rule):
+    """Key sets around and above what a CTA flags in shared memory, all keys or one in ten occurring."""
+    rng = np.random.default_rng([keys, spread, rule])
+    v = VOCAB
+    t, n = (np.arange(keys) + 10), 120_000
+    up = rng.permutation(t)
+    term = v["subprop"] if rule == 7 else v["subclass"]
+    schema = np.stack([t, np.full(keys, term), up], 1)
+    seen = t[::10] if keys == 60_000 else t
+    if rule == 7:
+        data = np.stack([rng.integers(10, 9_000, n), rng.choice(seen, n), rng.integers(10, 9_000, n)], 1)
+    else:
+        data = np.stack([rng.integers(10, 40_000, n), np.full(n, v["type"]), rng.choice(seen, n)], 1)
+    rows = np.concatenate([schema, data])
+    rows = np.where(rows < 10, rows, (rows - 9) * spread + 9)
+    assert rows.max() < 2**31 - 1
+    st, cols = _store(ctx, rng, rows[:keys], rows[keys:])
+    h, stats = tb.tid_entail(ctx, st, rule, v)
+    want, wstats = orc.entail(*cols, rule, v)
+    assert stats == wstats
+    assert np.array_equal(_rows(h), want.rows)
+    tb.tid_store_free(st)
