@@ -27,7 +27,10 @@ def shape(request, ctx):
     tb.tid_ctx_test_batch_shape(ctx, -1)
 
 
-def _check(ctx, orc, cols, keys, shape, per):
+_known = {}  # the oracle's lists, one set for the four shapes
+
+
+def _check(ctx, orc, cols, keys, shape, per, name):
     tb.tid_ctx_test_batch_shape(ctx, shape, per)
     st = tb.tid_load(ctx, *cols)
     hs = tb.tid_match_batch(ctx, st, keys)
@@ -38,7 +41,9 @@ def _check(ctx, orc, cols, keys, shape, per):
     for k, h in zip(keys, hs):
         got = tb.tid_set_to_host(h)[:, 0]
         tb.tid_set_free(h)
-        assert np.array_equal(got, orc.match(*cols, k)), k
+        if (name, k) not in _known:
+            _known[name, k] = orc.match(*cols, k)
+        assert np.array_equal(got, _known[name, k]), k
     tb.tid_store_free(st)
 
 
@@ -48,7 +53,7 @@ def test_every_mask(ctx, orc, shape, n):
     rng = np.random.default_rng(n)
     cols = [rng.integers(1, hi, n).astype(np.int32) for hi in (4, 3, 5)]
     keys = [(s, p, o) for s in range(5) for p in range(4) for o in range(6)]
-    _check(ctx, orc, cols, keys, shape, tb.TID_BATCH_KEYS)
+    _check(ctx, orc, cols, keys, shape, tb.TID_BATCH_KEYS, ("every", n))
 
 
 @pytest.mark.parametrize("n", [1000, 300_001, 5_000_003])
@@ -59,17 +64,17 @@ def test_few_candidates(ctx, orc, shape, n):
     rows = list(rng.integers(0, n, 40)) + [0, n - 1]
     keys = [tuple(int(c[r]) if m >> j & 1 else 0 for j, c in enumerate(cols)) for i, r in enumerate(rows)
             for m in (1, 4, 5, 3 + 3 * (i % 2), 7)]
-    _check(ctx, orc, cols, keys, shape, tb.TID_BATCH_KEYS)
+    _check(ctx, orc, cols, keys, shape, tb.TID_BATCH_KEYS, ("few", n))
 
 
 @pytest.mark.parametrize("per", [1, 100, 1152, tb.TID_BATCH_KEYS])
 def test_sub_batches(ctx, orc, shape, per):
     st = synth.tiny_store()
     rng = np.random.default_rng(per)
-    rows = rng.integers(0, st.n, min(3 * tb.TID_BATCH_KEYS, 8 * per))
+    rows = rng.integers(0, st.n, min(5 * tb.TID_BATCH_KEYS // 2, 8 * per))
     cols = (st.s, st.p, st.o)
     keys = [tuple(int(c[r]) if (1 + i % 7) >> j & 1 else 0 for j, c in enumerate(cols)) for i, r in enumerate(rows)]
-    _check(ctx, orc, cols, keys, shape, per)
+    _check(ctx, orc, cols, keys, shape, per, "tiny")
 
 
 def test_bad_shapes_are_refused(ctx):
