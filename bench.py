@@ -83,22 +83,32 @@ def _peaks():
 K1_REGION = ("// ---- k1_scan: mark and expand", "int launch_scan(")  # the kernels, their grids and launches
 
 
-def _kernel_region_sha1(kernel_src):
+CSRC = os.path.join(ROOT, "paper_1807_01409_gb300", "csrc")
+SIZING = ("int sel_scratch(", "\n}\n")  # of compact.cu: ranges, hence grids, of the search kernels
+
+
+def _kernel_region_sha1(kernel_src, csrc=CSRC):
+    """Hash of the scan's code: its section of match.cu (`kernel_src`), the device code the kernels are made of
+    (select.cuh) and the function that sizes their grids, of `csrc`."""
     src = open(kernel_src).read()
     a, b = src.index(K1_REGION[0]), src.index(K1_REGION[1])
-    return hashlib.sha1(src[a:b].encode()).hexdigest()
+    sizing = open(os.path.join(csrc, "compact.cu")).read()
+    c = sizing.index(SIZING[0])
+    h = hashlib.sha1(src[a:b].encode())
+    h.update(open(os.path.join(csrc, "select.cuh"), "rb").read())
+    h.update(sizing[c:sizing.index(SIZING[1], c)].encode())
+    return h.hexdigest()
 
 
-def _traffic_record(kernel_src):
-    """Per-launch DRAM bytes of the scan kernel from the committed ncu record,
-    valid only while the kernel's code (its device code, grid and launch) is
-    unchanged since the capture."""
+def _traffic_record(kernel_src, csrc=CSRC):
+    """DRAM bytes of the scan from the committed ncu record, valid only while the
+    kernels' code (device code, grids and launches) is unchanged since the capture."""
     p = os.path.join(ROOT, "profiles", "k1_scan_traffic.json")
     if not os.path.exists(p):
         return None
     d = json.load(open(p))
     try:
-        if d.get("kernel_region_sha1") != _kernel_region_sha1(kernel_src):
+        if d.get("kernel_region_sha1") != _kernel_region_sha1(kernel_src, csrc):
             return None
     except ValueError:  # the region markers moved: treat as changed
         return None
