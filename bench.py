@@ -613,12 +613,12 @@ def run_ours(args, rank, world, local):
             "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                          "frac": achieved / peak, "peak_kind": peak_kind,
                          "frac_of_8TBs_nominal": achieved / 8000.0,
-                         "traffic": traffic, "kernel": "k1_scan",
+                         "traffic": traffic, "kernel": "k1_mark + k1_expand",
                          "algorithmic_bytes_per_step": alg_bytes_step,
                          "avg_launch_us": total_kernel_ms * 1e3 / len(kernel_ms)},
             "e2e": {"value": e2e_value, "unit": UNIT, "h2d_bytes_per_step": h2d,
                     "d2h_bytes_per_step": d2h, "steps": e2e_steps},
-            "gpu_launches": nq * args.steps,
+            "gpu_launches": sum(2 if b else 1 for b in bound) * args.steps,  # k1_mark and k1_expand; (?,?,?) one
             "clocks": clk.summary(),
             "cpu_baseline": base,
             "rows": rows,

@@ -6,9 +6,9 @@
  * brute-force data-parallel scan (Section 3, Algorithm 1), then combines the
  * per-pattern results with union, join and filter (Section 4).  This library
  * is that hot path on one GPU: the store is resident in device memory as three
- * int32 columns (structure of arrays), patterns are matched by a single-pass
- * scan-and-compact kernel, and the results are tuple sets consumed by join,
- * union, filter and projection kernels.
+ * int32 columns (structure of arrays), patterns are matched by one read of their
+ * bound columns (a kernel that marks the hits, one that lists them), and the
+ * results are tuple sets consumed by join, union, filter and projection kernels.
  *
  * Conventions
  *  - IDs are int32 >= 1.  The value 0 in a pattern is the free variable "?"
@@ -197,15 +197,18 @@ int tid_batch_table_check(const tid_pattern *pats, int q, uint32_t seed, int *at
  * context that searched the store (the paper has no counterpart): the kernel
  * shape (TID_BATCH_DIRECT: every present mask looked up for every triple;
  * TID_BATCH_DIRECT_SKIP: the same, skipping masks no lane of a warp may answer;
- * TID_BATCH_QUEUE4 / TID_BATCH_QUEUE8: only the prefilter's candidates looked
- * up, queued across slots of 32 triples or slot by slot), the keys per sub-batch and the
- * number of sub-batches; -1, 0, 0 before any such call.  Any pointer may be
+ * TID_BATCH_QUEUE_ACROSS / TID_BATCH_QUEUE_BY_SLOT: only the prefilter's
+ * candidates looked up, queued across slots of 32 triples or slot by slot; QUEUE4
+ * and QUEUE8 are older names of the two), the keys per sub-batch and the number of
+ * sub-batches; -1, 0, 0 before any such call.  Any pointer may be
  * NULL.  The choice is timed on the first call for each (GPU, store size, masks
  * read, log2 of the distinct keys) and kept for the process. */
 #define TID_BATCH_DIRECT      0
 #define TID_BATCH_DIRECT_SKIP 1
 #define TID_BATCH_QUEUE4      2
 #define TID_BATCH_QUEUE8      3
+#define TID_BATCH_QUEUE_ACROSS  TID_BATCH_QUEUE4
+#define TID_BATCH_QUEUE_BY_SLOT TID_BATCH_QUEUE8
 int tid_batch_tuning(const tid_ctx *ctx, int32_t *shape, int32_t *keys_per_sub_batch, int32_t *sub_batches);
 
 /* Testing aid for tid_match_batch (the paper has no counterpart): the following

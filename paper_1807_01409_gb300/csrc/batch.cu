@@ -270,7 +270,7 @@ __global__ void __launch_bounds__(KB_THREADS) k_batch(BatchArgs a) {
         for (int k = lane; k < a.kids; k += 32) row[k] = cnt[k];
 }
 
-// QUEUE4 shape: only the (triple, mask) pairs the prefilter admits are looked up.
+// Queue across slots: only the (triple, mask) pairs the prefilter admits are looked up.
 // For each 32-triple slot and each mask that some lane may answer, the lanes'
 // candidates join a per-warp queue in lane order (a ballot places them), with the
 // triple's values, so for any one mask the queue is in triple order.  Whenever 32
@@ -389,7 +389,7 @@ __global__ void __launch_bounds__(KB_THREADS) k_batch_q(BatchArgs a) {
         for (int k = lane; k < a.kids; k += 32) row[k] = cnt[k];
 }
 
-// QUEUE8 shape: the same, slot by slot: lane l lists the masks its triple may answer,
+// Queue by slot: the same, slot by slot: lane l lists the masks its triple may answer,
 // an exclusive scan over the lanes' counts gives each lane its place in a queue of
 // (lane, mask) bytes, lane-major, and the queue is looked up 32 entries at a time, an
 // entry's values and mixed columns fetched from its lane by shuffle.  It costs a scan
@@ -541,8 +541,8 @@ __global__ void __launch_bounds__(32 * KS_PARTS) k_batch_scan(uint32_t *counts, 
 enum Shape {
     SH_DIRECT = TID_BATCH_DIRECT,
     SH_DIRECT_SKIP = TID_BATCH_DIRECT_SKIP,
-    SH_QUEUE4 = TID_BATCH_QUEUE4,
-    SH_QUEUE8 = TID_BATCH_QUEUE8,
+    SH_QUEUE_ACROSS = TID_BATCH_QUEUE_ACROSS,
+    SH_QUEUE_BY_SLOT = TID_BATCH_QUEUE_BY_SLOT,
     SH_COUNT = 4
 };
 
@@ -550,7 +550,7 @@ template <int U, bool WRITE, int SH>
 void *kernel_of() {
     if (SH == SH_DIRECT) return (void *)k_batch<U, WRITE, false>;
     if (SH == SH_DIRECT_SKIP) return (void *)k_batch<U, WRITE, true>;
-    if (SH == SH_QUEUE4) return (void *)k_batch_q<U, WRITE, 8>;
+    if (SH == SH_QUEUE_ACROSS) return (void *)k_batch_q<U, WRITE, 8>;
     return (void *)k_batch_slot<U, WRITE, 8>;
 }
 
@@ -603,8 +603,8 @@ int run_pass(cudaStream_t st, bool write, unsigned grid, size_t smem, const Batc
     switch (shape) {                                                               \
         case SH_DIRECT: KB_DISPATCH_U(SH_DIRECT, U, fn, __VA_ARGS__)               \
         case SH_DIRECT_SKIP: KB_DISPATCH_U(SH_DIRECT_SKIP, U, fn, __VA_ARGS__)     \
-        case SH_QUEUE4: KB_DISPATCH_U(SH_QUEUE4, U, fn, __VA_ARGS__)               \
-        default: KB_DISPATCH_U(SH_QUEUE8, U, fn, __VA_ARGS__)                      \
+        case SH_QUEUE_ACROSS: KB_DISPATCH_U(SH_QUEUE_ACROSS, U, fn, __VA_ARGS__)               \
+        default: KB_DISPATCH_U(SH_QUEUE_BY_SLOT, U, fn, __VA_ARGS__)                      \
     }
 
 int grid_of(int U, int shape, size_t smem, unsigned *grid) { KB_DISPATCH(shape, U, kb_grid, smem, grid) }
@@ -844,7 +844,7 @@ struct TuneKey {
     }
 };
 struct Choice {
-    int shape = SH_QUEUE8;
+    int shape = SH_QUEUE_BY_SLOT;
     int max_keys = KB_MAX_KIDS;
 };
 std::mutex g_tune_mu;

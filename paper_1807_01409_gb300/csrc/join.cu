@@ -9,9 +9,10 @@
 // Both algorithms follow the same three phases (the two-phase output sizing
 // of He et al. that the paper cites): count matches per row, exclusive-scan
 // the counts (one synchronisation reads the total to size the output), then
-// write every output row with one thread -- an output row finds its left row
-// by binary search over the scanned counts, so a key with millions of matches
-// is spread over as many threads (no per-row serial loops).
+// write every output row with one thread -- the output is cut into tiles of equal
+// work, and within a tile a running maximum over the rows' first output rows gives
+// every output row its left row -- so a key with millions of matches is spread
+// over as many threads (no per-row serial loops).
 //
 //  * runs: the right side leads with the key columns, so a key's rows are one run
 //    of it, ordered by its other columns; each left row, whatever its order by
@@ -139,9 +140,6 @@ __device__ __forceinline__ void warp_bracket(const Cols &RK, const Cols &LK, int
     *b0 = __shfl_sync(0xffffffffu, hi, 31);
 }
 
-
-
-// per left row: [lo, hi) of equal keys in the sorted right keys
 constexpr uint32_t NO_MATCH = 0xFFFFFFFFu;  // left outer join: a left row written once, padded
 
 // Where the right rows of a first-key term lie: bucket (order(term) - lo) >> shift

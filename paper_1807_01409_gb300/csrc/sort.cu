@@ -5,8 +5,9 @@
 // When the columns' value ranges fit 64 bits together (the usual case: entity
 // IDs need ~23 bits), each row is packed into one 32- or 64-bit key -- column
 // 0 most significant, each field rebased to (x - min) and as wide as
-// (max - min) needs -- and the keys alone are radix sorted, then unpacked (and
-// adjacent duplicates dropped) in one streaming pass.  Otherwise a row
+// (max - min) needs -- and the keys alone are radix sorted; the last digit pass
+// unpacks them into the result's columns, or (rows that may repeat) a row selection
+// over the sorted keys drops the repeats and unpacks the rest.  Otherwise a row
 // permutation is sorted: for each key column from the last to the first, the
 // (key, row) pairs are radix sorted stably, so the final permutation orders
 // rows lexicographically; again only the bits that vary are sorted.
@@ -14,7 +15,7 @@
 // One digit pass = per-tile histograms (k_tile_hist) + a scan of each digit's
 // tile counts (k_digit_scan, one CTA per digit) + one ranking-and-scatter
 // launch (k_onesweep): tiles of 4096
-// keys rank stably (the lanes of a warp with equal digits found by a match
+// keys (3072 for most 64-bit sorts) rank stably (the lanes of a warp with equal digits found by a match
 // instruction or by eight ballots, alternately, the first lane of each group
 // adding its size to a shared counter)
 // and scatter through shared memory so runs of equal digits are written
@@ -32,9 +33,10 @@
 // the distinct pass that a permutation of columns does not need; the sort of a
 // bind's 11.8M rows, four 32-bit passes, 370 -> 300 us.
 //
-// Sets of at most 4096 packed rows skip the passes: one CTA loads the keys into
-// shared memory, bitonic-sorts them, flags and block-scans the distinct ones
-// and unpacks them -- one launch, as the many small sets of a plan need.
+// Sets of at most 4096 packed rows skip the passes: one CTA keeps the keys in
+// registers, bitonic-sorts them (steps within a warp without shared memory), flags
+// and block-scans the distinct ones and unpacks them -- one launch, as the many
+// small sets of a plan need.
 
 #include <algorithm>
 
