@@ -1055,7 +1055,7 @@ extern "C" int tid_match_batch(tid_ctx *ctx, const tid_store *st, const tid_patt
     for (int i = 0; i < q; ++i)
         if (pats[i].s < 0 || pats[i].p < 0 || pats[i].o < 0)
             return fail(TID_ERR_ID, "tid_match_batch: negative ID in pattern %d", i);
-    DeviceGuard g(ctx->device);
+    CallGuard g(ctx);
     // distinct (mask, key) -> key id; (?,?,?) and an empty store go through tid_match
     std::vector<Key> keys;
     std::vector<int> kid_of;

@@ -714,7 +714,7 @@ extern "C" int tid_entail(tid_ctx *ctx, const tid_store *st, int rule, const tid
     const int32_t term[5] = {vocab->type, vocab->domain, vocab->range, vocab->sub_property_of, vocab->sub_class_of};
     for (int t = 0; t < 5; ++t)
         if (term[t] <= 0) return fail(TID_ERR_ID, "tid_entail: vocabulary ID %d is not positive", term[t]);
-    DeviceGuard g(ctx->device);
+    CallGuard g(ctx);
     cudaStream_t stream = ctx->stream;
     tid_entail_stats sx{};
     Sets hold;

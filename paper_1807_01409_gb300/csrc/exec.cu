@@ -272,6 +272,6 @@ extern "C" int tid_exec(tid_ctx *ctx, const tid_store *st, const tid_plan_node *
     *out = nullptr;
     if (st->ctx != ctx) return fail(TID_ERR_ARG, "tid_exec: store belongs to another context");
     TID_TRY(validate_plan(nodes, n_nodes));
-    DeviceGuard g(ctx->device);
+    CallGuard g(ctx);
     return exec_plan(ctx, st, nodes, n_nodes, nullptr, out);
 }

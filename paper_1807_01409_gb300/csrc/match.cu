@@ -387,7 +387,7 @@ extern "C" int tid_match(tid_ctx *ctx, const tid_store *st, tid_pattern pat, tid
     if (st->ctx != ctx) return fail(TID_ERR_ARG, "tid_match: store belongs to another context");
     if (pat.s < 0 || pat.p < 0 || pat.o < 0) return fail(TID_ERR_ID, "tid_match: negative ID in pattern");
     *out = nullptr;
-    DeviceGuard g(ctx->device);
+    CallGuard g(ctx);
     const int64_t n = st->n;
     const int8_t var = -1;
     tid_set *set = nullptr;

@@ -159,7 +159,7 @@ extern "C" int tid_match_multi(tid_ctx *ctx, const tid_store *st, const tid_patt
         if (pats[j].s < 0 || pats[j].p < 0 || pats[j].o < 0)
             return fail(TID_ERR_ID, "tid_match_multi: negative ID in pattern %d", j);
     }
-    DeviceGuard g(ctx->device);
+    CallGuard g(ctx);
     const int64_t n = st->n;
     int U = 0;
     for (int j = 0; j < m; ++j) U |= (pats[j].s != 0) | ((pats[j].p != 0) << 1) | ((pats[j].o != 0) << 2);

@@ -525,7 +525,7 @@ extern "C" int tid_bind(tid_ctx *ctx, const tid_store *st, tid_pattern pat, cons
     TID_TRY(check_set(ctx, idx, "tid_bind"));
     if (st->ctx != ctx) return fail(TID_ERR_ARG, "tid_bind: store belongs to another context");
     if (idx->k != 1 || idx->vars[0] != -1) return fail(TID_ERR_ARG, "tid_bind: idx must be an index set from tid_match");
-    DeviceGuard g(ctx->device);
+    CallGuard g(ctx);
     return bind_set(ctx, st, pat, idx, preds, n_preds, out, nullptr, 0);
 }
 
@@ -535,7 +535,7 @@ extern "C" int tid_filter(tid_ctx *ctx, const tid_set *in, const tid_pred *preds
     if (!ctx || !out) return fail(TID_ERR_ARG, "tid_filter: null argument");
     *out = nullptr;
     TID_TRY(check_set(ctx, in, "tid_filter"));
-    DeviceGuard g(ctx->device);
+    CallGuard g(ctx);
     return filter_set(ctx, in, preds, n_preds, out);
 }
 
@@ -546,7 +546,7 @@ extern "C" int tid_join(tid_ctx *ctx, const tid_set *L, const tid_set *R, int al
     *out = nullptr;
     TID_TRY(check_set(ctx, L, "tid_join"));
     TID_TRY(check_set(ctx, R, "tid_join"));
-    DeviceGuard g(ctx->device);
+    CallGuard g(ctx);
     return join_sets(ctx, L, R, algo, out);
 }
 
@@ -555,7 +555,7 @@ extern "C" int tid_union(tid_ctx *ctx, const tid_set *const *in, int k, tid_set 
     tid::Range nvtx_range("tid_union");
     if (!ctx || !out) return fail(TID_ERR_ARG, "tid_union: null argument");
     *out = nullptr;
-    DeviceGuard g(ctx->device);
+    CallGuard g(ctx);
     return union_sets(ctx, in, k, out);
 }
 
@@ -565,7 +565,7 @@ extern "C" int tid_project(tid_ctx *ctx, const tid_set *in, const int8_t *vars, 
     if (!ctx || !out) return fail(TID_ERR_ARG, "tid_project: null argument");
     *out = nullptr;
     TID_TRY(check_set(ctx, in, "tid_project"));
-    DeviceGuard g(ctx->device);
+    CallGuard g(ctx);
     return project_set(ctx, in, vars, n_vars, out);
 }
 
@@ -583,7 +583,7 @@ extern "C" int tid_set_from_host(tid_ctx *ctx, const int32_t *buf, int64_t rows,
         for (int d = 0; d < c; ++d)
             if (vars[d] == vars[c]) return fail(TID_ERR_ARG, "tid_set_from_host: variable %d twice", vars[c]);
     }
-    DeviceGuard g(ctx->device);
+    CallGuard g(ctx);
     if (rows == 0) return empty_set(ctx, cols, vars, out);
     // transpose on the host, one copy per column
     std::vector<int32_t> colbuf((size_t)rows * cols);

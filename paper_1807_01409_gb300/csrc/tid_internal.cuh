@@ -127,6 +127,7 @@ struct tid_ctx {
     std::deque<tid::PendingSlot> pending;
     std::vector<cudaEvent_t> free_events;  // of freed sets (at most MAX_FREE_EVENTS)
     std::mutex mu;
+    std::atomic<bool> in_graph{false};  // a graph is captured from the stream, as the last call found it
     tid::BlockCache blocks;
     std::atomic<bool> freed_twice{false};  // reported by the next check of the error word
     // the batched search's last plan on this context (tid_batch_tuning)
@@ -188,7 +189,12 @@ struct DeviceGuard {
     explicit DeviceGuard(int dev);
     ~DeviceGuard();
 };
-bool capturing(const tid_ctx *ctx);  // a graph is captured from the context's stream
+void note_capture(tid_ctx *ctx);  // whether a graph is captured from the context's stream, for capturing()
+inline bool capturing(const tid_ctx *ctx) { return ctx->in_graph.load(std::memory_order_relaxed); }
+// At the entry of a call that allocates, frees or launches.
+struct CallGuard : DeviceGuard {
+    explicit CallGuard(tid_ctx *ctx) : DeviceGuard(ctx->device) { note_capture(ctx); }
+};
 int keep_scratch(tid_ctx *ctx);      // the scratch a context keeps between calls
 int dev_alloc(tid_ctx *ctx, void **p, size_t bytes);
 void dev_free(tid_ctx *ctx, void *p);
