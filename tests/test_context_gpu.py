@@ -204,3 +204,38 @@ def test_look_backs_answer_after_one_gave_up(prog, orc):
         assert np.array_equal(_rows(tb.tid_filter(prog.ctx, h, [(1, "lt", 9, 0)])), want)
     tb.tid_ctx_sync(prog.ctx)
     tb.tid_set_free(h)
+
+
+def test_captured_operators(prog, orc):
+    """Operators that need no row count from the device, captured on long and short sets: FILTER, SELECT
+    DISTINCT (a prefix, and columns reordered), a join with keys and a union; run twice."""
+    key, pat = (0, 2, 0), tb.make_pattern(0, 2, 0, var=(0, -1, 1))
+    big = orc.bind(*prog.cols, key, (0, -1, 1), orc.match(*prog.cols, key))
+    small = orc.TupleSet((0, 1), big.rows[:900])
+    keys = orc.TupleSet((0,), np.unique(big.rows[::50, :1], axis=0))
+    hb, hs, hk = (tb.tid_set_from_host(prog.ctx, s.rows, s.vars) for s in (big, small, keys))
+    tb.tid_ctx_sync(prog.ctx)
+    for h in (hb, hs, hk):
+        tb.tid_set_rows(h)
+
+    def call():
+        out = []
+        for h in (hb, hs):
+            out += [tb.tid_filter(prog.ctx, h, [(1, "le", 300, 0)]), tb.tid_project(prog.ctx, h, (0,)),
+                    tb.tid_project(prog.ctx, h, (1, 0)), tb.tid_join(prog.ctx, hk, h), tb.tid_union(prog.ctx, [h, hs])]
+        return out
+    want = []
+    for s in (big, small):
+        want += [orc.filter(s, 1, "le", 300), orc.project(s, (0,)), orc.project(s, (1, 0)),
+                 orc.join(keys, s, method="sortmerge"), orc.union([s, small])]
+    for h, w in zip(call(), want):
+        assert np.array_equal(_rows(h), w.rows)
+    g, out = prog.captured(call)
+    assert np.array_equal(_rows(tb.tid_match(prog.ctx, prog.store, pat))[:, 0], orc.match(*prog.cols, key))
+    for _ in range(2):
+        g.replay()
+        torch.cuda.synchronize()
+        for h, w in zip(out, want):
+            assert np.array_equal(_read(h), w.rows)
+    for h in out + [hb, hs, hk]:
+        tb.tid_set_free(h)
